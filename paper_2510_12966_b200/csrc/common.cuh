@@ -117,6 +117,16 @@ template <> struct Elem<__nv_bfloat16> {
   }
 };
 
+// the inverse of unpack, for values that came from logits of the type
+template <typename T>
+__device__ __forceinline__ uint4 pack_vector(const float* x) {
+  if (sizeof(T) == 4) return make_uint4(__float_as_uint(x[0]), __float_as_uint(x[1]), __float_as_uint(x[2]), __float_as_uint(x[3]));
+  unsigned w[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) w[j] = (__float_as_uint(x[2 * j]) >> 16) | (__float_as_uint(x[2 * j + 1]) & 0xffff0000u);
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
 __device__ __forceinline__ uint4 ldg_vec(const void* base, long long vec_index) {
   return __ldg(reinterpret_cast<const uint4*>(base) + vec_index);
 }

@@ -219,7 +219,8 @@ int launch_rowstats(const StageParams& P, int dtype, int variant, int cluster_si
   bool use_cluster = false;
   psd::ClusterGeom geom{};
   if (variant != PSD_KERNEL_BASELINE) {
-    use_cluster = psd::cluster_geometry(P, dtype, cluster_size, variant == PSD_KERNEL_CLUSTER_STREAMED, allow_triples, &geom);
+    use_cluster = psd::cluster_geometry(P, dtype, cluster_size, variant == PSD_KERNEL_CLUSTER_STREAMED, allow_triples,
+                                        variant == PSD_KERNEL_AUTO, &geom);
     if (!use_cluster && variant != PSD_KERNEL_AUTO) return PSD_ERR_UNSUPPORTED;
   }
   TimedLaunch timed(stream, 0);
@@ -608,7 +609,7 @@ int verify_two_stage_locked(const psd_pyramid_args* a, StreamScratch* ss, int* s
       PS.seq_stride_small2 = Q.seq_stride_small; PS.seq_stride_large2 = Q.seq_stride_large;
       PS.K2 = K_q;
       psd::ClusterGeom g{};
-      if (variant != PSD_KERNEL_BASELINE && psd::cluster_geometry(PS, dtype, 0, false, false, &g)) s1.cluster_size = s2.cluster_size = g.cs;
+      if (variant != PSD_KERNEL_BASELINE && psd::cluster_geometry(PS, dtype, 0, false, false, variant == PSD_KERNEL_AUTO, &g)) s1.cluster_size = s2.cluster_size = g.cs;
       onepass = (variant == PSD_KERNEL_AUTO && psd::onepass_applies(PS, dtype, resid_any)) ? 1 : 0;
     }
     rc = run_stage_locked(&s1, ss, status, stream, window, n_window, K_q, fill_out, onepass);
@@ -1206,7 +1207,7 @@ int pyramidsd_cluster_occupancy(int B, int K, int V, psd_dtype dtype, int* out_c
   P.seq_stride_small = P.seq_stride_large = static_cast<long long>(K) * V;
   P.div_kind = PSD_DIV_JS;
   psd::ClusterGeom g{};
-  const bool ok = B > 0 && K > 0 && psd::cluster_geometry(P, dtype, 0, false, false, &g);
+  const bool ok = B > 0 && K > 0 && psd::cluster_geometry(P, dtype, 0, false, false, false, &g);
   if (out_cluster_size) *out_cluster_size = ok ? g.cs : 0;
   if (out_max_active_clusters) {
     *out_max_active_clusters = ok ? psd::cluster_max_active_any(dtype, PSD_DIV_JS, g.cs) : 0;

@@ -1,6 +1,6 @@
 // Baseline row-statistics kernel: one CTA per (sequence, position) row, three passes over global
 // memory (row maxima; sum-exps; divergence and residual mass). Works for any V, alignment and dtype;
-// the optimised cluster kernel falls back to it for shapes it does not take, and tests use it as a
+// the host takes it for vocabularies below 2048 (less than a chunk of the cluster kernel), and tests use it as a
 // second opinion on the GPU. Passes two and three mostly hit L2, but the row pair still crosses the
 // SM's load path three times.
 #pragma once

@@ -34,6 +34,14 @@
 // and normalised once -- and positions k >= K_q are ordinary pairs. A triple moves one chunk of three rows per
 // ring slot, a pair two chunks of two rows; each model's sums and each pair's terms are taken in the order of
 // the two-row form, so both forms return the same bits.
+//
+// Rows at any element boundary (template flag UA): an odd vocabulary, or a base or stride that is no multiple of 16
+// bytes. Bulk copies start at 16-byte boundaries, so a chunk is copied from the boundary at or before its first
+// logit and holds one vector fewer; each model's rows then sit at an offset of their own inside the slot. The
+// consumers take single logits (lane-consecutive, so shared memory still serves a warp in one go) instead of
+// 16-byte vectors; the rest of the pipeline is the same. What a copy reads besides the row lies in the same
+// 16-byte units as the row's first and last logit, which no page boundary cuts. It costs a load instruction per
+// logit: issue-bound, @@UA@@
 #pragma once
 
 #include <type_traits>
@@ -78,6 +86,7 @@ struct ClusterGeom {
                  // slice is streamed twice through slots of two chunks each, slots [0, ra) feed pass A and
                  // slots [ra, ring) feed pass B
   int lead;      // streamed twice: pass A hands row n to the agent once row n - lead has been released to pass B
+  int ua;        // 1: rows start at any element boundary (see the top)
   int tri;       // 1: the launch walks the two-stage wrapper's rows as triples (k < K2) and pairs, one item per stage-1 row
 };
 
@@ -324,12 +333,9 @@ __device__ __forceinline__ float lse_vector_sum(const uint4& u, float c, float r
   return v.x + v.y;
 }
 
-// the same as a packed pair of partial sums (their total is the vector sum)
-template <typename T>
-__device__ __forceinline__ float2 lse_vector_sum2(const uint4& u, float c, float ref) {
-  constexpr int N = Pairs<T>::kN;
-  float2 x[N];
-  Pairs<T>::load(u, x);
+// the same as a packed pair of partial sums (their total is the vector sum), from the vector's logits
+template <int N>
+__device__ __forceinline__ float2 lse_pairs_sum2(const float2 (&x)[N], float c, float ref) {
   const float2 cc = splat2(c), nref = splat2(-ref);
   float2 v = ex2_2(__ffma2_rn(x[0], cc, nref));
 #pragma unroll
@@ -369,15 +375,65 @@ __device__ __noinline__ float lse_slow_path(uint4 u, bool live, float c, float r
 }
 
 // Largest logit of one vector (-inf when the vector lies outside the slice), NaN ignored.
-template <typename T>
-__device__ __forceinline__ float vector_max(const uint4& u, bool live) {
-  constexpr int N = Pairs<T>::kN;
-  float2 x[N];
-  Pairs<T>::load(u, x);
+template <int N>
+__device__ __forceinline__ float pairs_max(const float2 (&x)[N], bool live) {
   float gm = fmaxf(x[0].x, x[0].y);
 #pragma unroll
   for (int j = 1; j < N; ++j) gm = fmaxf(gm, fmaxf(x[j].x, x[j].y));
   return live ? gm : -INFINITY;
+}
+
+template <typename T>
+__device__ __forceinline__ float vector_max(const uint4& u, bool live) {
+  float2 x[Pairs<T>::kN];
+  Pairs<T>::load(u, x);
+  return pairs_max(x, live);
+}
+
+// Rows at any element boundary: the N pairs of a lane's i-th group in a chunk, elements `t + 256 * j` of the chunk
+// (t: the lane's index among the 256 of the pass) in ascending j. Elements at or beyond `n`, the chunk's logits
+// inside the slice, come as -inf, which adds nothing to any sum.
+template <typename T>
+__device__ __forceinline__ float lds_logit(unsigned addr) {
+  if (sizeof(T) == 4) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
+    return v;
+  }
+  unsigned short h;
+  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(h) : "r"(addr));
+  return __uint_as_float(static_cast<unsigned>(h) << 16);
+}
+template <typename T>
+__device__ __forceinline__ void load_ragged(unsigned addr, int i, int t, int n, bool full, float2 (&x)[Pairs<T>::kN]) {
+  constexpr int E = Elem<T>::kPerVec, kLast = 16 / static_cast<int>(sizeof(T)) * 2 - 1;   // the last of a lane's elements
+  constexpr int kCap = (kClHalfBytes - 16) / static_cast<int>(sizeof(T));
+  float v[E];
+#pragma unroll
+  for (int q = 0; q < E; ++q) v[q] = lds_logit<T>(addr + static_cast<unsigned>((i * E + q) * 256 * sizeof(T)));
+  if (full) {   // only the last element of a full chunk can lie beyond it
+#pragma unroll
+    for (int q = 0; q < E; ++q)
+      if (i * E + q == kLast) v[q] = t + 256 * kLast < kCap ? v[q] : -INFINITY;
+  } else {
+#pragma unroll
+    for (int q = 0; q < E; ++q) v[q] = t + 256 * (i * E + q) < n ? v[q] : -INFINITY;
+  }
+#pragma unroll
+  for (int q = 0; q < E; q += 2) x[q / 2] = make_float2(v[q], v[q + 1]);
+}
+template <int N>
+__device__ __forceinline__ unsigned pairs_differ(const float2 (&a)[N], const float2 (&b)[N]) {
+  unsigned d = 0u;
+#pragma unroll
+  for (int j = 0; j < N; ++j)
+    d |= (__float_as_uint(a[j].x) ^ __float_as_uint(b[j].x)) | (__float_as_uint(a[j].y) ^ __float_as_uint(b[j].y));
+  return d;
+}
+template <int N>
+__device__ __forceinline__ void pairs_clamp(float2 (&x)[N], float floor_x) {
+#pragma unroll
+  for (int j = 0; j < N; ++j) x[j] = make_float2(fmaxf(x[j].x, floor_x), fmaxf(x[j].y, floor_x));
 }
 
 // Add one vector sum, taken against `ref_used`, to the state; all 32 lanes call this together. When an
@@ -494,15 +550,17 @@ __device__ __forceinline__ void release_dependent_launch() { asm volatile("gridd
 // larger than the ring (small clusters, which is what fills every SM of the device), so it is copied in
 // twice -- once for each pass, the second copy coming out of L2 -- through two rings of their own.
 // TRI (with RS only): the launch is a two-stage wrapper's, walked as row triples and pairs (see the top).
-template <typename T, int DIV, bool RS, bool TRI>
+// UA: rows start at any element boundary (see the top).
+template <typename T, int DIV, bool RS, bool TRI, bool UA>
 __global__ void __launch_bounds__(RS ? kClThreadsRS : kClThreads, 1) rowstats_cluster_kernel(const StageParams P, const ClusterGeom G) {
   static_assert(RS || !TRI, "row triples are streamed twice");
+  static_assert(kClAVec * Elem<T>::kPerVec * kClAWarps == kClBVec * Elem<T>::kPerVec * kClBWarps, "both passes cut a chunk alike");
   extern __shared__ unsigned char smem_raw[];
   unsigned char* ring = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
   ClusterCtl* ctl = reinterpret_cast<ClusterCtl*>(ring + static_cast<size_t>(kClSlots) * kClSlotBytes);
 
   constexpr int E = Elem<T>::kPerVec;              // logits per 16-byte vector
-  constexpr int CH = kClHalfBytes / sizeof(T);     // logits per chunk and model
+  constexpr int CH = (kClHalfBytes - (UA ? 16 : 0)) / sizeof(T);     // logits per chunk and model
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const unsigned rank = cluster_rank();
   const int cluster_id = blockIdx.x / G.cs;
@@ -566,13 +624,17 @@ __global__ void __launch_bounds__(RS ? kClThreadsRS : kClThreads, 1) rowstats_cl
                    : row_ptr<T>(P.large, P.seq_stride_large, w.r, K, V)) + slice_begin;
   };
 
+  // UA: bytes between the 16-byte boundary a row's copies start from and its first logit; the same for every chunk
+  auto lead_bytes = [](const T* p) { return static_cast<unsigned>(reinterpret_cast<uintptr_t>(p) & 15u); };
+
   if (warp < kClConsumerWarps) {
     const float c = P.c;
     const bool is_a = warp < kClAWarps;
     const int pw = is_a ? warp : warp - kClAWarps;    // index among the warps of this pass
     const int pass_warps = is_a ? kClAWarps : kClBWarps;
     // vectors pw*32 + lane + i * pass_warps * 32 of every chunk; `len[i]` > chunk offset while vector i lies inside the slice
-    const unsigned char* my = ring + (pw * 32 + lane) * 16;
+    const int t256 = pw * 32 + lane;
+    const unsigned char* my = ring + t256 * (UA ? static_cast<int>(sizeof(T)) : 16);
     constexpr int kMaxVec = kClAVec > kClBVec ? kClAVec : kClBVec;
     int len[kMaxVec];
 #pragma unroll
@@ -600,6 +662,9 @@ __global__ void __launch_bounds__(RS ? kClThreadsRS : kClThreads, 1) rowstats_cl
         float2 v[NM];
 #pragma unroll
         for (int m = 0; m < NM; ++m) { st[m].reset(); v[m] = make_float2(0.f, 0.f); }
+        unsigned lead[NM];   // UA: where the models' rows start inside a slot's parts
+#pragma unroll
+        for (int m = 0; m < NM; ++m) lead[m] = UA ? lead_bytes(model_row(w, m)) : 0u;
         const unsigned slot0 = slot;   // where the row starts in the ring
         int off = 0;   // chunk offset inside the slice, in logits
         for (int step = 0; step < steps; ++step) {
@@ -611,16 +676,27 @@ __global__ void __launch_bounds__(RS ? kClThreadsRS : kClThreads, 1) rowstats_cl
 #pragma unroll
           for (int sub = 0; sub < SUBN; ++sub, off += CH) {   // a chunk beyond the slice (odd count) has no live vector
             const unsigned char* base = sbase + sub * kClSlotBytes;
+            const int n = min(CH, slice_len - off);
             uint4 u[NM][kClAVec];
+            if (!UA) {
 #pragma unroll
-            for (int i = 0; i < kClAVec; ++i)
+              for (int i = 0; i < kClAVec; ++i)
 #pragma unroll
-              for (int m = 0; m < NM; ++m) u[m][i] = lds128(base + m * kClHalfBytes + i * kVecStride);
+                for (int m = 0; m < NM; ++m) u[m][i] = lds128(base + m * kClHalfBytes + i * kVecStride);
+            }
+            auto take = [&](int m, int i, float2 (&x)[Pairs<T>::kN]) {
+              if (UA) load_ragged<T>(smem_u32(base) + lead[m] + m * kClHalfBytes, i, t256, n, n == CH, x);
+              else Pairs<T>::load(u[m][i], x);
+            };
             if (step == 0 && sub == 0) {
               // the warp's largest logit of its first vectors (the floor keeps rows that start with -inf at 0)
               float g[NM];
 #pragma unroll
-              for (int m = 0; m < NM; ++m) g[m] = vector_max<T>(u[m][0], len[0] > 0);
+              for (int m = 0; m < NM; ++m) {
+                float2 x[Pairs<T>::kN];
+                take(m, 0, x);
+                g[m] = pairs_max(x, UA || len[0] > 0);
+              }
 #pragma unroll
               for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
@@ -628,12 +704,15 @@ __global__ void __launch_bounds__(RS ? kClThreadsRS : kClThreads, 1) rowstats_cl
 #pragma unroll
               for (int m = 0; m < NM; ++m) st[m].ref = fmaxf(g[m] * c, -1e30f);
             }
+            if (UA && n <= 0) continue;   // a chunk beyond the slice (odd count): nothing was copied
 #pragma unroll
             for (int i = 0; i < kClAVec; ++i) {
-              const bool live = len[i] > off;
+              const bool live = UA || len[i] > off;
 #pragma unroll
               for (int m = 0; m < NM; ++m) {
-                const float2 ps = lse_vector_sum2<T>(u[m][i], c, st[m].ref);
+                float2 x[Pairs<T>::kN];
+                take(m, i, x);
+                const float2 ps = lse_pairs_sum2(x, c, st[m].ref);
                 v[m] = __fadd2_rn(v[m], live ? ps : make_float2(0.f, 0.f));
               }
             }
@@ -662,11 +741,19 @@ __global__ void __launch_bounds__(RS ? kClThreadsRS : kClThreads, 1) rowstats_cl
 #pragma unroll 1
             for (int i = 0; i < kClAVec; ++i) {
               const int e = off + (pw * 32 + lane + i * kClAWarps * 32) * E;   // first logit of the vector, in the slice
-              const bool live = e < slice_len;
+              const bool live = UA || e < slice_len;
 #pragma unroll
               for (int m = 0; m < NM; ++m) {
                 uint4 v4 = make_uint4(0u, 0u, 0u, 0u);
-                if (RS) {
+                if (UA) {
+                  float z[E];
+#pragma unroll
+                  for (int q = 0; q < E; ++q) {
+                    const int idx = t256 + 256 * (i * E + q);
+                    z[q] = idx < min(CH, slice_len - off) ? Elem<T>::load(g[m], off + idx) : -INFINITY;
+                  }
+                  v4 = pack_vector<T>(z);
+                } else if (RS) {
                   if (live) v4 = *reinterpret_cast<const uint4*>(g[m] + e);
                 } else {
                   v4 = lds128(base + m * kClHalfBytes + i * kVecStride);
@@ -716,6 +803,9 @@ __global__ void __launch_bounds__(RS ? kClThreadsRS : kClThreads, 1) rowstats_cl
         const int d = w.n % kClDepth;
         wait_phase(&ctl->b_go[d], (w.n / kClDepth) & 1u);   // the row's constants are published: pass A is through
         const RowConsts rc = ctl->row_consts[d];
+        unsigned lead[NM];
+#pragma unroll
+        for (int m = 0; m < NM; ++m) lead[m] = UA ? lead_bytes(model_row(w, m)) : 0u;
         DivAcc acc, acc2;   // the pair (small, large); for a triple also the pair (large, third)
         acc.reset(); acc2.reset();
         int off = 0;
@@ -730,33 +820,51 @@ __global__ void __launch_bounds__(RS ? kClThreadsRS : kClThreads, 1) rowstats_cl
 #pragma unroll
           for (int sub = 0; sub < SUBN; ++sub, off += CH) {
             const unsigned char* base = sbase + sub * kClSlotBytes;
+            const int n = min(CH, slice_len - off);
+            if (UA && n <= 0) continue;   // a chunk beyond the slice: nothing was copied
             uint4 u[NM][kClBVec];
+            if (!UA) {
 #pragma unroll
-            for (int i = 0; i < kClBVec; ++i)
+              for (int i = 0; i < kClBVec; ++i)
 #pragma unroll
-              for (int m = 0; m < NM; ++m) u[m][i] = lds128(base + m * kClHalfBytes + i * kVecStride);
+                for (int m = 0; m < NM; ++m) u[m][i] = lds128(base + m * kClHalfBytes + i * kVecStride);
+            }
 #pragma unroll
             for (int i = 0; i < kClBVec; ++i) {
-              float2 xs[N], xl[N];
-              Pairs<T>::load_clamped(u[0][i], rc.floor_small, rc.floor2_small, xs);
-              Pairs<T>::load_clamped(u[1][i], rc.floor_large, rc.floor2_large, xl);
-              DivAcc local;
+              float2 xs[N], xl[N], xt[N];
+              DivAcc local, local2;
               local.reset();
-              local.differ = (u[0][i].x ^ u[1][i].x) | (u[0][i].y ^ u[1][i].y) | (u[0][i].z ^ u[1][i].z) | (u[0][i].w ^ u[1][i].w);
+              local2.reset();
+              if (UA) {
+                const unsigned a = smem_u32(base);
+                load_ragged<T>(a + lead[0], i, t256, n, n == CH, xs);
+                load_ragged<T>(a + lead[1] + kClHalfBytes, i, t256, n, n == CH, xl);
+                local.differ = pairs_differ(xs, xl);
+                if (NM == 3) {
+                  load_ragged<T>(a + lead[NM - 1] + 2 * kClHalfBytes, i, t256, n, n == CH, xt);
+                  local2.differ = pairs_differ(xl, xt);
+                  pairs_clamp(xt, rc.floor_third);
+                }
+                pairs_clamp(xs, rc.floor_small);
+                pairs_clamp(xl, rc.floor_large);
+              } else {
+                Pairs<T>::load_clamped(u[0][i], rc.floor_small, rc.floor2_small, xs);
+                Pairs<T>::load_clamped(u[1][i], rc.floor_large, rc.floor2_large, xl);
+                local.differ = (u[0][i].x ^ u[1][i].x) | (u[0][i].y ^ u[1][i].y) | (u[0][i].z ^ u[1][i].z) | (u[0][i].w ^ u[1][i].w);
+              }
               div_accumulate<DIV, N, PSI>(xl, xs, c, rc.off_large, rc.off_small, local);
-              const bool live = len[i] > off;   // a vector beyond the slice adds nothing
+              const bool live = UA || len[i] > off;   // a vector beyond the slice adds nothing
               if (live) {
                 acc.js = __fadd2_rn(acc.js, local.js);
                 acc.big = __fadd2_rn(acc.big, local.big);
                 acc.differ |= local.differ;
               }
               if (NM == 3) {
-                float2 xt[N];
-                Pairs<T>::load_clamped(u[NM - 1][i], rc.floor_third, rc.floor2_third, xt);
-                DivAcc local2;
-                local2.reset();
-                local2.differ = (u[1][i].x ^ u[NM - 1][i].x) | (u[1][i].y ^ u[NM - 1][i].y) | (u[1][i].z ^ u[NM - 1][i].z) |
-                                (u[1][i].w ^ u[NM - 1][i].w);
+                if (!UA) {
+                  Pairs<T>::load_clamped(u[NM - 1][i], rc.floor_third, rc.floor2_third, xt);
+                  local2.differ = (u[1][i].x ^ u[NM - 1][i].x) | (u[1][i].y ^ u[NM - 1][i].y) | (u[1][i].z ^ u[NM - 1][i].z) |
+                                  (u[1][i].w ^ u[NM - 1][i].w);
+                }
                 div_accumulate<DIV, N, PSI>(xt, xl, c, rc.off_third, rc.off_large, local2);
                 if (live) {
                   acc2.js = __fadd2_rn(acc2.js, local2.js);
@@ -809,19 +917,29 @@ __global__ void __launch_bounds__(RS ? kClThreadsRS : kClThreads, 1) rowstats_cl
       auto fill = [&](const T* const (&src)[3], int nm, int sub_n, int step, unsigned slot, unsigned fills) {
         if (fills > 0) wait_phase(&ctl->empty[slot], (fills - 1u) & 1u);
         if (dead) return false;   // the slot was never handed back: nothing more is copied into this ring
+        // bytes of model m's part of a chunk with n logits (UA: whole 16-byte units around them)
+        auto part_bytes = [&](int m, int n) {
+          const unsigned b = static_cast<unsigned>(n) * static_cast<unsigned>(sizeof(T));
+          return UA ? (lead_bytes(src[m]) + b + 15u) & ~15u : b;
+        };
         unsigned total = 0;
-        for (int sub = 0; sub < sub_n; ++sub) total += static_cast<unsigned>(max(0, min(CH, slice_len - (step * sub_n + sub) * CH)));
+        for (int sub = 0; sub < sub_n; ++sub) {
+          const int n = min(CH, slice_len - (step * sub_n + sub) * CH);
+          if (n > 0)
+            for (int m = 0; m < nm; ++m) total += part_bytes(m, n);
+        }
         if (total > 0) {
-          mbar_arrive_expect_tx(&ctl->full[slot], static_cast<unsigned>(nm) * total * static_cast<unsigned>(sizeof(T)));
+          mbar_arrive_expect_tx(&ctl->full[slot], total);
           for (int sub = 0; sub < sub_n; ++sub) {
             const int e0 = (step * sub_n + sub) * CH;
             const int n = min(CH, slice_len - e0);
             if (n > 0) {
-              const unsigned bytes = static_cast<unsigned>(n) * sizeof(T);
               unsigned char* dst = ring + static_cast<size_t>(slot) * kSlotStride + sub * kClSlotBytes;
               for (int m = 0; m < nm; ++m) {
-                if (RS) bulk_load_hint(dst + m * kClHalfBytes, src[m] + e0, bytes, &ctl->full[slot], policy);
-                else bulk_load(dst + m * kClHalfBytes, src[m] + e0, bytes, &ctl->full[slot]);
+                const unsigned bytes = part_bytes(m, n);
+                const unsigned char* from = reinterpret_cast<const unsigned char*>(src[m] + e0) - (UA ? lead_bytes(src[m]) : 0u);
+                if (RS) bulk_load_hint(dst + m * kClHalfBytes, from, bytes, &ctl->full[slot], policy);
+                else bulk_load(dst + m * kClHalfBytes, from, bytes, &ctl->full[slot]);
               }
             }
           }
@@ -1086,18 +1204,20 @@ __global__ void wait_timeout_selftest_kernel(int* status) {
 }
 
 // ---- host side --------------------------------------------------------------------------------------
-template <typename T, int DIV, bool RS, bool TRI>
+template <typename T, int DIV, bool RS, bool TRI, bool UA>
 inline cudaError_t cluster_prepare_one() {
-  cudaError_t e = cudaFuncSetAttribute(rowstats_cluster_kernel<T, DIV, RS, TRI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e = cudaFuncSetAttribute(rowstats_cluster_kernel<T, DIV, RS, TRI, UA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(kClSmemBytes));
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(rowstats_cluster_kernel<T, DIV, RS, TRI>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  return cudaFuncSetAttribute(rowstats_cluster_kernel<T, DIV, RS, TRI, UA>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
 }
 template <typename T, int DIV>
 inline cudaError_t cluster_prepare() {
-  cudaError_t e = cluster_prepare_one<T, DIV, false, false>();
-  if (e == cudaSuccess) e = cluster_prepare_one<T, DIV, true, false>();
-  if (e == cudaSuccess) e = cluster_prepare_one<T, DIV, true, true>();
+  cudaError_t e = cluster_prepare_one<T, DIV, false, false, false>();
+  if (e == cudaSuccess) e = cluster_prepare_one<T, DIV, true, false, false>();
+  if (e == cudaSuccess) e = cluster_prepare_one<T, DIV, true, true, false>();
+  if (e == cudaSuccess) e = cluster_prepare_one<T, DIV, false, false, true>();
+  if (e == cudaSuccess) e = cluster_prepare_one<T, DIV, true, false, true>();
   return e;
 }
 
@@ -1117,7 +1237,7 @@ inline int cluster_max_active_one(int cs) {
   cfg.attrs = at;
   cfg.numAttrs = 1;
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, rowstats_cluster_kernel<T, DIV, RS, TRI>, &cfg) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveClusters(&n, rowstats_cluster_kernel<T, DIV, RS, TRI, false>, &cfg) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -1184,15 +1304,15 @@ inline int cluster_sm_count() {
 }
 
 // Slice / chunk arithmetic for a vocabulary of V logits split over cs CTAs (pure host arithmetic).
-inline void cluster_slices(int V, int elem_bytes, int cs, int* slice, int* chunks) {
-  const int vec = 16 / elem_bytes, ch = kClHalfBytes / elem_bytes;
+inline void cluster_slices(int V, int elem_bytes, int cs, bool ua, int* slice, int* chunks) {
+  const int vec = 16 / elem_bytes, ch = (kClHalfBytes - (ua ? 16 : 0)) / elem_bytes;
   const int per = (V + cs - 1) / cs;
   *slice = (per + vec - 1) / vec * vec;
   *chunks = (*slice + ch - 1) / ch;
 }
 
-// The cluster kernel takes rows that can be copied in 16-byte units: V a multiple of the vector length,
-// 16-byte aligned bases and sequence strides, and at least one full vector per row.
+// Rows that can be copied in 16-byte units: V a multiple of the vector length, 16-byte aligned bases and sequence
+// strides, and at least one full vector per row.
 inline bool cluster_shape_ok(const StageParams& P, int dtype) {
   const int es = dtype == 0 ? 4 : 2, vec = 16 / es;
   if (P.V < 2048 || (P.V % vec) != 0) return false;
@@ -1207,9 +1327,11 @@ inline bool cluster_shape_ok(const StageParams& P, int dtype) {
 
 // Picks the cluster size (or takes `forced_cs`; a forced size whose slice exceeds the ring is streamed
 // twice), and sizes the grid to the clusters that can be co-resident. Returns false when the shape does not
-// fit the kernel.
-inline bool cluster_geometry(const StageParams& P, int dtype, int forced_cs, bool force_streamed, bool allow_triples, ClusterGeom* g) {
-  if (!cluster_shape_ok(P, dtype)) return false;
+// fit the kernel. `any_alignment`: rows that are not 16-byte units may go through the form that takes single logits.
+inline bool cluster_geometry(const StageParams& P, int dtype, int forced_cs, bool force_streamed, bool allow_triples, bool any_alignment,
+                             ClusterGeom* g) {
+  const bool ua = !cluster_shape_ok(P, dtype);
+  if (ua && (!any_alignment || P.V < 2048)) return false;
   const int es = dtype == 0 ? 4 : 2;
   const long long rows = static_cast<long long>(P.B) * (P.K + P.K2);
   int cs = 0, slice = 0, chunks = 0;
@@ -1217,7 +1339,7 @@ inline bool cluster_geometry(const StageParams& P, int dtype, int forced_cs, boo
   if (forced_cs > 0) {
     if (forced_cs > kClMaxRanks) return false;
     cs = forced_cs;
-    cluster_slices(P.V, es, cs, &slice, &chunks);
+    cluster_slices(P.V, es, cs, ua, &slice, &chunks);
     restream = chunks > kClSlots - 1 || force_streamed;   // a slice the ring cannot hold is streamed twice
   } else {
     // the smallest cluster whose slice leaves at least five ring slots beyond a row (measured: 4 CTAs for
@@ -1226,14 +1348,14 @@ inline bool cluster_geometry(const StageParams& P, int dtype, int forced_cs, boo
     bool found = false;
     for (int pass = 0; pass < 2 && !found; ++pass)
       for (cs = 1; cs <= (pass == 0 ? 8 : kClMaxRanks); ++cs) {   // sizes above 8 place few clusters: last resort
-        cluster_slices(P.V, es, cs, &slice, &chunks);
+        cluster_slices(P.V, es, cs, ua, &slice, &chunks);
         if (chunks <= wanted[pass] && cluster_max_active_any(dtype, P.div_kind, cs) > 0) { found = true; break; }
       }
     // few rows: spread each row over more CTAs so that more SMs pull on HBM
     const int sms = cluster_sm_count();
     while (found && cs < 8 && chunks >= 2 && rows * cs * 2 <= sms) {
       cs *= 2;
-      cluster_slices(P.V, es, cs, &slice, &chunks);
+      cluster_slices(P.V, es, cs, ua, &slice, &chunks);
     }
     // Small clusters fill more SMs (148 with one or two CTAs, 135 with three, 132 with four on B200; eight
     // CTAs place only 120), but for a large vocabulary their slice exceeds the ring and has to be streamed
@@ -1249,7 +1371,7 @@ inline bool cluster_geometry(const StageParams& P, int dtype, int forced_cs, boo
     double best = found ? (1.0 + 0.049 * cs) * rounds_per_cta(cs, cluster_max_active_any(dtype, P.div_kind, cs)) : 1e300;
     for (int c2 = 8; c2 >= 1; --c2) {
       int sl2 = 0, ch2 = 0;
-      cluster_slices(P.V, es, c2, &sl2, &ch2);
+      cluster_slices(P.V, es, c2, ua, &sl2, &ch2);
       if (ch2 <= wanted[0]) continue;   // fits the ring with room to spare: the rule above has seen it
       const int na = cluster_max_active_any(dtype, P.div_kind, c2);
       if (na <= 0) continue;
@@ -1264,6 +1386,7 @@ inline bool cluster_geometry(const StageParams& P, int dtype, int forced_cs, boo
   const int max_active = cluster_max_active_any(dtype, P.div_kind, cs);
   if (max_active <= 0) return false;
   g->cs = cs;
+  g->ua = ua ? 1 : 0;
   g->slice = slice;
   g->chunks = chunks;
   g->ring = max(chunks + 1, min(kClSlots, 3 * chunks - 1));
@@ -1277,7 +1400,7 @@ inline bool cluster_geometry(const StageParams& P, int dtype, int forced_cs, boo
   }
   // A wrapper launch whose second row set pairs the first set's large rows (the qualifier's, in place) with a
   // third tensor can be walked as row triples where it is streamed twice anyway.
-  g->tri = (allow_triples && restream && P.K2 > 0 && P.K2 <= P.K && P.n_valid == nullptr && P.small2 == P.large &&
+  g->tri = (allow_triples && restream && !ua && P.K2 > 0 && P.K2 <= P.K && P.n_valid == nullptr && P.small2 == P.large &&
             P.seq_stride_small2 == P.seq_stride_large) ? 1 : 0;
   const long long items = g->tri ? static_cast<long long>(P.B) * P.K : rows;
   g->n_clusters = static_cast<int>(items < max_active ? items : max_active);
@@ -1298,9 +1421,11 @@ inline cudaError_t cluster_launch_typed(const StageParams& P, const ClusterGeom&
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  if (g.ra > 0 && g.tri) return cudaLaunchKernelEx(&cfg, rowstats_cluster_kernel<T, DIV, true, true>, P, g);
-  if (g.ra > 0) return cudaLaunchKernelEx(&cfg, rowstats_cluster_kernel<T, DIV, true, false>, P, g);
-  return cudaLaunchKernelEx(&cfg, rowstats_cluster_kernel<T, DIV, false, false>, P, g);
+  if (g.ua && g.ra > 0) return cudaLaunchKernelEx(&cfg, rowstats_cluster_kernel<T, DIV, true, false, true>, P, g);
+  if (g.ua) return cudaLaunchKernelEx(&cfg, rowstats_cluster_kernel<T, DIV, false, false, true>, P, g);
+  if (g.ra > 0 && g.tri) return cudaLaunchKernelEx(&cfg, rowstats_cluster_kernel<T, DIV, true, true, false>, P, g);
+  if (g.ra > 0) return cudaLaunchKernelEx(&cfg, rowstats_cluster_kernel<T, DIV, true, false, false>, P, g);
+  return cudaLaunchKernelEx(&cfg, rowstats_cluster_kernel<T, DIV, false, false, false>, P, g);
 }
 
 // Launches the statistics pass with the cluster kernel. Returns 0, or -2 when the launch was refused.

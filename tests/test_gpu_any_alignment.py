@@ -1,0 +1,93 @@
+"""Rows that are no whole 16-byte units -- odd vocabularies, bases at any element -- through the cluster kernel's form
+that takes single logits, against the oracle: chunk edges (a chunk holds 4088 bf16 or 2044 fp32 logits), slices of one and
+several chunks, few rows (a row over many CTAs) and many (streamed twice), flagged, masked and overflowing rows."""
+import numpy as np
+import pytest
+import torch
+
+from parity_utils import TOL, compare_stage, gpu_stage_to_numpy, host_bits
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def psd():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2510_12966_b200 import binding
+    binding.load_library()
+    torch.cuda.set_device(0)
+    return binding
+
+
+def on_device(t, offset):
+    """A device copy of t whose first element sits `offset` elements behind a 16-byte boundary."""
+    buf = torch.empty(t.numel() + 16, dtype=t.dtype, device="cuda")
+    view = buf[offset:offset + t.numel()].view(t.shape)
+    view.copy_(t)
+    return view
+
+
+def check(psd, oracle, zs, zl, tok, tau, dtype, offs=(0, 0), n_valid=None, mode=0, div_kind=0):
+    nv = None if n_valid is None else torch.as_tensor(n_valid, dtype=torch.int32, device="cuda")
+    out = psd.verify_stage_ex(on_device(zs, offs[0]), on_device(zl, offs[1]), tok.cuda(), tau, mode, 3, 5, n_valid=nv, div_kind=div_kind)
+    torch.cuda.synchronize()
+    assert psd.last_status() == 0
+    gpu = gpu_stage_to_numpy(out)
+    orc = oracle.verify_stage(host_bits(zs), host_bits(zl), tok.numpy(), np.float32(tau), mode, 3, 5, n_valid=n_valid,
+                              div_kind=div_kind, n_threads=8)
+    return gpu, compare_stage(oracle, gpu, orc, host_bits(zs), host_bits(zl), dtype=dtype, mode=mode, tau=float(np.float32(tau)),
+                              seed=3, offset=5, n_valid=n_valid, div_kind=div_kind)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("V", [2049, 4087, 4089, 2 * 4088 + 1, 50257, 128257])
+def test_odd_vocabularies_and_bases(psd, oracle, V, dtype):
+    from paper_2510_12966_b200 import workloads as wl
+    zs, zl, tok = wl.make_stage_inputs(3, 4, V, dtype, seed=900 + V, sigma=0.8)
+    for offs, mode, div in (((0, 0), 0, 0), ((1, 6), 1, 1), ((3, 0), 2, 2)):
+        _, rep = check(psd, oracle, zs, zl, tok, 0.2, dtype, offs, mode=mode, div_kind=div)
+        assert rep["tie_div"] + rep["tie_coin"] + rep["tie_cdf"] <= 1
+
+
+@pytest.mark.parametrize("V,B,K,dtype,offs", [(4096, 40, 7, "bf16", (1, 0)), (32001, 48, 8, "f32", (0, 0)), (128257, 40, 16, "bf16", (0, 0)),
+                                              (152065, 24, 8, "f32", (2, 1))])
+def test_many_rows(psd, oracle, V, B, K, dtype, offs):
+    """Every cluster walks several rows: rings, exchange buffers and phases wrap, resident and streamed twice."""
+    from paper_2510_12966_b200 import workloads as wl
+    zs, zl, tok = wl.make_stage_inputs(B, K, V, dtype, seed=77, boost=(4.0, 12.0), sigma=0.7)
+    nv = [(3 * b) % (K + 1) for b in range(B)]
+    _, rep = check(psd, oracle, zs, zl, tok, 0.15, dtype, offs, n_valid=nv, mode=2)
+    assert rep["tie_div"] + rep["tie_coin"] + rep["tie_cdf"] <= 2
+    # the kernel's own accuracy: the arithmetic of the form over 16-byte vectors
+    assert rep["max_err_div"] < (2e-5 if dtype == "bf16" else TOL["f32"]["val"])
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_masked_flagged_identical_and_overflowing_rows(psd, oracle, dtype):
+    from paper_2510_12966_b200 import workloads as wl
+    V = 8191
+    zs, zl, tok = wl.make_stage_inputs(4, 3, V, dtype, seed=31, sigma=0.3)
+    zs[0, 1, 100:5000] = -float("inf")
+    zl[1, 0, :] = -float("inf")
+    zl[1, 0, 4321] = 2.0
+    zs[2, 1, 17] = float("nan")
+    zl[3, 0, V - 1] = float("inf")
+    zl[3, 2] = zs[3, 2]
+    zs[0, 0, :4000] = -3.0e38
+    zs[1, 2, V - 1] = 300.0                      # 2^127 above the row's first logits: the careful second go
+    gpu, _ = check(psd, oracle, zs, zl, tok, 1.0, dtype)
+    assert gpu["div"][3, 2] == 0.0 and gpu["row_flags"][2, 1] == 1 and gpu["row_flags"][3, 0] == 2
+
+
+def test_pyramid_schedules_agree(psd):
+    from paper_2510_12966_b200 import workloads as wl
+    t = [x.cuda() for x in wl.make_pyramid_inputs(20, 8, 4, 50257, "bf16", seed=23, sigma_q=0.6, sigma_d=1.2)]
+    outs = [psd.verify_ex(*t, 0.2, 0.15, psd.FUZZY, psd.FUZZY, 5, 9, schedule=s)
+            for s in (psd.TWO_STAGE_FUSED, psd.TWO_STAGE_SEPARATE, psd.TWO_STAGE_AUTO, psd.TWO_STAGE_FUSED_ROWS)]
+    n2 = outs[0]["n_window"].cpu()
+    live = torch.arange(4)[None, :] < n2[:, None]
+    for o in outs[1:]:
+        for k in ("accept_len_q", "next_token_q", "accept_len", "next_token", "window", "div_q", "resid_q"):
+            assert torch.equal(o[k], outs[0][k]), k
+        assert torch.equal(o["div_t"].cpu()[live], outs[0]["div_t"].cpu()[live])
