@@ -456,9 +456,9 @@ def run_single_stage(args):
 
 
 def run_fused(args):
-    """Config 5: the fused LM-head + target verify. A step = one pyramidsd_verify_fused_lmhead call (two GEMM
-    sweeps with the statistics in their epilogues, a row reduction, the finalisation). The bound is the
-    tensor pipe: achieved = 2 sweeps x 2*M*d*V flops / device time of the sweep kernels."""
+    """Config 5: the fused LM-head + target verify. A step = one pyramidsd_verify_fused_lmhead call (one GEMM
+    sweep that leaves the logits and the normalisers' partial sums, the divergence terms from them, the finalisation).
+    The bound is the tensor pipe: achieved = 2*M*d*V flops / device time of the sweep and the terms kernel."""
     from paper_2510_12966_b200 import binding, workloads
     if int(os.environ.get("WORLD_SIZE", "1")) > 1 and int(os.environ.get("RANK", "0")) != 0:
         return
@@ -513,11 +513,7 @@ def run_fused(args):
     if binding.last_status() != 0:
         raise SystemExit("bench.py: library status != 0")
     peaks, peak_kind = load_peaks()
-    # Jensen-Shannon runs the GEMM twice; KL once, plus a second sweep only when a rejected row needs residual masses:
-    # never in the assisted mode, and not in the threshold mode while every position is accepted
-    one_sweep = kl and (lm_mode == binding.ASSISTED or bool((out["accept_len"] == w.K_d).all().item()))
-    sweeps = 1 if one_sweep else 2
-    flops = sweeps * 2.0 * M * w.d_model * w.V
+    flops = 2.0 * M * w.d_model * w.V
     achieved = flops * n_sw / (ms_sweeps * 1e-3) / 1e12 if ms_sweeps > 0 else 0.0
     # end to end: activations and qualifier logits come from pinned host memory every step, results go back
     e2e = None
@@ -550,17 +546,16 @@ def run_fused(args):
         "vs_baseline": None, "dtype": "bf16 x bf16 -> f32 (GEMM), f32 (epilogue)", "data": "synthetic",
         "timed_regions": args.regions, "ms_per_step_min_max": [min(region_ms) / args.steps, max(region_ms) / args.steps],
         "config": {"workload": f"{w.name}: B={w.B}, K={w.K_d} (M={M}), d={w.d_model}, V={w.V}, LM-head weight bf16 [V, d], "
-                               f"qualifier logits bf16, tau_t={w.tau_t}, {args.lmhead_mode} mode, Philox seed 0, divergence {'KL(large||small)' if kl else 'Jensen-Shannon'}, {sweeps} GEMM sweep(s)",
+                               f"qualifier logits bf16, tau_t={w.tau_t}, {args.lmhead_mode} mode, Philox seed 0, divergence {'KL(large||small)' if kl else 'Jensen-Shannon'}",
                    "all_positions_accepted": bool((out["accept_len"] == w.K_d).all().item()),
-                   "l2_policy": "the weight (1.05 GB) is larger than L2 and is streamed twice per step"},
-        "roofline": {"bound": "tensor", "kernel": "lmhead_sweep (two tcgen05 GEMM sweeps + row reduction)",
+                   "l2_policy": "the weight (1.05 GB) is larger than L2 and is streamed once per step"},
+        "roofline": {"bound": "tensor", "kernel": "lmhead_sweep (tcgen05 GEMM) + lmhead_terms",
                      "achieved": achieved, "peak": tensor_peak, "unit": "TFLOP/s", "frac": achieved / tensor_peak,
                      "frac_of_burst": achieved / peaks["bf16_tflops"],
-                     "flops_counted": "the GEMM sweeps executed (%d); the method needs one h x W^T" % sweeps,
-                     "achieved_on_one_gemm": achieved / sweeps, "frac_on_one_gemm": achieved / sweeps / tensor_peak,
+                     "flops_counted": "one h x W^T, over the time of both kernels",
                      "peak_kind": tensor_kind, "traffic": None, "launches": n_sw,
                      "avg_launch_ms": ms_sweeps / max(n_sw, 1), "finalize_ms_per_launch": ms_fin / max(n_fin, 1),
-                     "weight_gb_per_s": sweeps * w.V * w.d_model * 2 * n_sw / (ms_sweeps * 1e-3) / 1e9 if ms_sweeps > 0 else 0.0},
+                     "weight_gb_per_s": w.V * w.d_model * 2 * n_sw / (ms_sweeps * 1e-3) / 1e9 if ms_sweeps > 0 else 0.0},
         "gpu_launches": launches, "clocks": clocks,
     }
     if e2e:

@@ -1,16 +1,18 @@
 // Fused LM-head + verification: the large model's logits z = hidden x W^T are produced by a tcgen05 GEMM
 // (bf16 operands staged by TMA into 128-byte-swizzled shared memory, fp32 accumulators in tensor memory)
-// and consumed in the epilogue by the same per-row arithmetic as the logits path (Sec. 3.1-3.2 for one
-// model pair), so the large model's logits never reach HBM.
+// and consumed by the same per-row arithmetic as the logits path (Sec. 3.1-3.2 for one model pair).
 //
-// The Jensen-Shannon terms need the large model's normaliser before they can be formed, and 256 x V fp32
-// logits fit nowhere on chip, so the GEMM runs twice:
-//   sweep 1  per (row, 128-column tile): partial (max, sum-exp) of the large logits (from the accumulator)
-//            and of the small logits (bf16, read from HBM);          -> lmhead_reduce_kernel -> per-row lse
-//   sweep 2  per (row, tile): sum of divergence terms, sum max(p,q), residual mass, mass of p
-//   final    per sequence: row totals, accept bits, accepted prefix, and the residual draw: the tile is found
-//            from the per-tile residual masses, and only that tile's 128 logits of the rejected row are
-//            recomputed (128 dot products) to place the token.
+// The divergence terms need the large model's normaliser before they can be formed, so a row is looked at twice.
+// The GEMM runs once and leaves its fp32 logits in scratch; what it would cost to run it a second time (the weight
+// streamed again: 1.05 GB and 269 GFLOP at M = 256, d = 4096, V = 128256) is far above what the logits cost
+// (131 MB written, 131 MB read):
+//   sweep    the GEMM; per (row, column part of a tile): the fp32 logits, and partial (max, sum-exp) of the large
+//            logits (from the accumulator) and of the small ones (bf16, read from HBM)
+//   terms    per (row, 512-column segment): divergence terms, residual mass and mass of p from both models' logits
+//   final    per sequence: row totals, accept bits, accepted prefix, and the residual draw: the segment is found
+//            from the per-segment masses, the token from that segment's logits
+// Measured, whole call: 551 -> 392 us at that size, 99.5 -> 50.4 us at M = 15, d = 2048, V = 32000, against two runs of
+// the GEMM with the terms in the second one's epilogue.
 //
 // One CTA = 10 warps: warp 0 lane 0 issues TMA loads, warp 1 lane 0 issues the MMAs (and owns the tensor
 // memory allocation), warps 2..9 are the epilogue (warp e reads TMEM lanes 32*(e%4).. of accumulator
@@ -39,23 +41,28 @@ constexpr int kLmEpiWarps = 8;
 constexpr size_t kLmSmemBytes = static_cast<size_t>(kLmStages) * kLmStageBytes + 1024 /*alignment*/ + 256 /*barriers*/;
 constexpr unsigned kLmSpinLimit = 1u << 24;
 
+// The call's rows are worked on in groups of whole sequences with at most kLmGroupRows rows, which bounds the
+// scratch the logits take (525 MB at V = 128256); a group's rows go through the GEMM in blocks of kLmM.
+constexpr int kLmGroupRows = 1024;
+constexpr int kLmSeg = 512;          // columns per segment of the terms kernel: 16 per lane of a warp
+
 struct LmParams {
   const __nv_bfloat16* small;     // [M, V] bf16 logits of the small model
   const int32_t* tokens;          // [M]
-  int M, d, V, n_tiles;
-  int row0;                       // first row of the 256-row block this launch works on
+  int M, d, V;                    // M: rows up to the end of the group this launch works on
+  int row0;                       // sweep: first row of the 256-row block this launch works on
+  int grp0;                       // first row of the group; scratch is indexed by row - grp0
+  int tile_n;                     // sweep: columns per tile (pair of CTAs: at most 256, a multiple of 32; one CTA: 128)
+  int n_tiles, n_part, n_seg;     // tiles; column parts with (max, sum) partials; segments
+  int w_once;                     // 1: every weight byte is read once in this call
+  long long ldz;                  // logits per row of z (a multiple of 32)
   float c;                        // log2(e) / T
-  float2* part_large;             // sweep 1: [M][n_tiles] (max in scaled base-2 domain, sum)
+  float* z;                       // [rows][ldz] fp32 logits of the large model
+  float2* part_large;             // [rows][n_part] (max in scaled base-2 domain, sum)
   float2* part_small;
-  float4* row_lse;                // [M] (m2_small, l2s_small, m2_large, l2s_large)
-  float4* part_div;               // sweep 2: [M][n_tiles] (js bits, sum max(p,q), residual mass, mass of p)
+  float4* row_lse;                // [rows] (m2_small, l2s_small, m2_large, l2s_large)
+  float4* part_div;               // [rows][n_seg] (divergence in bits, residual mass, mass of p, unused)
   int* status;
-  // KL(large || small) needs no second sweep for the divergence itself: sum_i p_i (log2 p_i - log2 q_i) =
-  // (1 / S_l) sum_i P_i (z_i - x_i) c - (lse_l - lse_s) with P_i = 2^(z_i c - m), which sweep 1 accumulates per
-  // tile next to (m, S_l), rescaled online like the sum.
-  float* part_t;                  // KL, sweep 1: [M][n_tiles] sum of P_i (z_i - x_i) c against the tile's own max
-  float* row_div;                 // KL: [M] the row's divergence in nats, written by the row reduction
-  int* need_sweep2;               // KL: set by the accept scan when a residual mass is needed after all; sweep 2 leaves at once if 0
 };
 
 // ---- tcgen05 / TMA wrappers -----------------------------------------------------------------------------
@@ -153,90 +160,42 @@ __device__ __forceinline__ void load_small32(const __nv_bfloat16* p, bool aligne
   }
 }
 
-// What one thread (= one row) leaves per 128-column tile.
-struct LmTilePartial {
-  float2 large, small;   // sweep 1: (max, sum) of both models
-  float kl_t;            // sweep 1, KL: sum of P_i (z_i - x_i) c against `large.x`
-  float4 div;            // sweep 2: (js bits, sum max(p,q), residual mass, mass of p)
-};
-
-// The epilogue of one 128-column tile for this thread's row: reads the accumulator from tensor memory 32
-// columns at a time (all 32 lanes execute the loads, whatever row_ok says) and the small model's logits
-// from global memory.
-template <int SWEEP, bool KL = false>
-__device__ __forceinline__ void lm_epilogue_tile(unsigned tacc, int n0, bool row_ok, const __nv_bfloat16* small_row, float c,
-                                                 float off_l, float off_s, int V, LmTilePartial& out) {
+// The epilogue of `width` columns of a tile for this thread's row: reads the accumulator from tensor memory 32
+// columns at a time (all 32 lanes execute the loads, whatever row_ok says) and the small model's logits from global
+// memory; leaves the logits in z and the columns' (max, sum) partials as part `part` of the row.
+__device__ __forceinline__ void lm_epilogue(const LmParams& P, unsigned tacc, int n0, int width, int row, int part) {
+  const bool row_ok = row < P.M;
+  const __nv_bfloat16* small_row = P.small + static_cast<size_t>(row_ok ? row : 0) * P.V;
+  const long long srow = row - P.grp0;
   OnlineLse ol, os;
   ol.init(); os.init();
-  float js = 0.f, big = 0.f, resid = 0.f, pmass = 0.f, kl_t = 0.f;
 #pragma unroll 1
-  for (int cb = 0; cb < kLmN / 32; ++cb) {
+  for (int cb = 0; cb * 32 < width; ++cb) {
     float z[32], x[32];
     tmem_ld32(tacc + static_cast<unsigned>(cb * 32), z);
     const int col0 = n0 + cb * 32;
-    const int nv = min(32, V - col0);   // columns of this group inside the vocabulary (<= 0: none)
+    const int nw = min(32, width - cb * 32);   // columns of this group that are the part's: a multiple of 16
+    const int nv = min(nw, P.V - col0);        // ... and inside the vocabulary (<= 0: none)
     if (row_ok && nv > 0) {
+      float4* zp = reinterpret_cast<float4*>(P.z + srow * P.ldz + col0);   // columns beyond V land in the row's padding
+#pragma unroll
+      for (int v = 0; v < 8; ++v)
+        if (v * 4 < nw) zp[v] = make_float4(z[4 * v], z[4 * v + 1], z[4 * v + 2], z[4 * v + 3]);
       const __nv_bfloat16* sp = small_row + col0;
       load_small32(sp, (reinterpret_cast<uintptr_t>(sp) & 15u) == 0, nv, x);
-      if (SWEEP == 1) {
-        const float m_before = ol.m;
-        ol.add<32>(z, c, nv);
-        os.add<32>(x, c, nv);
-        if (KL) {
-          kl_t *= ex2_approx(m_before - ol.m);   // the group may have raised the tile's max
-          float t = 0.f;
-#pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            if (i < nv) {
-              const float e = ex2_approx(fmaf(z[i], c, -ol.m));
-              if (e > 0.f) t = fmaf(e, (z[i] - x[i]) * c, t);   // q_i = 0 under p_i > 0 gives +inf, as it should
-            }
-          }
-          kl_t += t;
-        }
-      } else {
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          if (i < nv) {
-            const float a = fmaxf(fmaf(z[i], c, -off_l), -125.f), b = fmaxf(fmaf(x[i], c, -off_s), -125.f);   // log2 p, log2 q
-            const float E = ex2_approx(fmaxf(a, b));
-            const float dd = a - b;
-            const float u = ex2_approx(-fabsf(dd));
-            const float2 ps = psi_poly<7>(make_float2(u, u));
-            js = fmaf(E, fmaf(u, -fabsf(dd), ps.x), js);
-            big += E;
-            const float lo = E * u;                       // min(p, q)
-            resid += (dd > 0.f) ? E - lo : 0.f;           // max(0, p - q)
-            pmass += (dd >= 0.f) ? E : lo;                // p
-          }
-        }
-      }
+      ol.add<32>(z, P.c, nv);
+      os.add<32>(x, P.c, nv);
     }
   }
-  out.large = make_float2(ol.m, ol.s);
-  out.small = make_float2(os.m, os.s);
-  out.kl_t = kl_t;
-  out.div = make_float4(js, big, resid, pmass);
-}
-
-template <int SWEEP, bool KL = false>
-__device__ __forceinline__ void lm_store_partial(const LmParams& P, size_t idx, const LmTilePartial& part) {
-  if (SWEEP == 1) {
-    P.part_large[idx] = part.large;
-    P.part_small[idx] = part.small;
-    if (KL) P.part_t[idx] = part.kl_t;
-  } else {
-    P.part_div[idx] = part.div;
+  if (row_ok) {
+    P.part_large[srow * P.n_part + part] = make_float2(ol.m, ol.s);
+    P.part_small[srow * P.n_part + part] = make_float2(os.m, os.s);
   }
 }
 
-template <int SWEEP, bool KL = false>
 __global__ void __launch_bounds__(kLmThreads, 1)
 lmhead_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, const LmParams P) {
   extern __shared__ unsigned char lm_smem_raw[];
-  // KL: the second sweep only serves residual masses; when the accept scan found no use for them every CTA leaves
-  // here, before it has set up anything (the flag was written by an earlier kernel: the same answer for all)
-  if (SWEEP == 2 && P.need_sweep2 != nullptr && *reinterpret_cast<volatile const int*>(P.need_sweep2) == 0) return;
   unsigned char* tiles = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(lm_smem_raw) + 1023) & ~uintptr_t(1023));
   LmBarriers* bars = reinterpret_cast<LmBarriers*>(tiles + static_cast<size_t>(kLmStages) * kLmStageBytes);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -252,6 +211,7 @@ lmhead_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   __syncthreads();
   tc_fence_after();
   const unsigned tmem_base = bars->tmem_base;
+  release_dependent_launch();
 
   bool dead = false;
   auto wait_phase = [&](unsigned long long* bar, unsigned parity) {
@@ -324,12 +284,6 @@ lmhead_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     // a warp reads the TMEM lanes 32 * (its index in the CTA mod 4) ..; warps 2..5 take accumulator 0, 6..9 accumulator 1
     const int quarter = warp & 3, half = (warp - 2) >> 2;
     const int row = P.row0 + half * 128 + quarter * 32 + lane;   // this thread's row (TMEM lane + 128*half of the block)
-    const bool row_ok = row < P.M;
-    const float c = P.c;
-    const __nv_bfloat16* small_row = P.small + static_cast<size_t>(row_ok ? row : 0) * P.V;
-    float4 lse = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (SWEEP == 2 && row_ok) lse = P.row_lse[row];
-    const float off_s = lse.x + lse.y, off_l = lse.z + lse.w;
     int it = 0;
     for (int tile = blockIdx.x; tile < P.n_tiles; tile += gridDim.x, ++it) {
       const int buf = it & 1;
@@ -337,13 +291,10 @@ lmhead_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
       tc_fence_after();
       const unsigned tacc = tmem_base + static_cast<unsigned>(buf) * 256u + static_cast<unsigned>(half) * 128u +
                             (static_cast<unsigned>(quarter * 32) << 16);
-      const int n0 = tile * kLmN;
-      LmTilePartial part;
-      lm_epilogue_tile<SWEEP, KL>(tacc, n0, row_ok, small_row, c, off_l, off_s, P.V, part);
+      lm_epilogue(P, tacc, tile * kLmN, kLmN, row, tile);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&bars->tmem_empty[buf]);   // this warp has read its part of the accumulator
-      if (row_ok) lm_store_partial<SWEEP, KL>(P, static_cast<size_t>(row) * P.n_tiles + tile, part);
     }
   }
   tc_fence_before();
@@ -355,15 +306,15 @@ lmhead_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
 }
 
 // ---- two-SM variant -------------------------------------------------------------------------------------
-// A pair of CTAs (cluster of 2) shares one 256 x 256 tile: tcgen05.mma.cta_group::2 with M = 256 takes rows
+// A pair of CTAs (cluster of 2) shares one 256 x N tile, N = 256 or what leaves the last round of tiles fuller: tcgen05.mma.cta_group::2 with M = 256 takes rows
 // 0..127 of A from the even CTA's shared memory and rows 128..255 from the odd one's, and the two halves of
-// the 256 B rows likewise; each CTA keeps its 128 rows of the fp32 accumulator in its own tensor memory
+// the N B rows likewise; each CTA keeps its 128 rows of the fp32 accumulator in its own tensor memory
 // (256 columns, two buffers). Per K step a CTA stages 16 KB of A and 16 KB of B (six stages), so the hidden
 // matrix crosses L2 -> SM once per 256 columns instead of once per 128, and the ring holds 1.5x the K steps.
 // The even CTA issues the MMAs; both CTAs' TMA loads count their bytes on the even CTA's "full" barrier,
 // tcgen05.commit (multicast to both CTAs) frees the stages and publishes the accumulators, and the odd CTA's
 // epilogue warps arrive remotely on the even CTA's "accumulator drained" barrier.
-constexpr int kLm2N = 256;
+constexpr int kLm2N = 256;           // the largest N
 constexpr int kLm2Stages = 6;
 constexpr int kLm2HalfBytes = 128 * kLmK * 2;              // 16 KB: 128 rows x 64 bf16
 constexpr int kLm2StageBytes = 2 * kLm2HalfBytes;          // A half + B half
@@ -378,6 +329,13 @@ __device__ __forceinline__ void tma_load_2d_pair(void* smem_dst, const CUtensorM
   // the barrier address with the peer bit cleared names the even CTA's barrier at the same offset
   asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
                ::"r"(smem_u32(smem_dst)), "l"(map), "r"(smem_u32(bar) & 0xFEFFFFFFu), "r"(x), "r"(y) : "memory");
+}
+// the same with an L2 eviction priority
+__device__ __forceinline__ void tma_load_2d_pair_hint(void* smem_dst, const CUtensorMap* map, int x, int y, unsigned long long* bar,
+                                                      unsigned long long policy) {
+  asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint "
+               "[%0], [%1, {%3, %4}], [%2], %5;"
+               ::"r"(smem_u32(smem_dst)), "l"(map), "r"(smem_u32(bar) & 0xFEFFFFFFu), "r"(x), "r"(y), "l"(policy) : "memory");
 }
 __device__ __forceinline__ void tmem_alloc_pair(unsigned* smem_result, unsigned ncols) {   // same warp index in both CTAs
   asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(smem_result)), "r"(ncols) : "memory");
@@ -402,18 +360,16 @@ __device__ __forceinline__ void mbar_arrive_remote_release(unsigned cluster_addr
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 
-template <int SWEEP, bool KL = false>
 __global__ void __launch_bounds__(kLmThreads, 1)
 lmhead_sweep2sm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, const LmParams P) {
   extern __shared__ unsigned char lm_smem_raw[];
-  if (SWEEP == 2 && P.need_sweep2 != nullptr && *reinterpret_cast<volatile const int*>(P.need_sweep2) == 0) return;   // as in the one-SM kernel
   unsigned char* tiles = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(lm_smem_raw) + 1023) & ~uintptr_t(1023));
   Lm2Barriers* bars = reinterpret_cast<Lm2Barriers*>(tiles + static_cast<size_t>(kLm2Stages) * kLm2StageBytes);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const unsigned rank = cluster_rank();          // 0: issues the MMAs; 1: its peer
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
   const int k_steps = P.d / kLmK;
-  const int n_tiles2 = (P.n_tiles + 1) / 2;      // 256-column tiles
+  const int tile_n = P.tile_n, half_n = tile_n >> 1;
 
   if (tid == 0) {
     for (int s = 0; s < kLm2Stages; ++s) { mbar_init(&bars->full[s], 1); mbar_init(&bars->empty[s], 1); }
@@ -426,6 +382,7 @@ lmhead_sweep2sm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
   cluster_sync_all();        // both CTAs' barriers and allocations exist before either signals the other
   tc_fence_after();
   const unsigned tmem_base = bars->tmem_base;
+  release_dependent_launch();
 
   bool dead = false;
   auto wait_phase = [&](unsigned long long* bar, unsigned parity) {
@@ -439,15 +396,20 @@ lmhead_sweep2sm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
     // ================================ TMA producer (both CTAs) ================================
     if (lane == 0) {
       unsigned stage = 0, fills = 0;
-      for (int tile = pair; tile < n_tiles2 && !dead; tile += n_pairs) {
+      // the hidden rows, read by every pair, stay in L2; a weight that is read once is dropped first (M = 15, d = 2048,
+      // V = 32000: 69 us a call without priorities, 64 and 55 with either, 55 with both; no difference at M = 256)
+      const unsigned long long pol_a = l2_policy_keep(), pol_b = l2_policy_drop();
+      const unsigned pair_bytes = 2u * static_cast<unsigned>(kLm2HalfBytes + half_n * kLmK * 2);
+      for (int tile = pair; tile < P.n_tiles && !dead; tile += n_pairs) {
         for (int ks = 0; ks < k_steps; ++ks) {
           if (fills > 0) wait_phase(&bars->empty[stage], (fills - 1u) & 1u);
           if (dead) break;   // the stage never came back: nothing more is copied into this ring
           unsigned char* sa = tiles + static_cast<size_t>(stage) * kLm2StageBytes;
           // the even CTA's barrier counts the bytes of both CTAs
-          if (rank == 0) mbar_arrive_expect_tx(&bars->full[stage], 2u * kLm2StageBytes);
-          tma_load_2d_pair(sa, &map_a, ks * kLmK, P.row0 + static_cast<int>(rank) * 128, &bars->full[stage]);
-          tma_load_2d_pair(sa + kLm2HalfBytes, &map_b, ks * kLmK, tile * kLm2N + static_cast<int>(rank) * 128, &bars->full[stage]);
+          if (rank == 0) mbar_arrive_expect_tx(&bars->full[stage], pair_bytes);
+          tma_load_2d_pair_hint(sa, &map_a, ks * kLmK, P.row0 + static_cast<int>(rank) * 128, &bars->full[stage], pol_a);
+          if (P.w_once) tma_load_2d_pair_hint(sa + kLm2HalfBytes, &map_b, ks * kLmK, tile * tile_n + static_cast<int>(rank) * half_n, &bars->full[stage], pol_b);
+          else tma_load_2d_pair(sa + kLm2HalfBytes, &map_b, ks * kLmK, tile * tile_n + static_cast<int>(rank) * half_n, &bars->full[stage]);
           if (++stage == kLm2Stages) { stage = 0; ++fills; }
         }
       }
@@ -465,10 +427,10 @@ lmhead_sweep2sm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
   } else if (warp == 1) {
     // ================================ MMA issuer (even CTA only) ================================
     if (lane == 0 && rank == 0) {
-      constexpr unsigned idesc = umma_idesc_bf16(256, kLm2N);
+      const unsigned idesc = umma_idesc_bf16(256, tile_n);
       unsigned stage = 0, par = 0;
       int it = 0;
-      for (int tile = pair; tile < n_tiles2; tile += n_pairs, ++it) {
+      for (int tile = pair; tile < P.n_tiles; tile += n_pairs, ++it) {
         const int buf = it & 1;
         if (it >= 2) wait_phase(&bars->tmem_empty[buf], ((it >> 1) - 1) & 1u);   // both CTAs' epilogues have drained this buffer
         if (dead) break;
@@ -492,29 +454,20 @@ lmhead_sweep2sm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
     }
   } else {
     // ================================ epilogue (both CTAs) ================================
-    const int quarter = warp & 3, half = (warp - 2) >> 2;          // TMEM lanes 32*quarter.., columns 128*half..
+    const int quarter = warp & 3, half = (warp - 2) >> 2;          // TMEM lanes 32*quarter.., columns half_n*half..
     const int row = P.row0 + static_cast<int>(rank) * 128 + quarter * 32 + lane;
-    const bool row_ok = row < P.M;
-    const float c = P.c;
-    const __nv_bfloat16* small_row = P.small + static_cast<size_t>(row_ok ? row : 0) * P.V;
-    float4 lse = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (SWEEP == 2 && row_ok) lse = P.row_lse[row];
-    const float off_s = lse.x + lse.y, off_l = lse.z + lse.w;
     const unsigned drained = map_to_rank(&bars->tmem_empty[0], 0);   // the even CTA's barriers
     int it = 0;
-    for (int tile = pair; tile < n_tiles2; tile += n_pairs, ++it) {
+    for (int tile = pair; tile < P.n_tiles; tile += n_pairs, ++it) {
       const int buf = it & 1;
       wait_phase(&bars->tmem_full[buf], (it >> 1) & 1u);
       tc_fence_after();
-      const unsigned tacc = tmem_base + static_cast<unsigned>(buf) * 256u + static_cast<unsigned>(half) * 128u +
+      const unsigned tacc = tmem_base + static_cast<unsigned>(buf) * 256u + static_cast<unsigned>(half * half_n) +
                             (static_cast<unsigned>(quarter * 32) << 16);
-      const int tile128 = tile * 2 + half;
-      LmTilePartial part;
-      lm_epilogue_tile<SWEEP, KL>(tacc, tile128 * kLmN, row_ok, small_row, c, off_l, off_s, P.V, part);
+      lm_epilogue(P, tacc, tile * tile_n + half * half_n, half_n, row, tile * 2 + half);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_remote_release(drained + static_cast<unsigned>(buf) * 8u);
-      if (row_ok && tile128 < P.n_tiles) lm_store_partial<SWEEP, KL>(P, static_cast<size_t>(row) * P.n_tiles + tile128, part);
     }
   }
   tc_fence_before();
@@ -526,44 +479,117 @@ lmhead_sweep2sm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
   }
 }
 
-// Per row: combine the tiles' (max, sum) partials into the row's log-sum-exp (base 2), both models; with the KL
-// partials also the row's divergence KL(large || small) = ln 2 * (T / S_l - (lse_l - lse_s)), T rescaled to the
-// row's max like S_l.
-__global__ void __launch_bounds__(256) lmhead_reduce_kernel(const LmParams P) {
-  const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (row >= P.M) return;
-  const bool kl = P.part_t != nullptr;
-  float ml = -1e30f, sl = 0.f, ms = -1e30f, ss = 0.f;
-  for (int t = lane; t < P.n_tiles; t += 32) {
-    const float2 a = P.part_large[static_cast<size_t>(row) * P.n_tiles + t], b = P.part_small[static_cast<size_t>(row) * P.n_tiles + t];
-    lse_merge(ml, sl, a.x, a.y);
-    lse_merge(ms, ss, b.x, b.y);
-  }
+// ---- terms: both models' logits against the row's normalisers -----------------------------------------------
+// The (row, segment) items of the group are cut into one run of equal length per CTA, as many CTAs as are resident, so
+// a run touches a row or two. For each row the CTA merges the (max, sum) partials (a few KB out of L2, the same fixed
+// tree in every CTA, so all of a row's CTAs hold the same bits; a launch of its own for it took 15 us), then each
+// warp takes segment after segment, a lane four times four consecutive columns, so that 96 bytes per lane are in
+// flight. Memory-bound: 6 bytes per column.
+constexpr int kLmTermThreads = 256;
+constexpr int kLmTermCtas = 4;       // resident per SM
+
+__device__ __forceinline__ void lse_merge_warp(float& m, float& s) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    lse_merge(ml, sl, __shfl_xor_sync(0xffffffffu, ml, o), __shfl_xor_sync(0xffffffffu, sl, o));
-    lse_merge(ms, ss, __shfl_xor_sync(0xffffffffu, ms, o), __shfl_xor_sync(0xffffffffu, ss, o));
-  }
-  const float l2sl = lg2_approx(sl), l2ss = lg2_approx(ss);
-  if (lane == 0) P.row_lse[row] = make_float4(ms, l2ss, ml, l2sl);
-  if (kl) {
-    float tt = 0.f;   // sum over the tiles of T_t * 2^(m_t - ml): ml is the row's max after the merge above
-    for (int t = lane; t < P.n_tiles; t += 32) {
-      const float tv = P.part_t[static_cast<size_t>(row) * P.n_tiles + t];
-      const float f = ex2_approx(P.part_large[static_cast<size_t>(row) * P.n_tiles + t].x - ml);
-      if (f > 0.f) tt = fmaf(tv, f, tt);   // a tile without mass contributes nothing (0 * inf otherwise)
+  for (int o = 16; o > 0; o >>= 1) lse_merge(m, s, __shfl_xor_sync(0xffffffffu, m, o), __shfl_xor_sync(0xffffffffu, s, o));
+}
+
+template <int DIV>
+__global__ void __launch_bounds__(kLmTermThreads, kLmTermCtas) lmhead_terms_kernel(const LmParams P, const int items_per_cta) {
+  __shared__ float4 sh_part[kLmTermThreads / 32];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  constexpr int kWarps = kLmTermThreads / 32;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  release_dependent_launch();
+  const int items = (P.M - P.grp0) * P.n_seg;
+  int item = static_cast<int>(blockIdx.x) * items_per_cta;
+  const int end = min(items, item + items_per_cta);
+  while (item < end) {   // one row of the run
+    const int srow = item / P.n_seg, seg0 = item - srow * P.n_seg, seg_end = min(P.n_seg, seg0 + (end - item));
+    item += seg_end - seg0;
+    float ml = -1e30f, sl = 0.f, ms = -1e30f, ss = 0.f;
+    for (int t = tid; t < P.n_part; t += kLmTermThreads) {
+      const float2 a = P.part_large[static_cast<size_t>(srow) * P.n_part + t], b = P.part_small[static_cast<size_t>(srow) * P.n_part + t];
+      lse_merge(ml, sl, a.x, a.y);
+      lse_merge(ms, ss, b.x, b.y);
     }
-    tt = warp_reduce<OpSum>(tt);
-    if (lane == 0) P.row_div[row] = fmaxf(kLn2 * (__fdiv_rn(tt, sl) - ((ml + l2sl) - (ms + l2ss))), 0.f);
+    lse_merge_warp(ml, sl);
+    lse_merge_warp(ms, ss);
+    __syncthreads();   // the row before may still be being read
+    if (lane == 0) sh_part[warp] = make_float4(ml, sl, ms, ss);
+    __syncthreads();
+    const float4 v = lane < kWarps ? sh_part[lane] : make_float4(-1e30f, 0.f, -1e30f, 0.f);
+    ml = v.x; sl = v.y; ms = v.z; ss = v.w;
+    lse_merge_warp(ml, sl);
+    lse_merge_warp(ms, ss);
+    const float l2sl = lg2_approx(sl), l2ss = lg2_approx(ss);
+    if (seg0 == 0 && tid == 0) P.row_lse[srow] = make_float4(ms, l2ss, ml, l2sl);
+    const float off_l = ml + l2sl, off_s = ms + l2ss, c = P.c;
+
+    const float* zrow = P.z + srow * P.ldz;
+    const __nv_bfloat16* xrow = P.small + static_cast<size_t>(P.grp0 + srow) * P.V;
+    const bool x_vec = (reinterpret_cast<uintptr_t>(xrow) & 7u) == 0;
+    for (int seg = seg0 + warp; seg < seg_end; seg += kWarps) {
+      const int col0 = seg * kLmSeg + lane * 4;
+      float4 z4[4];
+      uint2 x4[4];
+      const bool whole = x_vec && (seg + 1) * kLmSeg <= P.V;
+      if (whole) {
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          z4[h] = __ldcg(reinterpret_cast<const float4*>(zrow + col0 + h * 128));   // written by the launch before
+          x4[h] = __ldg(reinterpret_cast<const uint2*>(xrow + col0 + h * 128));
+        }
+      }
+      float js = 0.f, resid = 0.f, pmass = 0.f;
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        float z[4], x[4];
+        if (whole) {
+          z[0] = z4[h].x; z[1] = z4[h].y; z[2] = z4[h].z; z[3] = z4[h].w;
+          x[0] = __uint_as_float(x4[h].x << 16); x[1] = __uint_as_float(x4[h].x & 0xffff0000u);
+          x[2] = __uint_as_float(x4[h].y << 16); x[3] = __uint_as_float(x4[h].y & 0xffff0000u);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int col = col0 + h * 128 + i;
+            z[i] = col < P.V ? __ldcg(zrow + col) : -INFINITY;
+            x[i] = col < P.V ? Elem<__nv_bfloat16>::load(xrow, col) : -INFINITY;
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          if (DIV == kDivKL) {
+            // KL(large || small) on unclamped logits: q = 0 under p > 0 gives +inf, as it should
+            const float a = fmaf(z[i], c, -off_l), b = fmaf(x[i], c, -off_s);
+            const float p = ex2_approx(a), q = ex2_approx(b);
+            if (p > 0.f) js = fmaf(p, a - b, js);
+            resid += fmaxf(p - q, 0.f);
+            pmass += p;
+          } else {
+            const bool in = whole || col0 + h * 128 + i < P.V;
+            const float a = fmaxf(fmaf(z[i], c, -off_l), -125.f), b = fmaxf(fmaf(x[i], c, -off_s), -125.f);   // log2 p, log2 q
+            const float E = in ? ex2_approx(fmaxf(a, b)) : 0.f;
+            const float dd = a - b;
+            const float u = ex2_approx(-fabsf(dd));
+            const float2 ps = psi_poly<7>(make_float2(u, u));
+            js = fmaf(E, fmaf(u, -fabsf(dd), ps.x), js);
+            const float lo = E * u;                       // min(p, q)
+            resid += (dd > 0.f) ? E - lo : 0.f;           // max(0, p - q)
+            pmass += (dd >= 0.f) ? E : lo;                // p
+          }
+        }
+      }
+      js = warp_reduce<OpSum>(js); resid = warp_reduce<OpSum>(resid); pmass = warp_reduce<OpSum>(pmass);
+      if (lane == 0) P.part_div[static_cast<size_t>(srow) * P.n_seg + seg] = make_float4(js, resid, pmass, 0.f);
+    }
   }
 }
 
 // ---- final kernel: one CTA per sequence ------------------------------------------------------------------
 struct LmFinalParams {
   LmParams lm;
-  const __nv_bfloat16* hidden;   // [M, d]
-  const __nv_bfloat16* w_t;      // [V, d]
-  int B, K;
+  int b0, K;             // first sequence of the group
+  int div_kind;
   float threshold;
   int mode;
   unsigned long long seed, offset;
@@ -572,77 +598,88 @@ struct LmFinalParams {
   int32_t* out_next_token;
   float* out_div;        // [B, K] or null
   float* out_resid;      // [B, K] or null
-  // KL: 0 = the usual pass over the second sweep's partials. 1 = accept scan only, before the second sweep: raises
-  // lm.need_sweep2 when some rejected row needs residual masses. 2 = full pass after a second sweep that may not
-  // have run (then every draw comes from p_large, whose tile masses the first sweep left).
-  int kl_phase;
 };
 
-// dot(hidden[row], w_t[col]) by one warp, fp32 accumulation in index order per lane then a shuffle tree
-__device__ __forceinline__ float lm_dot(const __nv_bfloat16* h, const __nv_bfloat16* w, int d, int lane) {
-  float acc = 0.f;
-  for (int j = lane * 8; j < d; j += 256) {
-    float a[8], b[8];
-    Elem<__nv_bfloat16>::unpack(__ldg(reinterpret_cast<const uint4*>(h + j)), a);
-    Elem<__nv_bfloat16>::unpack(__ldg(reinterpret_cast<const uint4*>(w + j)), b);
+constexpr int kLmFinalThreads = 256;
+static_assert(kLmSeg == 2 * kLmFinalThreads, "a thread of the final kernel takes two columns of the chosen segment");
+
+// One level of the inverse CDF by the whole CTA: thread t holds weight w (children in thread order). Leaves in *pick the
+// first thread whose inclusive cumulative weight exceeds `target`, else the last one with a positive weight (-1: none),
+// and in *before what lies before it. Every thread returns the same values.
+template <typename V>
+__device__ __forceinline__ void block_pick(V w, V target, V* sh_warp, int* sh_hit, V* sh_before, int* pick, V* before) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  V incl = w;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) acc = fmaf(a[i], b[i], acc);
+  for (int o = 1; o < 32; o <<= 1) {
+    const V up = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += up;
   }
-  return warp_reduce<OpSum>(acc);
+  __syncthreads();   // the shared words may still be read from the level before
+  if (lane == 31) sh_warp[warp] = incl;
+  if (tid == 0) { sh_hit[0] = kLmFinalThreads; sh_hit[1] = -1; }
+  __syncthreads();
+  V base = 0;
+  for (int k = 0; k < warp; ++k) base += sh_warp[k];
+  incl += base;
+  const bool live = w > static_cast<V>(0);
+  if (live && incl > target) atomicMin(&sh_hit[0], tid);
+  if (live) atomicMax(&sh_hit[1], tid);
+  __syncthreads();
+  const int p = sh_hit[0] < kLmFinalThreads ? sh_hit[0] : sh_hit[1];
+  if (tid == p) *sh_before = incl - w;
+  __syncthreads();
+  *pick = p;
+  *before = p >= 0 ? *sh_before : static_cast<V>(0);
 }
 
-__global__ void __launch_bounds__(256) lmhead_final_kernel(const LmFinalParams F) {
-  __shared__ float sh_div[32], sh_res[32], sh_px[32], sh_qx[32], sh_pm[32];
+__global__ void __launch_bounds__(kLmFinalThreads) lmhead_final_kernel(const LmFinalParams F) {
+  __shared__ float sh_div[32], sh_res[32], sh_px[32], sh_qx[32];
   __shared__ int sh_flag[32];
-  __shared__ float sh_w[kLmN];
-  __shared__ double sh_seg[256];
-  __shared__ int sh_L, sh_tile, sh_token;
-  __shared__ float sh_target, sh_u2;
+  __shared__ double sh_warp_d[kLmFinalThreads / 32], sh_before_d, sh_target;
+  __shared__ float sh_warp_f[kLmFinalThreads / 32], sh_before_f;
+  __shared__ int sh_hit[2];
+  __shared__ int sh_L, sh_seg, sh_token;
+  __shared__ float sh_u2;
   const LmParams& P = F.lm;
-  const int b = blockIdx.x, K = F.K, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nwarps = blockDim.x >> 5;
+  const int b = F.b0 + static_cast<int>(blockIdx.x), K = F.K, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  constexpr int nwarps = kLmFinalThreads / 32;
   const float c = P.c;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
 
-  // per row: totals over the tiles, and the probabilities of the row's token
+  // per row: totals over the segments, and the probabilities of the row's token
   for (int k = warp; k < K; k += nwarps) {
     const int r = b * K + k;
-    double js = 0.0, big = 0.0, res = 0.0, pm = 0.0;
-    // KL: the divergence comes from the row reduction; the second sweep's partials exist only if it ran
-    const bool have2 = F.kl_phase == 0 || (F.kl_phase == 2 && *reinterpret_cast<volatile const int*>(P.need_sweep2) != 0);
-    if (have2) {
-      for (int t = lane; t < P.n_tiles; t += 32) {
-        const float4 v = P.part_div[static_cast<size_t>(r) * P.n_tiles + t];
-        js += v.x; big += v.y; res += v.z; pm += v.w;
-      }
+    const size_t sr = static_cast<size_t>(r - P.grp0);
+    double js = 0.0, res = 0.0;
+    for (int t = lane; t < P.n_seg; t += 32) {
+      const float4 v = P.part_div[sr * P.n_seg + t];
+      js += v.x; res += v.y;
     }
-    js = warp_reduce<OpSum>(js); res = warp_reduce<OpSum>(res); pm = warp_reduce<OpSum>(pm);
-    const float4 lse = P.row_lse[r];
+    js = warp_reduce<OpSum>(js); res = warp_reduce<OpSum>(res);
+    const float4 lse = P.row_lse[sr];
     const int x = P.tokens[r];
-    (void)big;
     int flags = 0;
     if (!(fabsf(lse.x + lse.y) < INFINITY)) flags |= kFlagSmallNonfinite;
     if (!(fabsf(lse.z + lse.w) < INFINITY)) flags |= kFlagLargeNonfinite;
     if (x < 0 || x >= P.V) flags |= kFlagTokenRange;
-    float px = 0.f, qx = 0.f;
-    if (!flags) {
-      const float zx = lm_dot(F.hidden + static_cast<size_t>(r) * P.d, F.w_t + static_cast<size_t>(x) * P.d, P.d, lane);
-      px = ex2_approx(fmaf(zx, c, -lse.z) - lse.w);
-      qx = ex2_approx(fmaf(Elem<__nv_bfloat16>::load(P.small + static_cast<size_t>(r) * P.V, x), c, -lse.x) - lse.y);
-    }
     if (lane == 0) {
-      sh_div[k] = F.kl_phase != 0 ? P.row_div[r] : fmaxf(static_cast<float>(0.5 * 0.6931471805599453 * js), 0.f);
-      sh_res[k] = have2 ? fmaxf(static_cast<float>(res), 0.f) : __int_as_float(0x7fc00000);
-      sh_pm[k] = static_cast<float>(pm);
+      float px = 0.f, qx = 0.f;
+      if (!flags) {
+        px = ex2_approx(fmaf(P.z[sr * P.ldz + x], c, -lse.z) - lse.w);
+        qx = ex2_approx(fmaf(Elem<__nv_bfloat16>::load(P.small + static_cast<size_t>(r) * P.V, x), c, -lse.x) - lse.y);
+      }
+      const double scale = F.div_kind == kDivJS ? 0.5 * 0.6931471805599453 : 0.6931471805599453;   // bits -> nats, JS: its 1/2
+      sh_div[k] = fmaxf(static_cast<float>(scale * js), 0.f);
+      sh_res[k] = fmaxf(static_cast<float>(res), 0.f);
       sh_px[k] = px; sh_qx[k] = qx; sh_flag[k] = flags;
       const bool no_dist = (flags & (kFlagSmallNonfinite | kFlagLargeNonfinite)) != 0;   // a bad token leaves D and R intact
-      if (F.kl_phase != 1) {
-        if (F.out_div) F.out_div[r] = no_dist ? __int_as_float(0x7fc00000) : sh_div[k];
-        if (F.out_resid) F.out_resid[r] = no_dist ? __int_as_float(0x7fc00000) : sh_res[k];
-      }
+      if (F.out_div) F.out_div[r] = no_dist ? __int_as_float(0x7fc00000) : sh_div[k];
+      if (F.out_resid) F.out_resid[r] = no_dist ? __int_as_float(0x7fc00000) : sh_res[k];
     }
   }
   __syncthreads();
   // accept bits and prefix: lane k of warp 0 owns position k
-  float u2 = 0.f;
   if (warp == 0) {
     bool acc = true;
     float u = 0.f, uu2 = 0.f;
@@ -664,102 +701,68 @@ __global__ void __launch_bounds__(256) lmhead_final_kernel(const LmFinalParams F
   }
   __syncthreads();
   const int L = sh_L;
-  u2 = sh_u2;
-  if (F.kl_phase == 1) {
-    // scan only: a rejected row with a distribution draws from the residual unless the mode is the assisted one
-    if (tid == 0 && L < K && !(sh_flag[L] & (kFlagSmallNonfinite | kFlagLargeNonfinite)) && F.mode != kModeAssisted)
-      atomicExch(P.need_sweep2, 1);
-    return;
-  }
-  const bool have2 = F.kl_phase == 0 || *reinterpret_cast<volatile const int*>(P.need_sweep2) != 0;
   int next = -1;
   if (L < K) {
     if (sh_flag[L] & (kFlagSmallNonfinite | kFlagLargeNonfinite)) {
       next = -2;
     } else {
       const int r = b * K + L;
-      const bool from_large = (F.mode == kModeAssisted) || !have2 || !(sh_res[L] > 0.f);
-      const float4 lse_r = P.row_lse[r];
-      // weight of tile t: the second sweep's residual mass or mass of p; without a second sweep the mass of p from
-      // the first sweep's (max, sum) of the tile
-      auto tile_weight = [&](int t) -> double {
-        if (have2) {
-          const float4 v = P.part_div[static_cast<size_t>(r) * P.n_tiles + t];
-          return from_large ? v.w : v.z;
-        }
-        const float2 a = P.part_large[static_cast<size_t>(r) * P.n_tiles + t];
-        return static_cast<double>(a.y) * static_cast<double>(ex2_approx((a.x - lse_r.z) - lse_r.w));
+      const size_t sr = static_cast<size_t>(r - P.grp0);
+      const bool from_large = (F.mode == kModeAssisted) || !(sh_res[L] > 0.f);
+      const float4 lse = P.row_lse[sr];
+      // level 0, the segments: a thread sums a run of consecutive ones, the chosen thread walks its run
+      const int per = (P.n_seg + kLmFinalThreads - 1) / kLmFinalThreads, t0 = tid * per, t1 = min(P.n_seg, t0 + per);
+      auto seg_weight = [&](int t) -> double {
+        const float4 v = P.part_div[sr * P.n_seg + t];
+        return from_large ? v.z : v.y;
       };
-      // the tile that holds the target mass: first tile whose inclusive cumulative weight exceeds it. Two levels:
-      // every thread sums a run of consecutive tiles, one thread walks the 256 run sums and then the chosen run.
-      const int per = (P.n_tiles + static_cast<int>(blockDim.x) - 1) / static_cast<int>(blockDim.x);
-      {
-        double run = 0.0;
-        const int t0 = tid * per, t1 = min(P.n_tiles, t0 + per);
-        for (int t = t0; t < t1; ++t) run += tile_weight(t);
-        sh_seg[tid] = run;
-      }
+      double run = 0.0;
+      for (int t = t0; t < t1; ++t) run += seg_weight(t);
+      double total = warp_reduce<OpSum>(run);
+      if (lane == 0) sh_warp_d[warp] = total;
       __syncthreads();
-      if (tid == 0) {
-        double total = 0.0;
-        for (int g = 0; g < static_cast<int>(blockDim.x); ++g) total += sh_seg[g];
-        const double target = static_cast<double>(u2) * total;
-        int seg = -1, last_seg = -1;
-        double cum = 0.0, before_seg = 0.0, before_last_seg = 0.0;
-        for (int g = 0; g < static_cast<int>(blockDim.x); ++g) {
-          const double wgt = sh_seg[g];
-          if (wgt > 0.0) { last_seg = g; before_last_seg = cum; }
-          if (seg < 0 && cum + wgt > target && wgt > 0.0) { seg = g; before_seg = cum; }
-          cum += wgt;
-        }
-        if (seg < 0) { seg = last_seg; before_seg = before_last_seg; }
-        int pick = -1, last_pos = -1;
-        double before_pick = 0.0, before_last = 0.0;
-        if (seg >= 0) {
-          cum = before_seg;
-          for (int t = seg * per; t < min(P.n_tiles, (seg + 1) * per); ++t) {
-            const double wgt = tile_weight(t);
-            if (wgt > 0.0) { last_pos = t; before_last = cum; }
+      total = 0.0;
+      for (int k = 0; k < nwarps; ++k) total += sh_warp_d[k];
+      const double target = static_cast<double>(sh_u2) * total;
+      int who;
+      double before;
+      block_pick(run, target, sh_warp_d, sh_hit, &sh_before_d, &who, &before);
+      if (tid == (who >= 0 ? who : 0)) {
+        int pick = -1, last = -1;
+        double cum = before, before_pick = before, before_last = before;
+        if (who >= 0) {
+          for (int t = t0; t < t1; ++t) {
+            const double wgt = seg_weight(t);
+            if (wgt > 0.0) { last = t; before_last = cum; }
             if (pick < 0 && cum + wgt > target && wgt > 0.0) { pick = t; before_pick = cum; }
             cum += wgt;
           }
-          if (pick < 0) { pick = last_pos; before_pick = before_last; }
+          if (pick < 0) { pick = last; before_pick = before_last; }
         }
-        sh_tile = pick;
-        sh_target = static_cast<float>(target - before_pick);
+        sh_seg = pick;
+        sh_target = target - before_pick;
         sh_token = -1;
       }
       __syncthreads();
-      const int tile = sh_tile;
-      if (tile >= 0) {
-        // recompute the rejected row's logits of that tile only, and the weights from them
-        const float4 lse = P.row_lse[r];
-        for (int j = warp; j < kLmN; j += nwarps) {
-          const int col = tile * kLmN + j;
-          float w = 0.f;
+      const int seg = sh_seg;
+      if (seg >= 0) {
+        // level 1, the segment's columns, two per thread
+        const int col0 = seg * kLmSeg + tid * 2;
+        float w[2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const int col = col0 + j;
+          w[j] = 0.f;
           if (col < P.V) {
-            const float z = lm_dot(F.hidden + static_cast<size_t>(r) * P.d, F.w_t + static_cast<size_t>(col) * P.d, P.d, lane);
-            const float p = ex2_approx(fmaf(z, c, -lse.z) - lse.w);
+            const float p = ex2_approx(fmaf(P.z[sr * P.ldz + col], c, -lse.z) - lse.w);
             const float q = ex2_approx(fmaf(Elem<__nv_bfloat16>::load(P.small + static_cast<size_t>(r) * P.V, col), c, -lse.x) - lse.y);
-            w = from_large ? p : fmaxf(p - q, 0.f);
+            w[j] = from_large ? p : fmaxf(p - q, 0.f);
           }
-          if (lane == 0) sh_w[j] = w;
         }
-        __syncthreads();
-        if (tid == 0) {
-          const float t3 = sh_target;
-          float run = 0.f;
-          int choice = -1, last_pos = -1;
-          for (int j = 0; j < kLmN; ++j) {
-            run += sh_w[j];
-            if (sh_w[j] > 0.f) {
-              last_pos = j;
-              if (choice < 0 && run > t3) choice = j;
-            }
-          }
-          if (choice < 0) choice = last_pos;
-          sh_token = (choice >= 0) ? tile * kLmN + choice : -1;
-        }
+        const float t3 = static_cast<float>(sh_target);
+        float before_f;
+        block_pick(w[0] + w[1], t3, sh_warp_f, sh_hit, &sh_before_f, &who, &before_f);
+        if (tid == who) sh_token = col0 + ((w[0] > 0.f && (before_f + w[0] > t3 || !(w[1] > 0.f))) ? 0 : 1);
         __syncthreads();
         next = sh_token;
       }

@@ -301,9 +301,9 @@ bool split_finalize(long long units, int V, bool bonus, const StreamScratch* ss)
 // A launch that may begin while the launch before it on the stream drains (programmatic dependent launch): the
 // kernel itself waits, with griddepcontrol.wait, before it reads what that launch wrote.
 template <typename Kernel, typename... Args>
-cudaError_t launch_dependent(Kernel kernel, unsigned grid, unsigned block, cudaStream_t stream, Args... args) {
+cudaError_t launch_dependent(Kernel kernel, dim3 grid, unsigned block, cudaStream_t stream, Args... args) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
+  cfg.gridDim = grid;
   cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = 0;
   cfg.stream = stream;
@@ -901,10 +901,28 @@ int pyramidsd_verify_fused_lmhead_ex(const psd_lmhead_args* args) {
   int rc = scratch_for(stream, &ss);
   if (rc != PSD_OK) return rc;
   std::lock_guard<std::mutex> lock(ss->mu);
-  const int n_tiles = (V + psd::kLmN - 1) / psd::kLmN;
-  const size_t per = static_cast<size_t>(M) * n_tiles;
-  const size_t bytes = align_up(per * sizeof(float2)) * 2 + align_up(per * sizeof(float4)) + align_up(static_cast<size_t>(M) * sizeof(float4)) +
-                       align_up(per * sizeof(float)) + align_up(static_cast<size_t>(M) * sizeof(float)) + kAlign;
+  int sms = psd::cluster_sm_count();
+  if (sms <= 0) sms = 1;
+  // the two-SM (cta_group::2) sweep is the default
+  const bool use_pair = args->tile_variant != PSD_LMHEAD_TILES_ONE_SM;
+  // Columns per tile of the pair: the weight is streamed in rounds of one tile per pair, so the width that leaves the
+  // fewest columns per pair in all is taken (V = 32000: two rounds of 224 instead of two of 256, the second of them
+  // two thirds full), the widest of equals, which reads the hidden matrix least often.
+  int tile_n = psd::kLmN;
+  if (use_pair) {
+    const int pairs_max = sms / 2 > 0 ? sms / 2 : 1;
+    long long best = 1ll << 60;
+    for (int n = psd::kLm2N; n >= 128; n -= 32) {   // a pair's MMA takes N in steps of 32
+      const long long tiles = (V + n - 1) / n, cost = (tiles + pairs_max - 1) / pairs_max * n;
+      if (cost < best) { best = cost; tile_n = n; }
+    }
+  }
+  const int n_tiles = (V + tile_n - 1) / tile_n, n_part = use_pair ? 2 * n_tiles : n_tiles, n_seg = (V + psd::kLmSeg - 1) / psd::kLmSeg;
+  const long long ldz = (static_cast<long long>(n_tiles) * tile_n + 31) / 32 * 32;
+  const int group_seqs = psd::kLmGroupRows / K < B ? psd::kLmGroupRows / K : B;   // K <= 32: whole sequences
+  const size_t rows_max = static_cast<size_t>(group_seqs) * K;
+  const size_t bytes = align_up(rows_max * ldz * sizeof(float)) + align_up(rows_max * n_part * sizeof(float2)) * 2 +
+                       align_up(rows_max * n_seg * sizeof(float4)) + align_up(rows_max * sizeof(float4)) + kAlign;
   rc = ensure_status(ss);
   if (rc != PSD_OK) return rc;
   t_last_scratch = ss; t_last_status = ss->status; t_last_stream = stream;
@@ -938,95 +956,66 @@ int pyramidsd_verify_fused_lmhead_ex(const psd_lmhead_args* args) {
   psd::LmParams L{};
   L.small = static_cast<const __nv_bfloat16*>(logits_small);
   L.tokens = tokens;
-  L.M = static_cast<int>(M); L.d = d_model; L.V = V; L.n_tiles = n_tiles;
+  L.d = d_model; L.V = V;
+  L.tile_n = tile_n; L.n_tiles = n_tiles; L.n_part = n_part; L.n_seg = n_seg;
+  L.w_once = M <= psd::kLmM ? 1 : 0;
+  L.ldz = ldz;
   L.c = 1.4426950408889634f;
-  L.part_large = reinterpret_cast<float2*>(ws); ws += align_up(per * sizeof(float2));
-  L.part_small = reinterpret_cast<float2*>(ws); ws += align_up(per * sizeof(float2));
-  L.part_div = reinterpret_cast<float4*>(ws); ws += align_up(per * sizeof(float4));
-  L.row_lse = reinterpret_cast<float4*>(ws); ws += align_up(static_cast<size_t>(M) * sizeof(float4));
+  L.z = reinterpret_cast<float*>(ws); ws += align_up(rows_max * ldz * sizeof(float));
+  L.part_large = reinterpret_cast<float2*>(ws); ws += align_up(rows_max * n_part * sizeof(float2));
+  L.part_small = reinterpret_cast<float2*>(ws); ws += align_up(rows_max * n_part * sizeof(float2));
+  L.part_div = reinterpret_cast<float4*>(ws); ws += align_up(rows_max * n_seg * sizeof(float4));
+  L.row_lse = reinterpret_cast<float4*>(ws);
   L.status = ss->status;
-  if (kl) {
-    L.part_t = reinterpret_cast<float*>(ws); ws += align_up(per * sizeof(float));
-    L.row_div = reinterpret_cast<float*>(ws); ws += align_up(static_cast<size_t>(M) * sizeof(float));
-    L.need_sweep2 = reinterpret_cast<int*>(ws);
-    // the residual masses are wanted as an output: the second sweep runs whatever the accept scan finds
-    if (cudaMemsetAsync(L.need_sweep2, out_resid_mass != nullptr ? 1 : 0, sizeof(int), stream) != cudaSuccess) return PSD_ERR_CUDA;
-  }
   static bool attr_set[kMaxDevices] = {};
   int dev = 0;
   cudaGetDevice(&dev);
   if (!attr_set[dev]) {
     const int one = static_cast<int>(psd::kLmSmemBytes), two = static_cast<int>(psd::kLm2SmemBytes);
     const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    if (cudaFuncSetAttribute(psd::lmhead_sweep_kernel<1, false>, at, one) != cudaSuccess ||
-        cudaFuncSetAttribute(psd::lmhead_sweep_kernel<1, true>, at, one) != cudaSuccess ||
-        cudaFuncSetAttribute(psd::lmhead_sweep_kernel<2, false>, at, one) != cudaSuccess ||
-        cudaFuncSetAttribute(psd::lmhead_sweep2sm_kernel<1, false>, at, two) != cudaSuccess ||
-        cudaFuncSetAttribute(psd::lmhead_sweep2sm_kernel<1, true>, at, two) != cudaSuccess ||
-        cudaFuncSetAttribute(psd::lmhead_sweep2sm_kernel<2, false>, at, two) != cudaSuccess) {
+    if (cudaFuncSetAttribute(psd::lmhead_sweep_kernel, at, one) != cudaSuccess ||
+        cudaFuncSetAttribute(psd::lmhead_sweep2sm_kernel, at, two) != cudaSuccess) {
       cudaGetLastError();
       return PSD_ERR_CUDA;
     }
     attr_set[dev] = true;
   }
-  int sms = psd::cluster_sm_count();
-  if (sms <= 0) sms = 1;
-  // the two-SM (cta_group::2) sweeps are the default
-  const bool use_pair = args->tile_variant != PSD_LMHEAD_TILES_ONE_SM;
-  CUtensorMap map_a2, map_b2;   // the pair's A / B boxes are 64 x 128
+  CUtensorMap map_a2, map_b2;   // the pair's boxes: 64 x 128 of A, 64 x half a tile's columns of B
   if (use_pair) {
     const cuuint64_t dims_a[2] = {static_cast<cuuint64_t>(d_model), static_cast<cuuint64_t>(M)};
     const cuuint64_t dims_b[2] = {static_cast<cuuint64_t>(d_model), static_cast<cuuint64_t>(V)};
     const cuuint64_t strides[1] = {static_cast<cuuint64_t>(d_model) * 2};
-    const cuuint32_t box[2] = {psd::kLmK, 128}, estr[2] = {1, 1};
+    const cuuint32_t box[2] = {psd::kLmK, 128}, box_b[2] = {psd::kLmK, static_cast<cuuint32_t>(tile_n / 2)}, estr[2] = {1, 1};
     if (encode(&map_a2, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(hidden), dims_a, strides, box, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) return PSD_ERR_CUDA;
-    if (encode(&map_b2, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(w_t), dims_b, strides, box, estr,
+    if (encode(&map_b2, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(w_t), dims_b, strides, box_b, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) return PSD_ERR_CUDA;
   }
-  const int n_tiles2 = (n_tiles + 1) / 2;
-  const int pairs = n_tiles2 < sms / 2 ? n_tiles2 : sms / 2;
-  const unsigned grid_one = static_cast<unsigned>(n_tiles < sms ? n_tiles : sms);
-  // one GEMM sweep over every block of 256 rows (the weight is streamed once per block and sweep)
-  auto launch_sweep = [&](int sweep) -> bool {
+  const int pairs = n_tiles < sms / 2 ? n_tiles : sms / 2;
+  // the GEMM over one block of 256 rows
+  auto launch_sweep = [&]() -> cudaError_t {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
-    if (use_pair) {
-      cfg.gridDim = dim3(static_cast<unsigned>(2 * (pairs > 0 ? pairs : 1)));
-      cfg.dynamicSmemBytes = psd::kLm2SmemBytes;
-      at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-      cfg.attrs = at;
-      cfg.numAttrs = 1;
-    } else {
-      cfg.gridDim = dim3(grid_one);
-      cfg.dynamicSmemBytes = psd::kLmSmemBytes;
-    }
     cfg.blockDim = dim3(psd::kLmThreads);
     cfg.stream = stream;
-    for (int r0 = 0; r0 < M; r0 += psd::kLmM) {
-      L.row0 = r0;
-      cudaError_t e;
-      if (use_pair) {
-        if (sweep == 2) e = cudaLaunchKernelEx(&cfg, psd::lmhead_sweep2sm_kernel<2, false>, map_a2, map_b2, L);
-        else if (kl) e = cudaLaunchKernelEx(&cfg, psd::lmhead_sweep2sm_kernel<1, true>, map_a2, map_b2, L);
-        else e = cudaLaunchKernelEx(&cfg, psd::lmhead_sweep2sm_kernel<1, false>, map_a2, map_b2, L);
-      } else {
-        if (sweep == 2) e = cudaLaunchKernelEx(&cfg, psd::lmhead_sweep_kernel<2, false>, map_a, map_b, L);
-        else if (kl) e = cudaLaunchKernelEx(&cfg, psd::lmhead_sweep_kernel<1, true>, map_a, map_b, L);
-        else e = cudaLaunchKernelEx(&cfg, psd::lmhead_sweep_kernel<1, false>, map_a, map_b, L);
-      }
-      if (e != cudaSuccess) { cudaGetLastError(); return false; }
+    if (!use_pair) {
+      cfg.gridDim = dim3(static_cast<unsigned>(n_tiles < sms ? n_tiles : sms));
+      cfg.dynamicSmemBytes = psd::kLmSmemBytes;
+      return cudaLaunchKernelEx(&cfg, psd::lmhead_sweep_kernel, map_a, map_b, L);
     }
-    L.row0 = 0;
-    return true;
+    cfg.gridDim = dim3(static_cast<unsigned>(2 * (pairs > 0 ? pairs : 1)));
+    cfg.dynamicSmemBytes = psd::kLm2SmemBytes;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, psd::lmhead_sweep2sm_kernel, map_a2, map_b2, L);
   };
   psd::LmFinalParams F{};
-  F.hidden = static_cast<const __nv_bfloat16*>(hidden);
-  F.w_t = static_cast<const __nv_bfloat16*>(w_t);
-  F.B = B; F.K = K;
+  F.K = K;
+  F.div_kind = args->div_kind;
   F.threshold = threshold;
   F.mode = mode;
   F.seed = philox_seed; F.offset = offset;
@@ -1035,28 +1024,37 @@ int pyramidsd_verify_fused_lmhead_ex(const psd_lmhead_args* args) {
   F.out_next_token = out_next_token;
   F.out_div = out_div;
   F.out_resid = out_resid_mass;
-  uint64_t launches = 0;
-  {
-    TimedLaunch timed(stream, 0);
-    if (!launch_sweep(1)) return PSD_ERR_CUDA;
-    psd::lmhead_reduce_kernel<<<static_cast<unsigned>((M + 7) / 8), 256, 0, stream>>>(L);
-    if (kl) {
-      // Kullback-Leibler: the divergences are known after one sweep. The accept scan says whether any rejected row
-      // needs residual masses; only then does the second sweep do anything.
-      F.lm = L;
-      F.kl_phase = 1;
-      psd::lmhead_final_kernel<<<static_cast<unsigned>(B), 256, 0, stream>>>(F);
-      ++launches;
+  for (int b0 = 0; b0 < B; b0 += group_seqs) {
+    const int nb = B - b0 < group_seqs ? B - b0 : group_seqs, rows = nb * K;
+    L.grp0 = b0 * K;
+    L.M = L.grp0 + rows;
+    // the terms kernel: a CTA for every resident place, unless that left its warps without a segment each
+    const long long items = static_cast<long long>(rows) * n_seg;
+    const int warps = psd::kLmTermThreads / 32, places = psd::kLmTermCtas * sms;
+    long long ctas = (items + warps - 1) / warps;
+    if (ctas > places) ctas = places;
+    const int per_cta = static_cast<int>((items + ctas - 1) / ctas);
+    const dim3 grid(static_cast<unsigned>((items + per_cta - 1) / per_cta));
+    cudaError_t e = cudaSuccess;
+    {
+      TimedLaunch timed(stream, 0);
+      for (L.row0 = L.grp0; L.row0 < L.M && e == cudaSuccess; L.row0 += psd::kLmM) {
+        e = launch_sweep();
+        g_launches.fetch_add(1, std::memory_order_relaxed);
+      }
+      if (e == cudaSuccess)
+        e = kl ? launch_dependent(psd::lmhead_terms_kernel<psd::kDivKL>, grid, psd::kLmTermThreads, stream, L, per_cta)
+               : launch_dependent(psd::lmhead_terms_kernel<psd::kDivJS>, grid, psd::kLmTermThreads, stream, L, per_cta);
     }
-    if (!launch_sweep(2)) return PSD_ERR_CUDA;
+    F.lm = L;
+    F.b0 = b0;
+    if (e == cudaSuccess) {
+      TimedLaunch timed(stream, 1);
+      e = launch_dependent(psd::lmhead_final_kernel, dim3(static_cast<unsigned>(nb)), psd::kLmFinalThreads, stream, F);
+    }
+    g_launches.fetch_add(2, std::memory_order_relaxed);
+    if (e != cudaSuccess) { cudaGetLastError(); return PSD_ERR_CUDA; }
   }
-  F.lm = L;
-  F.kl_phase = kl ? 2 : 0;
-  {
-    TimedLaunch timed(stream, 1);
-    psd::lmhead_final_kernel<<<static_cast<unsigned>(B), 256, 0, stream>>>(F);
-  }
-  g_launches.fetch_add(launches + 2 + 2 * static_cast<uint64_t>((M + psd::kLmM - 1) / psd::kLmM), std::memory_order_relaxed);
   return check_launch();
 }
 

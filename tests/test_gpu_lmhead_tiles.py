@@ -1,0 +1,49 @@
+"""The LM-head form at the edges of its own cuts: tile widths other than 256 (two rounds of narrower tiles), segments of
+512 columns, rows that end a 256-row block or a group of 1024, against the oracle on the sequences sampled."""
+import numpy as np
+import pytest
+import torch
+
+from parity_utils import TOL
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,K,d,V", [(1, 1, 64, 100), (2, 3, 128, 511), (2, 3, 128, 513), (3, 5, 64, 16352), (32, 8, 64, 18945), (43, 6, 64, 2049),
+                                     (130, 8, 64, 1000)])
+def test_divergences_and_tokens(oracle, B, K, d, V):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2510_12966_b200 import binding as psd, workloads as wl
+    h, w_t, zs, tok = wl.make_fused_inputs(B, K, V, d, 40 + V, 0.7, device=torch.device("cuda"))
+    for mode, tau in ((psd.FUZZY, 0.03), (psd.ASSISTED, 0.0)):
+        out = psd.verify_fused_lmhead(h, w_t, zs, tok, tau, mode, 3, 1)
+        assert psd.last_status() == 0
+        # the same logits as a library GEMM in fp32 of the same bf16 operands gives
+        z = (h.float() @ w_t.float().T).view(B, K, V)
+        p, q = torch.softmax(z.double(), -1), torch.softmax(zs.double(), -1)
+        m = 0.5 * (p + q)
+        js = 0.5 * (torch.special.xlogy(p, p / m) + torch.special.xlogy(q, q / m)).nan_to_num(0.0).sum(-1)
+        assert (out["div"].double() - js).abs().max() < 2e-5
+        assert (out["resid_mass"].double() - (p - q).clamp(min=0).sum(-1)).abs().max() < 2e-5
+        L, nxt = out["accept_len"].cpu(), out["next_token"].cpu()
+        if mode == psd.FUZZY:
+            acc = (js.cpu() <= tau).int().cumprod(-1).sum(-1)
+            near = ((js.cpu() - tau).abs() < 1e-5).any(-1)
+            assert torch.equal(L[~near], acc.to(torch.int32)[~near])
+        ties = 0
+        for b in range(B):
+            k = int(L[b])
+            if k == K:
+                assert int(nxt[b]) == -1
+                continue
+            w = p[b, k] if mode == psd.ASSISTED else (p[b, k] - q[b, k]).clamp(min=0)
+            c = torch.cumsum(w, 0).cpu()
+            _, u2 = oracle.row_uniforms(3, 1, b * K + k)
+            t = u2 * float(c[-1])
+            x = int(nxt[b])
+            lo = float(c[x - 1]) if x else 0.0
+            slack = TOL["bf16"]["cdf"] * float(c[-1])   # the weights are fp32, the sums the library's
+            assert lo - slack <= t <= float(c[x]) + slack and float(w[x]) > 0
+            ties += not (lo <= t < float(c[x]))
+        assert ties <= max(1, B // 8)
