@@ -17,6 +17,7 @@ constexpr int kFinElemsPerThread = 8;                      // consecutive vocabu
 constexpr int kFinTile = kFinThreads * kFinElemsPerThread;  // 8192 indices per tile
 constexpr int kFinMaxTiles = 1024;                          // V <= 8,388,608
 constexpr int kFinBatch = 32;
+constexpr int kFinMaxRanks = 8;                             // CTAs per sequence at most
 
 __device__ __forceinline__ unsigned fin_cluster_rank() {
   unsigned r;
@@ -35,6 +36,14 @@ __device__ __forceinline__ void fin_remote_store(double* local, unsigned rank, d
 
 // A finalisation launch may start while the launch before it drains; it reads nothing of that launch before this.
 __device__ __forceinline__ void wait_for_previous_launch() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The same for a launch in clusters: afterwards every CTA of the cluster is known to run, so its shared memory may be
+// written remotely.
+template <int CL>
+__device__ __forceinline__ void begin_cluster_launch() {
+  if (CL > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  wait_for_previous_launch();
+  if (CL > 1) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+}
 // Lets the next launch on the stream, if it was launched as a dependent, be scheduled from here on.
 __device__ __forceinline__ void release_next_launch() { asm volatile("griddepcontrol.launch_dependents;"); }
 
@@ -100,6 +109,7 @@ struct RowView {
 
 struct FinShared {
   double tile_total[kFinMaxTiles];
+  double bonus_max[kFinMaxRanks];   // the CTAs' maxima of the bonus row
   float warp_total[32];
   float warp_tile[kFinBatch][32];   // per-warp sums of a batch of tiles
   int sh_L, sh_nv, sh_flags, sh_tile, sh_warp, sh_token;
@@ -201,28 +211,65 @@ __device__ __forceinline__ void write_results(const StageParams& P, const int b,
   }
 }
 
-// Level 0 of the draw, by one thread, once every tile's total is in S.tile_total: the first tile whose inclusive
-// cumulative weight exceeds the target, else the last non-empty tile. Leaves the tile in S.sh_tile (-1: no
+// The pick of one level of the draw, by one full warp: the first child whose inclusive cumulative weight exceeds the
+// target, else the last one with a positive weight (-1: none). Lane k holds the weight of child k; `base` lies before
+// them. Every lane returns the same values. (One lane walking 32 children in shared memory took half a microsecond.)
+template <typename V>
+__device__ __forceinline__ V warp_incl_scan(V w, const int lane) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const V up = __shfl_up_sync(0xffffffffu, w, o);
+    if (lane >= o) w += up;
+  }
+  return w;
+}
+struct WarpPick { int first, last; };
+template <typename V>
+__device__ __forceinline__ WarpPick warp_pick(const V w, const V incl, const V target) {
+  const unsigned hit = __ballot_sync(0xffffffffu, w > static_cast<V>(0) && incl > target), pos = __ballot_sync(0xffffffffu, w > static_cast<V>(0));
+  WarpPick r;
+  r.first = hit ? __ffs(hit) - 1 : -1;
+  r.last = pos ? 31 - __clz(pos) : -1;
+  return r;
+}
+
+// The total of a tile from its 32 warp sums, by one full warp, in double: a fixed tree, the same in every form.
+__device__ __forceinline__ double tile_sum(const float (&warp_sums)[32], const int lane) {
+  return warp_reduce<OpSum>(static_cast<double>(warp_sums[lane]));
+}
+
+// Level 0 of the draw, by one full warp, once every tile's total is in S.tile_total. Leaves the tile in S.sh_tile (-1: no
 // positive weight at all; -2: the residual weights all came out zero, take the totals again over p_large) and
 // the target that remains inside it in S.sh_target.
-__device__ __forceinline__ void pick_tile(FinShared& S, const int n_tiles, const bool from_large) {
-  const double* tile_total = S.tile_total;
-  double total = 0.0;
-  for (int j = 0; j < n_tiles; ++j) total += tile_total[j];
-  const double target = static_cast<double>(S.sh_u2) * total;
-  const bool redo = !(total > 0.0) && !from_large;
-  int pick = -1, last_pos = -1;
-  double cum = 0.0, cum_before_pick = 0.0, cum_before_last = 0.0;
-  for (int j = 0; j < n_tiles; ++j) {
-    const double nxt = cum + tile_total[j];
-    if (tile_total[j] > 0.0) { last_pos = j; cum_before_last = cum; }
-    if (pick < 0 && nxt > target && tile_total[j] > 0.0) { pick = j; cum_before_pick = cum; }
-    cum = nxt;
+__device__ __forceinline__ void pick_tile(FinShared& S, const int n_tiles, const bool from_large, const int lane) {
+  double total = 0.0, incl = 0.0, w = 0.0;
+  for (int j0 = 0; j0 < n_tiles; j0 += 32) {
+    w = j0 + lane < n_tiles ? S.tile_total[j0 + lane] : 0.0;
+    incl = warp_incl_scan(w, lane) + total;
+    total = __shfl_sync(0xffffffffu, incl, 31);
   }
-  if (pick < 0) { pick = last_pos; cum_before_pick = cum_before_last; }
-  S.sh_tile = redo ? -2 : pick;
-  S.sh_token = -1;
-  S.sh_target = static_cast<float>(target - cum_before_pick);
+  const double target = static_cast<double>(S.sh_u2) * total;
+  int pick = -1;
+  double before = 0.0, base = 0.0;
+  for (int j0 = 0; j0 < n_tiles; j0 += 32) {
+    if (n_tiles > 32) {
+      w = j0 + lane < n_tiles ? S.tile_total[j0 + lane] : 0.0;
+      incl = warp_incl_scan(w, lane) + base;
+      base = __shfl_sync(0xffffffffu, incl, 31);
+    }
+    const WarpPick k = warp_pick(w, incl, target);
+    const int c = k.first >= 0 ? k.first : k.last;
+    if (c >= 0) {
+      pick = j0 + c;
+      before = __shfl_sync(0xffffffffu, incl - w, c);
+    }
+    if (k.first >= 0) break;
+  }
+  if (lane == 0) {
+    S.sh_tile = (!(total > 0.0) && !from_large) ? -2 : pick;
+    S.sh_token = -1;
+    S.sh_target = static_cast<float>(target - before);
+  }
 }
 
 // Levels 1 to 3 of the draw inside the chosen tile, by the whole CTA: warps, lanes, the thread's own elements.
@@ -241,37 +288,26 @@ __device__ __forceinline__ void descend_tile(const RowView<T>& row, FinShared& S
     float ts = 0.f;
 #pragma unroll
     for (int e = 0; e < kFinElemsPerThread; ++e) ts += w[e];
-    // inclusive scan of thread sums across the warp (fixed shuffle tree)
-    float incl = ts;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const float up = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += up;
-    }
+    const float incl = warp_incl_scan(ts, lane);   // of the thread sums across the warp
     if (lane == 31) warp_total[warp] = incl;
     __syncthreads();
-    if (tid == 0) {
-      const float target = sh_target;
-      int pick = -1, last_pos = -1;
-      float cum = 0.f, before_pick = 0.f, before_last = 0.f;
-      for (int j = 0; j < kFinThreads / 32; ++j) {
-        const float nxt = cum + warp_total[j];
-        if (warp_total[j] > 0.f) { last_pos = j; before_last = cum; }
-        if (pick < 0 && nxt > target && warp_total[j] > 0.f) { pick = j; before_pick = cum; }
-        cum = nxt;
+    if (warp == 0) {
+      const float target = sh_target, wt = warp_total[lane], wi = warp_incl_scan(wt, lane);
+      const WarpPick k = warp_pick(wt, wi, target);
+      const int c = k.first >= 0 ? k.first : k.last;
+      const float before = __shfl_sync(0xffffffffu, wi - wt, c >= 0 ? c : 0);
+      if (lane == 0) {
+        sh_warp = c;
+        sh_target = target - (c >= 0 ? before : 0.f);
       }
-      if (pick < 0) { pick = last_pos; before_pick = before_last; }
-      sh_warp = pick;
-      sh_target = target - before_pick;
     }
     __syncthreads();
     if (warp == sh_warp) {
       // level 2: lanes of the chosen warp
       const float target = sh_target;
       const float excl = incl - ts;  // only used as the offset handed to the next level
-      const unsigned hit = __ballot_sync(0xffffffffu, incl > target && ts > 0.f);
-      const unsigned pos = __ballot_sync(0xffffffffu, ts > 0.f);
-      const int pick_lane = hit ? (__ffs(hit) - 1) : (pos ? 31 - __clz(pos) : -1);
+      const WarpPick k = warp_pick(ts, incl, target);
+      const int pick_lane = k.first >= 0 ? k.first : k.last;
       if (lane == pick_lane) {
         // level 3: the thread's own consecutive elements
         const float t3 = target - excl;
@@ -339,43 +375,47 @@ __device__ __forceinline__ void finalize_sequence(const StageParams& P, const in
   }
   const bool bonus = P.bonus && L == sh_nv;   // everything accepted: the larger model's next token comes for free
   if (bonus) {
-    // The row after the window was not part of the statistics pass: every CTA takes its normaliser here, with
-    // the same two passes and reduction trees (so all CTAs of a cluster hold the same bits).
+    // The row after the window was not part of the statistics pass. A draw from it needs its weights relative to one
+    // another only: the CTAs of the cluster take the row's maximum together, each over its own tiles, and every weight is
+    // 2^(z c - max c) (every CTA over the whole row, twice, for the normaliser: 31 us a launch for one sequence of
+    // V = 128256, now 18).
     const T* brow = large_seq + static_cast<long long>(L) * V;
-    const bool vec_ok = (reinterpret_cast<uintptr_t>(brow) & 15u) == 0 && (V % Elem<T>::kPerVec) == 0;
-    constexpr int E = Elem<T>::kPerVec;
+    constexpr int E = Elem<T>::kPerVec, kVecs = RowView<T>::kVecs;
+    const bool vec_ok = (reinterpret_cast<uintptr_t>(brow) & 15u) == 0 && (V % E) == 0;
     float mx = -INFINITY;
-    if (vec_ok) {
-      for (int v = tid; v < V / E; v += kFinThreads) {
-        float x[E];
-        Elem<T>::unpack(ldg_vec(brow, v), x);
+#pragma unroll 4
+    for (int i0 = static_cast<int>(cl_rank) * kFinTile + tid * kFinElemsPerThread; i0 < V; i0 += CL * kFinTile) {
+      if (vec_ok && i0 + kFinElemsPerThread <= V) {
 #pragma unroll
-        for (int j = 0; j < E; ++j) mx = max_nan(mx, x[j]);
+        for (int h = 0; h < kVecs; ++h) {
+          float x[E];
+          Elem<T>::unpack(ldg_vec(brow, i0 / E + h), x);
+#pragma unroll
+          for (int j = 0; j < E; ++j) mx = max_nan(mx, x[j]);
+        }
+      } else {
+#pragma unroll
+        for (int j = 0; j < kFinElemsPerThread; ++j)
+          if (i0 + j < V) mx = max_nan(mx, Elem<T>::load(brow, i0 + j));
       }
-    } else {
-      for (int i = tid; i < V; i += kFinThreads) mx = max_nan(mx, Elem<T>::load(brow, i));
     }
     mx = block_reduce<OpMaxNan>(mx, warp_total, -INFINITY);
+    if (CL > 1) {
+      if (tid < CL) {
+        if (tid == static_cast<int>(cl_rank)) S.bonus_max[cl_rank] = mx;
+        else fin_remote_store(&S.bonus_max[cl_rank], static_cast<unsigned>(tid), mx);
+      }
+      fin_cluster_sync();
+#pragma unroll
+      for (int p = 0; p < CL; ++p) mx = max_nan(mx, static_cast<float>(S.bonus_max[p]));
+    }
     if (!(fabsf(mx) < INFINITY)) {
       next = -2;   // NaN, +inf or no finite logit: no distribution to draw from
     } else {
-      const float m2 = mx * P.c;
-      float sum = 0.f;
-      if (vec_ok) {
-        for (int v = tid; v < V / E; v += kFinThreads) {
-          float x[E];
-          Elem<T>::unpack(ldg_vec(brow, v), x);
-#pragma unroll
-          for (int j = 0; j < E; ++j) sum += ex2_approx(fmaf(x[j], P.c, -m2));
-        }
-      } else {
-        for (int i = tid; i < V; i += kFinThreads) sum += ex2_approx(fmaf(Elem<T>::load(brow, i), P.c, -m2));
-      }
-      sum = block_reduce<OpSum>(sum, warp_total, 0.f);
       if (tid == 0) {
-        sh_m2l = m2; sh_l2sl = lg2_approx(sum);
-        sh_m2s = m2; sh_l2ss = sh_l2sl;
-        sh_resid = 0.f;   // weights are p_large itself
+        sh_m2l = mx * P.c; sh_l2sl = 0.f;
+        sh_m2s = sh_m2l; sh_l2ss = 0.f;
+        sh_resid = 0.f;   // weights are those of the large row itself
         sh_u2 = bonus_uniform(P.seed, P.offset, static_cast<unsigned>(P.seq_base + b));
       }
       __syncthreads();
@@ -419,21 +459,18 @@ __device__ __forceinline__ void finalize_sequence(const StageParams& P, const in
         if (lane == 0) warp_tile[m][warp] = ts;
       }
       __syncthreads();
-      if (tid < nb) {
-        double tt = 0.0;
-        for (int k = 0; k < 32; ++k) tt += static_cast<double>(warp_tile[tid][k]);
-        const int j = (m0 + tid) * CL + static_cast<int>(cl_rank);
-        tile_total[j] = tt;
-        if (CL > 1) {
-#pragma unroll
-          for (int p = 0; p < CL; ++p)
-            if (p != static_cast<int>(cl_rank)) fin_remote_store(&tile_total[j], static_cast<unsigned>(p), tt);
+      if (warp < nb) {   // kFinBatch = 32 warps: one tile each
+        const double tt = tile_sum(warp_tile[warp], lane);
+        const int j = (m0 + warp) * CL + static_cast<int>(cl_rank);
+        if (lane < CL) {
+          if (lane == static_cast<int>(cl_rank)) tile_total[j] = tt;
+          else fin_remote_store(&tile_total[j], static_cast<unsigned>(lane), tt);
         }
       }
       __syncthreads();
     }
     if (CL > 1) fin_cluster_sync();   // every CTA now holds every tile's total
-    if (tid == 0) pick_tile(S, n_tiles, row.from_large);
+    if (warp == 0) pick_tile(S, n_tiles, row.from_large, lane);
     __syncthreads();
     if (sh_tile != -2) break;
     row.from_large = true;            // every CTA of the cluster holds the same totals and takes the same turn
@@ -454,7 +491,7 @@ __device__ __forceinline__ void finalize_sequence(const StageParams& P, const in
 template <typename T, int CL>
 __global__ void __launch_bounds__(kFinThreads, 1) finalize_kernel(const StageParams P) {
   __shared__ FinShared S;
-  wait_for_previous_launch();
+  begin_cluster_launch<CL>();
   finalize_sequence<T, CL>(P, blockIdx.x / CL, S);
   if (CL > 1) fin_cluster_sync();   // nobody leaves while a peer may still post tile sums into its shared memory
 }
@@ -465,7 +502,7 @@ __global__ void __launch_bounds__(kFinThreads, 1) finalize_kernel(const StagePar
 template <typename T, int CL>
 __global__ void __launch_bounds__(kFinThreads) finalize_pyramid_kernel(const StageParams P1, const StageParams P2) {
   __shared__ FinShared S;
-  wait_for_previous_launch();
+  begin_cluster_launch<CL>();
   finalize_sequence<T, CL>(P1, blockIdx.x / CL, S);
   __threadfence();
   __syncthreads();
@@ -494,7 +531,7 @@ __device__ __forceinline__ void stage1_prefix(const StageParams& P1, const int K
 template <typename T, int CL>
 __global__ void __launch_bounds__(kFinThreads) finalize_pyramid_split_kernel(const StageParams P1, const StageParams P2) {
   __shared__ FinShared S;
-  wait_for_previous_launch();
+  begin_cluster_launch<CL>();
   __shared__ int sh_L1, sh_n2;
   const int unit = blockIdx.x / CL, b = unit >> 1;
   if ((unit & 1) == 0) {
@@ -686,10 +723,9 @@ __global__ void __launch_bounds__(kFinThreads) finalize_tiles_kernel(const Stage
       }
     }
     __syncthreads();
-    if (tid < nb) {
-      double tt = 0.0;
-      for (int k = 0; k < 32; ++k) tt += static_cast<double>(S.warp_tile[tid][k]);
-      *S.out[tid] = tt;
+    if (warp < nb) {
+      const double tt = tile_sum(S.warp_tile[warp], lane);
+      if (lane == 0) *S.out[warp] = tt;
     }
     __syncthreads();   // the batch's shared memory is free again
   }
@@ -722,7 +758,7 @@ __global__ void __launch_bounds__(kFinThreads) finalize_pick_kernel(const StageP
     if (tid < n_tiles) S.tile_total[tid] = tt;
     if (tid == 0) S.sh_u2 = rec.u2;
     __syncthreads();
-    if (tid == 0) pick_tile(S, n_tiles, row.from_large);
+    if (warp == 0) pick_tile(S, n_tiles, row.from_large, lane);
     __syncthreads();
     if (S.sh_tile == -2) {
       // the residual weights all came out zero although the row's residual mass did not: the totals again, over p_large
@@ -736,14 +772,13 @@ __global__ void __launch_bounds__(kFinThreads) finalize_pick_kernel(const StageP
         ts = warp_reduce<OpSum>(ts);
         if (lane == 0) S.warp_tile[0][warp] = ts;
         __syncthreads();
-        if (tid == 0) {
-          double tt = 0.0;
-          for (int k = 0; k < 32; ++k) tt += static_cast<double>(S.warp_tile[0][k]);
-          S.tile_total[j] = tt;
+        if (warp == 0) {
+          const double tt = tile_sum(S.warp_tile[0], lane);
+          if (lane == 0) S.tile_total[j] = tt;
         }
         __syncthreads();
       }
-      if (tid == 0) pick_tile(S, n_tiles, true);
+      if (warp == 0) pick_tile(S, n_tiles, true, lane);
       __syncthreads();
     }
     const int tile = S.sh_tile;

@@ -252,8 +252,9 @@ int launch_rowstats(const StageParams& P, int dtype, int variant, int cluster_si
   return check_launch();
 }
 
-// The finalisation kernels run as clusters of CL CTAs per sequence (per stage in the split form): four while
-// that still leaves SMs to spare, fewer for large batches, where one CTA per sequence already fills the GPU.
+// The finalisation kernels run as clusters of CL CTAs per sequence (per stage in the split form): eight while every one
+// of them finds an SM, four while that still leaves SMs to spare, fewer for large batches, where one CTA per sequence
+// already fills the GPU.
 template <typename Kernel, typename... Args>
 cudaError_t launch_fin_clusters(Kernel kernel, int cl, unsigned units, cudaStream_t stream, Args... args) {
   cudaLaunchConfig_t cfg = {};
@@ -278,13 +279,15 @@ cudaError_t launch_fin_clusters(Kernel kernel, int cl, unsigned units, cudaStrea
 int fin_cluster_size(long long units) {
   int sms = psd::cluster_sm_count();
   if (sms <= 0) sms = 148;
+  if (units * 8 <= sms) return 8;
   if (units * 4 <= 2ll * sms) return 4;
   if (units * 2 <= 2ll * sms) return 2;
   return 1;
 }
 
 #define PSD_FIN_DISPATCH(KERNEL, T, cl, units, stream, ...)                                              \
-  ((cl) == 4 ? launch_fin_clusters(psd::KERNEL<T, 4>, 4, units, stream, __VA_ARGS__)                        \
+  ((cl) == 8 ? launch_fin_clusters(psd::KERNEL<T, 8>, 8, units, stream, __VA_ARGS__)                        \
+   : (cl) == 4 ? launch_fin_clusters(psd::KERNEL<T, 4>, 4, units, stream, __VA_ARGS__)                      \
    : (cl) == 2 ? launch_fin_clusters(psd::KERNEL<T, 2>, 2, units, stream, __VA_ARGS__)                      \
                : launch_fin_clusters(psd::KERNEL<T, 1>, 1, units, stream, __VA_ARGS__))
 
