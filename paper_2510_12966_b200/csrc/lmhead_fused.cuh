@@ -11,7 +11,7 @@
 //   terms    per (row, 512-column segment): divergence terms, residual mass and mass of p from both models' logits
 //   final    per sequence: row totals, accept bits, accepted prefix, and the residual draw: the segment is found
 //            from the per-segment masses, the token from that segment's logits
-// Measured, whole call: 551 -> 392 us at that size, 99.5 -> 50.4 us at M = 15, d = 2048, V = 32000, against two runs of
+// Measured, whole call: 607 -> 370 us at that size, 99.8 -> 50.6 us at M = 15, d = 2048, V = 32000, against two runs of
 // the GEMM with the terms in the second one's epilogue.
 //
 // One CTA = 10 warps: warp 0 lane 0 issues TMA loads, warp 1 lane 0 issues the MMAs (and owns the tensor
@@ -484,9 +484,10 @@ lmhead_sweep2sm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
 // a run touches a row or two. For each row the CTA merges the (max, sum) partials (a few KB out of L2, the same fixed
 // tree in every CTA, so all of a row's CTAs hold the same bits; a launch of its own for it took 15 us), then each
 // warp takes segment after segment, a lane four times four consecutive columns, so that 96 bytes per lane are in
-// flight. Memory-bound: 6 bytes per column.
+// flight while the 96 before are worked on. Memory-bound: 6 bytes per column, 197 MB in 46 us at M = 256, V = 128256
+// (56 us without the second set of registers, at four CTAs per SM).
 constexpr int kLmTermThreads = 256;
-constexpr int kLmTermCtas = 4;       // resident per SM
+constexpr int kLmTermCtas = 3;       // resident per SM
 
 __device__ __forceinline__ void lse_merge_warp(float& m, float& s) {
 #pragma unroll
@@ -528,59 +529,78 @@ __global__ void __launch_bounds__(kLmTermThreads, kLmTermCtas) lmhead_terms_kern
     const float* zrow = P.z + srow * P.ldz;
     const __nv_bfloat16* xrow = P.small + static_cast<size_t>(P.grp0 + srow) * P.V;
     const bool x_vec = (reinterpret_cast<uintptr_t>(xrow) & 7u) == 0;
-    for (int seg = seg0 + warp; seg < seg_end; seg += kWarps) {
-      const int col0 = seg * kLmSeg + lane * 4;
-      float4 z4[4];
-      uint2 x4[4];
-      const bool whole = x_vec && (seg + 1) * kLmSeg <= P.V;
-      if (whole) {
+    // a segment's vectors are asked for before the one before it is worked on
+    float4 z4[2][4];
+    uint2 x4[2][4];
+    auto fetch = [&](int seg, float4 (&fz)[4], uint2 (&fx)[4]) {
+      if (seg < seg_end && x_vec && (seg + 1) * kLmSeg <= P.V) {
 #pragma unroll
         for (int h = 0; h < 4; ++h) {
-          z4[h] = __ldcg(reinterpret_cast<const float4*>(zrow + col0 + h * 128));   // written by the launch before
-          x4[h] = __ldg(reinterpret_cast<const uint2*>(xrow + col0 + h * 128));
+          fz[h] = __ldcg(reinterpret_cast<const float4*>(zrow + seg * kLmSeg + h * 128 + lane * 4));   // written by the launch before
+          fx[h] = __ldg(reinterpret_cast<const uint2*>(xrow + seg * kLmSeg + h * 128 + lane * 4));
         }
-      }
-      float js = 0.f, resid = 0.f, pmass = 0.f;
+      } else if (seg < seg_end) {   // the row's last segment, or logits that do not start at 8 bytes
 #pragma unroll
-      for (int h = 0; h < 4; ++h) {
-        float z[4], x[4];
-        if (whole) {
-          z[0] = z4[h].x; z[1] = z4[h].y; z[2] = z4[h].z; z[3] = z4[h].w;
-          x[0] = __uint_as_float(x4[h].x << 16); x[1] = __uint_as_float(x4[h].x & 0xffff0000u);
-          x[2] = __uint_as_float(x4[h].y << 16); x[3] = __uint_as_float(x4[h].y & 0xffff0000u);
-        } else {
+        for (int h = 0; h < 4; ++h) {
+          float z[4];
+          unsigned x[4];
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
-            const int col = col0 + h * 128 + i;
+            const int col = seg * kLmSeg + h * 128 + lane * 4 + i;
             z[i] = col < P.V ? __ldcg(zrow + col) : -INFINITY;
-            x[i] = col < P.V ? Elem<__nv_bfloat16>::load(xrow, col) : -INFINITY;
+            x[i] = col < P.V ? __ldg(reinterpret_cast<const unsigned short*>(xrow) + col) : 0xff80u;
           }
+          fz[h] = make_float4(z[0], z[1], z[2], z[3]);
+          fx[h] = make_uint2(x[0] | (x[1] << 16), x[2] | (x[3] << 16));
         }
+      }
+    };
+    fetch(seg0 + warp, z4[0], x4[0]);
+    auto segment = [&](int seg, const float4 (&fz)[4], const uint2 (&fx)[4]) {
+      float2 js2 = make_float2(0.f, 0.f);
+      float resid = 0.f, pmass = 0.f;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+      for (int h = 0; h < 4; ++h) {
+        const float2 zz[2] = {make_float2(fz[h].x, fz[h].y), make_float2(fz[h].z, fz[h].w)};
+        const float2 xx[2] = {Pairs<__nv_bfloat16>::widen(fx[h].x), Pairs<__nv_bfloat16>::widen(fx[h].y)};
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const float2 cc = splat2(c);
+          float2 a = __ffma2_rn(zz[i], cc, splat2(-off_l)), b = __ffma2_rn(xx[i], cc, splat2(-off_s));   // log2 p, log2 q
           if (DIV == kDivKL) {
             // KL(large || small) on unclamped logits: q = 0 under p > 0 gives +inf, as it should
-            const float a = fmaf(z[i], c, -off_l), b = fmaf(x[i], c, -off_s);
-            const float p = ex2_approx(a), q = ex2_approx(b);
-            if (p > 0.f) js = fmaf(p, a - b, js);
-            resid += fmaxf(p - q, 0.f);
-            pmass += p;
+            const float2 p = ex2_2(a), q = ex2_2(b);
+            if (p.x > 0.f) js2.x = fmaf(p.x, a.x - b.x, js2.x);
+            if (p.y > 0.f) js2.y = fmaf(p.y, a.y - b.y, js2.y);
+            resid += fmaxf(p.x - q.x, 0.f) + fmaxf(p.y - q.y, 0.f);
+            pmass += p.x + p.y;
           } else {
-            const bool in = whole || col0 + h * 128 + i < P.V;
-            const float a = fmaxf(fmaf(z[i], c, -off_l), -125.f), b = fmaxf(fmaf(x[i], c, -off_s), -125.f);   // log2 p, log2 q
-            const float E = in ? ex2_approx(fmaxf(a, b)) : 0.f;
-            const float dd = a - b;
-            const float u = ex2_approx(-fabsf(dd));
-            const float2 ps = psi_poly<7>(make_float2(u, u));
-            js = fmaf(E, fmaf(u, -fabsf(dd), ps.x), js);
-            const float lo = E * u;                       // min(p, q)
-            resid += (dd > 0.f) ? E - lo : 0.f;           // max(0, p - q)
-            pmass += (dd >= 0.f) ? E : lo;                // p
+            // beyond the vocabulary both are -inf: 2^-125, which no sum of positive masses sees
+            a = make_float2(fmaxf(a.x, -125.f), fmaxf(a.y, -125.f));
+            b = make_float2(fmaxf(b.x, -125.f), fmaxf(b.y, -125.f));
+            const float2 e = make_float2(ex2_approx(fmaxf(a.x, b.x)), ex2_approx(fmaxf(a.y, b.y)));   // max(p, q)
+            const float2 dd = __ffma2_rn(b, splat2(-1.f), a);
+            const float2 u = make_float2(ex2_approx(-fabsf(dd.x)), ex2_approx(-fabsf(dd.y)));
+            const float2 ps = psi_poly<7>(u);
+            js2 = __ffma2_rn(e, make_float2(fmaf(u.x, -fabsf(dd.x), ps.x), fmaf(u.y, -fabsf(dd.y), ps.y)), js2);
+            const float2 lo = __fmul2_rn(e, u);             // min(p, q)
+            resid += (dd.x > 0.f) ? e.x - lo.x : 0.f;       // max(0, p - q)
+            resid += (dd.y > 0.f) ? e.y - lo.y : 0.f;
+            pmass += (dd.x >= 0.f) ? e.x : lo.x;            // p
+            pmass += (dd.y >= 0.f) ? e.y : lo.y;
           }
         }
       }
+      float js = js2.x + js2.y;
       js = warp_reduce<OpSum>(js); resid = warp_reduce<OpSum>(resid); pmass = warp_reduce<OpSum>(pmass);
       if (lane == 0) P.part_div[static_cast<size_t>(srow) * P.n_seg + seg] = make_float4(js, resid, pmass, 0.f);
+    };
+    for (int seg = seg0 + warp; seg < seg_end; seg += 2 * kWarps) {
+      fetch(seg + kWarps, z4[1], x4[1]);
+      segment(seg, z4[0], x4[0]);
+      if (seg + kWarps >= seg_end) break;
+      fetch(seg + 2 * kWarps, z4[0], x4[0]);
+      segment(seg + kWarps, z4[1], x4[1]);
     }
   }
 }

@@ -908,15 +908,16 @@ int pyramidsd_verify_fused_lmhead_ex(const psd_lmhead_args* args) {
   if (sms <= 0) sms = 1;
   // the two-SM (cta_group::2) sweep is the default
   const bool use_pair = args->tile_variant != PSD_LMHEAD_TILES_ONE_SM;
-  // Columns per tile of the pair: the weight is streamed in rounds of one tile per pair, so the width that leaves the
-  // fewest columns per pair in all is taken (V = 32000: two rounds of 224 instead of two of 256, the second of them
-  // two thirds full), the widest of equals, which reads the hidden matrix least often.
+  // Columns per tile of the pair: the weight is streamed in rounds of one tile per pair, so a width that leaves fewer
+  // columns per pair in all is taken (V = 32000: two rounds of 224 instead of two of 256, the second of them two thirds
+  // full), but a tile also costs the hidden rows it multiplies, which counts as 64 columns (V = 128256, M = 256: seven
+  // rounds of 256 take 291 us with the terms, eleven of 160, a few columns fewer, 329).
   int tile_n = psd::kLmN;
   if (use_pair) {
     const int pairs_max = sms / 2 > 0 ? sms / 2 : 1;
     long long best = 1ll << 60;
     for (int n = psd::kLm2N; n >= 128; n -= 32) {   // a pair's MMA takes N in steps of 32
-      const long long tiles = (V + n - 1) / n, cost = (tiles + pairs_max - 1) / pairs_max * n;
+      const long long tiles = (V + n - 1) / n, cost = (tiles + pairs_max - 1) / pairs_max * (n + 64);
       if (cost < best) { best = cost; tile_n = n; }
     }
   }
