@@ -284,7 +284,8 @@ int pyramidsd_verify_fused_lmhead(const void* hidden, const void* w_t, const voi
 
 /* The same call with every option exposed. Zero-initialise, set struct_size, fill what you need.
  *   seq_index_base  as in psd_stage_args.
- *   tile_variant    PSD_LMHEAD_TILES_AUTO (pairs of CTAs on 256 x 256 tiles, tcgen05 cta_group::2) or
+ *   tile_variant    PSD_LMHEAD_TILES_AUTO (up to 128 rows: one CTA per 128 rows of the weight; more: pairs of CTAs on
+ *                   256 x 256 tiles, tcgen05 cta_group::2) or
  *                   PSD_LMHEAD_TILES_ONE_SM (one CTA per 256 x 128 tile); same results within rounding.
  *   div_kind        PSD_DIV_KL: KL(large || small), whose terms separate -- sum_i p_i (log p_i - log q_i) needs the
  *                   normalisers only at the end -- so the divergences are known after ONE sweep of the GEMM. The second

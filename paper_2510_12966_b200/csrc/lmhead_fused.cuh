@@ -11,7 +11,7 @@
 //   terms    per (row, 512-column segment): divergence terms, residual mass and mass of p from both models' logits
 //   final    per sequence: row totals, accept bits, accepted prefix, and the residual draw: the segment is found
 //            from the per-segment masses, the token from that segment's logits
-// Measured, whole call: 607 -> 370 us at that size, 99.8 -> 50.6 us at M = 15, d = 2048, V = 32000, against two runs of
+// Measured, whole call: 574 -> 348 us at that size, 105 -> 36.9 us at M = 15, d = 2048, V = 32000, against two runs of
 // the GEMM with the terms in the second one's epilogue.
 //
 // One CTA = 10 warps: warp 0 lane 0 issues TMA loads, warp 1 lane 0 issues the MMAs (and owns the tensor
@@ -101,6 +101,16 @@ __device__ __forceinline__ void tmem_ld32(unsigned taddr, float (&v)[32]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// 8 consecutive fp32 columns of this thread's TMEM lane
+__device__ __forceinline__ void tmem_ld8(unsigned taddr, float (&v)[8]) {
+  unsigned r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(taddr) : "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 // Shared-memory matrix descriptor of a K-major bf16 tile whose rows are 128 bytes, 128-byte swizzled:
@@ -476,6 +486,187 @@ lmhead_sweep2sm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc_pair(tmem_base, 512);
+  }
+}
+
+// ---- few rows --------------------------------------------------------------------------------------------
+// Up to 128 rows the weight's bytes are the bound, and the tiles above multiply 256 rows whatever the call has: 512
+// cycles per 16 KB of weight and SM, longer than HBM takes for them. Here the operands change places: 128 rows of the
+// weight are the M of the MMA, the call's rows its N (rounded up to 16), so an MMA costs what the rows are worth; a
+// tile's accumulator has a vocabulary index per lane and a row per column, which makes every store to z and every read
+// of the small logits a run of consecutive indices. A tile may load fewer than 128 weight rows (what the MMA makes of the rest
+// of the shared-memory tile is never read), which lets the host cut the vocabulary into equal rounds. A warp keeps the
+// (max, sum) of its columns of a row over all its tiles (lane r: row r of the warp's half) and leaves one partial.
+// Measured at M = 15, d = 2048, V = 32000: the launch 40 -> 29 us (131 MB of weight), the whole call 50.6 -> 36.9 us.
+constexpr int kLmFewRows = 128;
+constexpr int kLmFewMaxStages = 12;
+constexpr int kLmFewRing = 200 * 1024;
+
+struct LmFewBarriers {
+  unsigned long long full[kLmFewMaxStages], empty[kLmFewMaxStages], tmem_full[2], tmem_empty[2];
+  unsigned tmem_base;
+};
+constexpr size_t kLmFewSmemBytes = static_cast<size_t>(kLmFewRing) + 1024 + 512;
+static_assert(sizeof(LmFewBarriers) <= 512, "the barriers' share of the shared memory");
+
+__device__ __forceinline__ void tma_load_2d_hint(void* smem_dst, const CUtensorMap* map, int x, int y, unsigned long long* bar, unsigned long long policy) {
+  asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4}], [%2], %5;"
+               ::"r"(smem_u32(smem_dst)), "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y), "l"(policy) : "memory");
+}
+
+// P.tile_n: weight rows per tile (a multiple of 8, at most 128); `n_rows`: the call's rows rounded up to 16.
+__global__ void __launch_bounds__(kLmThreads, 1)
+lmhead_sweep_few_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUtensorMap map_w, const LmParams P, const int n_rows,
+                        const int stages) {
+  extern __shared__ unsigned char lm_smem_raw[];
+  unsigned char* tiles = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(lm_smem_raw) + 1023) & ~uintptr_t(1023));
+  LmFewBarriers* bars = reinterpret_cast<LmFewBarriers*>(tiles + kLmFewRing);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int k_steps = P.d / kLmK;
+  const int h_bytes = n_rows * kLmK * 2;                  // a multiple of 2 KB
+  const int stage_bytes = 128 * kLmK * 2 + h_bytes;       // the weight's part, then the hidden rows'
+
+  if (tid == 0) {
+    for (int s = 0; s < stages; ++s) { mbar_init(&bars->full[s], 1); mbar_init(&bars->empty[s], 1); }
+    for (int b = 0; b < 2; ++b) { mbar_init(&bars->tmem_full[b], 1); mbar_init(&bars->tmem_empty[b], kLmEpiWarps); }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) tmem_alloc(&bars->tmem_base, 256);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const unsigned tmem_base = bars->tmem_base;
+  release_dependent_launch();
+
+  bool dead = false;
+  auto wait_phase = [&](unsigned long long* bar, unsigned parity) {
+    if (mbar_test(bar, parity)) return;
+    unsigned spins = 0;
+    while (!dead && !mbar_try(bar, parity))
+      if (++spins > kLmSpinLimit) { dead = true; atomicExch(P.status, 1); }
+  };
+
+  if (warp == 0) {
+    // ================================ TMA producer ================================
+    if (lane == 0) {
+      const unsigned long long pol_h = l2_policy_keep(), pol_w = l2_policy_drop();
+      const unsigned bytes = static_cast<unsigned>(P.tile_n * kLmK * 2 + h_bytes);
+      int stage = 0;
+      unsigned fills = 0;
+      for (int tile = blockIdx.x; tile < P.n_tiles && !dead; tile += gridDim.x) {
+        for (int ks = 0; ks < k_steps; ++ks) {
+          if (fills > 0) wait_phase(&bars->empty[stage], (fills - 1u) & 1u);
+          if (dead) break;   // the stage never came back: nothing more is copied into this ring
+          unsigned char* sw = tiles + static_cast<size_t>(stage) * stage_bytes;
+          mbar_arrive_expect_tx(&bars->full[stage], bytes);
+          tma_load_2d_hint(sw, &map_w, ks * kLmK, tile * P.tile_n, &bars->full[stage], pol_w);
+          tma_load_2d_hint(sw + 128 * kLmK * 2, &map_h, ks * kLmK, P.row0, &bars->full[stage], pol_h);
+          if (++stage == stages) { stage = 0; ++fills; }
+        }
+      }
+      // as in the kernels above: after a wait gave up, the copies issued are seen to land (bounded)
+      if (dead || *reinterpret_cast<volatile int*>(P.status) != 0) {
+        for (int s = 0; s < stages; ++s) {
+          const unsigned turns = fills + (s < stage ? 1u : 0u);
+          if (turns == 0) continue;
+          unsigned spins = 0;
+          while (!mbar_try(&bars->full[s], (turns - 1u) & 1u) && ++spins <= kLmSpinLimit) {}
+        }
+      }
+    }
+  } else if (warp == 1) {
+    // ================================ MMA issuer ================================
+    if (lane == 0) {
+      const unsigned idesc = umma_idesc_bf16(128, n_rows);
+      int stage = 0, it = 0;
+      unsigned par = 0;
+      for (int tile = blockIdx.x; tile < P.n_tiles; tile += gridDim.x, ++it) {
+        const int buf = it & 1;
+        if (it >= 2) wait_phase(&bars->tmem_empty[buf], ((it >> 1) - 1) & 1u);   // the epilogue has drained this buffer
+        if (dead) break;
+        tc_fence_after();
+        const unsigned acc = tmem_base + static_cast<unsigned>(buf) * kLmFewRows;
+        for (int ks = 0; ks < k_steps; ++ks) {
+          wait_phase(&bars->full[stage], par);
+          if (dead) break;   // no MMA on operands that have not arrived
+          tc_fence_after();
+          const unsigned sw = smem_u32(tiles + static_cast<size_t>(stage) * stage_bytes);
+          const unsigned long long dw = umma_desc_k128(sw), dh = umma_desc_k128(sw + 128 * kLmK * 2);
+#pragma unroll
+          for (int kk = 0; kk < kLmK / 16; ++kk) tc_mma_bf16(acc, dw + 2ull * kk, dh + 2ull * kk, idesc, (ks | kk) != 0 ? 1u : 0u);
+          tc_commit(&bars->empty[stage]);
+          if (++stage == stages) { stage = 0; par ^= 1u; }
+        }
+        if (dead) break;
+        tc_commit(&bars->tmem_full[buf]);
+      }
+    }
+  } else {
+    // ================================ epilogue ================================
+    const int quarter = warp & 3, half = (warp - 2) >> 2;          // TMEM lanes 32*quarter.., the half's rows
+    const int half_rows = n_rows >> 1, r0 = half * half_rows;      // at most 64 rows: two (max, sum) per lane and model
+    const int rows = min(half_rows, P.M - P.row0 - r0);            // rows that exist (<= 0: none)
+    const float c = P.c;
+    float ml[2] = {-1e30f, -1e30f}, sl[2] = {0.f, 0.f}, ms[2] = {-1e30f, -1e30f}, ss[2] = {0.f, 0.f};
+    int it = 0;
+    for (int tile = blockIdx.x; tile < P.n_tiles; tile += gridDim.x, ++it) {
+      const int buf = it & 1;
+      wait_phase(&bars->tmem_full[buf], (it >> 1) & 1u);
+      tc_fence_after();
+      const unsigned tacc = tmem_base + static_cast<unsigned>(buf * kLmFewRows + r0) + (static_cast<unsigned>(quarter * 32) << 16);
+      const int in_tile = quarter * 32 + lane, col = tile * P.tile_n + in_tile;
+      const bool col_ok = in_tile < P.tile_n && col < P.V;
+#pragma unroll 1
+      for (int g = 0; g < rows; g += 8) {   // uniform across the warp
+        float z[8], x[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          x[i] = (col_ok && g + i < rows) ? Elem<__nv_bfloat16>::load(P.small + static_cast<size_t>(P.row0 + r0 + g + i) * P.V, col) : -INFINITY;
+        tmem_ld8(tacc + static_cast<unsigned>(g), z);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          if (g + i >= rows) break;
+          const size_t srow = static_cast<size_t>(P.row0 - P.grp0 + r0 + g + i);
+          if (col_ok) P.z[srow * P.ldz + col] = z[i];
+          const float zv = col_ok ? z[i] : -INFINITY;
+          float gl = zv, gs = x[i];
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) {
+            gl = fmaxf(gl, __shfl_xor_sync(0xffffffffu, gl, o));
+            gs = fmaxf(gs, __shfl_xor_sync(0xffffffffu, gs, o));
+          }
+          const float rl = fmaxf(gl * c, -1e30f), rs = fmaxf(gs * c, -1e30f);
+          // NaN and +inf logits poison the sums, as they should
+          const float tl = warp_reduce<OpSum>(col_ok ? ex2_approx(fmaf(z[i], c, -rl)) : 0.f);
+          const float ts = warp_reduce<OpSum>(col_ok ? ex2_approx(fmaf(x[i], c, -rs)) : 0.f);
+          const int r = g + i;
+          if ((r & 31) == lane) {
+            const int h = r >> 5;
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+              if (k == h) { lse_merge(ml[k], sl[k], rl, tl); lse_merge(ms[k], ss[k], rs, ts); }
+          }
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bars->tmem_empty[buf]);   // this warp has read its part of the accumulator
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int r = k * 32 + lane;
+      if (r < rows) {
+        const size_t idx = static_cast<size_t>(P.row0 - P.grp0 + r0 + r) * P.n_part + blockIdx.x * 4 + quarter;
+        P.part_large[idx] = make_float2(ml[k], sl[k]);
+        P.part_small[idx] = make_float2(ms[k], ss[k]);
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem_base, 256);
   }
 }
 

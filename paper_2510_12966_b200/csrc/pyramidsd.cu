@@ -906,8 +906,10 @@ int pyramidsd_verify_fused_lmhead_ex(const psd_lmhead_args* args) {
   std::lock_guard<std::mutex> lock(ss->mu);
   int sms = psd::cluster_sm_count();
   if (sms <= 0) sms = 1;
-  // the two-SM (cta_group::2) sweep is the default
-  const bool use_pair = args->tile_variant != PSD_LMHEAD_TILES_ONE_SM;
+  // the two-SM (cta_group::2) sweep is the default, unless the call has so few rows that the weight is streamed faster
+  // than its 256-row tiles multiply
+  const bool use_few = args->tile_variant == PSD_LMHEAD_TILES_AUTO && M <= psd::kLmFewRows;
+  const bool use_pair = !use_few && args->tile_variant != PSD_LMHEAD_TILES_ONE_SM;
   // Columns per tile of the pair: the weight is streamed in rounds of one tile per pair, so a width that leaves fewer
   // columns per pair in all is taken (V = 32000: two rounds of 224 instead of two of 256, the second of them two thirds
   // full), but a tile also costs the hidden rows it multiplies, which counts as 64 columns (V = 128256, M = 256: seven
@@ -921,7 +923,16 @@ int pyramidsd_verify_fused_lmhead_ex(const psd_lmhead_args* args) {
       if (cost < best) { best = cost; tile_n = n; }
     }
   }
-  const int n_tiles = (V + tile_n - 1) / tile_n, n_part = use_pair ? 2 * n_tiles : n_tiles, n_seg = (V + psd::kLmSeg - 1) / psd::kLmSeg;
+  if (use_few) {   // the same for one CTA per SM and at most 128 weight rows; every tile ends with a hand-over worth a few rows
+    long long best = 1ll << 60;
+    for (int n = 128; n >= 64; n -= 8) {
+      const long long tiles = (V + n - 1) / n, cost = (tiles + sms - 1) / sms * (n + 4);
+      if (cost < best) { best = cost; tile_n = n; }
+    }
+  }
+  const int n_tiles = (V + tile_n - 1) / tile_n;
+  const int n_ctas = n_tiles < sms ? n_tiles : sms;   // of the sweeps that take one tile per CTA
+  const int n_part = use_pair ? 2 * n_tiles : use_few ? 4 * n_ctas : n_tiles, n_seg = (V + psd::kLmSeg - 1) / psd::kLmSeg;
   const long long ldz = (static_cast<long long>(n_tiles) * tile_n + 31) / 32 * 32;
   const int group_seqs = psd::kLmGroupRows / K < B ? psd::kLmGroupRows / K : B;   // K <= 32: whole sequences
   const size_t rows_max = static_cast<size_t>(group_seqs) * K;
@@ -932,7 +943,6 @@ int pyramidsd_verify_fused_lmhead_ex(const psd_lmhead_args* args) {
   t_last_scratch = ss; t_last_status = ss->status; t_last_stream = stream;
   rc = grow(ss, &ss->lm_ws, &ss->lm_ws_bytes, bytes);
   if (rc != PSD_OK) return rc;
-  // tensor maps: hidden [M, d] and W^T [V, d], bf16, K innermost, boxes of 64 x 256 / 64 x 128, 128-byte swizzle
   typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
                                const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -943,19 +953,19 @@ int pyramidsd_verify_fused_lmhead_ex(const psd_lmhead_args* args) {
     return reinterpret_cast<EncodeFn>(fn);
   }();
   if (encode == nullptr) return PSD_ERR_CUDA;
-  CUtensorMap map_a, map_b;
-  {
-    const cuuint64_t dims_a[2] = {static_cast<cuuint64_t>(d_model), static_cast<cuuint64_t>(M)};
-    const cuuint64_t dims_b[2] = {static_cast<cuuint64_t>(d_model), static_cast<cuuint64_t>(V)};
+  // tensor maps: hidden [M, d] and W^T [V, d], bf16, K innermost, boxes of 64 x the rows a load takes, 128-byte swizzle
+  const int n_rows16 = static_cast<int>((M + 15) / 16 * 16);   // few rows: the N of the MMA
+  auto encode_rows = [&](CUtensorMap* map, const void* base, long long n, int box_rows) -> bool {
+    const cuuint64_t dims[2] = {static_cast<cuuint64_t>(d_model), static_cast<cuuint64_t>(n)};
     const cuuint64_t strides[1] = {static_cast<cuuint64_t>(d_model) * 2};
-    const cuuint32_t box_a[2] = {psd::kLmK, psd::kLmM}, box_b[2] = {psd::kLmK, psd::kLmN}, estr[2] = {1, 1};
-    if (encode(&map_a, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(hidden), dims_a, strides, box_a, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) return PSD_ERR_CUDA;
-    if (encode(&map_b, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(w_t), dims_b, strides, box_b, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) return PSD_ERR_CUDA;
-  }
+    const cuuint32_t box[2] = {psd::kLmK, static_cast<cuuint32_t>(box_rows)}, estr[2] = {1, 1};
+    return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  };
+  CUtensorMap map_h, map_w;
+  if (!encode_rows(&map_h, hidden, M, use_few ? n_rows16 : use_pair ? psd::kLmM / 2 : psd::kLmM) ||
+      !encode_rows(&map_w, w_t, V, use_pair ? tile_n / 2 : tile_n))   // a pair's CTAs load half of either operand each
+    return PSD_ERR_CUDA;
   char* ws = static_cast<char*>(ss->lm_ws);
   psd::LmParams L{};
   L.small = static_cast<const __nv_bfloat16*>(logits_small);
@@ -978,36 +988,30 @@ int pyramidsd_verify_fused_lmhead_ex(const psd_lmhead_args* args) {
     const int one = static_cast<int>(psd::kLmSmemBytes), two = static_cast<int>(psd::kLm2SmemBytes);
     const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
     if (cudaFuncSetAttribute(psd::lmhead_sweep_kernel, at, one) != cudaSuccess ||
-        cudaFuncSetAttribute(psd::lmhead_sweep2sm_kernel, at, two) != cudaSuccess) {
+        cudaFuncSetAttribute(psd::lmhead_sweep2sm_kernel, at, two) != cudaSuccess ||
+        cudaFuncSetAttribute(psd::lmhead_sweep_few_kernel, at, static_cast<int>(psd::kLmFewSmemBytes)) != cudaSuccess) {
       cudaGetLastError();
       return PSD_ERR_CUDA;
     }
     attr_set[dev] = true;
   }
-  CUtensorMap map_a2, map_b2;   // the pair's boxes: 64 x 128 of A, 64 x half a tile's columns of B
-  if (use_pair) {
-    const cuuint64_t dims_a[2] = {static_cast<cuuint64_t>(d_model), static_cast<cuuint64_t>(M)};
-    const cuuint64_t dims_b[2] = {static_cast<cuuint64_t>(d_model), static_cast<cuuint64_t>(V)};
-    const cuuint64_t strides[1] = {static_cast<cuuint64_t>(d_model) * 2};
-    const cuuint32_t box[2] = {psd::kLmK, 128}, box_b[2] = {psd::kLmK, static_cast<cuuint32_t>(tile_n / 2)}, estr[2] = {1, 1};
-    if (encode(&map_a2, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(hidden), dims_a, strides, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) return PSD_ERR_CUDA;
-    if (encode(&map_b2, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(w_t), dims_b, strides, box_b, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) return PSD_ERR_CUDA;
-  }
   const int pairs = n_tiles < sms / 2 ? n_tiles : sms / 2;
-  // the GEMM over one block of 256 rows
+  // the GEMM over one block of 256 rows (few rows: over all of them)
   auto launch_sweep = [&]() -> cudaError_t {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
     cfg.blockDim = dim3(psd::kLmThreads);
     cfg.stream = stream;
+    if (use_few) {
+      const int stage = 128 * psd::kLmK * 2 + n_rows16 * psd::kLmK * 2, fit = psd::kLmFewRing / stage;
+      cfg.gridDim = dim3(static_cast<unsigned>(n_ctas));
+      cfg.dynamicSmemBytes = psd::kLmFewSmemBytes;
+      return cudaLaunchKernelEx(&cfg, psd::lmhead_sweep_few_kernel, map_h, map_w, L, n_rows16, fit < psd::kLmFewMaxStages ? fit : psd::kLmFewMaxStages);
+    }
     if (!use_pair) {
-      cfg.gridDim = dim3(static_cast<unsigned>(n_tiles < sms ? n_tiles : sms));
+      cfg.gridDim = dim3(static_cast<unsigned>(n_ctas));
       cfg.dynamicSmemBytes = psd::kLmSmemBytes;
-      return cudaLaunchKernelEx(&cfg, psd::lmhead_sweep_kernel, map_a, map_b, L);
+      return cudaLaunchKernelEx(&cfg, psd::lmhead_sweep_kernel, map_h, map_w, L);
     }
     cfg.gridDim = dim3(static_cast<unsigned>(2 * (pairs > 0 ? pairs : 1)));
     cfg.dynamicSmemBytes = psd::kLm2SmemBytes;
@@ -1015,7 +1019,7 @@ int pyramidsd_verify_fused_lmhead_ex(const psd_lmhead_args* args) {
     at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, psd::lmhead_sweep2sm_kernel, map_a2, map_b2, L);
+    return cudaLaunchKernelEx(&cfg, psd::lmhead_sweep2sm_kernel, map_h, map_w, L);
   };
   psd::LmFinalParams F{};
   F.K = K;

@@ -1,5 +1,5 @@
-"""The LM-head form at the edges of its own cuts: tile widths other than 256 (two rounds of narrower tiles), segments of
-512 columns, rows that end a 256-row block or a group of 1024, against the oracle on the sequences sampled."""
+"""The LM-head form at the edges of its own cuts: 16, 17, 128 and 129 rows (the weight or the rows as the MMA's M), tile
+widths other than 256 or 128 (equal rounds of narrower tiles), one and several rounds, segments of 512 columns, rows that end a 256-row block or a group of 1024, against the oracle on the sequences sampled."""
 import numpy as np
 import pytest
 import torch
@@ -9,8 +9,8 @@ from parity_utils import TOL
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("B,K,d,V", [(1, 1, 64, 100), (2, 3, 128, 511), (2, 3, 128, 513), (3, 5, 64, 16352), (32, 8, 64, 18945), (43, 6, 64, 2049),
-                                     (130, 8, 64, 1000)])
+@pytest.mark.parametrize("B,K,d,V", [(1, 1, 64, 100), (2, 3, 128, 511), (2, 3, 128, 513), (3, 5, 64, 16352), (4, 4, 192, 37889), (17, 1, 64, 5000),
+                                     (16, 8, 448, 19001), (43, 3, 64, 2049), (32, 8, 64, 18945), (43, 6, 64, 2049), (130, 8, 64, 1000)])
 def test_divergences_and_tokens(oracle, B, K, d, V):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
