@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import struct
 from typing import Optional
 
 import torch
@@ -91,6 +92,24 @@ class LmheadArgs(C.Structure):
     ]
 
 
+class _Packed:
+    """An argument structure as one ``struct`` format: filling a ctypes structure field by field costs a few microseconds
+    a call, packing all fields at once half a microsecond. Values come in field order, after ``struct_size``."""
+    _CODES = {C.c_uint32: "I", C.c_int32: "i", C.c_float: "f", C.c_int64: "q", C.c_uint64: "Q", C.c_void_p: "P", C.c_size_t: "N"}
+
+    def __init__(self, cls):
+        self.size = C.sizeof(cls)
+        fmt = "@" + "".join(self._CODES[t] for _, t in cls._fields_)
+        tail = self.size - struct.calcsize(fmt)      # C pads the end of a structure, struct does not
+        self.pack = struct.Struct(fmt + f"{tail}x").pack
+        for i, (name, _) in enumerate(cls._fields_):
+            assert getattr(cls, name).offset == struct.calcsize(fmt[:i + 2]) - getattr(cls, name).size, name
+
+
+_U64 = (1 << 64) - 1
+_STAGE, _PYRAMID, _LMHEAD = _Packed(StageArgs), _Packed(PyramidArgs), _Packed(LmheadArgs)
+
+
 class PyramidSDError(RuntimeError):
     def __init__(self, status: int, where: str):
         self.status = status
@@ -161,6 +180,10 @@ def load_library(path: Optional[str] = None):
     lib.pyramidsd_version.restype = C.c_char_p
     lib.pyramidsd_status_string.argtypes = [i32]
     lib.pyramidsd_status_string.restype = C.c_char_p
+    for name in ("verify_stage_ex", "verify_ex", "verify_fused_lmhead_ex"):   # the same entry points, given packed bytes
+        f = lib["pyramidsd_" + name]
+        f.argtypes, f.restype = [C.c_char_p], i32
+        setattr(lib, "packed_" + name, f)
     if path is None:
         _lib = lib
     return lib
@@ -194,9 +217,34 @@ def _dev_ptr(t: Optional[torch.Tensor], dtype=None, name="tensor") -> Optional[i
         raise ValueError(f"{name} must live in device memory")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
-    if dtype is not None and t.dtype != dtype:
+    if dtype is not None and t.dtype is not dtype:
         raise TypeError(f"{name} must be {dtype}, got {t.dtype}")
     return t.data_ptr()
+
+
+_current_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)   # absent from CPU-only builds of torch
+
+
+def _stream_handle(stream: Optional[torch.cuda.Stream]) -> int:
+    """The handle of ``stream`` or of the current device's current stream (without building a Stream object)."""
+    if stream is not None:
+        return stream.cuda_stream
+    if _current_raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _current_raw_stream(torch._C._cuda_getDevice())
+
+
+def _rows(device, dtype, *shapes):
+    """Contiguous 1-D or 2-D tensors of these shapes, cut out of one allocation (an allocation costs 2 us, a cut 1)."""
+    if len(shapes) == 1:
+        return [torch.empty(shapes[0], dtype=dtype, device=device)]
+    sizes = [s[0] * s[1] if len(s) == 2 else s[0] for s in shapes]
+    buf = torch.empty(sum(sizes), dtype=dtype, device=device)
+    out, at = [], 0
+    for s, n in zip(shapes, sizes):
+        out.append(buf.as_strided(s, (s[1], 1) if len(s) == 2 else (1,), at))
+        at += n
+    return out
 
 
 def set_stream(stream: Optional[torch.cuda.Stream] = None) -> None:
@@ -297,39 +345,19 @@ def verify_fused_lmhead(hidden, w_t, logits_small, tokens, threshold, mode=FUZZY
     d = hidden.shape[1]
     assert hidden.shape[0] == B * K and w_t.shape == (V, d)
     dev = hidden.device
-    out = {"accept_len": torch.empty(B, dtype=torch.int32, device=dev),
-           "next_token": torch.empty(B, dtype=torch.int32, device=dev)}
+    out = dict(zip(("accept_len", "next_token"), _rows(dev, torch.int32, (B,), (B,))))
     want_resid = want_rows if want_resid is None else want_resid
-    if want_rows:
-        out["div"] = torch.empty((B, K), dtype=torch.float32, device=dev)
-    if want_resid:
-        out["resid_mass"] = torch.empty((B, K), dtype=torch.float32, device=dev)
-    s = torch.cuda.current_stream() if stream is None else stream
-    if tile_variant is None and seq_index_base == 0 and div_kind == DIV_JS:
-        rc = load_library().pyramidsd_verify_fused_lmhead(
-            _dev_ptr(hidden, torch.bfloat16, "hidden"), _dev_ptr(w_t, torch.bfloat16, "w_t"),
-            _dev_ptr(logits_small, torch.bfloat16, "logits_small"), _dev_ptr(tokens, torch.int32, "tokens"),
-            B, K, d, V, float(threshold), int(mode), int(philox_seed), int(offset),
-            out["accept_len"].data_ptr(), out["next_token"].data_ptr(),
-            out["div"].data_ptr() if want_rows else None, out["resid_mass"].data_ptr() if want_resid else None,
-            C.c_void_p(s.cuda_stream))
-    else:
-        a = LmheadArgs()
-        a.struct_size = C.sizeof(LmheadArgs)
-        a.mode = int(mode)
-        a.hidden, a.w_t = _dev_ptr(hidden, torch.bfloat16, "hidden"), _dev_ptr(w_t, torch.bfloat16, "w_t")
-        a.logits_small = _dev_ptr(logits_small, torch.bfloat16, "logits_small")
-        a.tokens = _dev_ptr(tokens, torch.int32, "tokens")
-        a.B, a.K, a.d_model, a.V = B, K, d, V
-        a.threshold, a.tile_variant, a.div_kind = float(threshold), int(tile_variant or 0), int(div_kind)
-        a.philox_seed, a.philox_offset, a.seq_index_base = int(philox_seed), int(offset), int(seq_index_base)
-        a.out_accept_len, a.out_next_token = out["accept_len"].data_ptr(), out["next_token"].data_ptr()
-        if want_rows:
-            a.out_div = out["div"].data_ptr()
-        if want_resid:
-            a.out_resid_mass = out["resid_mass"].data_ptr()
-        a.stream = s.cuda_stream
-        rc = load_library().pyramidsd_verify_fused_lmhead_ex(C.byref(a))
+    names = (("div",) if want_rows else ()) + (("resid_mass",) if want_resid else ())
+    if names:
+        out.update(zip(names, _rows(dev, torch.float32, *[(B, K)] * len(names))))
+    rc = load_library().packed_verify_fused_lmhead_ex(_LMHEAD.pack(
+        _LMHEAD.size, int(mode),
+        _dev_ptr(hidden, torch.bfloat16, "hidden") or 0, _dev_ptr(w_t, torch.bfloat16, "w_t") or 0,
+        _dev_ptr(logits_small, torch.bfloat16, "logits_small") or 0, _dev_ptr(tokens, torch.int32, "tokens") or 0,
+        B, K, d, V, C.c_float(threshold).value, int(tile_variant or 0), int(div_kind), 0,
+        int(philox_seed) & _U64, int(offset) & _U64, int(seq_index_base),
+        out["accept_len"].data_ptr(), out["next_token"].data_ptr(),
+        out["div"].data_ptr() if want_rows else 0, out["resid_mass"].data_ptr() if want_resid else 0, _stream_handle(stream)))
     out["status"] = rc
     if raise_on_error:
         _check(rc, "pyramidsd_verify_fused_lmhead")
@@ -355,12 +383,11 @@ def verify_stage_noalloc(logits_small, logits_large, draft_tokens, threshold, mo
     callers that may not allocate device memory. Every output tensor is the caller's (this wrapper
     creates none); B * K is limited to NOALLOC_MAX_ROWS. Returns the status code."""
     B, K, V = logits_small.shape
-    s = torch.cuda.current_stream() if stream is None else stream
     rc = load_library().pyramidsd_verify_stage_noalloc(
         _dev_ptr(logits_small, name="logits_small"), _dev_ptr(logits_large, name="logits_large"),
         _dev_ptr(draft_tokens, torch.int32, "draft_tokens"), B, K, V, dtype_code(logits_small), float(threshold),
         int(mode), int(philox_seed), int(offset), _dev_ptr(out_accept_len, torch.int32),
-        _dev_ptr(out_next_token, torch.int32), _dev_ptr(out_wait_timeout, torch.int32), C.c_void_p(s.cuda_stream))
+        _dev_ptr(out_next_token, torch.int32), _dev_ptr(out_wait_timeout, torch.int32), _stream_handle(stream))
     if raise_on_error:
         _check(rc, "pyramidsd_verify_stage_noalloc")
     return rc
@@ -379,45 +406,22 @@ def verify_stage_ex(logits_small, logits_large, tokens, threshold, mode=FUZZY, p
         assert tuple(logits_large.shape) == (B, K + (1 if large_has_bonus_row else 0), V)
     dt = dtype_code(logits_small)
     dev = logits_small.device
-    out = {"accept_len": torch.empty(B, dtype=torch.int32, device=dev),
-           "next_token": torch.empty(B, dtype=torch.int32, device=dev)}
     want_resid = want_rows if want_resid is None else (want_resid and want_rows)
+    names_f = ("div", "p_small_tok", "p_large_tok") + (("resid_mass",) if want_resid else ()) if want_rows else ()
+    names_i = ("accept_len", "next_token") + (("row_flags",) if want_rows else ())
+    out = dict(zip(names_i, _rows(dev, torch.int32, (B,), (B,), *[(B, K)] * (len(names_i) - 2))))
     if want_rows:
-        for k in ("div", "p_small_tok", "p_large_tok") + (("resid_mass",) if want_resid else ()):
-            out[k] = torch.empty((B, K), dtype=torch.float32, device=dev)
-        out["row_flags"] = torch.empty((B, K), dtype=torch.int32, device=dev)
-    a = StageArgs()
-    a.struct_size = C.sizeof(StageArgs)
-    a.dtype = dt
-    a.logits_small = logits_small.data_ptr()
-    a.logits_large = logits_large.data_ptr()
-    a.tokens = _dev_ptr(tokens, torch.int32, "tokens")
-    a.B, a.K, a.V = B, K, V
-    a.mode, a.div_kind = int(mode), int(div_kind)
-    a.threshold, a.inv_temperature = float(threshold), float(inv_temperature)
-    a.seq_stride_small, a.seq_stride_large = int(seq_stride_small), int(seq_stride_large)
-    a.philox_seed, a.philox_offset = int(philox_seed), int(offset)
-    a.n_valid = _dev_ptr(n_valid, torch.int32, "n_valid")
-    a.out_accept_len = out["accept_len"].data_ptr()
-    a.out_next_token = out["next_token"].data_ptr()
-    if want_rows:
-        a.out_div = out["div"].data_ptr()
-        a.out_p_small_tok = out["p_small_tok"].data_ptr()
-        a.out_p_large_tok = out["p_large_tok"].data_ptr()
-        if want_resid:
-            a.out_resid_mass = out["resid_mass"].data_ptr()
-        a.out_row_flags = out["row_flags"].data_ptr()
-    if workspace is not None:
-        a.workspace = workspace.data_ptr()
-        a.workspace_bytes = workspace.numel() * workspace.element_size()
-    s = torch.cuda.current_stream() if stream is None else stream
-    a.stream = s.cuda_stream
-    a.use_stream_field = 1
-    a.kernel_variant = int(kernel_variant)
-    a.cluster_size = int(cluster_size)
-    a.large_has_bonus_row = 1 if large_has_bonus_row else 0
-    a.seq_index_base = int(seq_index_base)
-    rc = load_library().pyramidsd_verify_stage_ex(C.byref(a))
+        out.update(zip(names_f, _rows(dev, torch.float32, *[(B, K)] * len(names_f))))
+    rc = load_library().packed_verify_stage_ex(_STAGE.pack(
+        _STAGE.size, dt, logits_small.data_ptr(), logits_large.data_ptr(), _dev_ptr(tokens, torch.int32, "tokens") or 0, B, K, V,
+        int(mode), int(div_kind), C.c_float(threshold).value, C.c_float(inv_temperature).value, int(seq_stride_small), int(seq_stride_large),
+        int(philox_seed) & _U64, int(offset) & _U64, _dev_ptr(n_valid, torch.int32, "n_valid") or 0,
+        out["accept_len"].data_ptr(), out["next_token"].data_ptr(),
+        *((out["div"].data_ptr(), out["p_small_tok"].data_ptr(), out["p_large_tok"].data_ptr(),
+           out["resid_mass"].data_ptr() if want_resid else 0, out["row_flags"].data_ptr()) if want_rows else (0, 0, 0, 0, 0)),
+        0 if workspace is None else workspace.data_ptr(),
+        0 if workspace is None else workspace.numel() * workspace.element_size(),
+        _stream_handle(stream), 1, int(kernel_variant), int(cluster_size), 1 if large_has_bonus_row else 0, 0, int(seq_index_base)))
     out["status"] = rc
     if raise_on_error:
         _check(rc, "pyramidsd_verify_stage_ex")
@@ -461,39 +465,27 @@ def verify_ex(logits_draft, logits_qual, logits_target, draft_tokens, tau_q, tau
                for k in ("accept_len_q", "next_token_q", "accept_len", "next_token")}
     else:
         out = dict(out)
-    a = PyramidArgs()
-    a.struct_size = C.sizeof(PyramidArgs)
-    a.dtype = dtype_code(logits_draft)
-    a.logits_draft = _dev_ptr(logits_draft, name="logits_draft")
-    a.logits_qual = _dev_ptr(logits_qual, logits_draft.dtype, "logits_qual")
-    a.logits_target = _dev_ptr(logits_target, logits_draft.dtype, "logits_target")
-    a.draft_tokens = _dev_ptr(draft_tokens, torch.int32, "draft_tokens")
-    a.B, a.K_d, a.K_q, a.V = B, K_d, K_q, V
-    a.mode_q, a.mode_t = int(mode_q), int(mode_q if mode_t is None else mode_t)
-    a.tau_q, a.tau_t = float(tau_q), float(tau_t)
-    a.inv_temperature, a.div_kind = float(inv_temperature), int(div_kind)
-    a.philox_seed, a.philox_offset, a.seq_index_base = int(philox_seed), int(offset), int(seq_index_base)
-    a.target_has_bonus_row, a.schedule = (1 if target_has_bonus_row else 0), int(schedule)
-    for k in ("accept_len_q", "next_token_q", "accept_len", "next_token"):
-        setattr(a, "out_" + k, _dev_ptr(out[k], torch.int32, k))
+    results = [_dev_ptr(out[k], torch.int32, k) or 0 for k in ("accept_len_q", "next_token_q", "accept_len", "next_token")]
     want_resid = want_rows if want_resid is None else (want_resid and want_rows)
-    if want_rows:
-        for k, n in (("div_q", K_d), ("resid_q", K_d), ("div_t", K_q), ("resid_t", K_q)):
-            if k.startswith("resid") and not want_resid:
-                continue   # without residual masses the KL divergence takes the one-pass statistics kernel
-            out[k] = torch.empty((B, n), dtype=torch.float32, device=dev)
-            setattr(a, "out_" + k, out[k].data_ptr())
+    rows = [0, 0, 0, 0]   # div_q, resid_q, div_t, resid_t
+    if want_rows:         # without residual masses the KL divergence takes the one-pass statistics kernel
+        names = ("div_q", "resid_q", "div_t", "resid_t") if want_resid else ("div_q", "div_t")
+        out.update(zip(names, _rows(dev, torch.float32, *[(B, K_d if k.endswith("q") else K_q) for k in names])))
+        rows = [out[k].data_ptr() if k in names else 0 for k in ("div_q", "resid_q", "div_t", "resid_t")]
+    window = (0, 0)
     if want_window:
-        out["window"] = torch.empty((B, K_q), dtype=torch.int32, device=dev)
-        out["n_window"] = torch.empty(B, dtype=torch.int32, device=dev)
-        a.out_window, a.out_n_window = out["window"].data_ptr(), out["n_window"].data_ptr()
-    if workspace is not None:
-        a.workspace = workspace.data_ptr()
-        a.workspace_bytes = workspace.numel() * workspace.element_size()
-    s = torch.cuda.current_stream() if stream is None else stream
-    a.stream, a.use_stream_field = s.cuda_stream, 1
-    a.kernel_variant = int(kernel_variant)
-    rc = load_library().pyramidsd_verify_ex(C.byref(a))
+        out["window"], out["n_window"] = _rows(dev, torch.int32, (B, K_q), (B,))
+        window = (out["window"].data_ptr(), out["n_window"].data_ptr())
+    dt = logits_draft.dtype
+    rc = load_library().packed_verify_ex(_PYRAMID.pack(
+        _PYRAMID.size, dtype_code(logits_draft), _dev_ptr(logits_draft, name="logits_draft") or 0, _dev_ptr(logits_qual, dt, "logits_qual") or 0,
+        _dev_ptr(logits_target, dt, "logits_target") or 0, _dev_ptr(draft_tokens, torch.int32, "draft_tokens") or 0,
+        B, K_d, K_q, V, int(mode_q), int(mode_q if mode_t is None else mode_t), C.c_float(tau_q).value, C.c_float(tau_t).value,
+        C.c_float(inv_temperature).value, int(div_kind), int(philox_seed) & _U64, int(offset) & _U64, int(seq_index_base),
+        1 if target_has_bonus_row else 0, int(schedule), *results, *rows, *window,
+        0 if workspace is None else workspace.data_ptr(),
+        0 if workspace is None else workspace.numel() * workspace.element_size(),
+        _stream_handle(stream), 1, int(kernel_variant)))
     out["status"] = rc
     if raise_on_error:
         _check(rc, "pyramidsd_verify_ex")
