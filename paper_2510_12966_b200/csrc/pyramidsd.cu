@@ -252,9 +252,10 @@ int launch_rowstats(const StageParams& P, int dtype, int variant, int cluster_si
   return check_launch();
 }
 
-// The finalisation kernels run as clusters of CL CTAs per sequence (per stage in the split form): eight while every one
-// of them finds an SM, four while that still leaves SMs to spare, fewer for large batches, where one CTA per sequence
-// already fills the GPU.
+// The finalisation kernels run as clusters of CL CTAs per sequence (per stage in the split form), the largest CL with
+// which all clusters are resident at once: a CTA takes an SM's registers, and the device places 15 clusters of eight, 33
+// of four, 74 of two (cudaOccupancyMaxActiveClusters). One cluster more and the last ones wait for a whole
+// finalisation: 18 sequences in clusters of eight 106 us a call, of four @@ us.
 template <typename Kernel, typename... Args>
 cudaError_t launch_fin_clusters(Kernel kernel, int cl, unsigned units, cudaStream_t stream, Args... args) {
   cudaLaunchConfig_t cfg = {};
@@ -279,9 +280,9 @@ cudaError_t launch_fin_clusters(Kernel kernel, int cl, unsigned units, cudaStrea
 int fin_cluster_size(long long units) {
   int sms = psd::cluster_sm_count();
   if (sms <= 0) sms = 148;
-  if (units * 8 <= sms) return 8;
-  if (units * 4 <= 2ll * sms) return 4;
-  if (units * 2 <= 2ll * sms) return 2;
+  if (units * 10 <= sms) return 8;
+  if (units * 9 <= 2ll * sms) return 4;
+  if (units * 2 <= sms) return 2;
   return 1;
 }
 
