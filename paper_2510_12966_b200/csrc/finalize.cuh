@@ -43,6 +43,7 @@ __device__ __forceinline__ void begin_cluster_launch() {
   if (CL > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   wait_for_previous_launch();
   if (CL > 1) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;");   // the next call's statistics launch may set itself up
 }
 // Lets the next launch on the stream, if it was launched as a dependent, be scheduled from here on.
 __device__ __forceinline__ void release_next_launch() { asm volatile("griddepcontrol.launch_dependents;"); }
@@ -738,6 +739,7 @@ __global__ void __launch_bounds__(kFinThreads) finalize_pick_kernel(const StageP
   __shared__ FinShared S;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   wait_for_previous_launch();
+  release_next_launch();
   const int n_tiles = (P1.V + kFinTile - 1) / kFinTile;
   // the first draw's record and totals are asked for together with the count (stale but allocated memory if this
   // CTA has no draw)

@@ -27,6 +27,7 @@ struct __align__(16) OpCtl {
   unsigned long long full[6], empty[6];
   unsigned long long part_done[2], part_free[2];   // the warps' partials of a row are in / have been read (rows alternate)
   float4 part[2][kOpWarps];                        // (ref_0, S_0, ref_1, S_1) per warp: the pair's small and large model
+  RowList list;                                    // n_valid given: this CTA's rows
   float4 part_x[2][kOpWarps];                      // (T_10, T_21, ref_2, S_2): the cross sums, and a triple's third model
 };
 constexpr size_t kOpSmemBytes = static_cast<size_t>(kOpRingBytes) + sizeof(OpCtl) + 128;
@@ -41,6 +42,7 @@ __global__ void __launch_bounds__(kOpThreads, 1) rowstats_kl_onepass_kernel(cons
   unsigned char* ring = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
   OpCtl* ctl = reinterpret_cast<OpCtl*>(ring + static_cast<size_t>(kOpRingBytes));
 
+  using Walk = typename std::conditional<TRI, RowWalk<true>, ListWalk>::type;
   constexpr int E = Elem<T>::kPerVec;
   constexpr int CH = kOpHalfBytes / sizeof(T);   // logits per step and model
   constexpr int kMaxModels = TRI ? 3 : 2;
@@ -62,8 +64,10 @@ __global__ void __launch_bounds__(kOpThreads, 1) rowstats_kl_onepass_kernel(cons
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // launched as a dependent of what precedes it on the stream
   __syncthreads();
   release_dependent_launch();
+  build_row_list(P, static_cast<int>(blockIdx.x), static_cast<int>(gridDim.x), ctl->list);
 
   bool dead = false;    // this thread gave up on a wait: stop waiting, just run to the end
   auto give_up = [&]() {
@@ -77,20 +81,20 @@ __global__ void __launch_bounds__(kOpThreads, 1) rowstats_kl_onepass_kernel(cons
       if (++spins > kClSpinLimit) give_up();
   };
   // model m of the walk's current item: 0 the pair's small model, 1 its large one, 2 (triples) the target
-  auto model_row = [&](const RowWalk& w, int m) -> const T* {
-    if (TRI) {
-      if (m == 0) return row_ptr<T>(P.small, P.seq_stride_small, w.r, K, V);
-      if (m == 1) return row_ptr<T>(P.large, P.seq_stride_large, w.r, K, V);
-      return row_ptr<T>(P.large2, P.seq_stride_large2, w.r2, P.K2, V);
+  auto model_row = [&](const Walk& w, int m) -> const T* {
+    const int r = w.row();
+    if constexpr (TRI) {
+      if (m == 0) return row_ptr<T>(P.small, P.seq_stride_small, r, K, V);
+      if (m == 1) return row_ptr<T>(P.large, P.seq_stride_large, r, K, V);
+      return row_ptr<T>(P.large2, P.seq_stride_large2, w.row2(), P.K2, V);
     }
-    const bool second = w.r >= rows1;   // second row set: stage 2 of the wrapper
-    if (m == 0) return second ? row_ptr<T>(P.small2, P.seq_stride_small2, w.r - rows1, P.K2, V)
-                              : row_ptr<T>(P.small, P.seq_stride_small, w.r, K, V);
-    return second ? row_ptr<T>(P.large2, P.seq_stride_large2, w.r - rows1, P.K2, V)
-                  : row_ptr<T>(P.large, P.seq_stride_large, w.r, K, V);
+    const bool second = r >= rows1;   // second row set: stage 2 of the wrapper
+    if (m == 0) return second ? row_ptr<T>(P.small2, P.seq_stride_small2, r - rows1, P.K2, V)
+                              : row_ptr<T>(P.small, P.seq_stride_small, r, K, V);
+    return second ? row_ptr<T>(P.large2, P.seq_stride_large2, r - rows1, P.K2, V)
+                  : row_ptr<T>(P.large, P.seq_stride_large, r, K, V);
   };
-  RowWalk w;
-  w.init(P, blockIdx.x, gridDim.x, TRI);
+  Walk w(P, static_cast<int>(blockIdx.x), static_cast<int>(gridDim.x), &ctl->list);
 
   if (warp < kOpWarps) {
     // ================================ consumers ================================
@@ -304,9 +308,10 @@ __global__ void __launch_bounds__(kOpThreads, 1) rowstats_kl_onepass_kernel(cons
       }
       if (lane == 0) {
         const RowStats st = make_stats(m0, l0, m1, l1, T10, S1);
-        if (TRI || w.r < rows1) P.stats[w.r] = st;
-        else P.stats2[w.r - rows1] = st;
-        if (tri) P.stats2[w.r2] = make_stats(m1, l1, m2, l2, T21, S2);
+        const int r = w.row();
+        if (TRI || r < rows1) P.stats[r] = st;
+        else P.stats2[r - rows1] = st;
+        if constexpr (TRI) if (tri) P.stats2[w.row2()] = make_stats(m1, l1, m2, l2, T21, S2);
       }
     }
   }
@@ -335,8 +340,17 @@ inline cudaError_t onepass_launch_typed(const StageParams& P, int sms, cudaStrea
     if (e != cudaSuccess) return e;
     prepared[dev] = true;
   }
-  rowstats_kl_onepass_kernel<T, TRI><<<sms, kOpThreads, kOpSmemBytes, stream>>>(P);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(sms));
+  cfg.blockDim = dim3(kOpThreads);
+  cfg.dynamicSmemBytes = kOpSmemBytes;
+  cfg.stream = stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, rowstats_kl_onepass_kernel<T, TRI>, P);
 }
 
 // Whether a wrapper launch can be walked as row triples: its second row set pairs the first set's large rows (the
