@@ -28,6 +28,8 @@ thread_local int t_two_stage_policy = PSD_TWO_STAGE_AUTO;
 
 constexpr int kMaxDevices = 64;
 constexpr size_t kAlign = 256;
+constexpr size_t kHostOverlapBytes = 2u << 20;   // pyramidsd_verify_host: from here on the copies overlap stage 1 (B = 4, K = 8 / 4,
+                                                // V = 128256: 469 -> 436 us a call, 390 of them copies; at 1.5 MB the gain is gone)
 
 // Scratch of pyramidsd_verify_stage_noalloc: per-row statistics for up to PSD_NOALLOC_MAX_ROWS rows, then one
 // 256-byte line whose first word is the wait-timeout flag. It is part of the library image, so every
@@ -62,6 +64,8 @@ struct StreamScratch {
   size_t lm_ws_bytes = 0;
   void* draw = nullptr;     // records and tile totals of the three-launch finalisation
   size_t draw_bytes = 0;
+  cudaStream_t copy_stream = nullptr;   // the host entry point's copies of large inputs
+  cudaEvent_t copy_ev[3] = {nullptr, nullptr, nullptr};   // the stream's earlier work; stage 1's inputs; all inputs
 };
 struct DeviceState {
   std::mutex mu;
@@ -129,6 +133,22 @@ int grow(StreamScratch* ss, void** ptr, size_t* have, size_t want) {
   }
   if (cudaMalloc(ptr, want) != cudaSuccess) { cudaGetLastError(); return PSD_ERR_CUDA; }
   *have = want;
+  return PSD_OK;
+}
+
+// with ss->mu held: the copy stream and its events, made on first use
+int ensure_copy_stream(StreamScratch* ss) {
+  if (ss->copy_stream == nullptr && cudaStreamCreateWithFlags(&ss->copy_stream, cudaStreamNonBlocking) != cudaSuccess) {
+    cudaGetLastError();
+    ss->copy_stream = nullptr;
+    return PSD_ERR_CUDA;
+  }
+  for (cudaEvent_t& e : ss->copy_ev)
+    if (e == nullptr && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {
+      cudaGetLastError();
+      e = nullptr;
+      return PSD_ERR_CUDA;
+    }
   return PSD_OK;
 }
 
@@ -498,8 +518,10 @@ int validate_pyramid(const psd_pyramid_args* a) {
   return PSD_OK;
 }
 
-// Both stages of the pyramid with the scratch entry `ss` held by the caller.
-int verify_two_stage_locked(const psd_pyramid_args* a, StreamScratch* ss, int* status, cudaStream_t stream) {
+// Both stages of the pyramid with the scratch entry `ss` held by the caller. `target_ready`: the target's logits are
+// there only once this event has come; the call then runs stage by stage and waits for it between the stages.
+int verify_two_stage_locked(const psd_pyramid_args* a, StreamScratch* ss, int* status, cudaStream_t stream,
+                            cudaEvent_t target_ready = nullptr) {
   const int B = a->B, K_d = a->K_d, K_q = a->K_q, V = a->V, dtype = a->dtype;
   DeviceState* ds = nullptr;
   int rc = current_device_state(&ds);
@@ -561,7 +583,8 @@ int verify_two_stage_locked(const psd_pyramid_args* a, StreamScratch* ss, int* s
   rc = validate_stage(&s1);
   if (rc == PSD_OK) rc = validate_stage(&s2);
   if (rc != PSD_OK) return rc;
-  const int policy = a->schedule != PSD_TWO_STAGE_DEFAULT ? a->schedule : t_two_stage_policy;
+  const int policy = target_ready != nullptr ? PSD_TWO_STAGE_SEPARATE
+                     : a->schedule != PSD_TWO_STAGE_DEFAULT ? a->schedule : t_two_stage_policy;
   bool separate = policy == PSD_TWO_STAGE_SEPARATE;
   int32_t* fill_out = nullptr;
   if (policy == PSD_TWO_STAGE_AUTO) {
@@ -618,6 +641,7 @@ int verify_two_stage_locked(const psd_pyramid_args* a, StreamScratch* ss, int* s
     }
     rc = run_stage_locked(&s1, ss, status, stream, window, n_window, K_q, fill_out, onepass);
     if (rc != PSD_OK) return rc;
+    if (target_ready != nullptr && cudaStreamWaitEvent(stream, target_ready, 0) != cudaSuccess) return PSD_ERR_CUDA;
     return run_stage_locked(&s2, ss, status, stream, nullptr, nullptr, 0, nullptr, onepass);
   }
   // Two launches for the whole pyramid. The statistics of both stages are independent of the stage-1
@@ -790,19 +814,36 @@ int pyramidsd_verify_host(const void* logits_draft, const void* logits_qual, con
   }
   rc = grow(ss, &ss->out4, &ss->out4_bytes, static_cast<size_t>(4) * B * 4);
   if (rc != PSD_OK) return rc;
+  if (n_d + n_t >= kHostOverlapBytes) {
+    rc = ensure_copy_stream(ss);
+    if (rc != PSD_OK) return rc;
+  }
+  // Large inputs: the copies go through a stream of their own, so that stage 1 runs while the target's logits are on
+  // their way. Below a few megabytes the copies are shorter than what the two streams' events cost.
+  const bool overlap = n_d + n_t >= kHostOverlapBytes;
+  const cudaStream_t cs = overlap ? ss->copy_stream : s;
   const void* src[4] = {logits_draft, logits_qual, logits_target, draft_tokens};
-  for (int i = 0; i < 4; ++i)
-    if (cudaMemcpyAsync(ss->stage[i], src[i], want[i], cudaMemcpyHostToDevice, s) != cudaSuccess) return PSD_ERR_CUDA;
+  auto copy_in = [&](int i) { return cudaMemcpyAsync(ss->stage[i], src[i], want[i], cudaMemcpyHostToDevice, cs) == cudaSuccess; };
+  if (overlap && (cudaEventRecord(ss->copy_ev[0], s) != cudaSuccess || cudaStreamWaitEvent(cs, ss->copy_ev[0], 0) != cudaSuccess)) return PSD_ERR_CUDA;
+  if (!copy_in(3) || !copy_in(0) || !copy_in(1)) return PSD_ERR_CUDA;
+  if (overlap && (cudaEventRecord(ss->copy_ev[1], cs) != cudaSuccess || cudaStreamWaitEvent(s, ss->copy_ev[1], 0) != cudaSuccess)) return PSD_ERR_CUDA;
+  if (!copy_in(2)) return PSD_ERR_CUDA;
+  if (overlap && cudaEventRecord(ss->copy_ev[2], cs) != cudaSuccess) return PSD_ERR_CUDA;
   int32_t* o = static_cast<int32_t*>(ss->out4);
   a.logits_draft = ss->stage[0]; a.logits_qual = ss->stage[1]; a.logits_target = ss->stage[2];
   a.draft_tokens = static_cast<const int32_t*>(ss->stage[3]);
   a.out_accept_len_q = o; a.out_next_token_q = o + B; a.out_accept_len = o + 2 * B; a.out_next_token = o + 3 * B;
-  rc = verify_two_stage_locked(&a, ss, ss->status, s);
-  if (rc != PSD_OK) return rc;
+  rc = verify_two_stage_locked(&a, ss, ss->status, s, overlap ? ss->copy_ev[2] : nullptr);
+  if (rc != PSD_OK) {
+    if (overlap) cudaStreamSynchronize(cs);   // the caller's buffers are read by copies still in flight
+    return rc;
+  }
   int32_t* dst[4] = {out_accept_len_q, out_next_token_q, out_accept_len, out_next_token};
-  for (int i = 0; i < 4; ++i)
-    if (cudaMemcpyAsync(dst[i], o + static_cast<size_t>(i) * B, static_cast<size_t>(B) * 4, cudaMemcpyDeviceToHost, s) != cudaSuccess)
-      return PSD_ERR_CUDA;
+  const size_t row = static_cast<size_t>(B) * 4;
+  // results that lie behind one another in the caller's memory, as they do here, come back in one copy
+  const bool joined = dst[1] == dst[0] + B && dst[2] == dst[1] + B && dst[3] == dst[2] + B;
+  for (int i = 0; i < (joined ? 1 : 4); ++i)
+    if (cudaMemcpyAsync(dst[i], o + static_cast<size_t>(i) * B, joined ? 4 * row : row, cudaMemcpyDeviceToHost, s) != cudaSuccess) return PSD_ERR_CUDA;
   return cudaStreamSynchronize(s) == cudaSuccess ? PSD_OK : PSD_ERR_CUDA;
 }
 
@@ -1143,6 +1184,12 @@ int pyramidsd_release_stream(void* cuda_stream) {
     }
     e.ws_bytes = e.out4_bytes = e.lm_ws_bytes = e.draw_bytes = 0;
     for (size_t& b : e.stage_bytes) b = 0;
+    if (e.copy_stream) cudaStreamDestroy(e.copy_stream);
+    e.copy_stream = nullptr;
+    for (cudaEvent_t& ev : e.copy_ev) {
+      if (ev) cudaEventDestroy(ev);
+      ev = nullptr;
+    }
     if (t_last_scratch == &e) { t_last_scratch = nullptr; t_last_status = nullptr; }
     e.used = false;
     e.stream = nullptr;

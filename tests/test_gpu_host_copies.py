@@ -1,0 +1,26 @@
+"""pyramidsd_verify_host below and above the size from which its copies overlap stage 1, with results in one block (one
+copy back) and in four, against the device entry point on the same inputs."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,K_d,K_q,V,pinned", [(2, 6, 3, 4096, True), (3, 8, 4, 50257, True), (1, 5, 5, 128256, True), (3, 8, 4, 32000, False)])
+def test_host_entry_point_matches_device(B, K_d, K_q, V, pinned):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2510_12966_b200 import binding as psd, workloads as wl
+    psd.load_library()
+    psd.set_stream()
+    names = ("accept_len_q", "next_token_q", "accept_len", "next_token")
+    for i in range(3):
+        t = wl.make_pyramid_inputs(B, K_d, K_q, V, "bf16", seed=70 + i, sigma_q=0.4, sigma_d=0.9)
+        want = psd.verify(*[x.cuda() for x in t], 0.2, 0.1, psd.FUZZY, 3, i)
+        host = [x.pin_memory() if pinned else x for x in t]
+        block = torch.full((4, B), -7, dtype=torch.int32)
+        apart = [torch.full((B + 1,), -7, dtype=torch.int32)[:B] for _ in names]
+        for out in (dict(zip(names, block)), dict(zip(names, apart))):
+            psd.verify_host(*host, 0.2, 0.1, psd.FUZZY, 3, i, out=out)
+            for k in names:
+                assert torch.equal(out[k], want[k].cpu()), (k, i)
