@@ -1450,6 +1450,14 @@ inline bool cluster_geometry(const StageParams& P, int dtype, int forced_cs, boo
       if (ch2 <= wanted[0]) continue;   // fits the ring with room to spare: the rule above has seen it
       const int na = cluster_max_active_any(dtype, P.div_kind, c2);
       if (na <= 0) continue;
+      if (ch2 <= wanted[1]) {
+        // Three ring slots beyond a row are enough where that leaves the rows on fewer CTAs (111 sequences, K = 8 / 1,
+        // V = 33344 bf16, nine chunks on one CTA: 72.8 us a call, streamed twice 77.5; B = 14, K = 12 / 12, V = 81344, ten
+        // chunks on two: 58.9 and 60.8).
+        const double t = (1.0 + 0.049 * c2) * rounds_per_cta(c2, na);
+        if (t < best) { best = t; cs = c2; slice = sl2; chunks = ch2; restream = false; found = true; }
+        continue;
+      }
       const double in_flight_mb = 2.0 * sl2 * es * static_cast<double>(na < rows ? na : rows) * c2 / 1048576.0;
       double factor = 1.0 + 0.056 * c2;
       if (in_flight_mb > 60.0) factor *= (es == 4 ? 1.5 : 1.08);
