@@ -221,6 +221,7 @@ lmhead_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   __syncthreads();
   tc_fence_after();
   const unsigned tmem_base = bars->tmem_base;
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // launched as a dependent: the set-up overlaps the launch before
   release_dependent_launch();
 
   bool dead = false;
@@ -392,6 +393,7 @@ lmhead_sweep2sm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
   cluster_sync_all();        // both CTAs' barriers and allocations exist before either signals the other
   tc_fence_after();
   const unsigned tmem_base = bars->tmem_base;
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // launched as a dependent: the set-up overlaps the launch before
   release_dependent_launch();
 
   bool dead = false;
@@ -536,6 +538,7 @@ lmhead_sweep_few_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_
   __syncthreads();
   tc_fence_after();
   const unsigned tmem_base = bars->tmem_base;
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // launched as a dependent: the set-up overlaps the launch before
   release_dependent_launch();
 
   bool dead = false;
@@ -857,6 +860,7 @@ __global__ void __launch_bounds__(kLmFinalThreads) lmhead_final_kernel(const LmF
   constexpr int nwarps = kLmFinalThreads / 32;
   const float c = P.c;
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  release_dependent_launch();
 
   // per row: totals over the segments, and the probabilities of the row's token
   for (int k = warp; k < K; k += nwarps) {

@@ -1041,9 +1041,13 @@ int pyramidsd_verify_fused_lmhead_ex(const psd_lmhead_args* args) {
   // the GEMM over one block of 256 rows (few rows: over all of them)
   auto launch_sweep = [&]() -> cudaError_t {
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     cfg.blockDim = dim3(psd::kLmThreads);
     cfg.stream = stream;
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
     if (use_few) {
       const int stage = 128 * psd::kLmK * 2 + n_rows16 * psd::kLmK * 2, fit = psd::kLmFewRing / stage;
       cfg.gridDim = dim3(static_cast<unsigned>(n_ctas));
@@ -1057,10 +1061,9 @@ int pyramidsd_verify_fused_lmhead_ex(const psd_lmhead_args* args) {
     }
     cfg.gridDim = dim3(static_cast<unsigned>(2 * (pairs > 0 ? pairs : 1)));
     cfg.dynamicSmemBytes = psd::kLm2SmemBytes;
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = 2; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+    cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, psd::lmhead_sweep2sm_kernel, map_h, map_w, L);
   };
   psd::LmFinalParams F{};
