@@ -264,18 +264,18 @@ int pyramidsd_verify_stage_noalloc(const void* logits_small, const void* logits_
                                    int32_t* out_wait_timeout, void* cuda_stream);
 
 /* One verification stage whose LARGE-model logits are produced inside the call: z_large = hidden x W^T
- * (the model's LM head), by a tensor-core GEMM whose epilogue does the softmax / divergence / residual
- * arithmetic of Sec. 3.1-3.2, so the large model's logits are never written to memory. Not in the paper
- * (it verifies logits the models have already produced); the rest of the stage is pyramidsd_verify_stage.
+ * (the model's LM head), by a tensor-core GEMM whose epilogue takes both models' normalisers and leaves the
+ * fp32 logits in library-owned scratch, from which the divergence and residual terms of Sec. 3.1-3.2 are
+ * formed. Not in the paper (it verifies logits the models have already produced); the rest of the stage is
+ * pyramidsd_verify_stage.
  *   hidden        [B*K, d_model] bf16, row-major (the large model's final hidden states), device
  *   w_t           [V, d_model]  bf16, row-major: the LM-head weight as checkpoints store it (out x in), device
  *   logits_small  [B, K, V] bf16, device; tokens [B, K] int32
  *   out_div, out_resid_mass  [B, K] float32 or NULL
  * Requires d_model a multiple of 64 (else PSD_ERR_UNSUPPORTED); hidden and w_t 16-byte aligned. Rows are
- * processed in blocks of 256 (B*K <= 256 is the intended case: one block, the weight streamed twice).
- * Jensen-Shannon divergence, temperature 1. Runs the GEMM twice (the divergence needs the large model's
- * normaliser first). Scratch (partial sums per row and 128-column tile) is library-owned, grown with
- * cudaMalloc on first use. Asynchronous on `cuda_stream`; device-side timeouts via pyramidsd_last_status(). */
+ * processed in blocks of 256 (B*K <= 256 is the intended case: one block, the weight streamed once).
+ * Jensen-Shannon divergence, temperature 1. Scratch (4 V bytes per row for at most 1024 rows at a time, and partial
+ * sums) is library-owned, grown with cudaMalloc on first use. Asynchronous on `cuda_stream`; device-side timeouts via pyramidsd_last_status(). */
 int pyramidsd_verify_fused_lmhead(const void* hidden, const void* w_t, const void* logits_small,
                                   const int32_t* tokens, int B, int K, int d_model, int V, float threshold,
                                   psd_mode mode, uint64_t philox_seed, uint64_t offset,
@@ -287,11 +287,7 @@ int pyramidsd_verify_fused_lmhead(const void* hidden, const void* w_t, const voi
  *   tile_variant    PSD_LMHEAD_TILES_AUTO (up to 128 rows: one CTA per 128 rows of the weight; more: pairs of CTAs on
  *                   256 x 256 tiles, tcgen05 cta_group::2) or
  *                   PSD_LMHEAD_TILES_ONE_SM (one CTA per 256 x 128 tile); same results within rounding.
- *   div_kind        PSD_DIV_KL: KL(large || small), whose terms separate -- sum_i p_i (log p_i - log q_i) needs the
- *                   normalisers only at the end -- so the divergences are known after ONE sweep of the GEMM. The second
- *                   sweep then only serves the residual masses: it is launched, and returns at once unless some rejected
- *                   row draws from the residual (any mode but the assisted one) or out_resid_mass is wanted. With
- *                   PSD_ASSISTED, or when every position is accepted, the weight is streamed once per call. */
+ *   div_kind        PSD_DIV_JS or PSD_DIV_KL (KL(large || small)). */
 #define PSD_LMHEAD_TILES_AUTO 0
 #define PSD_LMHEAD_TILES_ONE_SM 1
 typedef struct psd_lmhead_args {
