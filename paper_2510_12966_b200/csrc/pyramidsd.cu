@@ -220,9 +220,10 @@ int check_launch() {
 // walk its rows as (draft, qualifier, target) triples where the geometry streams them twice. `resid_wanted`: some
 // caller output takes the rows' residual masses (without them the KL divergence goes through the one-pass kernel).
 // `onepass`: 1 / 0 = the caller has decided for / against the one-pass kernel (a two-stage call decides once, on its
-// whole shape, so that all its schedules run the same arithmetic); -1 = decide here.
+// whole shape, so that all its schedules run the same arithmetic); -1 = decide here. `force_ua`: likewise decided by a
+// two-stage call for both its stages, see cluster_geometry.
 int launch_rowstats(const StageParams& P, int dtype, int variant, int cluster_size, cudaStream_t stream,
-                    bool allow_triples = false, bool resid_wanted = true, int onepass = -1) {
+                    bool allow_triples = false, bool resid_wanted = true, int onepass = -1, bool force_ua = false) {
   const long long rows = static_cast<long long>(P.B) * P.K;
   if (rows == 0 && P.K2 == 0) return PSD_OK;
   if (onepass < 0) onepass = (variant == PSD_KERNEL_AUTO && cluster_size == 0 && psd::onepass_applies(P, dtype, resid_wanted)) ? 1 : 0;
@@ -240,7 +241,7 @@ int launch_rowstats(const StageParams& P, int dtype, int variant, int cluster_si
   psd::ClusterGeom geom{};
   if (variant != PSD_KERNEL_BASELINE) {
     use_cluster = psd::cluster_geometry(P, dtype, cluster_size, variant == PSD_KERNEL_CLUSTER_STREAMED, allow_triples,
-                                        variant == PSD_KERNEL_AUTO, &geom);
+                                        variant == PSD_KERNEL_AUTO, &geom, force_ua);
     if (!use_cluster && variant != PSD_KERNEL_AUTO) return PSD_ERR_UNSUPPORTED;
   }
   TimedLaunch timed(stream, 0);
@@ -455,7 +456,7 @@ cudaStream_t pick_stream(const psd_stage_args* a) {
 // Runs one stage with the scratch entry `ss` (held by the caller); `window_out`/`n_window_out`/`K_window` non-null
 // make the finalisation also build the stage-2 window of the wrapper.
 int run_stage_locked(const psd_stage_args* a, StreamScratch* ss, int* status, cudaStream_t stream, int32_t* window_out,
-                     int32_t* n_window_out, int K_window, int32_t* fill_out = nullptr, int onepass = -1) {
+                     int32_t* n_window_out, int K_window, int32_t* fill_out = nullptr, int onepass = -1, bool force_ua = false) {
   int rc = PSD_OK;
   void* ws = a->workspace;
   if (ws == nullptr) {
@@ -470,7 +471,7 @@ int run_stage_locked(const psd_stage_args* a, StreamScratch* ss, int* status, cu
   P.fill_out = fill_out;
   P.fill_cap = kFillCap;
   if (a->K > 0) {
-    rc = launch_rowstats(P, a->dtype, a->kernel_variant, a->cluster_size, stream, false, P.out_resid_mass != nullptr, onepass);
+    rc = launch_rowstats(P, a->dtype, a->kernel_variant, a->cluster_size, stream, false, P.out_resid_mass != nullptr, onepass, force_ua);
     if (rc != PSD_OK) return rc;
   }
   return launch_finalize(P, a->dtype, stream, ss);
@@ -627,8 +628,10 @@ int verify_two_stage_locked(const psd_pyramid_args* a, StreamScratch* ss, int* s
   int onepass = 0;
   if (separate) {
     // stage by stage: stage 2's statistics run after stage 1 has fixed the windows and skip the rows beyond them.
-    // Both launches take the cluster size the single-launch schedule would pick, so a row's vocabulary is
-    // cut into the same slices and its statistics come out bit-identical under either policy.
+    // Both launches take the cluster size the single-launch schedule would pick, and its form: where one of the three
+    // tensors is no 16-byte units, that launch takes single logits of all rows. A row's vocabulary is then cut into the
+    // same slices and chunks and its statistics come out bit-identical under either policy.
+    bool force_ua = false;
     {
       StageParams PS = make_params(&s1, s1.workspace, nullptr);
       const StageParams Q = make_params(&s2, s2.workspace, nullptr);
@@ -636,13 +639,16 @@ int verify_two_stage_locked(const psd_pyramid_args* a, StreamScratch* ss, int* s
       PS.seq_stride_small2 = Q.seq_stride_small; PS.seq_stride_large2 = Q.seq_stride_large;
       PS.K2 = K_q;
       psd::ClusterGeom g{};
-      if (variant != PSD_KERNEL_BASELINE && psd::cluster_geometry(PS, dtype, 0, false, false, variant == PSD_KERNEL_AUTO, &g)) s1.cluster_size = s2.cluster_size = g.cs;
+      if (variant != PSD_KERNEL_BASELINE && psd::cluster_geometry(PS, dtype, 0, false, false, variant == PSD_KERNEL_AUTO, &g)) {
+        s1.cluster_size = s2.cluster_size = g.cs;
+        force_ua = g.ua != 0;
+      }
       onepass = (variant == PSD_KERNEL_AUTO && psd::onepass_applies(PS, dtype, resid_any)) ? 1 : 0;
     }
-    rc = run_stage_locked(&s1, ss, status, stream, window, n_window, K_q, fill_out, onepass);
+    rc = run_stage_locked(&s1, ss, status, stream, window, n_window, K_q, fill_out, onepass, force_ua);
     if (rc != PSD_OK) return rc;
     if (target_ready != nullptr && cudaStreamWaitEvent(stream, target_ready, 0) != cudaSuccess) return PSD_ERR_CUDA;
-    return run_stage_locked(&s2, ss, status, stream, nullptr, nullptr, 0, nullptr, onepass);
+    return run_stage_locked(&s2, ss, status, stream, nullptr, nullptr, 0, nullptr, onepass, force_ua);
   }
   // Two launches for the whole pyramid. The statistics of both stages are independent of the stage-1
   // outcome (only the token looked up in a row and the window length depend on it), so one launch of

@@ -1403,9 +1403,11 @@ inline bool cluster_shape_ok(const StageParams& P, int dtype) {
 // Picks the cluster size (or takes `forced_cs`; a forced size whose slice exceeds the ring is streamed
 // twice), and sizes the grid to the clusters that can be co-resident. Returns false when the shape does not
 // fit the kernel. `any_alignment`: rows that are not 16-byte units may go through the form that takes single logits.
+// `force_ua`: these rows take that form even if they are such units (the other half of a two-stage call is not, and both
+// halves have to be summed in the order that one launch over all of them would take).
 inline bool cluster_geometry(const StageParams& P, int dtype, int forced_cs, bool force_streamed, bool allow_triples, bool any_alignment,
-                             ClusterGeom* g) {
-  const bool ua = !cluster_shape_ok(P, dtype);
+                             ClusterGeom* g, bool force_ua = false) {
+  const bool ua = force_ua || !cluster_shape_ok(P, dtype);
   if (ua && (!any_alignment || P.V < 2048)) return false;
   const int es = dtype == 0 ? 4 : 2;
   const long long rows = static_cast<long long>(P.B) * (P.K + P.K2);

@@ -91,3 +91,22 @@ def test_pyramid_schedules_agree(psd):
         for k in ("accept_len_q", "next_token_q", "accept_len", "next_token", "window", "div_q", "resid_q"):
             assert torch.equal(o[k], outs[0][k]), k
         assert torch.equal(o["div_t"].cpu()[live], outs[0]["div_t"].cpu()[live])
+
+
+@pytest.mark.parametrize("which", [0, 1, 2])
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_schedules_agree_when_one_tensor_alone_is_off_a_boundary(psd, dtype, which):
+    """The single statistics launch takes single logits of every row then; stage by stage, the stage whose own two tensors
+    are aligned has to be summed in the same order."""
+    from paper_2510_12966_b200 import workloads as wl
+    t = list(wl.make_pyramid_inputs(32, 8, 4, 32000, dtype, seed=29, sigma_q=0.6, sigma_d=1.2))
+    t = [on_device(x, 1 if i == which else 0) if i < 3 else x.cuda() for i, x in enumerate(t)]
+    for div in (psd.DIV_JS, psd.DIV_KL):
+        outs = [psd.verify_ex(*t, 0.2, 0.15, psd.FUZZY, psd.FUZZY, 5, 9, schedule=s, div_kind=div)
+                for s in (psd.TWO_STAGE_FUSED, psd.TWO_STAGE_SEPARATE, psd.TWO_STAGE_FUSED_ROWS)]
+        live = torch.arange(4)[None, :] < outs[0]["n_window"].cpu()[:, None]
+        for o in outs[1:]:
+            for k in ("accept_len_q", "next_token_q", "accept_len", "next_token", "window", "div_q", "resid_q"):
+                assert torch.equal(o[k], outs[0][k]), k
+            for k in ("div_t", "resid_t"):
+                assert torch.equal(o[k].cpu()[live], outs[0][k].cpu()[live]), k
