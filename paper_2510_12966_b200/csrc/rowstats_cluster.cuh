@@ -101,13 +101,13 @@ struct ClusterGeom {
 
 // Per-row constants of pass B: -log2 of the normalisers in the scaled base-2 domain and the clamp floors.
 struct __align__(16) RowConsts {
-  float off_small, off_large;        // log2(sum_i exp(z_i / T)) of each model
+  float off_small, off_large;        // log2(sum_i exp(z_i / T)) of each model; UA: split_offset's logit, rest_* its rest
   float floor_small, floor_large;    // logits below these would give log2 p < -125
   unsigned floor2_small, floor2_large;   // the same floors as packed bf16 pairs
   unsigned floor2_third;             // row triples: the third model (the target)
-  unsigned pad0;
+  float rest_small;
   float off_third, floor_third;
-  unsigned pad1, pad2;
+  float rest_large, rest_third;
 };
 
 // Shared-memory control block behind the ring.
@@ -116,7 +116,7 @@ struct __align__(16) ClusterCtl {
   unsigned long long empty[kClSlots];
   unsigned long long a_done[kClDepth], b_done[kClDepth], lse_ready[kClDepth], fin_ready[kClDepth], b_go[kClDepth];
   float4 a_part[kClDepth][kClAWarps];              // (ref_small, sum_small, ref_large, sum_large) per pass-A warp
-  float4 b_part[kClDepth][kClBWarps];              // (divergence sum in bits, sum max(p,q), rows differ, unused) per pass-B warp
+  float4 b_part[kClDepth][kClBWarps];              // (divergence sum in bits, acc.big, rows differ, unused) per pass-B warp
   float4 row_lse[kClDepth];                        // (m2_small, l2s_small, m2_large, l2s_large) of the row
   RowConsts row_consts[kClDepth];                  // what pass B needs of the row, published by the agent
   float4 lse_in[kClDepth][kClMaxRanks];            // partials received from every rank of the cluster
@@ -530,6 +530,24 @@ __device__ __forceinline__ void lse_merge(float& ref, float& s, float oref, floa
   ref = m;
 }
 
+// log2 of a sum whose whole part goes into the reference it was taken against, so that what is left lies within 1/2 of zero
+// and loses nothing to the rounding of a larger number. As it is where the reference is no whole number (a row that went
+// through the slow path) or the sum no positive finite one.
+__device__ __forceinline__ float lg2_into(float s, float& ref) {
+  if (ref != rintf(ref) || !(s > 1e-30f && s < INFINITY)) return lg2_approx(s);
+  const int bits = __float_as_int(s), k = (bits - 0x3f3504f3) >> 23;   // s = 2^k f, f in [sqrt(1/2), sqrt(2))
+  ref += static_cast<float>(k);
+  return log2f(__int_as_float(bits - (k << 23)));
+}
+
+// The logit x0 of probability about 1 under a normaliser m2 + l2s, and what x0 c leaves of it: log2 p = (x - x0) c - rest.
+// The subtraction is exact or nearly so for the logits that weigh, and the rest, a difference of numbers below 1, is too.
+__device__ __forceinline__ void split_offset(float m2, float l2s, float c, float inv_c, float& x0, float& rest) {
+  x0 = (m2 + l2s) * inv_c;
+  if (!(fabsf(x0) < 1e30f)) x0 = 0.f;   // a vanishing 1 / T: the normaliser in one number
+  rest = fmaf(-x0, c, m2) + l2s;
+}
+
 // ---- pass B ------------------------------------------------------------------------------------------
 // With a = log2 p and b = log2 q (both linear in the logits once the normalisers are known), each
 // vocabulary index adds to the Jensen-Shannon divergence, in bits and before the factor 1/2,
@@ -577,7 +595,7 @@ __device__ __forceinline__ float2 psi_poly(float2 u) {
 constexpr int kPsiDegBf16 = 4;
 
 struct DivAcc {
-  float2 js, big;    // sum 2^M h(d); sum 2^M
+  float2 js, big;    // sum 2^M h(d); sum 2^M (UA: sum max(0, p - q))
   unsigned differ;   // OR of (small bits XOR large bits)
   __device__ __forceinline__ void reset() { js = big = make_float2(0.f, 0.f); differ = 0u; }
 };
@@ -609,8 +627,35 @@ __device__ __forceinline__ void div_accumulate(const float2 (&xl)[N], const floa
   }
 }
 
-template <typename V>
-__device__ __forceinline__ V warp_sum(V v) { return warp_reduce<OpSum>(v); }
+// The same for rows at any boundary, whose statistics keep the accuracy of the three-pass kernel. log2 p is taken as
+// (x - x0) c - rest with split_offset's pair: one rounding, where the normaliser as one number of about 20 scales every
+// probability by up to 1e-6. The residual mass is summed as such, in acc.big (the difference of two sums near 1 cannot tell
+// masses below 1e-6 from zero), and the polynomial is the one of degree 7 for bf16 too.
+template <int DIV, int N>
+__device__ __forceinline__ void div_accumulate_split(const float2 (&xl)[N], const float2 (&xs)[N], float c, float x0_l, float rest_l, float x0_s,
+                                                     float rest_s, DivAcc& acc) {
+  const float2 cc = splat2(c), x0l = splat2(-x0_l), x0s = splat2(-x0_s), rl = splat2(-rest_l), rs = splat2(-rest_s);
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    const float2 a = __ffma2_rn(__fadd2_rn(xl[j], x0l), cc, rl), b = __ffma2_rn(__fadd2_rn(xs[j], x0s), cc, rs);   // log2 p, log2 q
+    if (DIV == kDivJS) {
+      const float2 e = make_float2(ex2_approx(fmaxf(a.x, b.x)), ex2_approx(fmaxf(a.y, b.y)));   // max(p, q)
+      const float2 dd = __ffma2_rn(b, splat2(-1.f), a);
+      const float2 u = make_float2(ex2_approx(-fabsf(dd.x)), ex2_approx(-fabsf(dd.y)));
+      const float2 ps = psi_poly<7>(u), lo = __fmul2_rn(e, u);                                  // lo: min(p, q)
+      acc.js = __ffma2_rn(e, make_float2(fmaf(u.x, -fabsf(dd.x), ps.x), fmaf(u.y, -fabsf(dd.y), ps.y)), acc.js);
+      acc.big = __fadd2_rn(acc.big, make_float2(dd.x > 0.f ? e.x - lo.x : 0.f, dd.y > 0.f ? e.y - lo.y : 0.f));
+    } else {
+      const float2 p = ex2_2(a), q = ex2_2(b);
+      acc.big = __fadd2_rn(acc.big, make_float2(fmaxf(p.x - q.x, 0.f), fmaxf(p.y - q.y, 0.f)));
+      if (DIV == kDivKL) {
+        // KL(large || small) on unclamped logits: q == 0 with p > 0 gives +inf, as it should
+        if (p.x > 0.f) acc.js.x = fmaf(p.x, a.x - b.x, acc.js.x);
+        if (p.y > 0.f) acc.js.y = fmaf(p.y, a.y - b.y, acc.js.y);
+      }
+    }
+  }
+}
 
 // A next launch that was made a programmatic dependent of this one (the finalisation) may be scheduled once every
 // warp of every CTA has been here; it still waits for this grid's end before it reads a statistic. Every warp comes
@@ -778,7 +823,7 @@ __global__ void __launch_bounds__(RS ? kClThreadsRS : kClThreads, 1) rowstats_cl
 #pragma unroll
                 for (int m = 0; m < NM; ++m) g[m] = fmaxf(g[m], __shfl_xor_sync(0xffffffffu, g[m], o));
 #pragma unroll
-              for (int m = 0; m < NM; ++m) st[m].ref = fmaxf(g[m] * c, -1e30f);
+              for (int m = 0; m < NM; ++m) st[m].ref = fmaxf(UA ? rintf(g[m] * c) : g[m] * c, -1e30f);   // UA: a whole number, see lg2_into
             }
             if (UA && n <= 0) continue;   // a chunk beyond the slice (odd count): nothing was copied
 #pragma unroll
@@ -869,7 +914,7 @@ __global__ void __launch_bounds__(RS ? kClThreadsRS : kClThreads, 1) rowstats_cl
       if (RS) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kClRegsB));
       release_dependent_launch();
       constexpr int N = Pairs<T>::kN;
-      constexpr int PSI = sizeof(T) == 2 ? kPsiDegBf16 : 7;
+      constexpr int PSI = sizeof(T) == 2 ? kPsiDegBf16 : 7;   // of the form over 16-byte vectors
       constexpr int kVecStride = kClBWarps * 32 * 16;   // bytes between a lane's vectors
       if (RS) slot = static_cast<unsigned>(RB0);
       bool landed = false;   // as in pass A: the next chunk's barrier is tested one chunk early
@@ -928,7 +973,8 @@ __global__ void __launch_bounds__(RS ? kClThreadsRS : kClThreads, 1) rowstats_cl
                 Pairs<T>::load_clamped(u[1][i], rc.floor_large, rc.floor2_large, xl);
                 local.differ = (u[0][i].x ^ u[1][i].x) | (u[0][i].y ^ u[1][i].y) | (u[0][i].z ^ u[1][i].z) | (u[0][i].w ^ u[1][i].w);
               }
-              div_accumulate<DIV, N, PSI>(xl, xs, c, rc.off_large, rc.off_small, local);
+              if (UA) div_accumulate_split<DIV, N>(xl, xs, c, rc.off_large, rc.rest_large, rc.off_small, rc.rest_small, local);
+              else div_accumulate<DIV, N, PSI>(xl, xs, c, rc.off_large, rc.off_small, local);
               const bool live = UA || len[i] > off;   // a vector beyond the slice adds nothing
               if (live) {
                 acc.js = __fadd2_rn(acc.js, local.js);
@@ -941,7 +987,8 @@ __global__ void __launch_bounds__(RS ? kClThreadsRS : kClThreads, 1) rowstats_cl
                   local2.differ = (u[1][i].x ^ u[NM - 1][i].x) | (u[1][i].y ^ u[NM - 1][i].y) | (u[1][i].z ^ u[NM - 1][i].z) |
                                   (u[1][i].w ^ u[NM - 1][i].w);
                 }
-                div_accumulate<DIV, N, PSI>(xt, xl, c, rc.off_third, rc.off_large, local2);
+                if (UA) div_accumulate_split<DIV, N>(xt, xl, c, rc.off_third, rc.rest_third, rc.off_large, rc.rest_large, local2);
+                else div_accumulate<DIV, N, PSI>(xt, xl, c, rc.off_third, rc.off_large, local2);
                 if (live) {
                   acc2.js = __fadd2_rn(acc2.js, local2.js);
                   acc2.big = __fadd2_rn(acc2.big, local2.big);
@@ -1141,7 +1188,8 @@ __global__ void __launch_bounds__(RS ? kClThreadsRS : kClThreads, 1) rowstats_cl
           for (int j = 0; j < 4; ++j) stt = fmaf(v[j].y, ex2_approx(v[j].x - mt), stt);
         }
       }
-      const float l2ss = lg2_approx(ss), l2sl = lg2_approx(sl), l2st = lg2_approx(stt);
+      const float l2ss = UA ? lg2_into(ss, ms) : lg2_approx(ss), l2sl = UA ? lg2_into(sl, ml) : lg2_approx(sl),
+                  l2st = UA ? lg2_into(stt, mt) : lg2_approx(stt);
       if (lane == 0) {
         RowConsts rc;
         rc.off_small = ms + l2ss;
@@ -1154,7 +1202,12 @@ __global__ void __launch_bounds__(RS ? kClThreadsRS : kClThreads, 1) rowstats_cl
         rc.off_third = mt + l2st;
         rc.floor_third = (DIV == kDivKL) ? -INFINITY : (rc.off_third - 125.f) * inv_c;
         rc.floor2_third = Pairs<T>::floor_bits(rc.floor_third);
-        rc.pad0 = rc.pad1 = rc.pad2 = 0u;
+        rc.rest_small = rc.rest_large = rc.rest_third = 0.f;
+        if (UA) {
+          split_offset(ms, l2ss, P.c, inv_c, rc.off_small, rc.rest_small);
+          split_offset(ml, l2sl, P.c, inv_c, rc.off_large, rc.rest_large);
+          if (TRI) split_offset(mt, l2st, P.c, inv_c, rc.off_third, rc.rest_third);
+        }
         ctl->row_consts[d] = rc;
         ctl->row_lse[d] = make_float4(ms, l2ss, ml, l2sl);
         if (TRI) ctl->row_lse3[d] = make_float4(mt, l2st, 0.f, 0.f);
@@ -1196,7 +1249,7 @@ __global__ void __launch_bounds__(RS ? kClThreadsRS : kClThreads, 1) rowstats_cl
         st.m2_small = st.l2s_small = st.m2_large = st.l2s_large = st.div = st.resid = __int_as_float(0x7fc00000);
       } else {
         float D;
-        const float res = big - 1.f;   // sum max(p,q) - sum q = sum max(0, p - q)
+        const float res = UA ? big : big - 1.f;   // sum max(p,q) - sum q = sum max(0, p - q)
         if (DIV == kDivJS) D = (0.5f * kLn2) * js;   // bits -> nats, and the 1/2 of the definition
         else if (DIV == kDivKL) D = kLn2 * js;
         else D = res;

@@ -110,3 +110,32 @@ def test_schedules_agree_when_one_tensor_alone_is_off_a_boundary(psd, dtype, whi
                 assert torch.equal(o[k], outs[0][k]), k
             for k in ("div_t", "resid_t"):
                 assert torch.equal(o[k].cpu()[live], outs[0][k].cpu()[live]), k
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("V", [4033, 50257])
+@pytest.mark.parametrize("sigma", [2.0, 0.5, None])
+def test_accuracy_of_the_statistics(psd, V, dtype, sigma):
+    """Divergences and residual masses against 64 bits, down to rows that differ in three logits (sigma None). A probability
+    is off by at most 2^-22 (ex2.approx) and its row's normaliser by as much: 2^-21 of the masses. JS adds the polynomial's
+    5.6e-8 per unit of max(p, q) (at most 2, times ln 2 / 2), KL weighs the errors by |log p / q| + 1."""
+    torch.manual_seed(5)
+    z = torch.randn((4, 4, V), device="cuda") * 2
+    zs = z.to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+    zl = zs.clone()
+    if sigma is None:
+        idx = torch.randint(0, V, (4, 4, 3), device="cuda")
+        zl.scatter_(2, idx, (zs.gather(2, idx).float() + 0.05).to(zs.dtype))
+    else:
+        zl = (z + sigma * torch.randn_like(z)).to(zs.dtype)
+    tok = torch.zeros((4, 4), dtype=torch.int32, device="cuda")
+    a, b = torch.log_softmax(zl.double(), -1), torch.log_softmax(zs.double(), -1)
+    p, q = a.exp(), b.exp()
+    lm = torch.logaddexp(a, b) - np.log(2.0)
+    want = {psd.DIV_JS: 0.5 * (p * (a - lm) + q * (b - lm)).sum(-1), psd.DIV_TV: (p - q).clamp(min=0).sum(-1), psd.DIV_KL: (p * (a - b)).sum(-1)}
+    slack = {psd.DIV_JS: 3.9e-8 + 2.0 ** -21 * want[psd.DIV_JS], psd.DIV_TV: 2.0 ** -21 * torch.ones_like(a[..., 0]),
+             psd.DIV_KL: 2.0 ** -21 * (p * (a - b).abs()).sum(-1) + 2.0 ** -21}
+    for div in want:
+        out = psd.verify_stage_ex(zs, zl, tok, 0.1, psd.FUZZY, 1, 0, div_kind=div)
+        assert ((out["div"].double() - want[div]).abs() <= slack[div]).all(), (out["div"].double() - want[div]).abs().max()
+        assert ((out["resid_mass"].double() - want[psd.DIV_TV]).abs() <= slack[psd.DIV_TV]).all()
