@@ -492,7 +492,7 @@ lmhead_sweep2sm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
 }
 
 // ---- few rows --------------------------------------------------------------------------------------------
-// Up to 128 rows the weight's bytes are the bound, and the tiles above multiply 256 rows whatever the call has: 512
+// With few rows the weight's bytes are the bound, and the tiles above multiply 256 rows whatever the call has: 512
 // cycles per 16 KB of weight and SM, longer than HBM takes for them. Here the operands change places: 128 rows of the
 // weight are the M of the MMA, the call's rows its N (rounded up to 16), so an MMA costs what the rows are worth; a
 // tile's accumulator has a vocabulary index per lane and a row per column, which makes every store to z and every read
@@ -500,9 +500,14 @@ lmhead_sweep2sm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
 // of the shared-memory tile is never read), which lets the host cut the vocabulary into equal rounds. A warp keeps the
 // (max, sum) of its columns of a row over all its tiles (lane r: row r of the warp's half) and leaves one partial.
 // Measured at M = 15, d = 2048, V = 32000: the launch 40 -> 29 us (131 MB of weight), the whole call 50.6 -> 36.9 us.
-constexpr int kLmFewRows = 128;
+// Up to 32 rows: the epilogue takes a warp-wide maximum and sum per row, about 2.9 us a row at V = 128256, while a lane of the
+// pairs' epilogue has a row to itself. Whole calls in us, this form / pairs of CTAs: V = 152064, d = 1024: M = 16 92 / 138,
+// 32 134 / 136, 64 215 / 141, 128 385 / 197; V = 128256, d = 4096: 32 244 / 242, 64 256 / 272, 128 422 / 282;
+// V = 50257, d = 768: 32 74 / 95, 64 106 / 101, 128 173 / 118.
+constexpr int kLmFewRows = 32;
 constexpr int kLmFewMaxStages = 12;
 constexpr int kLmFewRing = 200 * 1024;
+static_assert(2 * kLmFewRows >= 32 && kLmFewRows <= 32, "tensor memory comes in 32 columns or more; a lane per row of a half");
 
 struct LmFewBarriers {
   unsigned long long full[kLmFewMaxStages], empty[kLmFewMaxStages], tmem_full[2], tmem_empty[2];
@@ -533,7 +538,7 @@ lmhead_sweep_few_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_
     for (int b = 0; b < 2; ++b) { mbar_init(&bars->tmem_full[b], 1); mbar_init(&bars->tmem_empty[b], kLmEpiWarps); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 1) tmem_alloc(&bars->tmem_base, 256);
+  if (warp == 1) tmem_alloc(&bars->tmem_base, 2 * kLmFewRows);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -607,10 +612,10 @@ lmhead_sweep_few_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_
   } else {
     // ================================ epilogue ================================
     const int quarter = warp & 3, half = (warp - 2) >> 2;          // TMEM lanes 32*quarter.., the half's rows
-    const int half_rows = n_rows >> 1, r0 = half * half_rows;      // at most 64 rows: two (max, sum) per lane and model
+    const int half_rows = n_rows >> 1, r0 = half * half_rows;      // at most 16 rows: a lane keeps the (max, sum) of one
     const int rows = min(half_rows, P.M - P.row0 - r0);            // rows that exist (<= 0: none)
     const float c = P.c;
-    float ml[2] = {-1e30f, -1e30f}, sl[2] = {0.f, 0.f}, ms[2] = {-1e30f, -1e30f}, ss[2] = {0.f, 0.f};
+    float ml = -1e30f, sl = 0.f, ms = -1e30f, ss = 0.f;
     int it = 0;
     for (int tile = blockIdx.x; tile < P.n_tiles; tile += gridDim.x, ++it) {
       const int buf = it & 1;
@@ -642,34 +647,24 @@ lmhead_sweep_few_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_
           // NaN and +inf logits poison the sums, as they should
           const float tl = warp_reduce<OpSum>(col_ok ? ex2_approx(fmaf(z[i], c, -rl)) : 0.f);
           const float ts = warp_reduce<OpSum>(col_ok ? ex2_approx(fmaf(x[i], c, -rs)) : 0.f);
-          const int r = g + i;
-          if ((r & 31) == lane) {
-            const int h = r >> 5;
-#pragma unroll
-            for (int k = 0; k < 2; ++k)
-              if (k == h) { lse_merge(ml[k], sl[k], rl, tl); lse_merge(ms[k], ss[k], rs, ts); }
-          }
+          if (g + i == lane) { lse_merge(ml, sl, rl, tl); lse_merge(ms, ss, rs, ts); }
         }
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&bars->tmem_empty[buf]);   // this warp has read its part of the accumulator
     }
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int r = k * 32 + lane;
-      if (r < rows) {
-        const size_t idx = static_cast<size_t>(P.row0 - P.grp0 + r0 + r) * P.n_part + blockIdx.x * 4 + quarter;
-        P.part_large[idx] = make_float2(ml[k], sl[k]);
-        P.part_small[idx] = make_float2(ms[k], ss[k]);
-      }
+    if (lane < rows) {
+      const size_t idx = static_cast<size_t>(P.row0 - P.grp0 + r0 + lane) * P.n_part + blockIdx.x * 4 + quarter;
+      P.part_large[idx] = make_float2(ml, sl);
+      P.part_small[idx] = make_float2(ms, ss);
     }
   }
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, 256);
+    tmem_dealloc(tmem_base, 2 * kLmFewRows);
   }
 }
 

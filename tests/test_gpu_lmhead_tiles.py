@@ -1,4 +1,4 @@
-"""The LM-head form at the edges of its own cuts: 16, 17, 128 and 129 rows (the weight or the rows as the MMA's M), tile
+"""The LM-head form at the edges of its own cuts: 16, 17, 32 and 33 rows (the weight or the rows as the MMA's M), 128 and 129, tile
 widths other than 256 or 128 (equal rounds of narrower tiles), one and several rounds, segments of 512 columns, rows that end a 256-row block or a group of 1024, against the oracle on the sequences sampled."""
 import numpy as np
 import pytest
@@ -10,7 +10,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("B,K,d,V", [(1, 1, 64, 100), (2, 3, 128, 511), (2, 3, 128, 513), (3, 5, 64, 16352), (4, 4, 192, 37889), (17, 1, 64, 5000),
-                                     (16, 8, 448, 19001), (43, 3, 64, 2049), (32, 8, 64, 18945), (43, 6, 64, 2049), (130, 8, 64, 1000)])
+                                     (16, 8, 448, 19001), (4, 8, 64, 5001), (11, 3, 128, 5001), (43, 3, 64, 2049), (32, 8, 64, 18945), (43, 6, 64, 2049), (130, 8, 64, 1000)])
 def test_divergences_and_tokens(oracle, B, K, d, V):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
@@ -47,3 +47,29 @@ def test_divergences_and_tokens(oracle, B, K, d, V):
             assert lo - slack <= t <= float(c[x]) + slack and float(w[x]) > 0
             ties += not (lo <= t < float(c[x]))
         assert ties <= max(1, B // 8)
+
+
+@pytest.mark.parametrize("V,d", [(152064, 1024), (128256, 2048)])
+def test_fewer_rows_take_no_longer(V, d):
+    """The form for few rows ends where the pairs of CTAs take over: a call with half of a tile's 256 rows (or a quarter, or
+    an eighth) is no slower than the full tile. Best of five; a tenth for what a shared GPU adds."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2510_12966_b200 import binding as psd, workloads as wl
+    h, w_t, zs, tok = wl.make_fused_inputs(32, 8, V, d, 4, 0.7, device=torch.device("cuda"))
+
+    def best(B):
+        args = h[:B * 8], w_t, zs[:B], tok[:B], 0.05
+        times = []
+        for i in range(7):
+            e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            e[0].record()
+            psd.verify_fused_lmhead(*args)
+            e[1].record()
+            torch.cuda.synchronize()
+            times.append(e[0].elapsed_time(e[1]))
+        return min(times[2:])
+
+    full = best(32)
+    for B in (16, 8, 4):
+        assert best(B) < 1.1 * full, (B, full)
