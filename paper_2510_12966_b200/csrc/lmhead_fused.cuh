@@ -9,6 +9,8 @@
 //   sweep    the GEMM; per (row, column part of a tile): the fp32 logits, and partial (max, sum-exp) of the large
 //            logits (from the accumulator) and of the small ones (bf16, read from HBM)
 //   terms    per (row, 512-column segment): divergence terms, residual mass and mass of p from both models' logits
+//            (KL(large || small) of large calls separates into sums the sweep takes along, sum_i P_i (z_i - x_i): where the
+//            caller takes no residual masses there is no such launch, and the final kernel forms those of the row it draws from)
 //   final    per sequence: row totals, accept bits, accepted prefix, and the residual draw: the segment is found
 //            from the per-segment masses, the token from that segment's logits
 // Measured, whole call: 574 -> 348 us at that size, 105 -> 36.9 us at M = 15, d = 2048, V = 32000, against two runs of
@@ -62,6 +64,7 @@ struct LmParams {
   float2* part_small;
   float4* row_lse;                // [rows] (m2_small, l2s_small, m2_large, l2s_large)
   float4* part_div;               // [rows][n_seg] (divergence in bits, residual mass, mass of p, unused)
+  float* part_t;                  // [rows][n_part] KL, sweeps of 256-row blocks: sum of P_i (z_i - x_i) c, P_i = 2^(z_i c - the part's max)
   int* status;
 };
 
@@ -170,15 +173,25 @@ __device__ __forceinline__ void load_small32(const __nv_bfloat16* p, bool aligne
   }
 }
 
+// 8 consecutive floats at a 32-byte boundary: a whole sector per lane, where the rows of a warp lie far apart (two stores of
+// 16 bytes: 291 us a call at M = 256, d = 4096, V = 128256, KL with everything accepted 263; this: 286 and 258)
+__device__ __forceinline__ void store8(float* p, const float* v) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+               ::"l"(p), "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])), "r"(__float_as_uint(v[3])),
+                 "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])), "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7])) : "memory");
+}
+
 // The epilogue of `width` columns of a tile for this thread's row: reads the accumulator from tensor memory 32
 // columns at a time (all 32 lanes execute the loads, whatever row_ok says) and the small model's logits from global
 // memory; leaves the logits in z and the columns' (max, sum) partials as part `part` of the row.
+template <bool KL>
 __device__ __forceinline__ void lm_epilogue(const LmParams& P, unsigned tacc, int n0, int width, int row, int part) {
   const bool row_ok = row < P.M;
   const __nv_bfloat16* small_row = P.small + static_cast<size_t>(row_ok ? row : 0) * P.V;
   const long long srow = row - P.grp0;
   OnlineLse ol, os;
   ol.init(); os.init();
+  float kl_t = 0.f;
 #pragma unroll 1
   for (int cb = 0; cb * 32 < width; ++cb) {
     float z[32], x[32];
@@ -187,22 +200,37 @@ __device__ __forceinline__ void lm_epilogue(const LmParams& P, unsigned tacc, in
     const int nw = min(32, width - cb * 32);   // columns of this group that are the part's: a multiple of 16
     const int nv = min(nw, P.V - col0);        // ... and inside the vocabulary (<= 0: none)
     if (row_ok && nv > 0) {
-      float4* zp = reinterpret_cast<float4*>(P.z + srow * P.ldz + col0);   // columns beyond V land in the row's padding
+      float* zp = P.z + srow * P.ldz + col0;   // columns beyond V land in the row's padding
 #pragma unroll
-      for (int v = 0; v < 8; ++v)
-        if (v * 4 < nw) zp[v] = make_float4(z[4 * v], z[4 * v + 1], z[4 * v + 2], z[4 * v + 3]);
+      for (int v = 0; v < 4; ++v)
+        if (v * 8 < nw) store8(zp + v * 8, z + v * 8);
       const __nv_bfloat16* sp = small_row + col0;
       load_small32(sp, (reinterpret_cast<uintptr_t>(sp) & 15u) == 0, nv, x);
+      const float m_before = ol.m;
       ol.add<32>(z, P.c, nv);
       os.add<32>(x, P.c, nv);
+      if (KL) {
+        kl_t *= ex2_approx(m_before - ol.m);   // the group may have raised the part's max
+        float t = 0.f;
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+          if (i < nv) {
+            const float e = ex2_approx(fmaf(z[i], P.c, -ol.m));
+            if (e > 0.f) t = fmaf(e, (z[i] - x[i]) * P.c, t);   // q_i = 0 under p_i > 0 gives +inf, as it should
+          }
+        }
+        kl_t += t;
+      }
     }
   }
   if (row_ok) {
     P.part_large[srow * P.n_part + part] = make_float2(ol.m, ol.s);
     P.part_small[srow * P.n_part + part] = make_float2(os.m, os.s);
+    if (KL) P.part_t[srow * P.n_part + part] = kl_t;
   }
 }
 
+template <bool KL>
 __global__ void __launch_bounds__(kLmThreads, 1)
 lmhead_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, const LmParams P) {
   extern __shared__ unsigned char lm_smem_raw[];
@@ -302,7 +330,7 @@ lmhead_sweep_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
       tc_fence_after();
       const unsigned tacc = tmem_base + static_cast<unsigned>(buf) * 256u + static_cast<unsigned>(half) * 128u +
                             (static_cast<unsigned>(quarter * 32) << 16);
-      lm_epilogue(P, tacc, tile * kLmN, kLmN, row, tile);
+      lm_epilogue<KL>(P, tacc, tile * kLmN, kLmN, row, tile);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&bars->tmem_empty[buf]);   // this warp has read its part of the accumulator
@@ -371,6 +399,7 @@ __device__ __forceinline__ void mbar_arrive_remote_release(unsigned cluster_addr
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 
+template <bool KL>
 __global__ void __launch_bounds__(kLmThreads, 1)
 lmhead_sweep2sm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, const LmParams P) {
   extern __shared__ unsigned char lm_smem_raw[];
@@ -476,7 +505,7 @@ lmhead_sweep2sm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
       tc_fence_after();
       const unsigned tacc = tmem_base + static_cast<unsigned>(buf) * 256u + static_cast<unsigned>(half * half_n) +
                             (static_cast<unsigned>(quarter * 32) << 16);
-      lm_epilogue(P, tacc, tile * tile_n + half * half_n, half_n, row, tile * 2 + half);
+      lm_epilogue<KL>(P, tacc, tile * tile_n + half * half_n, half_n, row, tile * 2 + half);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_remote_release(drained + static_cast<unsigned>(buf) * 8u);
@@ -683,6 +712,99 @@ __device__ __forceinline__ void lse_merge_warp(float& m, float& s) {
   for (int o = 16; o > 0; o >>= 1) lse_merge(m, s, __shfl_xor_sync(0xffffffffu, m, o), __shfl_xor_sync(0xffffffffu, s, o));
 }
 
+// One row as the terms of its segments are formed from it: its logits and the models' normalisers (base 2).
+struct LmRow {
+  const float* z;
+  const __nv_bfloat16* x;
+  int V;
+  float c, off_l, off_s;
+  bool x_vec;
+
+  __device__ __forceinline__ LmRow(const LmParams& P, long long srow, float off_large, float off_small)
+      : z(P.z + srow * P.ldz), x(P.small + static_cast<size_t>(P.grp0 + srow) * P.V), V(P.V), c(P.c), off_l(off_large), off_s(off_small),
+        x_vec((reinterpret_cast<uintptr_t>(x) & 7u) == 0) {}
+  // a lane's vectors of a segment
+  __device__ __forceinline__ void fetch(int seg, int lane, float4 (&fz)[4], uint2 (&fx)[4]) const {
+    if (x_vec && (seg + 1) * kLmSeg <= V) {
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        fz[h] = __ldcg(reinterpret_cast<const float4*>(z + seg * kLmSeg + h * 128 + lane * 4));   // written by the launch before
+        fx[h] = __ldg(reinterpret_cast<const uint2*>(x + seg * kLmSeg + h * 128 + lane * 4));
+      }
+    } else {   // the row's last segment, or logits that do not start at 8 bytes
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        float zz[4];
+        unsigned xx[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int col = seg * kLmSeg + h * 128 + lane * 4 + i;
+          zz[i] = col < V ? __ldcg(z + col) : -INFINITY;
+          xx[i] = col < V ? __ldg(reinterpret_cast<const unsigned short*>(x) + col) : 0xff80u;
+        }
+        fz[h] = make_float4(zz[0], zz[1], zz[2], zz[3]);
+        fx[h] = make_uint2(xx[0] | (xx[1] << 16), xx[2] | (xx[3] << 16));
+      }
+    }
+  }
+  // the segment's (divergence in bits, residual mass, mass of p), over the whole warp
+  template <int DIV>
+  __device__ __forceinline__ float4 terms(const float4 (&fz)[4], const uint2 (&fx)[4]) const {
+    float2 js2 = make_float2(0.f, 0.f);
+    float resid = 0.f, pmass = 0.f;
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const float2 zz[2] = {make_float2(fz[h].x, fz[h].y), make_float2(fz[h].z, fz[h].w)};
+      const float2 xx[2] = {Pairs<__nv_bfloat16>::widen(fx[h].x), Pairs<__nv_bfloat16>::widen(fx[h].y)};
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const float2 cc = splat2(c);
+        float2 a = __ffma2_rn(zz[i], cc, splat2(-off_l)), b = __ffma2_rn(xx[i], cc, splat2(-off_s));   // log2 p, log2 q
+        if (DIV == kDivKL) {
+          // KL(large || small) on unclamped logits: q = 0 under p > 0 gives +inf, as it should
+          const float2 p = ex2_2(a), q = ex2_2(b);
+          if (p.x > 0.f) js2.x = fmaf(p.x, a.x - b.x, js2.x);
+          if (p.y > 0.f) js2.y = fmaf(p.y, a.y - b.y, js2.y);
+          resid += fmaxf(p.x - q.x, 0.f) + fmaxf(p.y - q.y, 0.f);
+          pmass += p.x + p.y;
+        } else {
+          // beyond the vocabulary both are -inf: 2^-125, which no sum of positive masses sees
+          a = make_float2(fmaxf(a.x, -125.f), fmaxf(a.y, -125.f));
+          b = make_float2(fmaxf(b.x, -125.f), fmaxf(b.y, -125.f));
+          const float2 e = make_float2(ex2_approx(fmaxf(a.x, b.x)), ex2_approx(fmaxf(a.y, b.y)));   // max(p, q)
+          const float2 dd = __ffma2_rn(b, splat2(-1.f), a);
+          const float2 u = make_float2(ex2_approx(-fabsf(dd.x)), ex2_approx(-fabsf(dd.y)));
+          const float2 ps = psi_poly<7>(u);
+          js2 = __ffma2_rn(e, make_float2(fmaf(u.x, -fabsf(dd.x), ps.x), fmaf(u.y, -fabsf(dd.y), ps.y)), js2);
+          const float2 lo = __fmul2_rn(e, u);             // min(p, q)
+          resid += (dd.x > 0.f) ? e.x - lo.x : 0.f;       // max(0, p - q)
+          resid += (dd.y > 0.f) ? e.y - lo.y : 0.f;
+          pmass += (dd.x >= 0.f) ? e.x : lo.x;            // p
+          pmass += (dd.y >= 0.f) ? e.y : lo.y;
+        }
+      }
+    }
+    return make_float4(warp_reduce<OpSum>(js2.x + js2.y), warp_reduce<OpSum>(resid), warp_reduce<OpSum>(pmass), 0.f);
+  }
+  // the terms of segments first, first + stride, ... below `end` into out[], by one warp; a segment's vectors are asked
+  // for before the one before it is worked on
+  template <int DIV>
+  __device__ __forceinline__ void all_terms(int first, int stride, int end, int lane, float4* out) const {
+    float4 z4[2][4];
+    uint2 x4[2][4];
+    if (first < end) fetch(first, lane, z4[0], x4[0]);
+    for (int seg = first; seg < end; seg += 2 * stride) {
+      if (seg + stride < end) fetch(seg + stride, lane, z4[1], x4[1]);
+      const float4 v = terms<DIV>(z4[0], x4[0]);
+      if (lane == 0) out[seg] = v;
+      if (seg + stride >= end) break;
+      if (seg + 2 * stride < end) fetch(seg + 2 * stride, lane, z4[0], x4[0]);
+      const float4 w = terms<DIV>(z4[1], x4[1]);
+      if (lane == 0) out[seg + stride] = w;
+    }
+  }
+};
+
 template <int DIV>
 __global__ void __launch_bounds__(kLmTermThreads, kLmTermCtas) lmhead_terms_kernel(const LmParams P, const int items_per_cta) {
   __shared__ float4 sh_part[kLmTermThreads / 32];
@@ -713,84 +835,7 @@ __global__ void __launch_bounds__(kLmTermThreads, kLmTermCtas) lmhead_terms_kern
     lse_merge_warp(ms, ss);
     const float l2sl = lg2_approx(sl), l2ss = lg2_approx(ss);
     if (seg0 == 0 && tid == 0) P.row_lse[srow] = make_float4(ms, l2ss, ml, l2sl);
-    const float off_l = ml + l2sl, off_s = ms + l2ss, c = P.c;
-
-    const float* zrow = P.z + srow * P.ldz;
-    const __nv_bfloat16* xrow = P.small + static_cast<size_t>(P.grp0 + srow) * P.V;
-    const bool x_vec = (reinterpret_cast<uintptr_t>(xrow) & 7u) == 0;
-    // a segment's vectors are asked for before the one before it is worked on
-    float4 z4[2][4];
-    uint2 x4[2][4];
-    auto fetch = [&](int seg, float4 (&fz)[4], uint2 (&fx)[4]) {
-      if (seg < seg_end && x_vec && (seg + 1) * kLmSeg <= P.V) {
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-          fz[h] = __ldcg(reinterpret_cast<const float4*>(zrow + seg * kLmSeg + h * 128 + lane * 4));   // written by the launch before
-          fx[h] = __ldg(reinterpret_cast<const uint2*>(xrow + seg * kLmSeg + h * 128 + lane * 4));
-        }
-      } else if (seg < seg_end) {   // the row's last segment, or logits that do not start at 8 bytes
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-          float z[4];
-          unsigned x[4];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int col = seg * kLmSeg + h * 128 + lane * 4 + i;
-            z[i] = col < P.V ? __ldcg(zrow + col) : -INFINITY;
-            x[i] = col < P.V ? __ldg(reinterpret_cast<const unsigned short*>(xrow) + col) : 0xff80u;
-          }
-          fz[h] = make_float4(z[0], z[1], z[2], z[3]);
-          fx[h] = make_uint2(x[0] | (x[1] << 16), x[2] | (x[3] << 16));
-        }
-      }
-    };
-    fetch(seg0 + warp, z4[0], x4[0]);
-    auto segment = [&](int seg, const float4 (&fz)[4], const uint2 (&fx)[4]) {
-      float2 js2 = make_float2(0.f, 0.f);
-      float resid = 0.f, pmass = 0.f;
-#pragma unroll
-      for (int h = 0; h < 4; ++h) {
-        const float2 zz[2] = {make_float2(fz[h].x, fz[h].y), make_float2(fz[h].z, fz[h].w)};
-        const float2 xx[2] = {Pairs<__nv_bfloat16>::widen(fx[h].x), Pairs<__nv_bfloat16>::widen(fx[h].y)};
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          const float2 cc = splat2(c);
-          float2 a = __ffma2_rn(zz[i], cc, splat2(-off_l)), b = __ffma2_rn(xx[i], cc, splat2(-off_s));   // log2 p, log2 q
-          if (DIV == kDivKL) {
-            // KL(large || small) on unclamped logits: q = 0 under p > 0 gives +inf, as it should
-            const float2 p = ex2_2(a), q = ex2_2(b);
-            if (p.x > 0.f) js2.x = fmaf(p.x, a.x - b.x, js2.x);
-            if (p.y > 0.f) js2.y = fmaf(p.y, a.y - b.y, js2.y);
-            resid += fmaxf(p.x - q.x, 0.f) + fmaxf(p.y - q.y, 0.f);
-            pmass += p.x + p.y;
-          } else {
-            // beyond the vocabulary both are -inf: 2^-125, which no sum of positive masses sees
-            a = make_float2(fmaxf(a.x, -125.f), fmaxf(a.y, -125.f));
-            b = make_float2(fmaxf(b.x, -125.f), fmaxf(b.y, -125.f));
-            const float2 e = make_float2(ex2_approx(fmaxf(a.x, b.x)), ex2_approx(fmaxf(a.y, b.y)));   // max(p, q)
-            const float2 dd = __ffma2_rn(b, splat2(-1.f), a);
-            const float2 u = make_float2(ex2_approx(-fabsf(dd.x)), ex2_approx(-fabsf(dd.y)));
-            const float2 ps = psi_poly<7>(u);
-            js2 = __ffma2_rn(e, make_float2(fmaf(u.x, -fabsf(dd.x), ps.x), fmaf(u.y, -fabsf(dd.y), ps.y)), js2);
-            const float2 lo = __fmul2_rn(e, u);             // min(p, q)
-            resid += (dd.x > 0.f) ? e.x - lo.x : 0.f;       // max(0, p - q)
-            resid += (dd.y > 0.f) ? e.y - lo.y : 0.f;
-            pmass += (dd.x >= 0.f) ? e.x : lo.x;            // p
-            pmass += (dd.y >= 0.f) ? e.y : lo.y;
-          }
-        }
-      }
-      float js = js2.x + js2.y;
-      js = warp_reduce<OpSum>(js); resid = warp_reduce<OpSum>(resid); pmass = warp_reduce<OpSum>(pmass);
-      if (lane == 0) P.part_div[static_cast<size_t>(srow) * P.n_seg + seg] = make_float4(js, resid, pmass, 0.f);
-    };
-    for (int seg = seg0 + warp; seg < seg_end; seg += 2 * kWarps) {
-      fetch(seg + kWarps, z4[1], x4[1]);
-      segment(seg, z4[0], x4[0]);
-      if (seg + kWarps >= seg_end) break;
-      fetch(seg + 2 * kWarps, z4[0], x4[0]);
-      segment(seg + kWarps, z4[1], x4[1]);
-    }
+    LmRow(P, srow, ml + l2sl, ms + l2ss).all_terms<DIV>(seg0 + warp, kWarps, seg_end, lane, P.part_div + static_cast<size_t>(srow) * P.n_seg);
   }
 }
 
@@ -799,6 +844,7 @@ struct LmFinalParams {
   LmParams lm;
   int b0, K;             // first sequence of the group
   int div_kind;
+  int have_terms;        // the terms kernel has run (KL without residual masses: it has not)
   float threshold;
   int mode;
   unsigned long long seed, offset;
@@ -809,13 +855,19 @@ struct LmFinalParams {
   float* out_resid;      // [B, K] or null
 };
 
+// Logits (rows x V) from which on a KL call's divergences come from the sweep. The terms kernel that this saves takes 46 us
+// at M = 256, V = 128256 (no residual masses, d = 4096: 292 -> 267 us a call where everything is accepted, 284 where every
+// sequence draws, its CTA then forming the masses of one row, 17 us) but 7 us at M = 160, V = 32000 (d = 2048: 88 us
+// either way with everything accepted, 81 -> 90 with draws).
+constexpr long long kLmKlPartsLogits = 1ll << 24;
 constexpr int kLmFinalThreads = 256;
+constexpr int kLmFinalKlThreads = 1024;   // of the final kernel that may have a row's masses to form
 static_assert(kLmSeg == 2 * kLmFinalThreads, "a thread of the final kernel takes two columns of the chosen segment");
 
-// One level of the inverse CDF by the whole CTA: thread t holds weight w (children in thread order). Leaves in *pick the
-// first thread whose inclusive cumulative weight exceeds `target`, else the last one with a positive weight (-1: none),
-// and in *before what lies before it. Every thread returns the same values.
-template <typename V>
+// One level of the inverse CDF by the whole CTA of NT threads: thread t holds weight w (children in thread order). Leaves in
+// *pick the first thread whose inclusive cumulative weight exceeds `target`, else the last one with a positive weight (-1:
+// none), and in *before what lies before it. Every thread returns the same values.
+template <int NT, typename V>
 __device__ __forceinline__ void block_pick(V w, V target, V* sh_warp, int* sh_hit, V* sh_before, int* pick, V* before) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   V incl = w;
@@ -826,7 +878,7 @@ __device__ __forceinline__ void block_pick(V w, V target, V* sh_warp, int* sh_hi
   }
   __syncthreads();   // the shared words may still be read from the level before
   if (lane == 31) sh_warp[warp] = incl;
-  if (tid == 0) { sh_hit[0] = kLmFinalThreads; sh_hit[1] = -1; }
+  if (tid == 0) { sh_hit[0] = NT; sh_hit[1] = -1; }
   __syncthreads();
   V base = 0;
   for (int k = 0; k < warp; ++k) base += sh_warp[k];
@@ -835,39 +887,87 @@ __device__ __forceinline__ void block_pick(V w, V target, V* sh_warp, int* sh_hi
   if (live && incl > target) atomicMin(&sh_hit[0], tid);
   if (live) atomicMax(&sh_hit[1], tid);
   __syncthreads();
-  const int p = sh_hit[0] < kLmFinalThreads ? sh_hit[0] : sh_hit[1];
+  const int p = sh_hit[0] < NT ? sh_hit[0] : sh_hit[1];
   if (tid == p) *sh_before = incl - w;
   __syncthreads();
   *pick = p;
   *before = p >= 0 ? *sh_before : static_cast<V>(0);
 }
 
-__global__ void __launch_bounds__(kLmFinalThreads) lmhead_final_kernel(const LmFinalParams F) {
+// Rows' normalisers and KL divergences from the sweep's partials, KL = ln 2 (T / S_l - (lse_l - lse_s)) with T rescaled to
+// the row's maximum like S_l; the CTA's warps are shared out evenly among the K rows. Leaves sh_lse[k] = (m2_small,
+// l2s_small, m2_large, l2s_large) and sh_div[k] (nats).
+__device__ __forceinline__ void kl_rows(const LmParams& P, long long srow0, int K, float4* sh_warp, float* sh_t, float4* sh_lse, float* sh_div) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int per_row = (kLmFinalKlThreads / 32) / K, k = warp / per_row, first = (warp - k * per_row) * 32 + lane;   // K <= 32
+  const size_t at = static_cast<size_t>(srow0 + k) * P.n_part;
+  float ml = -1e30f, sl = 0.f, ms = -1e30f, ss = 0.f;
+  if (k < K) {
+    for (int t = first; t < P.n_part; t += per_row * 32) {
+      const float2 a = P.part_large[at + t], b = P.part_small[at + t];
+      lse_merge(ml, sl, a.x, a.y);
+      lse_merge(ms, ss, b.x, b.y);
+    }
+    lse_merge_warp(ml, sl);
+    lse_merge_warp(ms, ss);
+    if (lane == 0) sh_warp[warp] = make_float4(ml, sl, ms, ss);
+  }
+  __syncthreads();
+  if (k < K) {
+    const float4 v = lane < per_row ? sh_warp[k * per_row + lane] : make_float4(-1e30f, 0.f, -1e30f, 0.f);
+    ml = v.x; sl = v.y; ms = v.z; ss = v.w;
+    lse_merge_warp(ml, sl);
+    lse_merge_warp(ms, ss);
+    float tt = 0.f;   // sum over the parts of T_t * 2^(m_t - ml)
+    for (int t = first; t < P.n_part; t += per_row * 32) {
+      const float tv = P.part_t[at + t], f = ex2_approx(P.part_large[at + t].x - ml);
+      if (f > 0.f) tt = fmaf(tv, f, tt);   // a part without mass contributes nothing (0 * inf otherwise)
+    }
+    tt = warp_reduce<OpSum>(tt);
+    if (lane == 0) sh_t[warp] = tt;
+  }
+  __syncthreads();
+  if (k < K && warp == k * per_row && lane == 0) {
+    float tt = 0.f;
+    for (int j = 0; j < per_row; ++j) tt += sh_t[warp + j];
+    const float l2sl = lg2_approx(sl), l2ss = lg2_approx(ss);
+    sh_lse[k] = make_float4(ms, l2ss, ml, l2sl);
+    sh_div[k] = fmaxf(kLn2 * (__fdiv_rn(tt, sl) - ((ml + l2sl) - (ms + l2ss))), 0.f);
+  }
+  __syncthreads();
+}
+
+// PARTS: the divergences come from the sweep's partials (KL after a sweep of 256-row blocks), else from the terms kernel.
+template <bool PARTS>
+__global__ void __launch_bounds__(PARTS ? kLmFinalKlThreads : kLmFinalThreads) lmhead_final_kernel(const LmFinalParams F) {
+  constexpr int kThreads = PARTS ? kLmFinalKlThreads : kLmFinalThreads, nwarps = kThreads / 32;
   __shared__ float sh_div[32], sh_res[32], sh_px[32], sh_qx[32];
+  __shared__ float4 sh_lse[32], sh_part[PARTS ? nwarps : 1];
+  __shared__ float sh_t[PARTS ? nwarps : 1];
   __shared__ int sh_flag[32];
-  __shared__ double sh_warp_d[kLmFinalThreads / 32], sh_before_d, sh_target;
-  __shared__ float sh_warp_f[kLmFinalThreads / 32], sh_before_f;
+  __shared__ double sh_warp_d[nwarps], sh_before_d, sh_target;
+  __shared__ float sh_warp_f[nwarps], sh_before_f;
   __shared__ int sh_hit[2];
   __shared__ int sh_L, sh_seg, sh_token;
   __shared__ float sh_u2;
   const LmParams& P = F.lm;
   const int b = F.b0 + static_cast<int>(blockIdx.x), K = F.K, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  constexpr int nwarps = kLmFinalThreads / 32;
   const float c = P.c;
   asm volatile("griddepcontrol.wait;" ::: "memory");
   release_dependent_launch();
 
+  if (PARTS) kl_rows(P, static_cast<long long>(b) * K - P.grp0, K, sh_part, sh_t, sh_lse, sh_div);
   // per row: totals over the segments, and the probabilities of the row's token
   for (int k = warp; k < K; k += nwarps) {
     const int r = b * K + k;
     const size_t sr = static_cast<size_t>(r - P.grp0);
     double js = 0.0, res = 0.0;
-    for (int t = lane; t < P.n_seg; t += 32) {
+    for (int t = lane; t < P.n_seg && (!PARTS || F.have_terms); t += 32) {
       const float4 v = P.part_div[sr * P.n_seg + t];
       js += v.x; res += v.y;
     }
     js = warp_reduce<OpSum>(js); res = warp_reduce<OpSum>(res);
-    const float4 lse = P.row_lse[sr];
+    const float4 lse = PARTS ? sh_lse[k] : P.row_lse[sr];
     const int x = P.tokens[r];
     int flags = 0;
     if (!(fabsf(lse.x + lse.y) < INFINITY)) flags |= kFlagSmallNonfinite;
@@ -880,7 +980,10 @@ __global__ void __launch_bounds__(kLmFinalThreads) lmhead_final_kernel(const LmF
         qx = ex2_approx(fmaf(Elem<__nv_bfloat16>::load(P.small + static_cast<size_t>(r) * P.V, x), c, -lse.x) - lse.y);
       }
       const double scale = F.div_kind == kDivJS ? 0.5 * 0.6931471805599453 : 0.6931471805599453;   // bits -> nats, JS: its 1/2
-      sh_div[k] = fmaxf(static_cast<float>(scale * js), 0.f);
+      if (!PARTS) {
+        sh_div[k] = fmaxf(static_cast<float>(scale * js), 0.f);
+        sh_lse[k] = lse;
+      }
       sh_res[k] = fmaxf(static_cast<float>(res), 0.f);
       sh_px[k] = px; sh_qx[k] = qx; sh_flag[k] = flags;
       const bool no_dist = (flags & (kFlagSmallNonfinite | kFlagLargeNonfinite)) != 0;   // a bad token leaves D and R intact
@@ -918,10 +1021,20 @@ __global__ void __launch_bounds__(kLmFinalThreads) lmhead_final_kernel(const LmF
     } else {
       const int r = b * K + L;
       const size_t sr = static_cast<size_t>(r - P.grp0);
+      const float4 lse = sh_lse[L];
+      if (PARTS && !F.have_terms) {
+        // the masses of this row's segments, which nothing has formed yet
+        LmRow(P, static_cast<long long>(sr), lse.z + lse.w, lse.x + lse.y).all_terms<kDivKL>(warp, nwarps, P.n_seg, lane, P.part_div + sr * P.n_seg);
+        __syncthreads();
+        double res = 0.0;
+        for (int t = lane; t < P.n_seg; t += 32) res += P.part_div[sr * P.n_seg + t].y;
+        res = warp_reduce<OpSum>(res);   // every warp the same sum
+        if (tid == 0) sh_res[L] = fmaxf(static_cast<float>(res), 0.f);
+        __syncthreads();
+      }
       const bool from_large = (F.mode == kModeAssisted) || !(sh_res[L] > 0.f);
-      const float4 lse = P.row_lse[sr];
       // level 0, the segments: a thread sums a run of consecutive ones, the chosen thread walks its run
-      const int per = (P.n_seg + kLmFinalThreads - 1) / kLmFinalThreads, t0 = tid * per, t1 = min(P.n_seg, t0 + per);
+      const int per = (P.n_seg + kThreads - 1) / kThreads, t0 = tid * per, t1 = min(P.n_seg, t0 + per);
       auto seg_weight = [&](int t) -> double {
         const float4 v = P.part_div[sr * P.n_seg + t];
         return from_large ? v.z : v.y;
@@ -936,7 +1049,7 @@ __global__ void __launch_bounds__(kLmFinalThreads) lmhead_final_kernel(const LmF
       const double target = static_cast<double>(sh_u2) * total;
       int who;
       double before;
-      block_pick(run, target, sh_warp_d, sh_hit, &sh_before_d, &who, &before);
+      block_pick<kThreads>(run, target, sh_warp_d, sh_hit, &sh_before_d, &who, &before);
       if (tid == (who >= 0 ? who : 0)) {
         int pick = -1, last = -1;
         double cum = before, before_pick = before, before_last = before;
@@ -963,7 +1076,7 @@ __global__ void __launch_bounds__(kLmFinalThreads) lmhead_final_kernel(const LmF
         for (int j = 0; j < 2; ++j) {
           const int col = col0 + j;
           w[j] = 0.f;
-          if (col < P.V) {
+          if (tid < kLmFinalThreads && col < P.V) {
             const float p = ex2_approx(fmaf(P.z[sr * P.ldz + col], c, -lse.z) - lse.w);
             const float q = ex2_approx(fmaf(Elem<__nv_bfloat16>::load(P.small + static_cast<size_t>(r) * P.V, col), c, -lse.x) - lse.y);
             w[j] = from_large ? p : fmaxf(p - q, 0.f);
@@ -971,7 +1084,7 @@ __global__ void __launch_bounds__(kLmFinalThreads) lmhead_final_kernel(const LmF
         }
         const float t3 = static_cast<float>(sh_target);
         float before_f;
-        block_pick(w[0] + w[1], t3, sh_warp_f, sh_hit, &sh_before_f, &who, &before_f);
+        block_pick<kThreads>(w[0] + w[1], t3, sh_warp_f, sh_hit, &sh_before_f, &who, &before_f);
         if (tid == who) sh_token = col0 + ((w[0] > 0.f && (before_f + w[0] > t3 || !(w[1] > 0.f))) ? 0 : 1);
         __syncthreads();
         next = sh_token;

@@ -978,6 +978,9 @@ int pyramidsd_verify_fused_lmhead_ex(const psd_lmhead_args* args) {
       if (cost < best) { best = cost; tile_n = n; }
     }
   }
+  // KL: the sweep takes the divergence's sums along, from the size on where that is worth it (see kLmKlPartsLogits)
+  const bool kl_parts = kl && !use_few && M * V >= psd::kLmKlPartsLogits;
+  const bool terms = !kl_parts || out_resid_mass != nullptr;
   const int n_tiles = (V + tile_n - 1) / tile_n;
   const int n_ctas = n_tiles < sms ? n_tiles : sms;   // of the sweeps that take one tile per CTA
   const int n_part = use_pair ? 2 * n_tiles : use_few ? 4 * n_ctas : n_tiles, n_seg = (V + psd::kLmSeg - 1) / psd::kLmSeg;
@@ -985,6 +988,7 @@ int pyramidsd_verify_fused_lmhead_ex(const psd_lmhead_args* args) {
   const int group_seqs = psd::kLmGroupRows / K < B ? psd::kLmGroupRows / K : B;   // K <= 32: whole sequences
   const size_t rows_max = static_cast<size_t>(group_seqs) * K;
   const size_t bytes = align_up(rows_max * ldz * sizeof(float)) + align_up(rows_max * n_part * sizeof(float2)) * 2 +
+                       (kl_parts ? align_up(rows_max * n_part * sizeof(float)) : 0) +
                        align_up(rows_max * n_seg * sizeof(float4)) + align_up(rows_max * sizeof(float4)) + kAlign;
   rc = ensure_status(ss);
   if (rc != PSD_OK) return rc;
@@ -1027,7 +1031,8 @@ int pyramidsd_verify_fused_lmhead_ex(const psd_lmhead_args* args) {
   L.part_large = reinterpret_cast<float2*>(ws); ws += align_up(rows_max * n_part * sizeof(float2));
   L.part_small = reinterpret_cast<float2*>(ws); ws += align_up(rows_max * n_part * sizeof(float2));
   L.part_div = reinterpret_cast<float4*>(ws); ws += align_up(rows_max * n_seg * sizeof(float4));
-  L.row_lse = reinterpret_cast<float4*>(ws);
+  L.row_lse = reinterpret_cast<float4*>(ws); ws += align_up(rows_max * sizeof(float4));
+  L.part_t = kl_parts ? reinterpret_cast<float*>(ws) : nullptr;
   L.status = ss->status;
   static bool attr_set[kMaxDevices] = {};
   int dev = 0;
@@ -1035,8 +1040,10 @@ int pyramidsd_verify_fused_lmhead_ex(const psd_lmhead_args* args) {
   if (!attr_set[dev]) {
     const int one = static_cast<int>(psd::kLmSmemBytes), two = static_cast<int>(psd::kLm2SmemBytes);
     const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    if (cudaFuncSetAttribute(psd::lmhead_sweep_kernel, at, one) != cudaSuccess ||
-        cudaFuncSetAttribute(psd::lmhead_sweep2sm_kernel, at, two) != cudaSuccess ||
+    if (cudaFuncSetAttribute(psd::lmhead_sweep_kernel<false>, at, one) != cudaSuccess ||
+        cudaFuncSetAttribute(psd::lmhead_sweep_kernel<true>, at, one) != cudaSuccess ||
+        cudaFuncSetAttribute(psd::lmhead_sweep2sm_kernel<false>, at, two) != cudaSuccess ||
+        cudaFuncSetAttribute(psd::lmhead_sweep2sm_kernel<true>, at, two) != cudaSuccess ||
         cudaFuncSetAttribute(psd::lmhead_sweep_few_kernel, at, static_cast<int>(psd::kLmFewSmemBytes)) != cudaSuccess) {
       cudaGetLastError();
       return PSD_ERR_CUDA;
@@ -1063,18 +1070,21 @@ int pyramidsd_verify_fused_lmhead_ex(const psd_lmhead_args* args) {
     if (!use_pair) {
       cfg.gridDim = dim3(static_cast<unsigned>(n_ctas));
       cfg.dynamicSmemBytes = psd::kLmSmemBytes;
-      return cudaLaunchKernelEx(&cfg, psd::lmhead_sweep_kernel, map_h, map_w, L);
+      return kl_parts ? cudaLaunchKernelEx(&cfg, psd::lmhead_sweep_kernel<true>, map_h, map_w, L)
+                      : cudaLaunchKernelEx(&cfg, psd::lmhead_sweep_kernel<false>, map_h, map_w, L);
     }
     cfg.gridDim = dim3(static_cast<unsigned>(2 * (pairs > 0 ? pairs : 1)));
     cfg.dynamicSmemBytes = psd::kLm2SmemBytes;
     at[1].id = cudaLaunchAttributeClusterDimension;
     at[1].val.clusterDim.x = 2; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, psd::lmhead_sweep2sm_kernel, map_h, map_w, L);
+    return kl_parts ? cudaLaunchKernelEx(&cfg, psd::lmhead_sweep2sm_kernel<true>, map_h, map_w, L)
+                    : cudaLaunchKernelEx(&cfg, psd::lmhead_sweep2sm_kernel<false>, map_h, map_w, L);
   };
   psd::LmFinalParams F{};
   F.K = K;
   F.div_kind = args->div_kind;
+  F.have_terms = terms ? 1 : 0;
   F.threshold = threshold;
   F.mode = mode;
   F.seed = philox_seed; F.offset = offset;
@@ -1101,7 +1111,7 @@ int pyramidsd_verify_fused_lmhead_ex(const psd_lmhead_args* args) {
         e = launch_sweep();
         g_launches.fetch_add(1, std::memory_order_relaxed);
       }
-      if (e == cudaSuccess)
+      if (e == cudaSuccess && terms)
         e = kl ? launch_dependent(psd::lmhead_terms_kernel<psd::kDivKL>, grid, psd::kLmTermThreads, stream, L, per_cta)
                : launch_dependent(psd::lmhead_terms_kernel<psd::kDivJS>, grid, psd::kLmTermThreads, stream, L, per_cta);
     }
@@ -1109,9 +1119,10 @@ int pyramidsd_verify_fused_lmhead_ex(const psd_lmhead_args* args) {
     F.b0 = b0;
     if (e == cudaSuccess) {
       TimedLaunch timed(stream, 1);
-      e = launch_dependent(psd::lmhead_final_kernel, dim3(static_cast<unsigned>(nb)), psd::kLmFinalThreads, stream, F);
+      e = kl_parts ? launch_dependent(psd::lmhead_final_kernel<true>, dim3(static_cast<unsigned>(nb)), psd::kLmFinalKlThreads, stream, F)
+                   : launch_dependent(psd::lmhead_final_kernel<false>, dim3(static_cast<unsigned>(nb)), psd::kLmFinalThreads, stream, F);
     }
-    g_launches.fetch_add(2, std::memory_order_relaxed);
+    g_launches.fetch_add(terms ? 2 : 1, std::memory_order_relaxed);
     if (e != cudaSuccess) { cudaGetLastError(); return PSD_ERR_CUDA; }
   }
   return check_launch();

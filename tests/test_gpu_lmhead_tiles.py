@@ -49,6 +49,52 @@ def test_divergences_and_tokens(oracle, B, K, d, V):
         assert ties <= max(1, B // 8)
 
 
+@pytest.mark.parametrize("B,K,d,V", [(4, 8, 64, 5001), (11, 3, 128, 511), (8, 32, 64, 2049), (32, 8, 64, 18945),
+                                     (300, 1, 64, 56001), (32, 8, 64, 65537), (10, 32, 64, 53000), (43, 7, 64, 56000), (130, 8, 64, 16200)])
+@pytest.mark.parametrize("tile_variant", [None, 1])
+def test_kl_with_and_without_residual_masses(oracle, B, K, d, V, tile_variant):
+    """KL(large || small) from the terms of the stored logits, and from 2^24 logits on out of the sweep's own sums: the same
+    divergences, accept lengths and tokens whether the masses of all rows are formed or those of the rejected rows alone; any
+    number of positions per sequence (the final kernel shares its warps out among them), tiles of 160 columns (V = 18945),
+    several row blocks."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2510_12966_b200 import binding as psd, workloads as wl
+    h, w_t, zs, tok = wl.make_fused_inputs(B, K, V, d, 40 + V, 0.7, device=torch.device("cuda"))
+    z = (h.double() @ w_t.double().T).view(B, K, V)
+    lp, lq = torch.log_softmax(z, -1), torch.log_softmax(zs.double(), -1)
+    p, q = lp.exp(), lq.exp()
+    kl, resid = (p * (lp - lq)).sum(-1), (p - q).clamp(min=0).sum(-1)
+    large = B * K * V >= 1 << 24
+    for mode, tau in ((psd.FUZZY, 0.06), (psd.FUZZY, float(kl.median())), (psd.STRICT, 0.0), (psd.ASSISTED, 0.0), (psd.FUZZY, 1e9)):
+        n0 = psd.launch_count()
+        a = psd.verify_fused_lmhead(h, w_t, zs, tok, tau, mode, 3, 1, div_kind=psd.DIV_KL, want_resid=True, tile_variant=tile_variant)
+        n1 = psd.launch_count()
+        c = psd.verify_fused_lmhead(h, w_t, zs, tok, tau, mode, 3, 1, div_kind=psd.DIV_KL, want_resid=False, tile_variant=tile_variant)
+        n2 = psd.launch_count()
+        assert psd.last_status() == 0
+        assert n2 - n1 < n1 - n0 if large else n2 - n1 == n1 - n0   # no launch forms a large call's masses if nobody takes them
+        assert (a["div"].double() - kl).abs().max() < 1e-5 and (a["resid_mass"].double() - resid).abs().max() < 1e-5
+        assert torch.equal(a["div"], c["div"]) and torch.equal(a["accept_len"], c["accept_len"])
+        L, nxt, other = a["accept_len"].cpu(), a["next_token"].cpu(), c["next_token"].cpu()
+        assert ((nxt >= 0) == (L < K)).all()
+        ties = 0
+        for b in range(B):
+            k = int(L[b])
+            if k == K:
+                assert int(nxt[b]) == int(other[b]) == -1
+                continue
+            w = p[b, k] if mode == psd.ASSISTED else (p[b, k] - q[b, k]).clamp(min=0)
+            cum = torch.cumsum(w, 0).cpu()
+            _, u2 = oracle.row_uniforms(3, 1, b * K + k)
+            t, slack = u2 * float(cum[-1]), TOL["bf16"]["cdf"] * float(cum[-1])
+            for x in {int(nxt[b]), int(other[b])}:
+                lo = float(cum[x - 1]) if x else 0.0
+                assert lo - slack <= t <= float(cum[x]) + slack and float(w[x]) > 0
+                ties += not (lo <= t < float(cum[x]))
+        assert ties <= max(1, B // 8)
+
+
 @pytest.mark.parametrize("V,d", [(152064, 1024), (128256, 2048)])
 def test_fewer_rows_take_no_longer(V, d):
     """The form for few rows ends where the pairs of CTAs take over: a call with half of a tile's 256 rows (or a quarter, or
