@@ -274,8 +274,8 @@ int pyramidsd_verify_stage_noalloc(const void* logits_small, const void* logits_
  *   out_div, out_resid_mass  [B, K] float32 or NULL
  * Requires d_model a multiple of 64 (else PSD_ERR_UNSUPPORTED); hidden and w_t 16-byte aligned. Rows are
  * processed in blocks of 256 (B*K <= 256 is the intended case: one block, the weight streamed once).
- * Jensen-Shannon divergence, temperature 1. Scratch (4 V bytes per row for at most 1024 rows at a time, and partial
- * sums) is library-owned, grown with cudaMalloc on first use. Asynchronous on `cuda_stream`; device-side timeouts via pyramidsd_last_status(). */
+ * Jensen-Shannon divergence, temperature 1. Scratch (4 V bytes per row for one block of rows at a time, or as
+ * many as take 160 MB: 135 MB at V = 128256, K = 8; and partial sums) is library-owned, grown with cudaMalloc on first use. Asynchronous on `cuda_stream`; device-side timeouts via pyramidsd_last_status(). */
 int pyramidsd_verify_fused_lmhead(const void* hidden, const void* w_t, const void* logits_small,
                                   const int32_t* tokens, int B, int K, int d_model, int V, float threshold,
                                   psd_mode mode, uint64_t philox_seed, uint64_t offset,

@@ -43,17 +43,22 @@ constexpr int kLmEpiWarps = 8;
 constexpr size_t kLmSmemBytes = static_cast<size_t>(kLmStages) * kLmStageBytes + 1024 /*alignment*/ + 256 /*barriers*/;
 constexpr unsigned kLmSpinLimit = 1u << 24;
 
-// The call's rows are worked on in groups of whole sequences with at most kLmGroupRows rows, which bounds the
-// scratch the logits take (525 MB at V = 128256); a group's rows go through the GEMM in blocks of kLmM.
-constexpr int kLmGroupRows = 1024;
+// The call's rows go through the GEMM in blocks of kLmM; after every kLmGroupBytes of logits (one block at V = 128256, up
+// to four at small vocabularies, so that the launches behind the sweep have work for the whole device) the sequences that
+// are complete by then are finished. Scratch is a ring over the rows, one group and what a sequence may have begun of it
+// in the group before: 135 MB at V = 128256, K = 8. (Four blocks there would take 525 MB and save nothing: the weight is
+// streamed once per block either way.)
+constexpr int kLmGroupBlocks = 4;
+constexpr long long kLmGroupBytes = 160ll << 20;
 constexpr int kLmSeg = 512;          // columns per segment of the terms kernel: 16 per lane of a warp
 
 struct LmParams {
   const __nv_bfloat16* small;     // [M, V] bf16 logits of the small model
   const int32_t* tokens;          // [M]
-  int M, d, V;                    // M: rows up to the end of the group this launch works on
+  int M, d, V;
   int row0;                       // sweep: first row of the 256-row block this launch works on
-  int grp0;                       // first row of the group; scratch is indexed by row - grp0
+  int ring;                       // rows of scratch; row r of the call sits at r mod ring
+  int term_row0, term_rows;       // terms: the rows this launch works on
   int tile_n;                     // sweep: columns per tile (pair of CTAs: at most 256, a multiple of 32; one CTA: 128)
   int n_tiles, n_part, n_seg;     // tiles; column parts with (max, sum) partials; segments
   int w_once;                     // 1: every weight byte is read once in this call
@@ -188,7 +193,7 @@ template <bool KL>
 __device__ __forceinline__ void lm_epilogue(const LmParams& P, unsigned tacc, int n0, int width, int row, int part) {
   const bool row_ok = row < P.M;
   const __nv_bfloat16* small_row = P.small + static_cast<size_t>(row_ok ? row : 0) * P.V;
-  const long long srow = row - P.grp0;
+  const long long srow = row % P.ring;
   OnlineLse ol, os;
   ol.init(); os.init();
   float kl_t = 0.f;
@@ -663,7 +668,7 @@ lmhead_sweep_few_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
           if (g + i >= rows) break;
-          const size_t srow = static_cast<size_t>(P.row0 - P.grp0 + r0 + g + i);
+          const size_t srow = static_cast<size_t>(P.row0 + r0 + g + i);   // one block: the ring holds every row
           if (col_ok) P.z[srow * P.ldz + col] = z[i];
           const float zv = col_ok ? z[i] : -INFINITY;
           float gl = zv, gs = x[i];
@@ -684,7 +689,7 @@ lmhead_sweep_few_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_
       if (lane == 0) mbar_arrive(&bars->tmem_empty[buf]);   // this warp has read its part of the accumulator
     }
     if (lane < rows) {
-      const size_t idx = static_cast<size_t>(P.row0 - P.grp0 + r0 + lane) * P.n_part + blockIdx.x * 4 + quarter;
+      const size_t idx = static_cast<size_t>(P.row0 + r0 + lane) * P.n_part + blockIdx.x * 4 + quarter;
       P.part_large[idx] = make_float2(ml, sl);
       P.part_small[idx] = make_float2(ms, ss);
     }
@@ -698,7 +703,7 @@ lmhead_sweep_few_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_
 }
 
 // ---- terms: both models' logits against the row's normalisers -----------------------------------------------
-// The (row, segment) items of the group are cut into one run of equal length per CTA, as many CTAs as are resident, so
+// The (row, segment) items of the launch are cut into one run of equal length per CTA, as many CTAs as are resident, so
 // a run touches a row or two. For each row the CTA merges the (max, sum) partials (a few KB out of L2, the same fixed
 // tree in every CTA, so all of a row's CTAs hold the same bits; a launch of its own for it took 15 us), then each
 // warp takes segment after segment, a lane four times four consecutive columns, so that 96 bytes per lane are in
@@ -720,8 +725,8 @@ struct LmRow {
   float c, off_l, off_s;
   bool x_vec;
 
-  __device__ __forceinline__ LmRow(const LmParams& P, long long srow, float off_large, float off_small)
-      : z(P.z + srow * P.ldz), x(P.small + static_cast<size_t>(P.grp0 + srow) * P.V), V(P.V), c(P.c), off_l(off_large), off_s(off_small),
+  __device__ __forceinline__ LmRow(const LmParams& P, int row, float off_large, float off_small)
+      : z(P.z + (row % P.ring) * P.ldz), x(P.small + static_cast<size_t>(row) * P.V), V(P.V), c(P.c), off_l(off_large), off_s(off_small),
         x_vec((reinterpret_cast<uintptr_t>(x) & 7u) == 0) {}
   // a lane's vectors of a segment
   __device__ __forceinline__ void fetch(int seg, int lane, float4 (&fz)[4], uint2 (&fx)[4]) const {
@@ -812,11 +817,12 @@ __global__ void __launch_bounds__(kLmTermThreads, kLmTermCtas) lmhead_terms_kern
   constexpr int kWarps = kLmTermThreads / 32;
   asm volatile("griddepcontrol.wait;" ::: "memory");
   release_dependent_launch();
-  const int items = (P.M - P.grp0) * P.n_seg;
+  const int items = P.term_rows * P.n_seg;
   int item = static_cast<int>(blockIdx.x) * items_per_cta;
   const int end = min(items, item + items_per_cta);
   while (item < end) {   // one row of the run
-    const int srow = item / P.n_seg, seg0 = item - srow * P.n_seg, seg_end = min(P.n_seg, seg0 + (end - item));
+    const int nth = item / P.n_seg, seg0 = item - nth * P.n_seg, seg_end = min(P.n_seg, seg0 + (end - item));
+    const int row = P.term_row0 + nth, srow = row % P.ring;
     item += seg_end - seg0;
     float ml = -1e30f, sl = 0.f, ms = -1e30f, ss = 0.f;
     for (int t = tid; t < P.n_part; t += kLmTermThreads) {
@@ -835,14 +841,14 @@ __global__ void __launch_bounds__(kLmTermThreads, kLmTermCtas) lmhead_terms_kern
     lse_merge_warp(ms, ss);
     const float l2sl = lg2_approx(sl), l2ss = lg2_approx(ss);
     if (seg0 == 0 && tid == 0) P.row_lse[srow] = make_float4(ms, l2ss, ml, l2sl);
-    LmRow(P, srow, ml + l2sl, ms + l2ss).all_terms<DIV>(seg0 + warp, kWarps, seg_end, lane, P.part_div + static_cast<size_t>(srow) * P.n_seg);
+    LmRow(P, row, ml + l2sl, ms + l2ss).all_terms<DIV>(seg0 + warp, kWarps, seg_end, lane, P.part_div + static_cast<size_t>(srow) * P.n_seg);
   }
 }
 
 // ---- final kernel: one CTA per sequence ------------------------------------------------------------------
 struct LmFinalParams {
   LmParams lm;
-  int b0, K;             // first sequence of the group
+  int b0, K;             // first sequence of this launch
   int div_kind;
   int have_terms;        // the terms kernel has run (KL without residual masses: it has not)
   float threshold;
@@ -897,10 +903,10 @@ __device__ __forceinline__ void block_pick(V w, V target, V* sh_warp, int* sh_hi
 // Rows' normalisers and KL divergences from the sweep's partials, KL = ln 2 (T / S_l - (lse_l - lse_s)) with T rescaled to
 // the row's maximum like S_l; the CTA's warps are shared out evenly among the K rows. Leaves sh_lse[k] = (m2_small,
 // l2s_small, m2_large, l2s_large) and sh_div[k] (nats).
-__device__ __forceinline__ void kl_rows(const LmParams& P, long long srow0, int K, float4* sh_warp, float* sh_t, float4* sh_lse, float* sh_div) {
+__device__ __forceinline__ void kl_rows(const LmParams& P, int row0, int K, float4* sh_warp, float* sh_t, float4* sh_lse, float* sh_div) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int per_row = (kLmFinalKlThreads / 32) / K, k = warp / per_row, first = (warp - k * per_row) * 32 + lane;   // K <= 32
-  const size_t at = static_cast<size_t>(srow0 + k) * P.n_part;
+  const size_t at = static_cast<size_t>((row0 + k) % P.ring) * P.n_part;
   float ml = -1e30f, sl = 0.f, ms = -1e30f, ss = 0.f;
   if (k < K) {
     for (int t = first; t < P.n_part; t += per_row * 32) {
@@ -956,11 +962,11 @@ __global__ void __launch_bounds__(PARTS ? kLmFinalKlThreads : kLmFinalThreads) l
   asm volatile("griddepcontrol.wait;" ::: "memory");
   release_dependent_launch();
 
-  if (PARTS) kl_rows(P, static_cast<long long>(b) * K - P.grp0, K, sh_part, sh_t, sh_lse, sh_div);
+  if (PARTS) kl_rows(P, b * K, K, sh_part, sh_t, sh_lse, sh_div);
   // per row: totals over the segments, and the probabilities of the row's token
   for (int k = warp; k < K; k += nwarps) {
     const int r = b * K + k;
-    const size_t sr = static_cast<size_t>(r - P.grp0);
+    const size_t sr = static_cast<size_t>(r % P.ring);
     double js = 0.0, res = 0.0;
     for (int t = lane; t < P.n_seg && (!PARTS || F.have_terms); t += 32) {
       const float4 v = P.part_div[sr * P.n_seg + t];
@@ -1020,11 +1026,11 @@ __global__ void __launch_bounds__(PARTS ? kLmFinalKlThreads : kLmFinalThreads) l
       next = -2;
     } else {
       const int r = b * K + L;
-      const size_t sr = static_cast<size_t>(r - P.grp0);
+      const size_t sr = static_cast<size_t>(r % P.ring);
       const float4 lse = sh_lse[L];
       if (PARTS && !F.have_terms) {
         // the masses of this row's segments, which nothing has formed yet
-        LmRow(P, static_cast<long long>(sr), lse.z + lse.w, lse.x + lse.y).all_terms<kDivKL>(warp, nwarps, P.n_seg, lane, P.part_div + sr * P.n_seg);
+        LmRow(P, r, lse.z + lse.w, lse.x + lse.y).all_terms<kDivKL>(warp, nwarps, P.n_seg, lane, P.part_div + sr * P.n_seg);
         __syncthreads();
         double res = 0.0;
         for (int t = lane; t < P.n_seg; t += 32) res += P.part_div[sr * P.n_seg + t].y;

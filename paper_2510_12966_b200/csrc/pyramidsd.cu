@@ -985,8 +985,10 @@ int pyramidsd_verify_fused_lmhead_ex(const psd_lmhead_args* args) {
   const int n_ctas = n_tiles < sms ? n_tiles : sms;   // of the sweeps that take one tile per CTA
   const int n_part = use_pair ? 2 * n_tiles : use_few ? 4 * n_ctas : n_tiles, n_seg = (V + psd::kLmSeg - 1) / psd::kLmSeg;
   const long long ldz = (static_cast<long long>(n_tiles) * tile_n + 31) / 32 * 32;
-  const int group_seqs = psd::kLmGroupRows / K < B ? psd::kLmGroupRows / K : B;   // K <= 32: whole sequences
-  const size_t rows_max = static_cast<size_t>(group_seqs) * K;
+  const long long block_bytes = psd::kLmM * ldz * static_cast<long long>(sizeof(float));
+  const long long room = psd::kLmGroupBytes / block_bytes, blocks = room < 1 ? 1 : room < psd::kLmGroupBlocks ? room : psd::kLmGroupBlocks;
+  const long long group_rows = blocks * psd::kLmM;
+  const size_t rows_max = static_cast<size_t>(M <= group_rows ? M : group_rows + K - 1 < M ? group_rows + K - 1 : M);   // K <= 32
   const size_t bytes = align_up(rows_max * ldz * sizeof(float)) + align_up(rows_max * n_part * sizeof(float2)) * 2 +
                        (kl_parts ? align_up(rows_max * n_part * sizeof(float)) : 0) +
                        align_up(rows_max * n_seg * sizeof(float4)) + align_up(rows_max * sizeof(float4)) + kAlign;
@@ -1093,10 +1095,15 @@ int pyramidsd_verify_fused_lmhead_ex(const psd_lmhead_args* args) {
   F.out_next_token = out_next_token;
   F.out_div = out_div;
   F.out_resid = out_resid_mass;
-  for (int b0 = 0; b0 < B; b0 += group_seqs) {
-    const int nb = B - b0 < group_seqs ? B - b0 : group_seqs, rows = nb * K;
-    L.grp0 = b0 * K;
-    L.M = L.grp0 + rows;
+  L.M = static_cast<int>(M);
+  L.ring = static_cast<int>(rows_max);
+  int b0 = 0;
+  for (long long row_end = 0; row_end < M;) {
+    const long long row_begin = row_end;
+    row_end = M - row_begin < group_rows ? M : row_begin + group_rows;
+    const int nb = static_cast<int>(row_end / K) - b0, rows = nb * K;   // the sequences that end in this group
+    L.term_row0 = b0 * K;
+    L.term_rows = rows;
     // the terms kernel: a CTA for every resident place, unless that left its warps without a segment each
     const long long items = static_cast<long long>(rows) * n_seg;
     const int warps = psd::kLmTermThreads / 32, places = psd::kLmTermCtas * sms;
@@ -1107,7 +1114,7 @@ int pyramidsd_verify_fused_lmhead_ex(const psd_lmhead_args* args) {
     cudaError_t e = cudaSuccess;
     {
       TimedLaunch timed(stream, 0);
-      for (L.row0 = L.grp0; L.row0 < L.M && e == cudaSuccess; L.row0 += psd::kLmM) {
+      for (L.row0 = static_cast<int>(row_begin); L.row0 < row_end && e == cudaSuccess; L.row0 += psd::kLmM) {
         e = launch_sweep();
         g_launches.fetch_add(1, std::memory_order_relaxed);
       }
@@ -1124,6 +1131,7 @@ int pyramidsd_verify_fused_lmhead_ex(const psd_lmhead_args* args) {
     }
     g_launches.fetch_add(terms ? 2 : 1, std::memory_order_relaxed);
     if (e != cudaSuccess) { cudaGetLastError(); return PSD_ERR_CUDA; }
+    b0 += nb;
   }
   return check_launch();
 }

@@ -1,5 +1,6 @@
 """The LM-head form at the edges of its own cuts: 16, 17, 32 and 33 rows (the weight or the rows as the MMA's M), 128 and 129, tile
-widths other than 256 or 128 (equal rounds of narrower tiles), one and several rounds, segments of 512 columns, rows that end a 256-row block or a group of 1024, against the oracle on the sequences sampled."""
+widths other than 256 or 128 (equal rounds of narrower tiles), one and several rounds, segments of 512 columns, rows that end a
+256-row block or a group of blocks (with sequences that begin in one group and end in the next), against the oracle on the sequences sampled."""
 import numpy as np
 import pytest
 import torch
@@ -10,7 +11,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("B,K,d,V", [(1, 1, 64, 100), (2, 3, 128, 511), (2, 3, 128, 513), (3, 5, 64, 16352), (4, 4, 192, 37889), (17, 1, 64, 5000),
-                                     (16, 8, 448, 19001), (4, 8, 64, 5001), (11, 3, 128, 5001), (43, 3, 64, 2049), (32, 8, 64, 18945), (43, 6, 64, 2049), (130, 8, 64, 1000)])
+                                     (16, 8, 448, 19001), (4, 8, 64, 5001), (11, 3, 128, 5001), (43, 3, 64, 2049), (32, 8, 64, 18945), (43, 6, 64, 2049), (130, 8, 64, 1000), (90, 7, 64, 56000), (150, 7, 64, 2049), (21, 31, 64, 44032)])
 def test_divergences_and_tokens(oracle, B, K, d, V):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
@@ -119,3 +120,22 @@ def test_fewer_rows_take_no_longer(V, d):
     full = best(32)
     for B in (16, 8, 4):
         assert best(B) < 1.1 * full, (B, full)
+
+
+def test_scratch_is_one_block_of_logits():
+    """A call of 1024 rows at V = 128256 keeps one block of 256 rows of logits, not 525 MB of them."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2510_12966_b200 import binding as psd, workloads as wl
+    h, w_t, zs, tok = wl.make_fused_inputs(128, 8, 128256, 64, 4, 0.7, device=torch.device("cuda"))
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        out = torch.zeros(1 << 22, device="cuda")   # what torch itself takes on a new stream
+        del out
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        psd.verify_fused_lmhead(h, w_t, zs, tok, 0.05)
+        torch.cuda.synchronize()
+        taken = before - torch.cuda.mem_get_info()[0]
+    psd.release_stream(stream)
+    assert taken < 200 << 20, taken
