@@ -229,12 +229,16 @@ int launch_rowstats(const StageParams& P, int dtype, int variant, int cluster_si
   if (onepass < 0) onepass = (variant == PSD_KERNEL_AUTO && cluster_size == 0 && psd::onepass_applies(P, dtype, resid_wanted)) ? 1 : 0;
   if (onepass == 1) {
     TimedLaunch timed(stream, 0);
-    if (psd::launch_rowstats_onepass(P, dtype, stream, allow_triples) != 0) {
-      const cudaError_t e = cudaGetLastError();
-      std::fprintf(stderr, "pyramidsd: one-pass kernel launch failed: %s\n", cudaGetErrorString(e));
-      return PSD_ERR_CUDA;
+    const int n_seq = psd::list_sequences(P, psd::cluster_sm_count());
+    for (int b0 = 0; b0 < P.B; b0 += n_seq) {
+      const StageParams Q = n_seq == P.B ? P : psd::slice_sequences(P, static_cast<int>(elem_size(dtype)), b0, P.B - b0 < n_seq ? P.B - b0 : n_seq);
+      if (psd::launch_rowstats_onepass(Q, dtype, stream, allow_triples) != 0) {
+        const cudaError_t e = cudaGetLastError();
+        std::fprintf(stderr, "pyramidsd: one-pass kernel launch failed: %s\n", cudaGetErrorString(e));
+        return PSD_ERR_CUDA;
+      }
+      g_launches.fetch_add(1, std::memory_order_relaxed);
     }
-    g_launches.fetch_add(1, std::memory_order_relaxed);
     return check_launch();
   }
   bool use_cluster = false;
@@ -246,10 +250,17 @@ int launch_rowstats(const StageParams& P, int dtype, int variant, int cluster_si
   }
   TimedLaunch timed(stream, 0);
   if (use_cluster) {
-    if (psd::launch_rowstats_cluster(P, dtype, geom, stream) != 0) {
-      const cudaError_t e = cudaGetLastError();
-      std::fprintf(stderr, "pyramidsd: cluster kernel launch failed: %s\n", cudaGetErrorString(e));
-      return PSD_ERR_CUDA;
+    const int n_seq = geom.ra > 0 ? P.B : psd::list_sequences(P, geom.n_clusters);   // the streamed-twice form has no lists
+    for (int b0 = 0; b0 < P.B; b0 += n_seq) {
+      const StageParams Q = n_seq == P.B ? P : psd::slice_sequences(P, static_cast<int>(elem_size(dtype)), b0, P.B - b0 < n_seq ? P.B - b0 : n_seq);
+      psd::ClusterGeom slice = geom;   // cut as the whole call is: the same statistics
+      if (n_seq != P.B && static_cast<long long>(Q.B) * Q.K < slice.n_clusters) slice.n_clusters = Q.B * Q.K;
+      if (psd::launch_rowstats_cluster(Q, dtype, slice, stream) != 0) {
+        const cudaError_t e = cudaGetLastError();
+        std::fprintf(stderr, "pyramidsd: cluster kernel launch failed: %s\n", cudaGetErrorString(e));
+        return PSD_ERR_CUDA;
+      }
+      if (b0 > 0) g_launches.fetch_add(1, std::memory_order_relaxed);
     }
   } else {
     const dim3 block(1024);

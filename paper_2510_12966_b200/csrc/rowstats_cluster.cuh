@@ -283,42 +283,84 @@ struct RowWalk<true> {
   __device__ __forceinline__ int row2() const { return r / K * K2 + r % K; }   // a triple's stage-2 row b * K2 + k
 };
 
-// Fills the list: the j-th valid candidate goes to cluster j mod n_clusters. By every thread of the CTA; counts are taken
-// by ballots, a block of candidates at a time. No list without n_valid, or where it might not hold the cluster's rows: then
-// every row is taken, and the finalisation looks at the valid ones.
-__device__ __forceinline__ void build_row_list(const StageParams& P, int cluster_id, int n_clusters, RowList& list) {
+// Fills the list: the j-th valid candidate goes to cluster j mod n_clusters. By every thread of the CTA, kEach consecutive
+// candidates per thread at a time; returns the number of valid ones.
+template <int kEach>
+__device__ __forceinline__ int deal_valid_rows(const StageParams& P, int cluster_id, int n_clusters, RowList& list) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, warps = blockDim.x >> 5;
   const int rows = P.B * P.K;
-  if (P.n_valid == nullptr || P.K2 != 0 || rows > kClListRows * n_clusters) {   // n_valid speaks of the first row set only
-    if (tid == 0) {
-      list.len = (P.B * (P.K + P.K2) - cluster_id + n_clusters - 1) / n_clusters;
-      list.given = 0;
-    }
-    __syncthreads();
-    return;
-  }
   int seen = 0;   // valid candidates before this block
-  for (int base = 0; base < rows; base += static_cast<int>(blockDim.x)) {
-    const int cand = base + tid;
-    const int k = cand / P.B, b = cand - k * P.B;
-    const bool valid = cand < rows && k < P.n_valid[b];
-    const unsigned m = __ballot_sync(0xffffffffu, valid);
+  for (int base = 0; base < rows; base += static_cast<int>(blockDim.x) * kEach) {
+    const int cand = base + tid * kEach, k0 = cand / P.B, b0 = cand - k0 * P.B;
+    unsigned valid = 0u;
+#pragma unroll
+    for (int i = 0, k = k0, b = b0; i < kEach; ++i) {
+      if (cand + i < rows && k < P.n_valid[b]) valid |= 1u << i;
+      if (++b == P.B) { b = 0; ++k; }
+    }
+    int incl = __popc(valid);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int up = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += up;
+    }
+    __syncthreads();   // the counts may still be being read
+    if (lane == 31) list.warp[warp] = incl;
     __syncthreads();
-    if (lane == 0) list.warp[warp] = __popc(m);
-    __syncthreads();
-    int j = seen + __popc(m & ((1u << lane) - 1u));
+    int j = seen + incl - __popc(valid);
     for (int w = 0; w < warps; ++w) {
       const int c = list.warp[w];
       if (w < warp) j += c;
       seen += c;
     }
-    if (valid && j % n_clusters == cluster_id) list.row[j / n_clusters] = b * P.K + k;
+#pragma unroll
+    for (int i = 0, k = k0, b = b0; i < kEach; ++i) {
+      if (valid >> i & 1u) {
+        if (j % n_clusters == cluster_id) list.row[j / n_clusters] = b * P.K + k;
+        ++j;
+      }
+      if (++b == P.B) { b = 0; ++k; }
+    }
   }
-  if (tid == 0) {
-    list.len = seen / n_clusters + (cluster_id < seen % n_clusters ? 1 : 0);
-    list.given = 1;
+  return seen;
+}
+// The cluster's list. None without n_valid. The host launches no more candidates than lists hold, see list_sequences.
+// Two candidates per thread where that takes one go (256 sequences, K = 32, V = 4032 bf16: 78 us a call with one candidate
+// per thread, 72 with eight; 2048 sequences, K = 32, V = 2048: 486 and 432; 48 sequences, K = 16, V = 32000 fp32: 40.5, with
+// eight 41.2).
+__device__ __forceinline__ void build_row_list(const StageParams& P, int cluster_id, int n_clusters, RowList& list) {
+  if (P.n_valid == nullptr || P.K2 != 0) {   // n_valid speaks of the first row set only
+    if (threadIdx.x == 0) {
+      list.len = (P.B * (P.K + P.K2) - cluster_id + n_clusters - 1) / n_clusters;
+      list.given = 0;
+    }
+  } else {
+    const int seen = P.B * P.K <= 2 * static_cast<int>(blockDim.x) ? deal_valid_rows<2>(P, cluster_id, n_clusters, list)
+                                                                   : deal_valid_rows<8>(P, cluster_id, n_clusters, list);
+    if (threadIdx.x == 0) {
+      list.len = seen / n_clusters + (cluster_id < seen % n_clusters ? 1 : 0);
+      list.given = 1;
+    }
   }
   __syncthreads();
+}
+
+// Sequences whose candidate rows fit the lists of a launch of `n_clusters`: all of them, unless n_valid is given and there
+// are many (the host then launches slices; streaming what is not valid instead took 1760 us where 1170 do).
+inline int list_sequences(const StageParams& P, int n_clusters) {
+  if (P.n_valid == nullptr || P.K2 != 0 || P.K == 0) return P.B;
+  const long long most = static_cast<long long>(kClListRows) * n_clusters / P.K;
+  return most < P.B ? (most > 1 ? static_cast<int>(most) : 1) : P.B;
+}
+// The launch's sequences [b0, b0 + n) as a launch of their own.
+inline StageParams slice_sequences(const StageParams& P, int elem_bytes, int b0, int n) {
+  StageParams Q = P;
+  Q.small = static_cast<const char*>(P.small) + b0 * P.seq_stride_small * elem_bytes;
+  Q.large = static_cast<const char*>(P.large) + b0 * P.seq_stride_large * elem_bytes;
+  Q.n_valid = P.n_valid + b0;
+  Q.stats = P.stats + static_cast<long long>(b0) * P.K;
+  Q.B = n;
+  return Q;
 }
 
 template <typename T>

@@ -1,0 +1,75 @@
+"""Stages with n_valid: the statistics kernels' lists of valid rows, at the sizes where they are built in another way (two
+candidates per thread, eight, several blocks of them), and with more candidates than the lists hold, where the same results
+come out as for the same sequences in slices that fit and the positions beyond n_valid cost nothing."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("div_kind", [0, 2])   # JS: the cluster kernel; KL without residual masses: the one-pass kernel
+def test_more_rows_than_the_lists_hold(div_kind):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2510_12966_b200 import binding as psd
+    psd.load_library()
+    B, K, V = 4800, 32, 2048      # 153600 candidates; 148 lists of 1024
+    g = torch.Generator(device="cuda").manual_seed(3)
+    zs = torch.randn((B, K, V), generator=g, device="cuda", dtype=torch.bfloat16)
+    zl = zs + 0.3 * torch.randn((B, K, V), generator=g, device="cuda", dtype=torch.bfloat16)
+    tok = torch.randint(0, V, (B, K), generator=g, device="cuda", dtype=torch.int32)
+    few = torch.randint(0, 4, (B,), generator=g, device="cuda", dtype=torch.int32)
+
+    def call(n_valid, lo=0, hi=B):
+        return psd.verify_stage_ex(zs[lo:hi], zl[lo:hi], tok[lo:hi], 0.02, psd.FUZZY_SD_FALLBACK, 7, 0, n_valid=n_valid[lo:hi],
+                                   div_kind=div_kind, want_resid=div_kind == 0, seq_index_base=lo)
+
+    whole = call(few)
+    assert psd.last_status() == 0
+    for lo in range(0, B, 1600):
+        part = call(few, lo, lo + 1600)
+        for k in ("accept_len", "next_token", "div", "p_small_tok", "p_large_tok", "row_flags"):
+            assert torch.equal(part[k], whole[k][lo:lo + 1600]), k
+
+    def best(n_valid):
+        times = []
+        for _ in range(6):
+            e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            e[0].record()
+            call(n_valid)
+            e[1].record()
+            torch.cuda.synchronize()
+            times.append(e[0].elapsed_time(e[1]))
+        return min(times[1:])
+
+    # a twentieth of the rows takes part; the rest of the call does not shrink with them
+    assert best(few) < 0.5 * best(torch.full_like(few, K))
+
+
+@pytest.mark.parametrize("B,K", [(1, 32), (3, 1), (40, 32), (43, 31), (160, 32), (161, 32), (700, 17)])
+@pytest.mark.parametrize("div_kind", [0, 2])
+def test_lists_against_single_sequences(B, K, div_kind):
+    """Windows of every length, empty ones and ones beyond K among them."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2510_12966_b200 import binding as psd
+    psd.load_library()
+    V = 2048
+    g = torch.Generator(device="cuda").manual_seed(B)
+    zs = torch.randn((B, K, V), generator=g, device="cuda")
+    zl = zs + 0.3 * torch.randn((B, K, V), generator=g, device="cuda")
+    tok = torch.randint(0, V, (B, K), generator=g, device="cuda", dtype=torch.int32)
+    for n_valid in (torch.randint(-2, K + 3, (B,), generator=g, device="cuda", dtype=torch.int32), torch.zeros(B, dtype=torch.int32, device="cuda"),
+                    torch.full((B,), K, dtype=torch.int32, device="cuda")):
+        out = psd.verify_stage_ex(zs, zl, tok, 0.03, psd.FUZZY, 7, 0, n_valid=n_valid, div_kind=div_kind, want_resid=div_kind == 0)
+        assert psd.last_status() == 0
+        p, q = torch.log_softmax(zl.double(), -1), torch.log_softmax(zs.double(), -1)
+        if div_kind == 2:
+            want = (p.exp() * (p - q)).sum(-1)
+        else:
+            m = torch.logaddexp(p, q) - np.log(2.0)
+            want = 0.5 * (p.exp() * (p - m) + q.exp() * (q - m)).sum(-1)
+        live = torch.arange(K, device="cuda")[None, :] < n_valid[:, None]
+        assert ((out["div"].double() - want)[live].abs() < 1e-5).all() and (out["div"][~live] == 0).all()
+        assert torch.equal(out["accept_len"], ((out["div"] <= 0.03) & live).int().cumprod(-1).sum(-1).int())
