@@ -12,6 +12,7 @@
 
 #include "common.cuh"
 #include "finalize.cuh"
+#include "host_copies.h"
 #include "rowstats_baseline.cuh"
 #include "rowstats_cluster.cuh"
 #include "rowstats_onepass.cuh"
@@ -831,37 +832,41 @@ int pyramidsd_verify_host(const void* logits_draft, const void* logits_qual, con
   }
   rc = grow(ss, &ss->out4, &ss->out4_bytes, static_cast<size_t>(4) * B * 4);
   if (rc != PSD_OK) return rc;
-  if (n_d + n_t >= kHostOverlapBytes) {
+  // below a few megabytes the copies are shorter than what the two streams' events cost
+  const bool overlap = n_d + n_t >= kHostOverlapBytes;
+  if (overlap) {
     rc = ensure_copy_stream(ss);
     if (rc != PSD_OK) return rc;
   }
-  // Large inputs: the copies go through a stream of their own, so that stage 1 runs while the target's logits are on
-  // their way. Below a few megabytes the copies are shorter than what the two streams' events cost.
-  const bool overlap = n_d + n_t >= kHostOverlapBytes;
-  const cudaStream_t cs = overlap ? ss->copy_stream : s;
-  const void* src[4] = {logits_draft, logits_qual, logits_target, draft_tokens};
-  auto copy_in = [&](int i) { return cudaMemcpyAsync(ss->stage[i], src[i], want[i], cudaMemcpyHostToDevice, cs) == cudaSuccess; };
-  if (overlap && (cudaEventRecord(ss->copy_ev[0], s) != cudaSuccess || cudaStreamWaitEvent(cs, ss->copy_ev[0], 0) != cudaSuccess)) return PSD_ERR_CUDA;
-  if (!copy_in(3) || !copy_in(0) || !copy_in(1)) return PSD_ERR_CUDA;
-  if (overlap && (cudaEventRecord(ss->copy_ev[1], cs) != cudaSuccess || cudaStreamWaitEvent(s, ss->copy_ev[1], 0) != cudaSuccess)) return PSD_ERR_CUDA;
-  if (!copy_in(2)) return PSD_ERR_CUDA;
-  if (overlap && cudaEventRecord(ss->copy_ev[2], cs) != cudaSuccess) return PSD_ERR_CUDA;
   int32_t* o = static_cast<int32_t*>(ss->out4);
   a.logits_draft = ss->stage[0]; a.logits_qual = ss->stage[1]; a.logits_target = ss->stage[2];
   a.draft_tokens = static_cast<const int32_t*>(ss->stage[3]);
   a.out_accept_len_q = o; a.out_next_token_q = o + B; a.out_accept_len = o + 2 * B; a.out_next_token = o + 3 * B;
-  rc = verify_two_stage_locked(&a, ss, ss->status, s, overlap ? ss->copy_ev[2] : nullptr);
-  if (rc != PSD_OK) {
-    if (overlap) cudaStreamSynchronize(cs);   // the caller's buffers are read by copies still in flight
-    return rc;
-  }
-  int32_t* dst[4] = {out_accept_len_q, out_next_token_q, out_accept_len, out_next_token};
-  const size_t row = static_cast<size_t>(B) * 4;
-  // results that lie behind one another in the caller's memory, as they do here, come back in one copy
-  const bool joined = dst[1] == dst[0] + B && dst[2] == dst[1] + B && dst[3] == dst[2] + B;
-  for (int i = 0; i < (joined ? 1 : 4); ++i)
-    if (cudaMemcpyAsync(dst[i], o + static_cast<size_t>(i) * B, joined ? 4 * row : row, cudaMemcpyDeviceToHost, s) != cudaSuccess) return PSD_ERR_CUDA;
-  return cudaStreamSynchronize(s) == cudaSuccess ? PSD_OK : PSD_ERR_CUDA;
+  struct Api {
+    StreamScratch* ss;
+    cudaStream_t streams[2];
+    const void* src[4];
+    const size_t* bytes;
+    const psd_pyramid_args* a;
+    int32_t* o;
+    int32_t* dst[4];
+    bool overlap;
+    bool record(int e, int s) { return cudaEventRecord(ss->copy_ev[e], streams[s]) == cudaSuccess; }
+    bool wait(int s, int e) { return cudaStreamWaitEvent(streams[s], ss->copy_ev[e], 0) == cudaSuccess; }
+    bool copy_in(int i, int s) { return cudaMemcpyAsync(ss->stage[i], src[i], bytes[i], cudaMemcpyHostToDevice, streams[s]) == cudaSuccess; }
+    int run() { return verify_two_stage_locked(a, ss, ss->status, streams[0], overlap ? ss->copy_ev[2] : nullptr); }
+    bool copy_out() {
+      const size_t row = static_cast<size_t>(a->B) * 4;
+      // results that lie behind one another in the caller's memory, as they do here, come back in one copy
+      const bool joined = dst[1] == dst[0] + a->B && dst[2] == dst[1] + a->B && dst[3] == dst[2] + a->B;
+      for (int i = 0; i < (joined ? 1 : 4); ++i)
+        if (cudaMemcpyAsync(dst[i], o + static_cast<size_t>(i) * a->B, joined ? 4 * row : row, cudaMemcpyDeviceToHost, streams[0]) != cudaSuccess) return false;
+      return true;
+    }
+    bool sync(int s) { return cudaStreamSynchronize(streams[s]) == cudaSuccess; }
+  } api{ss, {s, ss->copy_stream}, {logits_draft, logits_qual, logits_target, draft_tokens}, want, &a, o,
+        {out_accept_len_q, out_next_token_q, out_accept_len, out_next_token}, overlap};
+  return psd::host_pipeline(api, overlap, PSD_OK, PSD_ERR_CUDA);
 }
 
 int pyramidsd_verify_stage_noalloc(const void* logits_small, const void* logits_large, const int32_t* draft_tokens,
