@@ -61,6 +61,8 @@ struct StreamScratch {
   size_t stage_bytes[4] = {0, 0, 0, 0};
   void* out4 = nullptr;     // 4 x [B] results of the host entry point
   size_t out4_bytes = 0;
+  void* out4_host = nullptr;   // the same in pinned host memory, from where they go to the caller's four arrays
+  size_t out4_host_bytes = 0;
   void* lm_ws = nullptr;    // partial sums of the fused LM-head path
   size_t lm_ws_bytes = 0;
   void* draw = nullptr;     // records and tile totals of the three-launch finalisation
@@ -134,6 +136,24 @@ int grow(StreamScratch* ss, void** ptr, size_t* have, size_t want) {
   }
   if (cudaMalloc(ptr, want) != cudaSuccess) { cudaGetLastError(); return PSD_ERR_CUDA; }
   *have = want;
+  return PSD_OK;
+}
+
+// with ss->mu held: the pinned buffer of the results
+int grow_pinned(StreamScratch* ss, size_t want) {
+  if (ss->out4_host_bytes >= want) return PSD_OK;
+  if (ss->out4_host) {
+    if (cudaStreamSynchronize(ss->stream) != cudaSuccess) return PSD_ERR_CUDA;
+    cudaFreeHost(ss->out4_host);
+    ss->out4_host = nullptr;
+    ss->out4_host_bytes = 0;
+  }
+  if (cudaHostAlloc(&ss->out4_host, want, cudaHostAllocDefault) != cudaSuccess) {
+    cudaGetLastError();
+    ss->out4_host = nullptr;
+    return PSD_ERR_CUDA;
+  }
+  ss->out4_host_bytes = want;
   return PSD_OK;
 }
 
@@ -830,7 +850,9 @@ int pyramidsd_verify_host(const void* logits_draft, const void* logits_qual, con
     rc = grow(ss, &ss->stage[i], &ss->stage_bytes[i], want[i]);
     if (rc != PSD_OK) return rc;
   }
-  rc = grow(ss, &ss->out4, &ss->out4_bytes, static_cast<size_t>(4) * B * 4);
+  const size_t n_out = static_cast<size_t>(4) * B * 4;
+  rc = grow(ss, &ss->out4, &ss->out4_bytes, n_out);
+  if (rc == PSD_OK) rc = grow_pinned(ss, n_out);
   if (rc != PSD_OK) return rc;
   // below a few megabytes the copies are shorter than what the two streams' events cost
   const bool overlap = n_d + n_t >= kHostOverlapBytes;
@@ -848,25 +870,22 @@ int pyramidsd_verify_host(const void* logits_draft, const void* logits_qual, con
     const void* src[4];
     const size_t* bytes;
     const psd_pyramid_args* a;
-    int32_t* o;
-    int32_t* dst[4];
+    size_t n_out;
     bool overlap;
     bool record(int e, int s) { return cudaEventRecord(ss->copy_ev[e], streams[s]) == cudaSuccess; }
     bool wait(int s, int e) { return cudaStreamWaitEvent(streams[s], ss->copy_ev[e], 0) == cudaSuccess; }
     bool copy_in(int i, int s) { return cudaMemcpyAsync(ss->stage[i], src[i], bytes[i], cudaMemcpyHostToDevice, streams[s]) == cudaSuccess; }
     int run() { return verify_two_stage_locked(a, ss, ss->status, streams[0], overlap ? ss->copy_ev[2] : nullptr); }
-    bool copy_out() {
-      const size_t row = static_cast<size_t>(a->B) * 4;
-      // results that lie behind one another in the caller's memory, as they do here, come back in one copy
-      const bool joined = dst[1] == dst[0] + a->B && dst[2] == dst[1] + a->B && dst[3] == dst[2] + a->B;
-      for (int i = 0; i < (joined ? 1 : 4); ++i)
-        if (cudaMemcpyAsync(dst[i], o + static_cast<size_t>(i) * a->B, joined ? 4 * row : row, cudaMemcpyDeviceToHost, streams[0]) != cudaSuccess) return false;
-      return true;
-    }
+    // one copy for all four, into memory that is known to be one allocation (arrays of the caller's that lie behind one
+    // another may still be pinned one by one, which no copy may span)
+    bool copy_out() { return cudaMemcpyAsync(ss->out4_host, ss->out4, n_out, cudaMemcpyDeviceToHost, streams[0]) == cudaSuccess; }
     bool sync(int s) { return cudaStreamSynchronize(streams[s]) == cudaSuccess; }
-  } api{ss, {s, ss->copy_stream}, {logits_draft, logits_qual, logits_target, draft_tokens}, want, &a, o,
-        {out_accept_len_q, out_next_token_q, out_accept_len, out_next_token}, overlap};
-  return psd::host_pipeline(api, overlap, PSD_OK, PSD_ERR_CUDA);
+  } api{ss, {s, ss->copy_stream}, {logits_draft, logits_qual, logits_target, draft_tokens}, want, &a, n_out, overlap};
+  rc = psd::host_pipeline(api, overlap, PSD_OK, PSD_ERR_CUDA);
+  if (rc != PSD_OK) return rc;
+  int32_t* dst[4] = {out_accept_len_q, out_next_token_q, out_accept_len, out_next_token};
+  for (int i = 0; i < 4; ++i) std::memcpy(dst[i], static_cast<const int32_t*>(ss->out4_host) + static_cast<size_t>(i) * B, static_cast<size_t>(B) * 4);
+  return PSD_OK;
 }
 
 int pyramidsd_verify_stage_noalloc(const void* logits_small, const void* logits_large, const int32_t* draft_tokens,
@@ -1228,6 +1247,9 @@ int pyramidsd_release_stream(void* cuda_stream) {
     }
     e.ws_bytes = e.out4_bytes = e.lm_ws_bytes = e.draw_bytes = 0;
     for (size_t& b : e.stage_bytes) b = 0;
+    if (e.out4_host) cudaFreeHost(e.out4_host);
+    e.out4_host = nullptr;
+    e.out4_host_bytes = 0;
     if (e.copy_stream) cudaStreamDestroy(e.copy_stream);
     e.copy_stream = nullptr;
     for (cudaEvent_t& ev : e.copy_ev) {

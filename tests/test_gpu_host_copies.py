@@ -24,3 +24,29 @@ def test_host_entry_point_matches_device(B, K_d, K_q, V, pinned):
             psd.verify_host(*host, 0.2, 0.1, psd.FUZZY, 3, i, out=out)
             for k in names:
                 assert torch.equal(out[k], want[k].cpu()), (k, i)
+
+
+def test_results_in_neighbouring_buffers_pinned_one_by_one():
+    """Four result arrays that happen to lie behind one another, each a page pinned on its own: no copy may span them."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2510_12966_b200 import binding as psd, workloads as wl
+    psd.load_library()
+    psd.set_stream()
+    B = 1024                                               # 4096 bytes of int32 each
+    names = ("accept_len_q", "next_token_q", "accept_len", "next_token")
+    t = wl.make_pyramid_inputs(B, 1, 1, 2048, "bf16", seed=5, sigma_q=0.4, sigma_d=0.9)
+    want = psd.verify(*[x.cuda() for x in t], 0.2, 0.1, psd.FUZZY, 3, 0)
+    raw = torch.zeros(6 * 4096, dtype=torch.uint8)
+    first = -raw.data_ptr() % 4096
+    pages = [raw[first + 4096 * i:first + 4096 * (i + 1)].view(torch.int32) for i in range(4)]
+    rt = torch.cuda.cudart()
+    for p in pages:
+        assert int(rt.cudaHostRegister(p.data_ptr(), 4096, 0)) == 0
+    try:
+        psd.verify_host(*[x.pin_memory() for x in t], 0.2, 0.1, psd.FUZZY, 3, 0, out=dict(zip(names, pages)))
+        for p, k in zip(pages, names):
+            assert torch.equal(p, want[k].cpu()), k
+    finally:
+        for p in pages:
+            rt.cudaHostUnregister(p.data_ptr())
