@@ -227,7 +227,9 @@ int pyramidsd_verify_bonus(const void* logits_draft, const void* logits_qual, co
 
 /* pyramidsd_verify with HOST pointers for every array: copies the three logits tensors and the tokens
  * to library-owned device staging buffers, runs both stages, copies the four [B] results back and
- * synchronises the stream before returning. For callers whose logits live in host memory; the copies
+ * synchronises the stream before returning, whatever the status. From 2 MB of logits on the copies go through a stream of
+ * the library's own and the call runs stage by stage, stage 1 while the target's logits are on their way, unless the
+ * thread's policy (pyramidsd_set_two_stage_policy) is one of the two-step ones: those start after the last copy. For callers whose logits live in host memory; the copies
  * are part of the call. Pinned host memory makes the copies asynchronous up to the final sync. */
 int pyramidsd_verify_host(const void* logits_draft, const void* logits_qual, const void* logits_target,
                           const int32_t* draft_tokens, int B, int K_d, int K_q, int V, psd_dtype dtype,

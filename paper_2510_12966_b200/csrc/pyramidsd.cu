@@ -854,8 +854,9 @@ int pyramidsd_verify_host(const void* logits_draft, const void* logits_qual, con
   rc = grow(ss, &ss->out4, &ss->out4_bytes, n_out);
   if (rc == PSD_OK) rc = grow_pinned(ss, n_out);
   if (rc != PSD_OK) return rc;
-  // below a few megabytes the copies are shorter than what the two streams' events cost
-  const bool overlap = n_d + n_t >= kHostOverlapBytes;
+  // below a few megabytes the copies are shorter than what the two streams' events cost; a thread that asked for two steps
+  // gets them, behind all copies
+  const bool overlap = n_d + n_t >= kHostOverlapBytes && (t_two_stage_policy == PSD_TWO_STAGE_AUTO || t_two_stage_policy == PSD_TWO_STAGE_SEPARATE);
   if (overlap) {
     rc = ensure_copy_stream(ss);
     if (rc != PSD_OK) return rc;

@@ -50,3 +50,24 @@ def test_results_in_neighbouring_buffers_pinned_one_by_one():
     finally:
         for p in pages:
             rt.cudaHostUnregister(p.data_ptr())
+
+
+def test_schedule_of_a_large_call_is_the_threads():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2510_12966_b200 import binding as psd, workloads as wl
+    psd.load_library()
+    psd.set_stream()
+    t = [x.pin_memory() for x in wl.make_pyramid_inputs(3, 8, 4, 50264, "bf16", seed=9, sigma_q=0.4, sigma_d=0.9)]
+    outs, launches = [], []
+    try:
+        for policy in (psd.TWO_STAGE_FUSED, psd.TWO_STAGE_SEPARATE, psd.TWO_STAGE_FUSED_ROWS, psd.TWO_STAGE_AUTO):
+            psd.set_two_stage_policy(policy)
+            n0 = psd.launch_count()
+            outs.append(psd.verify_host(*t, 0.2, 0.1, psd.FUZZY, 3, 1))
+            launches.append(psd.launch_count() - n0)
+    finally:
+        psd.set_two_stage_policy(psd.TWO_STAGE_DEFAULT)
+    assert launches == [2, 4, 2, 4]
+    for o in outs[1:]:
+        assert all(torch.equal(o[k], outs[0][k]) for k in o)
