@@ -234,17 +234,12 @@ def _stream_handle(stream: Optional[torch.cuda.Stream]) -> int:
     return _current_raw_stream(torch._C._cuda_getDevice())
 
 
-def _rows(device, dtype, *shapes):
-    """Contiguous 1-D or 2-D tensors of these shapes, cut out of one allocation (an allocation costs 2 us, a cut 1)."""
-    if len(shapes) == 1:
-        return [torch.empty(shapes[0], dtype=dtype, device=device)]
-    sizes = [s[0] * s[1] if len(s) == 2 else s[0] for s in shapes]
-    buf = torch.empty(sum(sizes), dtype=dtype, device=device)
-    out, at = [], 0
-    for s, n in zip(shapes, sizes):
-        out.append(buf.as_strided(s, (s[1], 1) if len(s) == 2 else (1,), at))
-        at += n
-    return out
+def _rows(device, dtype, shape, n):
+    """``n`` tensors of this shape, each an allocation of its own: cut out of one they could not be viewed as another type,
+    changed in place under autograd, detached in place or saved apart from one another. (Some 5 us a call with six of
+    them; empty_like costs half of empty.)"""
+    first = torch.empty(shape, dtype=dtype, device=device)
+    return (first, *[torch.empty_like(first) for _ in range(n - 1)])
 
 
 def set_stream(stream: Optional[torch.cuda.Stream] = None) -> None:
@@ -345,11 +340,11 @@ def verify_fused_lmhead(hidden, w_t, logits_small, tokens, threshold, mode=FUZZY
     d = hidden.shape[1]
     assert hidden.shape[0] == B * K and w_t.shape == (V, d)
     dev = hidden.device
-    out = dict(zip(("accept_len", "next_token"), _rows(dev, torch.int32, (B,), (B,))))
+    out = dict(zip(("accept_len", "next_token"), _rows(dev, torch.int32, (B,), 2)))
     want_resid = want_rows if want_resid is None else want_resid
     names = (("div",) if want_rows else ()) + (("resid_mass",) if want_resid else ())
     if names:
-        out.update(zip(names, _rows(dev, torch.float32, *[(B, K)] * len(names))))
+        out.update(zip(names, _rows(dev, torch.float32, (B, K), len(names))))
     rc = load_library().packed_verify_fused_lmhead_ex(_LMHEAD.pack(
         _LMHEAD.size, int(mode),
         _dev_ptr(hidden, torch.bfloat16, "hidden") or 0, _dev_ptr(w_t, torch.bfloat16, "w_t") or 0,
@@ -408,10 +403,10 @@ def verify_stage_ex(logits_small, logits_large, tokens, threshold, mode=FUZZY, p
     dev = logits_small.device
     want_resid = want_rows if want_resid is None else (want_resid and want_rows)
     names_f = ("div", "p_small_tok", "p_large_tok") + (("resid_mass",) if want_resid else ()) if want_rows else ()
-    names_i = ("accept_len", "next_token") + (("row_flags",) if want_rows else ())
-    out = dict(zip(names_i, _rows(dev, torch.int32, (B,), (B,), *[(B, K)] * (len(names_i) - 2))))
+    out = dict(zip(("accept_len", "next_token"), _rows(dev, torch.int32, (B,), 2)))
     if want_rows:
-        out.update(zip(names_f, _rows(dev, torch.float32, *[(B, K)] * len(names_f))))
+        out["row_flags"] = torch.empty((B, K), dtype=torch.int32, device=dev)
+        out.update(zip(names_f, _rows(dev, torch.float32, (B, K), len(names_f))))
     rc = load_library().packed_verify_stage_ex(_STAGE.pack(
         _STAGE.size, dt, logits_small.data_ptr(), logits_large.data_ptr(), _dev_ptr(tokens, torch.int32, "tokens") or 0, B, K, V,
         int(mode), int(div_kind), C.c_float(threshold).value, C.c_float(inv_temperature).value, int(seq_stride_small), int(seq_stride_large),
@@ -470,11 +465,14 @@ def verify_ex(logits_draft, logits_qual, logits_target, draft_tokens, tau_q, tau
     rows = [0, 0, 0, 0]   # div_q, resid_q, div_t, resid_t
     if want_rows:         # without residual masses the KL divergence takes the one-pass statistics kernel
         names = ("div_q", "resid_q", "div_t", "resid_t") if want_resid else ("div_q", "div_t")
-        out.update(zip(names, _rows(dev, torch.float32, *[(B, K_d if k.endswith("q") else K_q) for k in names])))
+        for k in "qt":
+            of_stage = [name for name in names if name.endswith(k)]
+            out.update(zip(of_stage, _rows(dev, torch.float32, (B, K_d if k == "q" else K_q), len(of_stage))))
         rows = [out[k].data_ptr() if k in names else 0 for k in ("div_q", "resid_q", "div_t", "resid_t")]
     window = (0, 0)
     if want_window:
-        out["window"], out["n_window"] = _rows(dev, torch.int32, (B, K_q), (B,))
+        out["window"] = torch.empty((B, K_q), dtype=torch.int32, device=dev)
+        out["n_window"] = torch.empty(B, dtype=torch.int32, device=dev)
         window = (out["window"].data_ptr(), out["n_window"].data_ptr())
     dt = logits_draft.dtype
     rc = load_library().packed_verify_ex(_PYRAMID.pack(
