@@ -94,19 +94,27 @@ class LmheadArgs(C.Structure):
 
 class _Packed:
     """An argument structure as one ``struct`` format: filling a ctypes structure field by field costs a few microseconds
-    a call, packing all fields at once half a microsecond. Values come in field order, after ``struct_size``."""
+    a call, packing all fields at once half a microsecond. Values come in field order, ``struct_size`` first. What struct
+    refuses -- an integer beyond its field, a float beyond binary32 -- goes through the ctypes field, which wraps or
+    rounds it as ever: whether such a value is valid is for the library to say."""
     _CODES = {C.c_uint32: "I", C.c_int32: "i", C.c_float: "f", C.c_int64: "q", C.c_uint64: "Q", C.c_void_p: "P", C.c_size_t: "N"}
 
     def __init__(self, cls):
         self.size = C.sizeof(cls)
         fmt = "@" + "".join(self._CODES[t] for _, t in cls._fields_)
         tail = self.size - struct.calcsize(fmt)      # C pads the end of a structure, struct does not
-        self.pack = struct.Struct(fmt + f"{tail}x").pack
+        self._pack = struct.Struct(fmt + f"{tail}x").pack
+        self._types = [t for _, t in cls._fields_]
         for i, (name, _) in enumerate(cls._fields_):
             assert getattr(cls, name).offset == struct.calcsize(fmt[:i + 2]) - getattr(cls, name).size, name
 
+    def pack(self, *values):
+        try:
+            return self._pack(*values)
+        except (struct.error, OverflowError):
+            return self._pack(*[t(v).value or 0 for t, v in zip(self._types, values)])
 
-_U64 = (1 << 64) - 1
+
 _STAGE, _PYRAMID, _LMHEAD = _Packed(StageArgs), _Packed(PyramidArgs), _Packed(LmheadArgs)
 
 
@@ -349,8 +357,8 @@ def verify_fused_lmhead(hidden, w_t, logits_small, tokens, threshold, mode=FUZZY
         _LMHEAD.size, int(mode),
         _dev_ptr(hidden, torch.bfloat16, "hidden") or 0, _dev_ptr(w_t, torch.bfloat16, "w_t") or 0,
         _dev_ptr(logits_small, torch.bfloat16, "logits_small") or 0, _dev_ptr(tokens, torch.int32, "tokens") or 0,
-        B, K, d, V, C.c_float(threshold).value, int(tile_variant or 0), int(div_kind), 0,
-        int(philox_seed) & _U64, int(offset) & _U64, int(seq_index_base),
+        B, K, d, V, float(threshold), int(tile_variant or 0), int(div_kind), 0,
+        int(philox_seed), int(offset), int(seq_index_base),
         out["accept_len"].data_ptr(), out["next_token"].data_ptr(),
         out["div"].data_ptr() if want_rows else 0, out["resid_mass"].data_ptr() if want_resid else 0, _stream_handle(stream)))
     out["status"] = rc
@@ -409,8 +417,8 @@ def verify_stage_ex(logits_small, logits_large, tokens, threshold, mode=FUZZY, p
         out.update(zip(names_f, _rows(dev, torch.float32, (B, K), len(names_f))))
     rc = load_library().packed_verify_stage_ex(_STAGE.pack(
         _STAGE.size, dt, logits_small.data_ptr(), logits_large.data_ptr(), _dev_ptr(tokens, torch.int32, "tokens") or 0, B, K, V,
-        int(mode), int(div_kind), C.c_float(threshold).value, C.c_float(inv_temperature).value, int(seq_stride_small), int(seq_stride_large),
-        int(philox_seed) & _U64, int(offset) & _U64, _dev_ptr(n_valid, torch.int32, "n_valid") or 0,
+        int(mode), int(div_kind), float(threshold), float(inv_temperature), int(seq_stride_small), int(seq_stride_large),
+        int(philox_seed), int(offset), _dev_ptr(n_valid, torch.int32, "n_valid") or 0,
         out["accept_len"].data_ptr(), out["next_token"].data_ptr(),
         *((out["div"].data_ptr(), out["p_small_tok"].data_ptr(), out["p_large_tok"].data_ptr(),
            out["resid_mass"].data_ptr() if want_resid else 0, out["row_flags"].data_ptr()) if want_rows else (0, 0, 0, 0, 0)),
@@ -478,8 +486,8 @@ def verify_ex(logits_draft, logits_qual, logits_target, draft_tokens, tau_q, tau
     rc = load_library().packed_verify_ex(_PYRAMID.pack(
         _PYRAMID.size, dtype_code(logits_draft), _dev_ptr(logits_draft, name="logits_draft") or 0, _dev_ptr(logits_qual, dt, "logits_qual") or 0,
         _dev_ptr(logits_target, dt, "logits_target") or 0, _dev_ptr(draft_tokens, torch.int32, "draft_tokens") or 0,
-        B, K_d, K_q, V, int(mode_q), int(mode_q if mode_t is None else mode_t), C.c_float(tau_q).value, C.c_float(tau_t).value,
-        C.c_float(inv_temperature).value, int(div_kind), int(philox_seed) & _U64, int(offset) & _U64, int(seq_index_base),
+        B, K_d, K_q, V, int(mode_q), int(mode_q if mode_t is None else mode_t), float(tau_q), float(tau_t),
+        float(inv_temperature), int(div_kind), int(philox_seed), int(offset), int(seq_index_base),
         1 if target_has_bonus_row else 0, int(schedule), *results, *rows, *window,
         0 if workspace is None else workspace.data_ptr(),
         0 if workspace is None else workspace.numel() * workspace.element_size(),

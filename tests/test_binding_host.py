@@ -1,4 +1,6 @@
 """The binding's own work on the host, without a GPU: output tensors and argument packing."""
+import ctypes as C
+
 import torch
 
 from paper_2510_12966_b200 import binding
@@ -18,3 +20,37 @@ def test_outputs_are_tensors_of_their_own():
     y.clamp_(min=0)                           # one of them in place while autograd holds another
     loss.backward()
     y.detach_()
+
+
+def test_values_beyond_their_fields_reach_the_library_as_ctypes_passes_them():
+    for packed, cls in ((binding._STAGE, binding.StageArgs), (binding._PYRAMID, binding.PyramidArgs), (binding._LMHEAD, binding.LmheadArgs)):
+        for seed, base, mode, tau in ((5, 7, 1, 0.25), (-1, -1, -3, float("inf")), (1 << 64, 1 << 63, 1 << 31, 1e300), ((1 << 70) + 9, (1 << 64) + 2, (1 << 32) + 1, -1e39)):
+            a, values = cls(), []
+            for name, t in cls._fields_:
+                v = {"philox_seed": seed, "philox_offset": seed, "seq_index_base": base}.get(name)
+                if v is None:
+                    v = tau if t is C.c_float else mode if t is C.c_int32 else 4096
+                setattr(a, name, v)
+                values.append(v)
+            assert packed.pack(*values) == bytes(a)
+
+
+def test_numbers_in_any_form_are_taken_as_thresholds():
+    """A threshold is what float() makes of it, as it was when it went through a ctypes call."""
+    z = torch.zeros((1, 2, 64))
+    tok = torch.zeros((1, 2), dtype=torch.int32)
+    seen = []
+
+    class Library:
+        def packed_verify_stage_ex(self, packed):
+            seen.append(binding.StageArgs.from_buffer_copy(packed))
+            return 0
+
+    saved = binding.load_library, binding._dev_ptr, binding._stream_handle
+    binding.load_library, binding._dev_ptr, binding._stream_handle = Library, lambda t, *a, **k: 0 if t is None else t.data_ptr(), lambda s: 0
+    try:
+        for tau in (0.25, "0.25", torch.tensor(0.25), 1):
+            binding.verify_stage_ex(z, z, tok, tau, seq_index_base=1 << 63)
+    finally:
+        binding.load_library, binding._dev_ptr, binding._stream_handle = saved
+    assert [a.threshold for a in seen] == [0.25, 0.25, 0.25, 1.0] and all(a.seq_index_base == -(1 << 63) for a in seen)
