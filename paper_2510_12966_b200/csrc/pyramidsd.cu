@@ -305,10 +305,6 @@ int launch_rowstats(const StageParams& P, int dtype, int variant, int cluster_si
   return check_launch();
 }
 
-// The finalisation kernels run as clusters of CL CTAs per sequence (per stage in the split form), the largest CL with
-// which all clusters are resident at once: a CTA takes an SM's registers, and the device places 15 clusters of eight, 33
-// of four, 74 of two (cudaOccupancyMaxActiveClusters). One cluster more and the last ones wait for a whole
-// finalisation: 18 sequences in clusters of eight 106 us a call, of four @@ us.
 template <typename Kernel, typename... Args>
 cudaError_t launch_fin_clusters(Kernel kernel, int cl, unsigned units, cudaStream_t stream, Args... args) {
   cudaLaunchConfig_t cfg = {};
@@ -330,12 +326,44 @@ cudaError_t launch_fin_clusters(Kernel kernel, int cl, unsigned units, cudaStrea
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// Clusters of `cl` CTAs of a finalisation kernel that are resident at once: a CTA takes an SM's registers, whatever the
+// kernel and the logits' type, so the answer for one of them serves all.
+template <int CL>
+int fin_resident_clusters() {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(CL);
+  cfg.blockDim = dim3(psd::kFinThreads);
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = CL;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, psd::finalize_kernel<float, CL>, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n;
+}
+
+// The finalisation kernels run as clusters of CL CTAs per sequence (per stage in the split form), the largest CL with
+// which all clusters are resident at once; a B200 places 15 clusters of eight, 33 of four, 74 of two. One cluster more and
+// the last ones wait for a whole finalisation: 18 draws at V = 128256, K = 4 in clusters of eight 32.9 us a call, of four
+// 27.5; 34 in clusters of four 45.4, of two 40.5.
 int fin_cluster_size(long long units) {
-  int sms = psd::cluster_sm_count();
-  if (sms <= 0) sms = 148;
-  if (units * 10 <= sms) return 8;
-  if (units * 9 <= 2ll * sms) return 4;
-  if (units * 2 <= sms) return 2;
+  static std::atomic<int> resident[kMaxDevices][3];   // of eight, four and two CTAs, plus one; 0: not asked yet
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 1;
+  for (int i = 0; i < 3; ++i) {
+    int n = resident[dev][i].load(std::memory_order_relaxed) - 1;
+    if (n < 0) {
+      n = i == 0 ? fin_resident_clusters<8>() : i == 1 ? fin_resident_clusters<4>() : fin_resident_clusters<2>();
+      resident[dev][i].store(n + 1, std::memory_order_relaxed);
+    }
+    if (units <= n) return 8 >> i;
+  }
   return 1;
 }
 

@@ -232,3 +232,21 @@ def test_three_launch_form_replayed_from_a_cuda_graph(psd, wl):
     finally:
         psd.set_two_stage_policy(psd.TWO_STAGE_DEFAULT)
     assert psd.last_status() == 0
+
+
+@pytest.mark.parametrize("B", [14, 15, 16, 33, 34, 63])
+def test_any_cluster_size_draws_the_same(psd, B):
+    """Either side of the batch sizes at which the finalisation goes to smaller clusters, with and without a bonus row,
+    against calls of one sequence each (statistics by the kernel whose bits do not depend on the batch)."""
+    from paper_2510_12966_b200 import workloads as wl
+    K, V = 3, 33001
+    zs, zl, tok = wl.make_stage_inputs(B, K + 1, V, "bf16", seed=B, sigma=0.6, device=torch.device("cuda"))
+    small, tokens = zs[:, :K].contiguous(), tok[:, :K].contiguous()
+    for mode, tau, bonus in ((psd.FUZZY, 1e-6, False), (psd.ASSISTED, 0.0, True), (psd.FUZZY, 1e9, True)):
+        large = zl if bonus else zl[:, :K].contiguous()
+        call = lambda lo, hi: psd.verify_stage_ex(small[lo:hi], large[lo:hi], tokens[lo:hi], tau, mode, 3, 1, seq_index_base=lo,
+                                                  large_has_bonus_row=bonus, kernel_variant=psd.KERNEL_BASELINE)
+        whole = call(0, B)
+        for b in range(B):
+            one = call(b, b + 1)
+            assert torch.equal(one["accept_len"], whole["accept_len"][b:b + 1]) and torch.equal(one["next_token"], whole["next_token"][b:b + 1]), b
