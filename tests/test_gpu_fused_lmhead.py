@@ -178,18 +178,17 @@ def test_fused_lmhead_one_sm_variant_agrees(psd, oracle):
 
 
 @pytest.mark.parametrize("tile_variant", [None, 1])
-def test_fused_lmhead_kl_single_sweep(psd, oracle, tile_variant):
-    """KL(large || small): the divergences come out of the first GEMM sweep; the second one only serves residual masses.
-    Threshold mode with a threshold that splits the rows (rejected rows draw from the residual: the second sweep runs),
-    the same without the residual output, everything accepted (no draw: it returns at once), the assisted mode (draws
-    from p_large off the first sweep's tile sums), strict mode, and a masked small logit under a live large one
-    (divergence +inf). Two row blocks, ragged last tile."""
+def test_fused_lmhead_kl(psd, oracle, tile_variant):
+    """KL(large || small) against the oracle: a threshold that splits the rows (rejected rows draw from the residual), the
+    same without the residual output (the same divergences, bit for bit), everything accepted, the assisted mode (draws from
+    p_large), strict mode, and a masked small logit under a live large one (divergence +inf). Two row blocks, ragged last
+    tile. (Large calls, whose divergences come from the sweep, are in test_gpu_lmhead_tiles.py.)"""
     KL = 2
     h, w_t, z_q, tok = make_case(40, 8, 256, 1500, seed=88, w_scale=0.08)
     probe, orc = run_both(psd, oracle, h, w_t, z_q, tok, 1e9, 0, div_kind=KL, tile_variant=tile_variant)
     check(oracle, probe, orc, 1e9, 0)
     assert np.all(probe["accept_len"] == 8) and np.all(probe["next_token"] == -1)
-    gpu, orc = run_both(psd, oracle, h, w_t, z_q, tok, 1e9, 0, div_kind=KL, want_resid=False, tile_variant=tile_variant)   # one sweep
+    gpu, orc = run_both(psd, oracle, h, w_t, z_q, tok, 1e9, 0, div_kind=KL, want_resid=False, tile_variant=tile_variant)
     check(oracle, gpu, orc, 1e9, 0)
     assert np.array_equal(gpu["div"], probe["div"])
     tau = float(np.float32(np.median(orc["div"])))
@@ -220,6 +219,51 @@ def test_fused_lmhead_more_than_one_row_block(psd, oracle):
     gpu, orc = run_both(psd, oracle, h, w_t, z_q, tok, tau, 0)
     check(oracle, gpu, orc, tau, 0, max_token_ties=3)
     assert 0 < orc["accept_len"][:32].sum() < 32 * 8 and 0 < orc["accept_len"][32:].sum() < 8 * 8
+
+
+@pytest.mark.parametrize("B,V,tile_variant", [(40, 1000, None), (40, 1000, 1), (4, 1000, 1), (80, 1000, None), (40, 106496, None), (40, 106496, 1)])
+@pytest.mark.parametrize("div_kind", [0, 2])
+def test_masked_and_poisoned_rows_in_every_sweep(psd, B, V, tile_variant, div_kind):
+    """The same flags in the last four sequences of calls that take the pairs of CTAs (the rows then sit in the odd CTA's half,
+    or in a second block of rows) or one CTA per tile, and (V = 106496) of KL calls whose divergences come from the sweep:
+    a masked small row, a NaN and an infinity in the hidden rows, a token out of range. The other rows against 64 bits."""
+    dev = torch.device("cuda:0")
+    g = torch.Generator(device=dev).manual_seed(B)
+    h = torch.randn((B * 4, 128), generator=g, device=dev).to(torch.bfloat16)
+    w_t = (torch.randn((V, 128), generator=g, device=dev) * 0.08).to(torch.bfloat16)
+    z_q = ((h.float() @ w_t.float().T) + 0.7 * torch.randn((B * 4, V), generator=g, device=dev)).to(torch.bfloat16).reshape(B, 4, V)
+    tok = torch.randint(0, V, (B, 4), generator=g, device=dev, dtype=torch.int32)
+    s = B - 4
+    z_q[s, 1, 100:700] = -float("inf")
+    h[(s + 1) * 4 + 3, 7] = float("inf")
+    h[(s + 2) * 4 + 1, 5] = float("nan")
+    tok[s + 3, 2] = V
+    z = (h.double() @ w_t.double().T).view(B, 4, V)
+    a, b = torch.log_softmax(z, -1), torch.log_softmax(z_q.double(), -1)
+    p, q = a.exp(), b.exp()
+    bad = torch.zeros((B, 4), dtype=torch.bool, device=dev)
+    bad[s + 1, 3] = bad[s + 2, 1] = True
+    if div_kind == 2:
+        want = (p * (a - b)).sum(-1)
+        assert torch.isinf(want[s, 1])
+    else:
+        m = torch.logaddexp(a, b) - np.log(2.0)
+        want = 0.5 * (p * (a - m) + torch.where(q > 0, q * (b - m), torch.zeros_like(q))).sum(-1)
+    for want_resid in (True, False):
+        out = psd.verify_fused_lmhead(h, w_t, z_q, tok, 1e9, psd.FUZZY, 3, 5, tile_variant=tile_variant, div_kind=div_kind, want_resid=want_resid)
+        assert psd.last_status() == 0
+        L, nxt = out["accept_len"].cpu(), out["next_token"].cpu()
+        assert (L[:s] == 4).all() and (nxt[:s] == -1).all()
+        assert int(L[s]) == (1 if div_kind == 2 else 4)              # KL of the masked row is +inf
+        assert int(L[s + 1]) == 3 and int(nxt[s + 1]) == -2
+        assert int(L[s + 2]) == 1 and int(nxt[s + 2]) == -2
+        assert int(L[s + 3]) == 2 and 0 <= int(nxt[s + 3]) < V       # its row has a distribution: the residual's token
+        assert torch.equal(torch.isnan(out["div"]), bad)
+        fin = torch.isfinite(want) & ~bad
+        assert (out["div"].double() - want)[fin].abs().max() < 2e-5
+        assert torch.equal(torch.isinf(out["div"]), torch.isinf(want) & ~bad)
+        if want_resid:
+            assert (out["resid_mass"].double() - (p - q).clamp(min=0).sum(-1))[~bad].abs().max() < 2e-5
 
 
 def test_fused_lmhead_masked_and_poisoned_rows(psd, oracle):
