@@ -22,7 +22,8 @@
  *   - All data pointers are DEVICE pointers owned by the caller; the library never frees or keeps them.
  *   - Logits are row-major [B, K, V], dtype float32 or bfloat16. Rows whose base address is 16-byte
  *     aligned with V * sizeof(element) a multiple of 16 take the vector path; other shapes take a
- *     scalar path — never an error. -inf logits are legal (probability 0). A row holding NaN or +inf,
+ *     scalar path — never an error; it may read, and ignore, the up to 14 bytes before a tensor's first
+ *     logit and after its last that share their 16-byte unit. -inf logits are legal (probability 0). A row holding NaN or +inf,
  *     or no finite entry, or a token outside [0, V), is flagged and rejected; a flagged non-finite row
  *     at the first rejection emits token -2. Finite logits are meant to be of ordinary size: beyond about
  *     1e9 in magnitude the product with log2(e)/T is rounded by more than the exponent range of a float and

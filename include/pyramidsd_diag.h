@@ -20,8 +20,8 @@ int pyramidsd_kernel_timing_end(double* ms_rowstats, int* n_rowstats, double* ms
 uint64_t pyramidsd_launch_count(void);
 
 /* The cluster size (CTAs per row pair) the library picks for a [B, K, V] stage of this dtype and the
- * number of such clusters the current device keeps resident at once; 0 and 0 when the shape takes the
- * baseline kernel. Lets a caller size batches to whole waves. Needs a CUDA device. */
+ * number of such clusters the current device keeps resident at once, for 16-byte aligned tensors; 0 and 0
+ * where their rows are no whole 16-byte units (V odd, say) or V is below 2048. Lets a caller size batches to whole waves. Needs a CUDA device. */
 int pyramidsd_cluster_occupancy(int B, int K, int V, psd_dtype dtype, int* out_cluster_size, int* out_max_active_clusters);
 
 /* Self-test of the path by which a bounded device-side wait reports that it gave up. Launches one small kernel

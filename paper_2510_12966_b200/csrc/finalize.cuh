@@ -16,7 +16,7 @@ constexpr int kFinThreads = 1024;
 constexpr int kFinElemsPerThread = 8;                      // consecutive vocabulary indices per thread and tile
 constexpr int kFinTile = kFinThreads * kFinElemsPerThread;  // 8192 indices per tile
 constexpr int kFinMaxTiles = 1024;                          // V <= 8,388,608
-constexpr int kFinBatch = 32;
+constexpr int kFinBatch = 32;                               // tiles summed between two CTA-wide barriers
 constexpr int kFinMaxRanks = 8;                             // CTAs per sequence at most
 
 __device__ __forceinline__ unsigned fin_cluster_rank() {
@@ -32,7 +32,7 @@ __device__ __forceinline__ void fin_remote_store(double* local, unsigned rank, d
   unsigned addr;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(static_cast<unsigned>(__cvta_generic_to_shared(local))), "r"(rank));
   asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(addr), "d"(v) : "memory");
-}                               // tiles summed between two CTA-wide barriers
+}
 
 // A finalisation launch may start while the launch before it drains; it reads nothing of that launch before this.
 __device__ __forceinline__ void wait_for_previous_launch() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -213,8 +213,7 @@ __device__ __forceinline__ void write_results(const StageParams& P, const int b,
 }
 
 // The pick of one level of the draw, by one full warp: the first child whose inclusive cumulative weight exceeds the
-// target, else the last one with a positive weight (-1: none). Lane k holds the weight of child k; `base` lies before
-// them. Every lane returns the same values. (One lane walking 32 children in shared memory took half a microsecond.)
+// target, else the last one with a positive weight (-1: none). Lane k holds child k's weight and inclusive sum. Every lane returns the same values. (One lane walking 32 children in shared memory took half a microsecond.)
 template <typename V>
 __device__ __forceinline__ V warp_incl_scan(V w, const int lane) {
 #pragma unroll
@@ -440,7 +439,7 @@ __device__ __forceinline__ void finalize_sequence(const StageParams& P, const in
     float w[kFinElemsPerThread];
     // level 0: total weight of every tile. CTA `cl_rank` of the cluster takes tiles cl_rank, cl_rank + CL, ...;
     // the tiles of a batch are independent (their loads overlap); each warp leaves its sum per tile, then one
-    // thread per tile adds the 32 warp sums in warp order and hands the total to every CTA of the cluster.
+    // warp per tile adds the 32 warp sums in a fixed tree and hands the total to every CTA of the cluster.
     const int my_tiles = (n_tiles - static_cast<int>(cl_rank) + CL - 1) / CL;
     // A second go happens only when the residual weights, taken again here in single precision, all come out
     // zero although the row's residual mass did not (two rows that differ only where both probabilities

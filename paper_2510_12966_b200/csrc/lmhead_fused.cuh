@@ -13,8 +13,8 @@
 //            caller takes no residual masses there is no such launch, and the final kernel forms those of the row it draws from)
 //   final    per sequence: row totals, accept bits, accepted prefix, and the residual draw: the segment is found
 //            from the per-segment masses, the token from that segment's logits
-// Measured, whole call: 574 -> 348 us at that size, 105 -> 36.9 us at M = 15, d = 2048, V = 32000, against two runs of
-// the GEMM with the terms in the second one's epilogue.
+// Measured against two runs of the GEMM with the terms in the second one's epilogue, whole calls: 602 -> 356 us at that
+// size, 103 -> 35.6 us at M = 15, d = 2048, V = 32000.
 //
 // One CTA = 10 warps: warp 0 lane 0 issues TMA loads, warp 1 lane 0 issues the MMAs (and owns the tensor
 // memory allocation), warps 2..9 are the epilogue (warp e reads TMEM lanes 32*(e%4).. of accumulator
@@ -533,7 +533,7 @@ lmhead_sweep2sm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
 // of the small logits a run of consecutive indices. A tile may load fewer than 128 weight rows (what the MMA makes of the rest
 // of the shared-memory tile is never read), which lets the host cut the vocabulary into equal rounds. A warp keeps the
 // (max, sum) of its columns of a row over all its tiles (lane r: row r of the warp's half) and leaves one partial.
-// Measured at M = 15, d = 2048, V = 32000: the launch 40 -> 29 us (131 MB of weight), the whole call 50.6 -> 36.9 us.
+// Measured at M = 15, d = 2048, V = 32000: the launch 40 -> 29 us (131 MB of weight), the whole call 50.6 -> 35.6 us.
 // Up to 32 rows: the epilogue takes a warp-wide maximum and sum per row, about 2.9 us a row at V = 128256, while a lane of the
 // pairs' epilogue has a row to itself. Whole calls in us, this form / pairs of CTAs: V = 152064, d = 1024: M = 16 92 / 138,
 // 32 134 / 136, 64 215 / 141, 128 385 / 197; V = 128256, d = 4096: 32 244 / 242, 64 256 / 272, 128 422 / 282;

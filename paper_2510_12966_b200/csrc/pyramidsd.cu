@@ -45,7 +45,7 @@ size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 // Library-owned scratch. Every (device, stream) pair that has been used without a caller workspace owns its own
 // buffers: the workspace of the stage / pyramid calls, the status word of the bounded waits, the staging
-// buffers of the host-pointer entry point and the partial sums of the fused LM-head. A call touches only the
+// buffers of the host-pointer entry point and the logits and partial sums of the fused LM-head. A call touches only the
 // buffers of the stream it runs on and holds that entry's mutex while it enqueues, so two host threads on two
 // streams share nothing and two threads on one stream take turns. Buffers are grown on demand (after waiting
 // for the stream's own earlier work, which is all that can still use them), never shrunk, and freed at
@@ -63,7 +63,7 @@ struct StreamScratch {
   size_t out4_bytes = 0;
   void* out4_host = nullptr;   // the same in pinned host memory, from where they go to the caller's four arrays
   size_t out4_host_bytes = 0;
-  void* lm_ws = nullptr;    // partial sums of the fused LM-head path
+  void* lm_ws = nullptr;    // the fused LM-head path's logits (one block of rows, or as many as kLmGroupBytes hold) and partial sums
   size_t lm_ws_bytes = 0;
   void* draw = nullptr;     // records and tile totals of the three-launch finalisation
   size_t draw_bytes = 0;
@@ -318,7 +318,7 @@ cudaError_t launch_fin_clusters(Kernel kernel, int cl, unsigned units, cudaStrea
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
   // a programmatic dependent of the statistics launch before it: its CTAs may be placed while that launch drains,
-  // and wait (griddepcontrol.wait, their first instruction) for its end before they read a statistic
+  // and wait (griddepcontrol.wait) for its end before they read a statistic
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
