@@ -244,8 +244,8 @@ def _stream_handle(stream: Optional[torch.cuda.Stream]) -> int:
 
 def _rows(device, dtype, shape, n):
     """``n`` tensors of this shape, each an allocation of its own: cut out of one they could not be viewed as another type,
-    changed in place under autograd, detached in place or saved apart from one another. (Some 5 us a call with six of
-    them; empty_like costs half of empty.)"""
+    changed in place under autograd, detached in place or saved apart from one another. (empty_like costs half of
+    empty.)"""
     first = torch.empty(shape, dtype=dtype, device=device)
     return (first, *[torch.empty_like(first) for _ in range(n - 1)])
 
@@ -410,18 +410,22 @@ def verify_stage_ex(logits_small, logits_large, tokens, threshold, mode=FUZZY, p
     dt = dtype_code(logits_small)
     dev = logits_small.device
     want_resid = want_rows if want_resid is None else (want_resid and want_rows)
-    names_f = ("div", "p_small_tok", "p_large_tok") + (("resid_mass",) if want_resid else ()) if want_rows else ()
-    out = dict(zip(("accept_len", "next_token"), _rows(dev, torch.int32, (B,), 2)))
+    accept_len = torch.empty(B, dtype=torch.int32, device=dev)
+    out = {"accept_len": accept_len, "next_token": torch.empty_like(accept_len)}
+    rows = (0, 0, 0, 0, 0)
     if want_rows:
-        out["row_flags"] = torch.empty((B, K), dtype=torch.int32, device=dev)
-        out.update(zip(names_f, _rows(dev, torch.float32, (B, K), len(names_f))))
+        out["row_flags"] = accept_len.new_empty((B, K))
+        out["div"] = div = torch.empty((B, K), dtype=torch.float32, device=dev)
+        out["p_small_tok"], out["p_large_tok"] = torch.empty_like(div), torch.empty_like(div)
+        if want_resid:
+            out["resid_mass"] = torch.empty_like(div)
+        rows = (div.data_ptr(), out["p_small_tok"].data_ptr(), out["p_large_tok"].data_ptr(),
+                out["resid_mass"].data_ptr() if want_resid else 0, out["row_flags"].data_ptr())
     rc = load_library().packed_verify_stage_ex(_STAGE.pack(
         _STAGE.size, dt, logits_small.data_ptr(), logits_large.data_ptr(), _dev_ptr(tokens, torch.int32, "tokens") or 0, B, K, V,
         int(mode), int(div_kind), float(threshold), float(inv_temperature), int(seq_stride_small), int(seq_stride_large),
         int(philox_seed), int(offset), _dev_ptr(n_valid, torch.int32, "n_valid") or 0,
-        out["accept_len"].data_ptr(), out["next_token"].data_ptr(),
-        *((out["div"].data_ptr(), out["p_small_tok"].data_ptr(), out["p_large_tok"].data_ptr(),
-           out["resid_mass"].data_ptr() if want_resid else 0, out["row_flags"].data_ptr()) if want_rows else (0, 0, 0, 0, 0)),
+        accept_len.data_ptr(), out["next_token"].data_ptr(), *rows,
         0 if workspace is None else workspace.data_ptr(),
         0 if workspace is None else workspace.numel() * workspace.element_size(),
         _stream_handle(stream), 1, int(kernel_variant), int(cluster_size), 1 if large_has_bonus_row else 0, 0, int(seq_index_base)))
@@ -470,18 +474,21 @@ def verify_ex(logits_draft, logits_qual, logits_target, draft_tokens, tau_q, tau
         out = dict(out)
     results = [_dev_ptr(out[k], torch.int32, k) or 0 for k in ("accept_len_q", "next_token_q", "accept_len", "next_token")]
     want_resid = want_rows if want_resid is None else (want_resid and want_rows)
-    rows = [0, 0, 0, 0]   # div_q, resid_q, div_t, resid_t
+    rows = (0, 0, 0, 0)   # div_q, resid_q, div_t, resid_t
     if want_rows:         # without residual masses the KL divergence takes the one-pass statistics kernel
-        names = ("div_q", "resid_q", "div_t", "resid_t") if want_resid else ("div_q", "div_t")
-        for k in "qt":
-            of_stage = [name for name in names if name.endswith(k)]
-            out.update(zip(of_stage, _rows(dev, torch.float32, (B, K_d if k == "q" else K_q), len(of_stage))))
-        rows = [out[k].data_ptr() if k in names else 0 for k in ("div_q", "resid_q", "div_t", "resid_t")]
+        out["div_q"] = div_q = torch.empty((B, K_d), dtype=torch.float32, device=dev)
+        if want_resid:
+            out["resid_q"] = torch.empty_like(div_q)
+        out["div_t"] = div_t = div_q.new_empty((B, K_q))
+        if want_resid:
+            out["resid_t"] = torch.empty_like(div_t)
+        rows = (div_q.data_ptr(), out["resid_q"].data_ptr() if want_resid else 0,
+                div_t.data_ptr(), out["resid_t"].data_ptr() if want_resid else 0)
     window = (0, 0)
     if want_window:
-        out["window"] = torch.empty((B, K_q), dtype=torch.int32, device=dev)
-        out["n_window"] = torch.empty(B, dtype=torch.int32, device=dev)
-        window = (out["window"].data_ptr(), out["n_window"].data_ptr())
+        out["window"] = win = torch.empty((B, K_q), dtype=torch.int32, device=dev)
+        out["n_window"] = n_win = win.new_empty(B)
+        window = (win.data_ptr(), n_win.data_ptr())
     dt = logits_draft.dtype
     rc = load_library().packed_verify_ex(_PYRAMID.pack(
         _PYRAMID.size, dtype_code(logits_draft), _dev_ptr(logits_draft, name="logits_draft") or 0, _dev_ptr(logits_qual, dt, "logits_qual") or 0,
