@@ -50,7 +50,9 @@ def test_numbers_in_any_form_are_taken_as_thresholds():
     binding.load_library, binding._dev_ptr, binding._stream_handle = Library, lambda t, *a, **k: 0 if t is None else t.data_ptr(), lambda s: 0
     try:
         for tau in (0.25, "0.25", torch.tensor(0.25), 1):
-            binding.verify_stage_ex(z, z, tok, tau, seq_index_base=1 << 63)
+            out = binding.verify_stage_ex(z, z, tok, tau, seq_index_base=1 << 63)
+            tensors = [t for t in out.values() if torch.is_tensor(t)]
+            assert len(tensors) == 7 and len({t.untyped_storage().data_ptr() for t in tensors}) == 7
     finally:
         binding.load_library, binding._dev_ptr, binding._stream_handle = saved
     assert [a.threshold for a in seen] == [0.25, 0.25, 0.25, 1.0] and all(a.seq_index_base == -(1 << 63) for a in seen)
