@@ -172,8 +172,9 @@ int pyramidsd_verify(const void* logits_draft, const void* logits_qual, const vo
  *                     (PSD_FUZZY, PSD_FUZZY); PSD_A (Sec. 3.4: assisted decoding in place of tau_Q, on rejection
  *                     a draw from the qualifier's own distribution, the target stage unchanged) is
  *                     (PSD_ASSISTED, PSD_FUZZY), and tau_q is then unused.
- *   seq_index_base    as in psd_stage_args: a call on sequences [base, base + B) of a batch returns, bit for
- *                     bit, what the call on the whole batch returns for them.
+ *   seq_index_base    as in psd_stage_args: a call on sequences [base, base + B) of a batch returns what the call
+ *                     on the whole batch returns for them, up to the rounding by which calls of different sizes differ
+ *                     (another number of CTAs per row, one launch or several).
  *   target_has_bonus_row  logits_target is [B, K_q + 1, V] (see pyramidsd_verify_bonus).
  *   out_div_q [B, K_d], out_resid_q [B, K_d], out_div_t [B, K_q], out_resid_t [B, K_q]: per-row divergence and
  *                     residual mass of the two stages, or NULL. Stage-2 rows at or beyond the window hold 0.
@@ -337,7 +338,14 @@ int pyramidsd_row_uniforms(uint64_t philox_seed, uint64_t offset, int n_rows, fl
 size_t pyramidsd_workspace_bytes(int B, int K, int V, psd_dtype dtype);
 
 /* How the two-stage calls schedule their launches (per host thread; every schedule returns the same results, bit
- * for bit: all of them cut a row over the CTAs of a cluster the same way). A "finalisation" below is one launch (a
+ * for bit: all of them cut a row over the CTAs of a cluster the same way).
+ *   PSD_TWO_STAGE_DEFAULT   no schedule asked for: PSD_TWO_STAGE_AUTO, except that small and medium calls on the
+ *                           library's own scratch go as ONE launch, whose clusters take a row pair each and finish a
+ *                           sequence when its last row is done. It sums in another order and, for bf16 logits, with
+ *                           a longer polynomial than the schedules below, so divergences and residual masses differ
+ *                           from theirs by rounding (at most 2e-5 and 1e-6 in absolute terms), as single stages of
+ *                           different batch sizes do, which go either way likewise.
+ * A "finalisation" below is one launch (a
  * cluster of CTAs per sequence), or, for batches that fill the GPU on calls that use the library's own scratch,
  * three small launches that hand over to one another (accept scan; the tile totals of every draw, spread over all
  * SMs; pick and descent) -- again with the same bits.
@@ -347,7 +355,7 @@ size_t pyramidsd_workspace_bytes(int B, int K, int V, psd_dtype dtype);
  *                           K_q tokens (Fig. 1).
  *   PSD_TWO_STAGE_SEPARATE  four steps, stage by stage; stage 2 then skips the rows beyond each window, which
  *                           wins when acceptance is low and windows are short.
- *   PSD_TWO_STAGE_AUTO      (the default) the library chooses between the two per call. Stage 1 also leaves each
+ *   PSD_TWO_STAGE_AUTO      the library chooses between the two per call. Stage 1 also leaves each
  *                           sequence's window length in a small host-mapped buffer (no copy, no synchronisation);
  *                           a later call with the same B and K_q on this device reads whatever lengths are there
  *                           -- those of a recent call -- and runs stage by stage when the unfilled part of the

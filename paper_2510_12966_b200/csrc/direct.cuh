@@ -1,0 +1,606 @@
+// Small and medium calls in ONE launch: the statistics of every row pair and, by whichever cluster is the last of a
+// sequence, that sequence's finalisation (accept scan, window, draw: Sec. 3.1-3.4).
+//
+// What bounds a small call is a chain of dependent latencies, not bytes. The ring kernel (rowstats_cluster.cuh) is built
+// for many rows per CTA: it fills a pipeline first, and a second launch then reads the rejected rows again to draw from
+// them. Here a cluster of `cs` CTAs takes one row pair. Every warp of the cluster copies a run of consecutive logits of both
+// rows into shared memory of its own and both passes run over that; the log-sum-exp partials cross the cluster once
+// (st.async: every warp's to every CTA), the pass-B partials once (to rank 0), among them the residual mass and the mass of
+// p of every warp's run. With these a draw is the work of one warp: runs, then the logits of one run. The cluster that
+// completes a sequence (a ticket per sequence, counted up in global memory) does it; no cluster waits for another.
+//
+// Whole calls, before (statistics launch, then finalisation) / now: 4 rows of 32000 fp32 with a draw 13.0 / 9.2 us; one
+// sequence through the pyramid, V = 128256, bonus row 19.7 / 15.4; 32 sequences, V = 50257 64.8 / 54.7; the rule in
+// direct_applies has more. Errors against 64 bits (rms over 36 row pairs, V = 32000): bf16 divergence 5.2e-6 / 2.2e-8, residual
+// mass 3.6e-7 / 4.9e-8; fp32 4.5e-8 / 2.1e-8 and 4.4e-7 / 4.8e-8. Of a warp's way through one small call (17000 cycles at the start, 4 rows
+// of 32000 fp32): set-up 700, copies 1600, pass A 1200, exchange and merge 1600, pass B 1100, partials to rank 0 and their sum 1900,
+// record and ticket 1700, accept scan 2000, draw 4200, results 500. Tried: both rows in registers with every loop unrolled (84
+// registers: half as many CTAs, 283 us for 1000 rows of 50256 where this takes 113), 512 threads, both loops unrolled further.
+//
+// Rows at any element boundary: the 16-byte units around a run are copied, and a group of eight logits is shifted into
+// place as it is read. The arithmetic is that of the ring kernel's form for such rows (div_accumulate_split: degree 7,
+// split normalisers, the residual mass summed as such) for every row.
+#pragma once
+
+#include "common.cuh"
+#include "finalize.cuh"
+#include "rowstats_cluster.cuh"
+
+namespace psd {
+
+constexpr int kDirMaxRanks = 8;
+constexpr int kDirThreads = 256;
+constexpr int kDirWarps = kDirThreads / 32;
+constexpr int kDirCtasPerSm = 4;
+constexpr int kDirMaxRuns = kDirMaxRanks * kDirWarps;        // warps of a cluster
+constexpr int kDirPer = kDirMaxRuns / 32;
+constexpr int kDirMaxSmem = 200 * 1024;
+constexpr int kDirSmemForFour = 52 * 1024;                   // of a CTA, so that kDirCtasPerSm of them share an SM
+constexpr unsigned kDirSpinLimit = 1u << 22;
+
+struct DirectParams {
+  StageParams s1, s2;      // s2: the two-stage wrapper's second stage (n_stages == 2)
+  int n_stages;
+  int cs;                  // CTAs per row pair
+  int n_groups;            // groups of 256 indices of a row
+  int run_bytes;           // shared memory of one model's run: its most groups and a 16-byte unit
+  int items_per_seq;       // row pairs of a sequence, and one more for the last stage's bonus row
+  float2* runs;            // [items][warps of a cluster]: (residual mass, mass of p_large)
+  RowStats* bonus_stats;   // [B]
+  int* ticket;             // [B], zero between calls
+};
+
+// First group of a cluster's run `nth` of `n`.
+__device__ __forceinline__ int run_begin(int nth, int n, int n_groups) { return nth * n_groups / n; }
+
+__device__ __forceinline__ float warp_max(float v) {   // NaN ignored
+  float r;
+  asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+  return r;
+}
+__device__ __forceinline__ float sum_of(const float (&w)[kFinElemsPerThread]) {
+  float ts = 0.f;
+#pragma unroll
+  for (int e = 0; e < kFinElemsPerThread; ++e) ts += w[e];
+  return ts;
+}
+
+// A run of one row in a warp's shared memory, copied from the 16-byte boundary at or before its first logit.
+template <typename T>
+struct Run {
+  unsigned at;      // shared-memory address
+  unsigned lead;    // bytes from there to the first logit, 0 .. 14
+  int n;            // logits
+
+  __device__ __forceinline__ Run(unsigned smem, const T* first, int count) : at(smem), lead(static_cast<unsigned>(reinterpret_cast<uintptr_t>(first) & 15u)), n(count) {}
+  // Starts the copy (cp.async) of the 16-byte units that hold logits [from, to) of the run and have not been copied with
+  // those before `from`. No unit without a logit of the run is read.
+  __device__ __forceinline__ void copy(const T* first, int from, int to, int lane) const {
+    const char* src = reinterpret_cast<const char*>(first) - lead;
+    auto units = [&](int logits) { return logits > 0 ? (static_cast<int>(lead) + logits * static_cast<int>(sizeof(T)) + 15) / 16 : 0; };
+#pragma unroll 4
+    for (int u = units(from) + lane; u < units(to); u += 32)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(at + 16u * static_cast<unsigned>(u)), "l"(src + 16 * static_cast<long long>(u)) : "memory");
+  }
+};
+__device__ __forceinline__ void run_copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int kPending>
+__device__ __forceinline__ void run_copies_wait() {   // for all but the last kPending commits
+  asm volatile("cp.async.wait_group %0;" ::"n"(kPending) : "memory");
+  __syncwarp();
+}
+
+// Eight consecutive logits as they lie in memory (bf16: 4 words, fp32: 8 words); those beyond the run's end as -inf.
+template <typename T>
+struct Group {
+  static constexpr int kWords = kFinElemsPerThread * static_cast<int>(sizeof(T)) / 4;
+  unsigned w[kWords];
+
+  __device__ __forceinline__ Group(const Run<T>& run, int first) {
+    unsigned u[kWords + 4];
+    const unsigned at = run.at + static_cast<unsigned>(first) * static_cast<unsigned>(sizeof(T));
+    auto unit = [&](int k) {
+      asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(u[4 * k]), "=r"(u[4 * k + 1]), "=r"(u[4 * k + 2]), "=r"(u[4 * k + 3]) : "r"(at + 16u * k) : "memory");
+    };
+#pragma unroll
+    for (int k = 0; k < kWords / 4; ++k) unit(k);
+    if (run.lead != 0) {   // uniform across the warp
+      unit(kWords / 4);
+      if (run.lead & 8u) {
+#pragma unroll
+        for (int j = 0; j < kWords + 2; ++j) u[j] = u[j + 2];
+      }
+      if (run.lead & 4u) {
+#pragma unroll
+        for (int j = 0; j < kWords + 1; ++j) u[j] = u[j + 1];
+      }
+      if (sizeof(T) == 2 && (run.lead & 2u)) {
+#pragma unroll
+        for (int j = 0; j < kWords; ++j) u[j] = __funnelshift_r(u[j], u[j + 1], 16);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < kWords; ++j) w[j] = u[j];
+    const int left = run.n - first;
+    if (left < kFinElemsPerThread) {
+#pragma unroll
+      for (int j = 0; j < kWords; ++j) {
+        if (sizeof(T) == 4) {
+          if (j >= left) w[j] = 0xff800000u;
+        } else {
+          if (2 * j >= left) w[j] = 0xff80ff80u;
+          else if (2 * j + 1 >= left) w[j] = (w[j] & 0xffffu) | 0xff800000u;
+        }
+      }
+    }
+  }
+  __device__ __forceinline__ float2 pair(int j) const {   // logits 2 j and 2 j + 1
+    if constexpr (sizeof(T) == 4) return make_float2(__uint_as_float(w[2 * j]), __uint_as_float(w[2 * j + 1]));
+    else return Pairs<__nv_bfloat16>::widen(w[j]);
+  }
+  // ... raised to at least the floor
+  __device__ __forceinline__ float2 pair_clamped(int j, float floor_x, unsigned floor2) const {
+    if constexpr (sizeof(T) == 4) {
+      const float2 x = pair(j);
+      return make_float2(fmaxf(x.x, floor_x), fmaxf(x.y, floor_x));
+    } else {
+      return Pairs<__nv_bfloat16>::widen(Pairs<__nv_bfloat16>::max_bf16x2(w[j], floor2));
+    }
+  }
+  __device__ __forceinline__ float max() const {   // NaN ignored
+    if constexpr (sizeof(T) == 4) {
+      float m = __uint_as_float(w[0]);
+#pragma unroll
+      for (int j = 1; j < kWords; ++j) m = fmaxf(m, __uint_as_float(w[j]));
+      return m;
+    } else {
+      unsigned m = w[0];
+#pragma unroll
+      for (int j = 1; j < kWords; ++j) m = Pairs<__nv_bfloat16>::max_bf16x2(m, w[j]);
+      const float2 x = Pairs<__nv_bfloat16>::widen(m);
+      return fmaxf(x.x, x.y);
+    }
+  }
+};
+
+// Both models' partials of a run: the reference in the scaled base-2 domain, a whole number (see lg2_into), and the sum of
+// 2^(x c - reference). The reference is that of the largest logit of the run's first group; only if a sum leaves the range
+// of a float (a logit 2^127 above it, or NaN / +inf) is it taken again from the whole run's. `half`: the groups whose
+// copies have landed; it waits for the others before it comes to them.
+template <typename T>
+__device__ __forceinline__ float4 run_lse(const Run<T>& xs, const Run<T>& xl, const int groups, const int half, const float c, const int lane) {
+  float rs = -1e30f, rl = -1e30f, ss = 0.f, sl = 0.f;
+#pragma unroll 1
+  for (int most = min(groups, 1); most > 0; most = most < groups ? groups : 0) {
+    float ms = -INFINITY, ml = -INFINITY;
+#pragma unroll 1
+    for (int g = 0; g < most; ++g) {
+      ms = fmaxf(ms, Group<T>(xs, g * kFinPart + lane * kFinElemsPerThread).max());
+      ml = fmaxf(ml, Group<T>(xl, g * kFinPart + lane * kFinElemsPerThread).max());
+    }
+    rs = fmaxf(rintf(warp_max(ms) * c), -1e30f);
+    rl = fmaxf(rintf(warp_max(ml) * c), -1e30f);
+    const float2 cc = splat2(c), ns = splat2(-rs), nl = splat2(-rl);
+    float2 vs = make_float2(0.f, 0.f), vl = vs;
+#pragma unroll 2
+    for (int g = 0; g < groups; ++g) {
+      if (g == half) run_copies_wait<0>();
+      const Group<T> a(xs, g * kFinPart + lane * kFinElemsPerThread), b(xl, g * kFinPart + lane * kFinElemsPerThread);
+#pragma unroll
+      for (int j = 0; j < kFinElemsPerThread / 2; ++j) {
+        vs = __fadd2_rn(vs, ex2_2(__ffma2_rn(a.pair(j), cc, ns)));
+        vl = __fadd2_rn(vl, ex2_2(__ffma2_rn(b.pair(j), cc, nl)));
+      }
+    }
+    ss = warp_reduce<OpSum>(vs.x + vs.y);
+    sl = warp_reduce<OpSum>(vl.x + vl.y);
+    if (ss + sl < INFINITY) break;   // uniform: every lane holds the same sums
+  }
+  return make_float4(rs, ss, rl, sl);
+}
+
+// The draw of one stage's row by one warp, from the row's runs. Returns the token (-1: none).
+template <typename T>
+__device__ __forceinline__ int direct_draw(const DirectParams& D, const StageParams& P, const T* large, const T* small, const float4 lse, const float2* runs,
+                                           const int n_runs, bool from_large, const float u2, const unsigned smem, const int lane) {
+  const int per = (n_runs + 31) / 32;   // consecutive runs per lane
+  float2 w[kDirPer];
+#pragma unroll
+  for (int j = 0; j < kDirPer; ++j) w[j] = (j < per && lane * per + j < n_runs) ? __ldcg(runs + lane * per + j) : make_float2(0.f, 0.f);
+  // The residual; if it has no positive weight (or none in single precision as the weights are taken here), p_large: a
+  // rejected row with a distribution always yields a token.
+#pragma unroll 1
+  for (;;) {
+    double sum = 0.0;
+#pragma unroll
+    for (int j = 0; j < kDirPer; ++j) sum += static_cast<double>(from_large ? w[j].y : w[j].x);
+    const double incl = warp_incl_scan(sum, lane);
+    const double target = static_cast<double>(u2) * __shfl_sync(0xffffffffu, incl, 31);
+    const WarpPick k = warp_pick(sum, incl, target);
+    const int who = k.first >= 0 ? k.first : k.last;
+    int token = -1;
+    if (who >= 0) {
+      double cum = incl - sum, before = 0.0;
+      int pick = -1;
+      bool past = false;   // the first run whose inclusive sum exceeds the target, else the last positive one
+#pragma unroll
+      for (int j = 0; j < kDirPer; ++j) {
+        const double wj = static_cast<double>(from_large ? w[j].y : w[j].x);
+        if (wj > 0.0 && !past) { pick = j; before = cum; past = cum + wj > target; }
+        cum += wj;
+      }
+      const int nth = __shfl_sync(0xffffffffu, lane * per + pick, who);
+      float left = __shfl_sync(0xffffffffu, static_cast<float>(target - before), who);
+      // the run's logits: groups, lanes, elements
+      const int g0 = run_begin(nth, n_runs, D.n_groups), groups = run_begin(nth + 1, n_runs, D.n_groups) - g0;
+      const int n = min(groups * kFinPart, P.V - g0 * kFinPart);
+      const Run<T> xs(smem, small + g0 * kFinPart, n), xl(smem + static_cast<unsigned>(D.run_bytes), large + g0 * kFinPart, n);
+      __syncwarp();
+      xs.copy(small + g0 * kFinPart, 0, n, lane);
+      xl.copy(large + g0 * kFinPart, 0, n, lane);
+      run_copies_commit();
+      run_copies_wait<0>();
+      // of the chosen group -- the first whose inclusive sum exceeds the target, else the last positive one --: this lane's
+      // weights and their sum, and the target inside it
+      float tw[kFinElemsPerThread], ts = 0.f, tt = 0.f;
+      int at = -1;
+#pragma unroll 1
+      for (int g = 0; g < groups; ++g) {
+        const Group<T> a(xs, g * kFinPart + lane * kFinElemsPerThread), b(xl, g * kFinPart + lane * kFinElemsPerThread);
+        float v[kFinElemsPerThread];
+#pragma unroll
+        for (int j = 0; j < kFinElemsPerThread / 2; ++j) {
+          const float2 x = b.pair(j), y = a.pair(j);
+          const float p0 = ex2_approx(fmaf(x.x, P.c, -lse.z) - lse.w), p1 = ex2_approx(fmaf(x.y, P.c, -lse.z) - lse.w);
+          const float q0 = ex2_approx(fmaf(y.x, P.c, -lse.x) - lse.y), q1 = ex2_approx(fmaf(y.y, P.c, -lse.x) - lse.y);
+          v[2 * j] = from_large ? p0 : fmaxf(p0 - q0, 0.f);
+          v[2 * j + 1] = from_large ? p1 : fmaxf(p1 - q1, 0.f);
+        }
+        const float vs = sum_of(v), total = warp_reduce<OpSum>(vs);
+        if (total > 0.f) {
+          at = g; tt = left; ts = vs;
+#pragma unroll
+          for (int j = 0; j < kFinElemsPerThread; ++j) tw[j] = v[j];
+          if (total > left) break;
+          left -= total;
+        }
+      }
+      if (at >= 0) {
+        const float in = warp_incl_scan(ts, lane);
+        const WarpPick l = warp_pick(ts, in, tt);
+        const float t3 = tt - (in - ts);
+        float run = 0.f;
+        int choice = -1;
+        bool hit = false;
+#pragma unroll
+        for (int j = 0; j < kFinElemsPerThread; ++j) {
+          run += tw[j];
+          if (tw[j] > 0.f && !hit) { choice = j; hit = run > t3; }
+        }
+        token = __shfl_sync(0xffffffffu, (g0 + at) * kFinPart + lane * kFinElemsPerThread + choice, l.first >= 0 ? l.first : l.last);
+      }
+    }
+    if (token >= 0 || from_large) return token;
+    from_large = true;
+  }
+}
+
+// One stage of sequence b by one warp, from the records and runs of its rows. `first_item`: the item of its position 0.
+template <typename T>
+__device__ __forceinline__ void direct_finish(const DirectParams& D, const StageParams& P, const int b, const int first_item, const int n_runs, const unsigned smem,
+                                              const int lane, const int nv_given, const int32_t* tokens_given, const int n_given) {
+  const ScanOut o = scan_unit<T>(P, b, lane, true, nv_given, tokens_given, n_given);
+  const bool bonus = P.bonus && o.L == o.nv;
+  int next = -1;
+  if (bonus || o.L < o.nv) {
+    float4 lse = make_float4(o.m2s, o.l2ss, o.m2l, o.l2sl);
+    int flags = o.flags;
+    float u2 = o.u2;
+    bool from_large = P.mode == kModeAssisted || !(o.resid > 0.f);
+    const T* large = static_cast<const T*>(P.large) + b * P.seq_stride_large + static_cast<long long>(o.L) * P.V;
+    const T* small = static_cast<const T*>(P.small) + b * P.seq_stride_small + static_cast<long long>(o.L) * P.V;
+    if (bonus) {   // the row after the last valid position
+      const RowStats* s = o.L < P.K ? P.stats + static_cast<long long>(b) * P.K + o.L : D.bonus_stats + b;
+      lse = __ldcg(reinterpret_cast<const float4*>(s));
+      lse.x = lse.z; lse.y = lse.w;
+      flags = __ldcg(&s->flags) & kFlagLargeNonfinite;
+      u2 = bonus_uniform(P.seed, P.offset, static_cast<unsigned>(P.seq_base + b));
+      from_large = true;
+      small = large;
+    }
+    if (flags & (kFlagSmallNonfinite | kFlagLargeNonfinite)) next = -2;   // no distribution to draw from
+    else next = direct_draw<T>(D, P, large, small, lse, D.runs + static_cast<size_t>(first_item + o.L) * n_runs, n_runs, from_large, u2, smem, lane);
+  }
+  write_results(P, b, o.L, next, lane);
+}
+
+template <typename T, int DIV>
+__global__ void __launch_bounds__(kDirThreads, kDirCtasPerSm) direct_kernel(const __grid_constant__ DirectParams D) {
+  constexpr int NW = kDirWarps;
+  extern __shared__ __align__(16) unsigned char dir_smem[];   // [warp][model][run_bytes]
+  __shared__ __align__(16) float4 lse_in[kDirMaxRuns];        // (ref_small, sum_small, ref_large, sum_large) of every warp of the cluster
+  __shared__ __align__(16) float4 done_in[kDirMaxRuns];       // rank 0: (divergence in bits, residual mass, mass of p, rows differ)
+  __shared__ unsigned long long lse_bar, done_bar;
+  __shared__ int sh_last;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int rank = static_cast<int>(cluster_rank()), cs = D.cs, n_runs = cs * NW;
+  const StageParams& P1 = D.s1;
+  if (tid == 0) {
+    mbar_init(&lse_bar, 1);
+    mbar_init(&done_bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    mbar_arrive_expect_tx(&lse_bar, static_cast<unsigned>(n_runs) * 16u);
+    if (rank == 0) mbar_arrive_expect_tx(&done_bar, static_cast<unsigned>(n_runs) * 16u);
+  }
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // waited for before the first remote post
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  release_dependent_launch();
+
+  // ---- the item ----
+  const int item = blockIdx.x / cs, b = item / D.items_per_seq, nth = item - b * D.items_per_seq;
+  const bool second = nth >= P1.K && D.n_stages == 2;
+  const StageParams& P = second ? D.s2 : P1;
+  const int k = second ? nth - P1.K : nth;    // position; k == P.K: the bonus row
+  const int V = P.V;
+  const unsigned smem = smem_u32(dir_smem) + static_cast<unsigned>(warp * 2 * D.run_bytes);
+  int nv = P.K;                               // n_valid comes with single stages only
+  if (D.n_stages == 1 && P1.n_valid != nullptr) nv = min(max(P1.n_valid[b], 0), P.K);
+  const int need = D.n_stages == 2 ? D.items_per_seq : nv + (P.bonus ? 1 : 0);   // items of the sequence that take part
+  if (!(k < nv || (P.bonus && k == nv))) {    // uniform across the cluster
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    // a sequence without a row: its first item's cluster has only to say so
+    if (need == 0 && k == 0 && rank == 0 && warp == 0) direct_finish<T>(D, P1, b, item, n_runs, smem, lane, -1, nullptr, 0);
+    return;
+  }
+  const bool single = k >= P.K;               // the bonus row has no small partner
+  const T* large = static_cast<const T*>(P.large) + b * P.seq_stride_large + static_cast<long long>(k) * V;
+  const T* small = single ? large : static_cast<const T*>(P.small) + b * P.seq_stride_small + static_cast<long long>(k) * V;
+
+  // ---- this warp's run ----
+  const int me = rank * NW + warp, g0 = run_begin(me, n_runs, D.n_groups), groups = run_begin(me + 1, n_runs, D.n_groups) - g0;
+  const int n = max(0, min(groups * kFinPart, V - g0 * kFinPart)), half = (groups + 1) / 2;
+  const Run<T> xs(smem, small + g0 * kFinPart, n), xl(smem + static_cast<unsigned>(D.run_bytes), large + g0 * kFinPart, n);
+#pragma unroll 1
+  for (int from = 0, to = min(n, half * kFinPart), i = 0; i < 2; ++i, from = to, to = n) {   // pass A begins with the first half
+    xs.copy(small + g0 * kFinPart, from, to, lane);
+    xl.copy(large + g0 * kFinPart, from, to, lane);
+    run_copies_commit();
+  }
+  run_copies_wait<1>();
+
+  // ---- pass A and the exchange: every warp's partials go to every CTA of the cluster ----
+  const float c = P.c;
+  const float4 mine = run_lse(xs, xl, groups, half, c, lane);
+  auto wait_bar = [&](unsigned long long* bar) {
+    unsigned spins = 0;
+    while (!mbar_try(bar, 0u))
+      if (++spins > kDirSpinLimit) { atomicExch(P.status, 1); break; }
+  };
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (lane < cs) remote_post_f4(map_to_rank(&lse_in[me], lane), mine, map_to_rank(&lse_bar, lane));
+  wait_bar(&lse_bar);
+  float ms = -1e30f, ml = -1e30f, ss = 0.f, sl = 0.f;
+  {
+    float4 v[kDirPer];
+#pragma unroll
+    for (int j = 0; j < kDirPer; ++j) {
+      v[j] = lane + 32 * j < n_runs ? lse_in[lane + 32 * j] : make_float4(-1e30f, 0.f, -1e30f, 0.f);
+      ms = fmaxf(ms, v[j].x); ml = fmaxf(ml, v[j].z);
+    }
+    ms = warp_max(ms); ml = warp_max(ml);
+#pragma unroll
+    for (int j = 0; j < kDirPer; ++j) {
+      ss = fmaf(v[j].y, ex2_approx(v[j].x - ms), ss);
+      sl = fmaf(v[j].w, ex2_approx(v[j].z - ml), sl);
+    }
+    ss = warp_reduce<OpSum>(ss);
+    sl = warp_reduce<OpSum>(sl);
+  }
+  const float l2ss = lg2_into(ss, ms), l2sl = lg2_into(sl, ml);
+
+  // ---- pass B: divergence terms, residual mass and mass of p ----
+  float2 js = make_float2(0.f, 0.f), r2 = js, p2 = js;
+  unsigned differ = 0u;
+  {
+    const float inv_c = 1.f / c;
+    float x0s, rests, x0l, restl;
+    split_offset(ms, l2ss, c, inv_c, x0s, rests);
+    split_offset(ml, l2sl, c, inv_c, x0l, restl);
+    const float floor_s = DIV == kDivKL ? -INFINITY : (ms + l2ss - 125.f) * inv_c, floor_l = DIV == kDivKL ? -INFINITY : (ml + l2sl - 125.f) * inv_c;
+    const unsigned floor2_s = Pairs<T>::floor_bits(floor_s), floor2_l = Pairs<T>::floor_bits(floor_l);
+    const float2 cc = splat2(c), n0l = splat2(-x0l), n0s = splat2(-x0s), nrl = splat2(-restl), nrs = splat2(-rests);
+#pragma unroll 1
+    for (int g = 0; g < groups; ++g) {
+      const Group<T> u(xs, g * kFinPart + lane * kFinElemsPerThread), v(xl, g * kFinPart + lane * kFinElemsPerThread);
+#pragma unroll
+      for (int j = 0; j < Group<T>::kWords; ++j) differ |= u.w[j] ^ v.w[j];
+#pragma unroll
+      for (int j = 0; j < kFinElemsPerThread / 2; ++j) {
+        const float2 a = __ffma2_rn(__fadd2_rn(v.pair_clamped(j, floor_l, floor2_l), n0l), cc, nrl);   // log2 p
+        const float2 d = __ffma2_rn(__fadd2_rn(u.pair_clamped(j, floor_s, floor2_s), n0s), cc, nrs);   // log2 q
+        if (DIV == kDivJS) {
+          const float2 e = make_float2(ex2_approx(fmaxf(a.x, d.x)), ex2_approx(fmaxf(a.y, d.y)));   // max(p, q)
+          const float2 dd = __ffma2_rn(d, splat2(-1.f), a);
+          const float2 t = make_float2(ex2_approx(-fabsf(dd.x)), ex2_approx(-fabsf(dd.y)));
+          const float2 ps = psi_poly<7>(t), lo = __fmul2_rn(e, t);                                  // lo: min(p, q)
+          js = __ffma2_rn(e, make_float2(fmaf(t.x, -fabsf(dd.x), ps.x), fmaf(t.y, -fabsf(dd.y), ps.y)), js);
+          r2 = __fadd2_rn(r2, make_float2(dd.x > 0.f ? e.x - lo.x : 0.f, dd.y > 0.f ? e.y - lo.y : 0.f));
+          p2 = __fadd2_rn(p2, make_float2(dd.x > 0.f ? e.x : lo.x, dd.y > 0.f ? e.y : lo.y));
+        } else {
+          const float2 p = ex2_2(a), q = ex2_2(d);
+          r2 = __fadd2_rn(r2, make_float2(fmaxf(p.x - q.x, 0.f), fmaxf(p.y - q.y, 0.f)));
+          p2 = __fadd2_rn(p2, p);
+          if (DIV == kDivKL) {
+            // KL(large || small) on unclamped logits: q == 0 with p > 0 gives +inf, as it should
+            if (p.x > 0.f) js.x = fmaf(p.x, a.x - d.x, js.x);
+            if (p.y > 0.f) js.y = fmaf(p.y, a.y - d.y, js.y);
+          }
+        }
+      }
+    }
+  }
+  {
+    const float js_w = warp_reduce<OpSum>(js.x + js.y), r_w = warp_reduce<OpSum>(r2.x + r2.y), p_w = warp_reduce<OpSum>(p2.x + p2.y);
+    const bool any = __any_sync(0xffffffffu, differ != 0u);
+    if (lane == 0) remote_post_f4(map_to_rank(&done_in[me], 0), make_float4(js_w, r_w, p_w, any ? 1.f : 0.f), map_to_rank(&done_bar, 0));
+  }
+
+  // ---- the row's record, by rank 0 ----
+  // No CTA leaves while a peer can still write into its shared memory: everyone says here that its posts are out (rank 0's
+  // first warp, once all of them have arrived) and waits for the others at the end.
+  __syncwarp();
+  if (rank != 0 || warp != 0) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  if (rank == 0) {
+    if (warp == 0) {
+      wait_bar(&done_bar);
+      __syncwarp();
+      asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+      float js_t = 0.f, res_t = 0.f, dif_t = 0.f;
+#pragma unroll
+      for (int j = 0; j < kDirPer; ++j) {
+        if (lane + 32 * j < n_runs) {
+          const float4 v = done_in[lane + 32 * j];
+          js_t += v.x; res_t += v.y; dif_t += v.w;
+          // what the clamp leaves of masked logits (2^-125 each) is no weight
+          __stcg(D.runs + static_cast<size_t>(item) * n_runs + lane + 32 * j, make_float2(v.y > 1e-30f ? v.y : 0.f, v.z > 1e-30f ? v.z : 0.f));
+        }
+      }
+      js_t = warp_reduce<OpSum>(js_t); res_t = warp_reduce<OpSum>(res_t); dif_t = warp_reduce<OpSum>(dif_t);
+      if (lane == 0) {
+        RowStats st{};
+        int flags = 0;
+        if (!(fabsf(ms + l2ss) < INFINITY)) flags |= kFlagSmallNonfinite;   // NaN, +inf, or no finite logit
+        if (!(fabsf(ml + l2sl) < INFINITY)) flags |= kFlagLargeNonfinite;
+        if (flags) {
+          st.m2_small = st.l2s_small = st.m2_large = st.l2s_large = st.div = st.resid = __int_as_float(0x7fc00000);
+        } else {
+          st.m2_small = ms; st.l2s_small = l2ss; st.m2_large = ml; st.l2s_large = l2sl;
+          st.div = fmaxf(DIV == kDivJS ? (0.5f * kLn2) * js_t : DIV == kDivKL ? kLn2 * js_t : res_t, 0.f);
+          st.resid = res_t;
+          if (dif_t == 0.f) { st.div = 0.f; st.resid = 0.f; }   // bitwise identical rows: exactly zero
+        }
+        st.flags = flags;
+        if (single) D.bonus_stats[b] = st;
+        else P.stats[static_cast<long long>(b) * P.K + k] = st;
+      }
+      __syncwarp();
+      if (lane == 0) {   // the record and the runs come before the ticket, and the others' before what follows it
+        int before;
+        asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(before) : "l"(D.ticket + b) : "memory");
+        if (before == need - 1) D.ticket[b] = 0;
+        sh_last = before == need - 1;
+      }
+    }
+    __syncthreads();
+    if (sh_last && warp < 2) {
+      // every row of the sequence is done: its finalisation, a warp per stage where stage 2 does not need stage 1's draw
+      const int item0 = b * D.items_per_seq;
+      const bool side = D.n_stages == 2 && D.s2.mode == kModeFuzzy;
+      int L1 = 0, n2 = -1;
+      const int32_t* tokens = nullptr;
+      if (warp == 1 && side) {
+        stage1_prefix<T>(P1, D.s2.K, b, lane, &L1, &n2);
+        tokens = P1.tokens + static_cast<long long>(b) * P1.K;
+      }
+#pragma unroll 1
+      for (int stage = warp; stage < D.n_stages; stage += side ? 2 : 1) {
+        if (warp == 1 && !side) break;
+        direct_finish<T>(D, stage ? D.s2 : P1, b, item0 + (stage ? P1.K : 0), n_runs, smem, lane, stage ? n2 : -1, tokens, L1);
+        __threadfence_block();   // the window, for a second stage by the same warp
+        __syncwarp();
+      }
+    }
+  }
+  __syncwarp();
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+}
+
+// ---- host side --------------------------------------------------------------------------------------
+inline int direct_run_bytes(int V, int elem_bytes, int cs) {
+  const int groups = (V + kFinPart - 1) / kFinPart, runs = cs * kDirWarps, most = (groups + runs - 1) / runs;
+  return most * kFinPart * elem_bytes + 16;
+}
+inline int direct_smem_bytes(int V, int elem_bytes, int cs) { return direct_run_bytes(V, elem_bytes, cs) * 2 * kDirWarps; }
+
+template <typename T, int DIV>
+inline cudaError_t direct_launch_typed(const DirectParams& D, unsigned items, cudaStream_t stream) {
+  static bool prepared[kClMaxDevices] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= kClMaxDevices) return cudaErrorInvalidDevice;
+  if (!prepared[dev]) {
+    e = cudaFuncSetAttribute(direct_kernel<T, DIV>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDirMaxSmem);
+    if (e != cudaSuccess) return e;
+    prepared[dev] = true;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(items * static_cast<unsigned>(D.cs));
+  cfg.blockDim = dim3(kDirThreads);
+  cfg.dynamicSmemBytes = static_cast<size_t>(D.run_bytes) * 2 * kDirWarps;
+  cfg.stream = stream;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = static_cast<unsigned>(D.cs);
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, direct_kernel<T, DIV>, D);
+}
+
+inline cudaError_t launch_direct(const DirectParams& D, int dtype, unsigned items, cudaStream_t stream) {
+  const int div = D.s1.div_kind;
+  if (dtype == 0)
+    return div == kDivJS ? direct_launch_typed<float, kDivJS>(D, items, stream) : div == kDivTV ? direct_launch_typed<float, kDivTV>(D, items, stream)
+                                                                                            : direct_launch_typed<float, kDivKL>(D, items, stream);
+  return div == kDivJS ? direct_launch_typed<__nv_bfloat16, kDivJS>(D, items, stream)
+         : div == kDivTV ? direct_launch_typed<__nv_bfloat16, kDivTV>(D, items, stream)
+                         : direct_launch_typed<__nv_bfloat16, kDivKL>(D, items, stream);
+}
+
+// Whether a call goes this way, by its index pairs (rows x V). Both ways were measured over V = 4096 to 128001, both types,
+// 0.5 to 32 million pairs, everything accepted and every sequence drawing; the limits are where this way stops being the
+// faster one. Two stages (the ring kernel's single finalisation launch finishes both, us a call ring / this, B, K = 8 / 4):
+// V = 8000 bf16 B = 10 18.7 / 11.0, 83 35.9 / 26.2, 167 65.9 / 44.8; V = 32000 B = 3 20.8 / 12.4, 21 29.7 / 28.9, 42 46.1 / 45.5,
+// 83 67.2 / 78.7; V = 128000 B = 10 63.5 / 45.1, 21 80.3 / 81.2. One stage (K = 8, every sequence drawing / accepting everything):
+// V = 8000 bf16 B = 125 29.4, 23.4 / 26.1, 23.1, 250 47.5, 37.1 / 45.2, 41.7; V = 32000 B = 4 15.8, 11.5 / 10.7, 9.6, 16 18.3, 14.3 /
+// 17.2, 14.8, 31 24.1, 19.9 / 27.8, 25.5. Rows that the ring kernel takes logit by logit (unaligned): V = 32001 bf16 two
+// stages B = 10 31.7 / 18.7, 83 96.1 / 85.9; one stage B = 16 25.9 / 18.8, 62 54.3 / 49.4. fp32 logits, twice the bytes to copy and
+// to hold, turn earlier. `onepass`: the KL kernel that reads every logit once would take the call.
+inline bool direct_applies(int V, int dtype, int n_stages, long long rows, bool unaligned, bool ragged, bool bonus, bool onepass) {
+  const double pairs = static_cast<double>(rows) * V;
+  if (V < 2048) return false;
+  double most;
+  if (n_stages == 2) {
+    if (onepass) most = V <= 16384 ? 8.2e6 : 4.1e6;
+    else if (dtype == 1) most = unaligned ? 33e6 : (V <= 8192 || V >= 49152) ? 16.5e6 : 8.2e6;
+    else if (unaligned) most = V <= 65536 ? 16.5e6 : 4.8e6;
+    else most = V > 4096 && V <= 16384 ? 4.1e6 : 8.2e6;
+  } else {
+    if (onepass) most = 0.0;
+    else if (dtype == 1) most = unaligned ? min(33e6, 5.2e11 / V) : min(8.2e6, 6.6e10 / V);
+    else if (V <= 4608) most = unaligned ? 16.5e6 : 4.1e6;
+    else most = min(2.2e6, 1.3e11 / V);
+    if (bonus) most *= 2.0;                  // a draw more from a row that the ring kernel has not seen
+    if (ragged) most = min(most, 4.0e6);     // the ring kernel deals out the valid rows alone
+  }
+  return pairs <= most;
+}
+
+// CTAs per row pair: what lets four CTAs share an SM, and more while all CTAs are resident at once and every warp has 256
+// indices (0: rows too long for the kernel). V = 32000 bf16, K = 8, one stage, clusters of 2 / 4 / 8: B = 4 11.1 / 10.0 / 8.9 us,
+// 8 11.3 / 11.7 / 11.0, 16 18.0 / 14.5 / 18.6.
+inline int direct_cluster_size(int V, int dtype, long long items) {
+  const int es = dtype == 0 ? 4 : 2, sms = cluster_sm_count(), groups = (V + kFinPart - 1) / kFinPart;
+  int cs = 1;
+  while (cs < kDirMaxRanks && direct_smem_bytes(V, es, cs) > kDirSmemForFour) ++cs;
+  if (direct_smem_bytes(V, es, cs) > kDirMaxSmem) return 0;
+  while (cs < kDirMaxRanks && (cs + 1) * kDirWarps <= groups && items * (cs + 1) <= static_cast<long long>(kDirCtasPerSm) * sms) ++cs;
+  return cs;
+}
+
+}  // namespace psd

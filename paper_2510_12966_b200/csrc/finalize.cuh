@@ -15,6 +15,7 @@ namespace psd {
 constexpr int kFinThreads = 1024;
 constexpr int kFinElemsPerThread = 8;                      // consecutive vocabulary indices per thread and tile
 constexpr int kFinTile = kFinThreads * kFinElemsPerThread;  // 8192 indices per tile
+constexpr int kFinPart = 32 * kFinElemsPerThread;           // what a warp takes of them
 constexpr int kFinMaxTiles = 1024;                          // V <= 8,388,608
 constexpr int kFinBatch = 32;                               // tiles summed between two CTA-wide barriers
 constexpr int kFinMaxRanks = 8;                             // CTAs per sequence at most
@@ -144,7 +145,10 @@ __device__ __forceinline__ ScanOut scan_unit(const StageParams& P, const int b, 
   int flags = 0;
   if (lane < nv) {
     const int r = b * K + lane;
-    st = P.stats[r];
+    // (past the first-level cache: the records may come from other CTAs of this very launch)
+    const float4 lse = __ldcg(reinterpret_cast<const float4*>(P.stats + r)), rest = __ldcg(reinterpret_cast<const float4*>(P.stats + r) + 1);
+    st.m2_small = lse.x; st.l2s_small = lse.y; st.m2_large = lse.z; st.l2s_large = lse.w;
+    st.div = rest.x; st.resid = rest.y; st.flags = __float_as_int(rest.z);
     const int x = (tokens_given != nullptr) ? (lane < n_given ? tokens_given[lane] : 0) : P.tokens[r];
     flags = st.flags | ((x < 0 || x >= V) ? kFlagTokenRange : 0);
     row_uniforms(P.seed, P.offset, static_cast<unsigned>((P.seq_base + b) * K + lane), &u, &u2);
@@ -197,18 +201,21 @@ __device__ __forceinline__ ScanOut scan_unit(const StageParams& P, const int b, 
   return o;
 }
 
-// The results of one sequence, by one thread: prefix length, next token, and in the two-stage wrapper the stage-2
+// The results of one sequence, by one full warp: prefix length, next token, and in the two-stage wrapper the stage-2
 // window (Fig. 1): accepted draft tokens, then the correction token.
-__device__ __forceinline__ void write_results(const StageParams& P, const int b, const int L, const int next) {
-  P.out_accept_len[b] = L;
-  P.out_next_token[b] = next;
+__device__ __forceinline__ void write_results(const StageParams& P, const int b, const int L, const int next, const int lane) {
+  if (lane == 0) {
+    P.out_accept_len[b] = L;
+    P.out_next_token[b] = next;
+  }
   if (P.window != nullptr) {
     const int have = L + (next >= 0 ? 1 : 0);
     const int n2 = min(have, P.K_window);
-    P.n_window[b] = n2;
-    if (P.fill_out != nullptr && b < P.fill_cap) P.fill_out[b] = n2;
-    for (int j = 0; j < P.K_window; ++j)
-      P.window[b * P.K_window + j] = (j < n2) ? ((j < L) ? P.tokens[b * P.K + j] : next) : 0;
+    if (lane == 0) {
+      P.n_window[b] = n2;
+      if (P.fill_out != nullptr && b < P.fill_cap) P.fill_out[b] = n2;
+    }
+    if (lane < P.K_window) P.window[b * P.K_window + lane] = (lane < n2) ? ((lane < L) ? P.tokens[b * P.K + lane] : next) : 0;
   }
 }
 
@@ -485,7 +492,7 @@ __device__ __forceinline__ void finalize_sequence(const StageParams& P, const in
     }
   }
 
-  if (tid == 0 && cl_rank == writer) write_results(P, b, L, next);
+  if (warp == 0 && cl_rank == writer) write_results(P, b, L, next, lane);
 }
 
 template <typename T, int CL>
@@ -599,22 +606,17 @@ __global__ void __launch_bounds__(kScanWarps * 32) finalize_scan_kernel(const St
     stage1_prefix<T>(P1, P2.K, b, lane, &L1, &n2);
     o = scan_unit<T>(P2, b, lane, true, n2, P1.tokens + b * P1.K, L1);
   }
+  const bool no_dist = o.L < o.nv && (o.flags & (kFlagSmallNonfinite | kFlagLargeNonfinite)) != 0;   // nothing to draw from
+  const bool draw = o.L < o.nv && !no_dist;
   if (lane == 0) {
-    int next = -1;
-    bool draw = false;
-    if (o.L < o.nv) {
-      if (o.flags & (kFlagSmallNonfinite | kFlagLargeNonfinite)) next = -2;   // no distribution to draw from
-      else draw = true;
-    }
     ds.need[unit] = draw ? 1 : 0;
     if (draw) {
       DrawRecord r;
       r.L = o.L; r.u2 = o.u2; r.m2l = o.m2l; r.l2sl = o.l2sl; r.m2s = o.m2s; r.l2ss = o.l2ss; r.resid = o.resid; r.unit = unit;
       ds.record[unit] = r;
-    } else {
-      write_results(second ? P2 : P1, b, o.L, next);
     }
   }
+  if (!draw) write_results(second ? P2 : P1, b, o.L, no_dist ? -2 : -1, lane);
 }
 
 template <typename T>
@@ -788,7 +790,7 @@ __global__ void __launch_bounds__(kFinThreads) finalize_pick_kernel(const StageP
       descend_tile<T>(row, S, tile);
       next = S.sh_token;
     }
-    if (tid == 0) write_results(P, b, rec.L, next);
+    if (warp == 0) write_results(P, b, rec.L, next, lane);
     __syncthreads();   // S is free for the next draw
   }
 }

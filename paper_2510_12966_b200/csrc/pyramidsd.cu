@@ -17,6 +17,7 @@
 #include "rowstats_cluster.cuh"
 #include "rowstats_onepass.cuh"
 #include "lmhead_fused.cuh"
+#include "direct.cuh"
 
 namespace {
 
@@ -25,7 +26,7 @@ using psd::StageParams;
 
 std::atomic<uint64_t> g_launches{0};
 thread_local cudaStream_t t_stream = nullptr;
-thread_local int t_two_stage_policy = PSD_TWO_STAGE_AUTO;
+thread_local int t_two_stage_policy = PSD_TWO_STAGE_DEFAULT;   // DEFAULT: as AUTO, and small calls go as one launch
 
 constexpr int kMaxDevices = 64;
 constexpr size_t kAlign = 256;
@@ -56,7 +57,7 @@ struct StreamScratch {
   cudaStream_t stream = nullptr;
   void* ws = nullptr;
   size_t ws_bytes = 0;
-  int* status = nullptr;
+  int* status = nullptr;    // and behind it, 256 bytes on, the tickets of the one-launch calls (zero between calls)
   void* stage[4] = {nullptr, nullptr, nullptr, nullptr};
   size_t stage_bytes[4] = {0, 0, 0, 0};
   void* out4 = nullptr;     // 4 x [B] results of the host entry point
@@ -81,6 +82,7 @@ struct DeviceState {
   unsigned fill_calls = 0;       // calls of that shape since the lengths were last asked for
 };
 constexpr int kFillCap = 4096;
+constexpr int kDirectMaxB = 4096;   // sequences of a one-launch call: a ticket each, behind the status word
 DeviceState g_dev[kMaxDevices];
 // what pyramidsd_last_status() looks at: the stream and the status word of this thread's most recent call (the word
 // sits in a scratch entry, or in the tail of the caller's workspace)
@@ -120,8 +122,9 @@ int scratch_for(cudaStream_t stream, StreamScratch** out) {
 // with ss->mu held
 int ensure_status(StreamScratch* ss) {
   if (ss->status) return PSD_OK;
-  if (cudaMalloc(reinterpret_cast<void**>(&ss->status), kAlign) != cudaSuccess) { cudaGetLastError(); return PSD_ERR_CUDA; }
-  if (cudaMemset(ss->status, 0, kAlign) != cudaSuccess) return PSD_ERR_CUDA;
+  const size_t bytes = kAlign + kDirectMaxB * sizeof(int);
+  if (cudaMalloc(reinterpret_cast<void**>(&ss->status), bytes) != cudaSuccess) { cudaGetLastError(); return PSD_ERR_CUDA; }
+  if (cudaMemset(ss->status, 0, bytes) != cudaSuccess) return PSD_ERR_CUDA;
   return PSD_OK;
 }
 
@@ -446,6 +449,48 @@ int launch_finalize(const StageParams& P, int dtype, cudaStream_t stream, Stream
   return check_launch();
 }
 
+// CTAs per row pair if the call goes as one launch (direct.cuh), else 0. For calls on the library's own scratch whose
+// schedule is the library's to choose.
+int direct_route(const StageParams& P1, const StageParams& P2, int n_stages, int dtype, int kernel_variant, int cluster_size) {
+  if (kernel_variant != PSD_KERNEL_AUTO || cluster_size != 0 || P1.K == 0 || P1.B > kDirectMaxB) return 0;
+  StageParams P = P1;
+  if (n_stages == 2) {
+    P.small2 = P2.small; P.large2 = P2.large;
+    P.seq_stride_small2 = P2.seq_stride_small; P.seq_stride_large2 = P2.seq_stride_large;
+    P.K2 = P2.K;
+  }
+  const bool resid_wanted = P1.out_resid_mass != nullptr || P2.out_resid_mass != nullptr;
+  const long long rows = static_cast<long long>(P.B) * (P.K + P.K2);
+  if (!psd::direct_applies(P.V, dtype, n_stages, rows, !psd::cluster_shape_ok(P, dtype), P1.n_valid != nullptr, P2.bonus != 0,
+                           psd::onepass_applies(P, dtype, resid_wanted))) return 0;
+  return psd::direct_cluster_size(P.V, dtype, rows);
+}
+
+// A stage (n_stages == 1) or both stages of the pyramid as that one launch, on the entry's own scratch.
+int launch_direct_call(const StageParams& P1, const StageParams& P2, int n_stages, int cs, int dtype, cudaStream_t stream, StreamScratch* ss) {
+  psd::DirectParams D{};
+  D.s1 = P1; D.s2 = P2;
+  D.n_stages = n_stages;
+  D.cs = cs;
+  D.n_groups = (P1.V + psd::kFinPart - 1) / psd::kFinPart;
+  D.run_bytes = psd::direct_run_bytes(P1.V, static_cast<int>(elem_size(dtype)), cs);
+  D.items_per_seq = P1.K + (n_stages == 2 ? P2.K : 0) + (P1.bonus || (n_stages == 2 && P2.bonus) ? 1 : 0);
+  const long long items = static_cast<long long>(P1.B) * D.items_per_seq;
+  const size_t stat = align_up(static_cast<size_t>(P1.B) * sizeof(RowStats));
+  const int rc = grow(ss, &ss->draw, &ss->draw_bytes, stat + static_cast<size_t>(items) * (cs * psd::kDirWarps) * sizeof(float2));
+  if (rc != PSD_OK) return rc;
+  D.bonus_stats = static_cast<RowStats*>(ss->draw);
+  D.runs = reinterpret_cast<float2*>(static_cast<char*>(ss->draw) + stat);
+  D.ticket = reinterpret_cast<int*>(reinterpret_cast<char*>(ss->status) + kAlign);
+  TimedLaunch timed(stream, 0);
+  if (psd::launch_direct(D, dtype, static_cast<unsigned>(items), stream) != cudaSuccess) {
+    std::fprintf(stderr, "pyramidsd: one-launch kernel failed to launch: %s\n", cudaGetErrorString(cudaGetLastError()));
+    return PSD_ERR_CUDA;
+  }
+  g_launches.fetch_add(1, std::memory_order_relaxed);
+  return check_launch();
+}
+
 int validate_stage(const psd_stage_args* a) {
   if (a == nullptr || a->struct_size != sizeof(psd_stage_args)) return PSD_ERR_INVALID_ARG;
   if (!valid_dtype(a->dtype) || !valid_mode(a->mode) || !valid_div(a->div_kind)) return PSD_ERR_INVALID_ARG;
@@ -516,7 +561,7 @@ cudaStream_t pick_stream(const psd_stage_args* a) {
 // Runs one stage with the scratch entry `ss` (held by the caller); `window_out`/`n_window_out`/`K_window` non-null
 // make the finalisation also build the stage-2 window of the wrapper.
 int run_stage_locked(const psd_stage_args* a, StreamScratch* ss, int* status, cudaStream_t stream, int32_t* window_out,
-                     int32_t* n_window_out, int K_window, int32_t* fill_out = nullptr, int onepass = -1, bool force_ua = false) {
+                     int32_t* n_window_out, int K_window, int32_t* fill_out = nullptr, int onepass = -1, bool force_ua = false, bool allow_direct = false) {
   int rc = PSD_OK;
   void* ws = a->workspace;
   if (ws == nullptr) {
@@ -530,6 +575,10 @@ int run_stage_locked(const psd_stage_args* a, StreamScratch* ss, int* status, cu
   P.K_window = K_window;
   P.fill_out = fill_out;
   P.fill_cap = kFillCap;
+  if (allow_direct) {
+    const int cs = direct_route(P, P, 1, a->dtype, a->kernel_variant, a->cluster_size);
+    if (cs > 0) return launch_direct_call(P, P, 1, cs, a->dtype, stream, ss);
+  }
   if (a->K > 0) {
     rc = launch_rowstats(P, a->dtype, a->kernel_variant, a->cluster_size, stream, false, P.out_resid_mass != nullptr, onepass, force_ua);
     if (rc != PSD_OK) return rc;
@@ -556,7 +605,7 @@ int run_stage(const psd_stage_args* a) {
   rc = ensure_status(ss);
   if (rc != PSD_OK) return rc;
   t_last_scratch = ss; t_last_status = ss->status; t_last_stream = stream;
-  return run_stage_locked(a, ss, ss->status, stream, nullptr, nullptr, 0);
+  return run_stage_locked(a, ss, ss->status, stream, nullptr, nullptr, 0, nullptr, -1, false, true);
 }
 
 size_t pyramid_workspace_bytes(int B, int K_d, int K_q) { return stage_workspace_bytes(B, K_d) + stage_workspace_bytes(B, K_q); }
@@ -644,8 +693,18 @@ int verify_two_stage_locked(const psd_pyramid_args* a, StreamScratch* ss, int* s
   rc = validate_stage(&s1);
   if (rc == PSD_OK) rc = validate_stage(&s2);
   if (rc != PSD_OK) return rc;
-  const int policy = target_ready != nullptr ? PSD_TWO_STAGE_SEPARATE
-                     : a->schedule != PSD_TWO_STAGE_DEFAULT ? a->schedule : t_two_stage_policy;
+  int policy = target_ready != nullptr ? PSD_TWO_STAGE_SEPARATE
+               : a->schedule != PSD_TWO_STAGE_DEFAULT ? a->schedule : t_two_stage_policy;
+  if (policy == PSD_TWO_STAGE_DEFAULT && ss != nullptr && a->workspace == nullptr) {
+    StageParams P1 = make_params(&s1, s1.workspace, status);
+    P1.window = window;
+    P1.n_window = n_window;
+    P1.K_window = K_q;
+    const StageParams P2 = make_params(&s2, s2.workspace, status);
+    const int cs = direct_route(P1, P2, 2, dtype, a->kernel_variant, 0);
+    if (cs > 0) return launch_direct_call(P1, P2, 2, cs, dtype, stream, ss);
+  }
+  if (policy == PSD_TWO_STAGE_DEFAULT) policy = PSD_TWO_STAGE_AUTO;
   bool separate = policy == PSD_TWO_STAGE_SEPARATE;
   int32_t* fill_out = nullptr;
   if (policy == PSD_TWO_STAGE_AUTO) {
@@ -884,7 +943,7 @@ int pyramidsd_verify_host(const void* logits_draft, const void* logits_qual, con
   if (rc != PSD_OK) return rc;
   // below a few megabytes the copies are shorter than what the two streams' events cost; a thread that asked for two steps
   // gets them, behind all copies
-  const bool overlap = n_d + n_t >= kHostOverlapBytes && (t_two_stage_policy == PSD_TWO_STAGE_AUTO || t_two_stage_policy == PSD_TWO_STAGE_SEPARATE);
+  const bool overlap = n_d + n_t >= kHostOverlapBytes && t_two_stage_policy != PSD_TWO_STAGE_FUSED && t_two_stage_policy != PSD_TWO_STAGE_FUSED_ROWS;
   if (overlap) {
     rc = ensure_copy_stream(ss);
     if (rc != PSD_OK) return rc;
@@ -1250,7 +1309,7 @@ size_t pyramidsd_pyramid_workspace_bytes(int B, int K_d, int K_q, int V, psd_dty
 
 int pyramidsd_set_two_stage_policy(int policy) {
   if (policy < PSD_TWO_STAGE_DEFAULT || policy > PSD_TWO_STAGE_FUSED_ROWS) return PSD_ERR_INVALID_ARG;
-  t_two_stage_policy = policy == PSD_TWO_STAGE_DEFAULT ? PSD_TWO_STAGE_AUTO : policy;
+  t_two_stage_policy = policy;
   return PSD_OK;
 }
 

@@ -1,0 +1,180 @@
+"""Small and medium calls as one launch (csrc/direct.cuh). Every form such a call accepts -- strides, bases at any element,
+types, modes, divergences, ragged windows, bonus rows, temperatures -- against the same call with a workspace of the
+caller's, which takes the statistics launch and the finalisation launch; and the sizes at which a row's runs and groups
+end against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+from parity_utils import compare_stage, gpu_stage_to_numpy, host_bits
+from test_gpu_any_alignment import on_device
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def psd():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2510_12966_b200 import binding
+    binding.load_library()
+    torch.cuda.set_device(0)
+    return binding
+
+
+def launches(psd, call):
+    n0 = psd.launch_count()
+    out = call()
+    torch.cuda.synchronize()
+    assert psd.last_status() == 0
+    return out, psd.launch_count() - n0
+
+
+def agree(a, b):
+    """Integers equal; floats within what the two arithmetics differ by (degree 4 against 7: 2e-5; sums of max(p, q) less 1
+    against the residual mass itself: 2e-6; probabilities: one rounding of a normaliser of about 20). Sequences whose
+    integers differ are counted."""
+    ints = [k for k in a if torch.is_tensor(a[k]) and a[k].dtype == torch.int32]
+    B = a["accept_len"].shape[0]
+    bad = sum((a[k] != b[k]).view(B, -1).any(1).long() for k in ints) > 0
+    for k in a:
+        if torch.is_tensor(a[k]) and a[k].dtype == torch.float32:
+            ok = ~bad
+            assert torch.allclose(a[k][ok], b[k][ok], rtol=5e-6, atol=2.5e-5, equal_nan=True), k
+    return int(bad.sum())
+
+
+def test_stage_forms_against_two_launches(psd):
+    from paper_2510_12966_b200 import workloads as wl
+    rng = np.random.default_rng(5)
+    bad = drew = n = 0
+    for i in range(60):
+        dtype = ("bf16", "f32")[i % 2]
+        V = int(rng.choice([2048, 2049, 2304, 2305, 4095, 5000, 8191, 10007, 16384, 20005]))
+        K, B = int(rng.integers(1, 33)), int(rng.integers(1, 5))
+        while B * K * V > 7e5:
+            K = (K + 1) // 2
+        bonus, ragged = i % 5 == 3, i % 3 == 2
+        zs, zl, tok = wl.make_stage_inputs(B, K + 1, V, dtype, seed=i, boost=(2.0, 10.0), sigma=0.6)
+        zl[B - 1, K - 1] = zs[B - 1, K - 1]                                  # identical rows: exactly zero
+        if i % 4 == 1:
+            zs[0, 0, 5], zl[0, K // 2, V - 1] = float("nan"), float("inf")
+            zl[B - 1, 0, : V // 2] = -float("inf")
+        tok = tok[:, :K].contiguous().cuda()
+        large = zl if bonus else zl[:, :K].contiguous()
+        pad = int(rng.integers(0, 9))                                       # a sequence stride beyond the rows
+        def strided(z):
+            buf = torch.zeros((B, z.shape[1] * V + pad), dtype=z.dtype)
+            buf[:, :z.shape[1] * V] = z.reshape(B, -1)
+            return on_device(buf, int(rng.integers(0, 8)) if i % 2 else 0), z.shape[1] * V + pad
+        (ds, ss), (dl, sl) = strided(zs[:, :K].contiguous()), strided(large)
+        kw = dict(B=B, K=K, V=V, seq_stride_small=ss, seq_stride_large=sl, large_has_bonus_row=bonus, seq_index_base=7 * i,
+                  inv_temperature=(0.0, 1 / 0.7)[i % 2], div_kind=(0, 0, 1, 2)[i % 4], want_resid=i % 4 != 3 or None)
+        if ragged:
+            kw["n_valid"] = torch.as_tensor(rng.integers(-1, K + 2, size=B), dtype=torch.int32, device="cuda")
+        mode, tau = (psd.FUZZY, psd.STRICT, psd.FUZZY_SD_FALLBACK, psd.ASSISTED)[i % 4], (0.03, -1.0, 1e9)[i % 3]
+        a, na = launches(psd, lambda: psd.verify_stage_ex(ds, dl, tok, tau, mode, 11, i, **kw))
+        ws = torch.empty(psd.workspace_bytes(B, K, V, psd.dtype_code(ds)), dtype=torch.uint8, device="cuda")
+        b, nb = launches(psd, lambda: psd.verify_stage_ex(ds, dl, tok, tau, mode, 11, i, workspace=ws, **kw))
+        assert (na, nb) == (1, 2), (i, V, B, K)
+        bad += agree(a, b)
+        drew += int((a["next_token"] >= 0).sum())
+        n += B
+    assert bad <= 1 and drew > n // 3      # a draw or a coin flip within rounding of its boundary
+
+
+def test_pyramid_forms_against_two_launches(psd):
+    from paper_2510_12966_b200 import workloads as wl
+    rng = np.random.default_rng(6)
+    bad = 0
+    for i in range(48):
+        dtype = ("bf16", "f32")[i % 2]
+        V = int(rng.choice([2048, 2051, 4096, 8001, 12345, 33001]))
+        K_d, B = int(rng.integers(1, 20)), int(rng.integers(1, 9))
+        K_q = int(rng.integers(1, K_d + 1))
+        while B > 1 and B * (K_d + K_q) * V > 3e6:
+            B //= 2
+        bonus = i % 4 == 1
+        zd, zq, zt, tok = wl.make_pyramid_inputs(B, K_d, max(K_q, 1), V, dtype, seed=i, sigma_q=0.4, sigma_d=0.8)
+        if bonus:
+            zt = torch.cat([zt, zt[:, :1].flip(-1)], 1).contiguous()
+        off = [int(x) for x in rng.integers(0, 8, 3)] if i % 3 == 2 else [0, 0, 0]
+        t = [on_device(z, o) for z, o in zip((zd, zq, zt), off)] + [tok.cuda()]
+        modes = [(0, 0), (1, 1), (3, 0), (2, 2), (0, 1), (1, 0)][i % 6]
+        kw = dict(target_has_bonus_row=bonus, inv_temperature=(0.0, 1 / 0.7)[i % 2], div_kind=(0, 0, 1, 2)[i % 4], seq_index_base=3 * i)
+        tau = (0.1, 0.05) if i % 2 else (0.3, 0.2)
+        a, na = launches(psd, lambda: psd.verify_ex(*t, *tau, *modes, 5, i, **kw))
+        ws = torch.empty(psd.pyramid_workspace_bytes(B, K_d, K_q, V, psd.dtype_code(t[0])), dtype=torch.uint8, device="cuda")
+        b, nb = launches(psd, lambda: psd.verify_ex(*t, *tau, *modes, 5, i, workspace=ws, schedule=psd.TWO_STAGE_FUSED, **kw))
+        assert (na, nb) == (1, 2), (i, V, B, K_d, K_q)
+        for k in ("div_t", "resid_t"):
+            inside = torch.arange(K_q, device="cuda")[None, :] < a["n_window"][:, None]
+            assert torch.all(a[k][~inside] == 0)
+        bad += agree(a, b)
+    assert bad <= 1
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("V,B,K", [(2048, 1, 1), (2303, 2, 3), (2305, 1, 32), (4096 + 255, 33, 4), (16385, 3, 2), (65536 + 1, 1, 4),
+                                   (128256, 1, 3), (128257, 1, 2)])
+def test_edges_of_runs_and_groups_against_the_oracle(psd, oracle, V, B, K, dtype):
+    from paper_2510_12966_b200 import workloads as wl
+    zs, zl, tok = wl.make_stage_inputs(B, K, V, dtype, seed=V + B, sigma=0.7)
+    zl[0, 0, V - 1] = 40.0                                   # nearly all of the mass on the row's last logit
+    zs[0, K - 1, : V - 3] = -float("inf")                    # a run that starts with no finite logit, and few at its end
+    for mode, tau in ((psd.FUZZY, 0.15), (psd.ASSISTED, 0.0)):
+        out, n = launches(psd, lambda: psd.verify_stage_ex(zs.cuda(), zl.cuda(), tok.cuda(), tau, mode, 3, 5))
+        assert n == 1
+        orc = oracle.verify_stage(host_bits(zs), host_bits(zl), tok.numpy(), np.float32(tau), mode, 3, 5, n_threads=8)
+        rep = compare_stage(oracle, gpu_stage_to_numpy(out), orc, host_bits(zs), host_bits(zl), dtype=dtype, mode=mode,
+                            tau=float(np.float32(tau)), seed=3, offset=5)
+        assert rep["tie_div"] + rep["tie_coin"] + rep["tie_cdf"] <= 1
+
+
+def test_from_two_threads_and_from_a_graph(psd):
+    """The tickets and the records belong to the stream a call runs on; a captured call replays on new contents."""
+    import threading
+    from paper_2510_12966_b200 import workloads as wl
+    sets = [[x.cuda() for x in wl.make_pyramid_inputs(6, 8, 4, 8192, "bf16", seed=s, sigma_q=0.4, sigma_d=0.8)] for s in range(3)]
+    ref = [psd.verify_ex(*t, 0.1, 0.05, 0, 0, 2, 8) for t in sets]
+    torch.cuda.synchronize()
+    errors = []
+    def work(k):
+        try:
+            stream = torch.cuda.Stream()
+            for _ in range(30):
+                out = psd.verify_ex(*sets[k], 0.1, 0.05, 0, 0, 2, 8, stream=stream)
+            stream.synchronize()
+            for key, v in out.items():
+                if torch.is_tensor(v) and not torch.equal(v, ref[k][key]):
+                    errors.append((k, key))
+            psd.release_stream(stream)
+        except Exception as e:
+            errors.append(repr(e))
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(3)]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join()
+    assert not errors, errors[:5]
+    bufs = [t.clone() for t in sets[0]]
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    out = {k: torch.empty(6, dtype=torch.int32, device="cuda") for k in ("accept_len_q", "next_token_q", "accept_len", "next_token")}
+    call = lambda: psd.verify_ex(*bufs, 0.1, 0.05, 0, 0, 2, 8, out=out, want_rows=False, want_window=False, stream=side)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(side):
+        call()
+        side.synchronize()
+        with torch.cuda.graph(g, stream=side):
+            call()
+    for t, r in zip(sets, ref):
+        for dst, src in zip(bufs, t):
+            dst.copy_(src)
+        torch.cuda.synchronize()
+        g.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(out[k], r[k]) for k in out)
+    del g
+    psd.release_stream(side)
+    assert psd.last_status() == 0
