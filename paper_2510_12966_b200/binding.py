@@ -13,7 +13,7 @@ from typing import Optional
 
 import torch
 
-from .build import LIB_PATH
+from .build import LIB_PATH, TENSORS_PATH
 
 F32, BF16 = 0, 1
 FUZZY, STRICT, FUZZY_SD_FALLBACK, ASSISTED = 0, 1, 2, 3
@@ -242,12 +242,26 @@ def _stream_handle(stream: Optional[torch.cuda.Stream]) -> int:
     return _current_raw_stream(torch._C._cuda_getDevice())
 
 
+def _load_tensors():
+    global _new_tensors
+    if not os.path.exists(TENSORS_PATH):
+        raise ImportError(f"{TENSORS_PATH} is missing: build it with `python -m paper_2510_12966_b200.build`")
+    from ._tensors import new_tensors
+    _new_tensors = new_tensors
+
+
+def _new_tensors(like, *spec):
+    """Output tensors on ``like``'s device, one per (kind, rows, cols) of ``spec``: int32 [rows, cols] (kind 0), float32
+    [rows, cols] (1) or int32 [rows] (2). Returns the tensors, then their addresses. Each is an allocation of its own: cut out of one they could not be
+    viewed as another type, changed in place under autograd, detached in place or saved apart from one another.
+    (The first call loads csrc/tensors.cpp, whose function takes this one's place.)"""
+    _load_tensors()
+    return _new_tensors(like, *spec)
+
+
 def _rows(device, dtype, shape, n):
-    """``n`` tensors of this shape, each an allocation of its own: cut out of one they could not be viewed as another type,
-    changed in place under autograd, detached in place or saved apart from one another. (empty_like costs half of
-    empty.)"""
-    first = torch.empty(shape, dtype=dtype, device=device)
-    return (first, *[torch.empty_like(first) for _ in range(n - 1)])
+    """``n`` tensors of this shape and type, each an allocation of its own."""
+    return tuple(torch.empty(shape, dtype=dtype, device=device) for _ in range(n))
 
 
 def set_stream(stream: Optional[torch.cuda.Stream] = None) -> None:
@@ -347,20 +361,17 @@ def verify_fused_lmhead(hidden, w_t, logits_small, tokens, threshold, mode=FUZZY
     B, K, V = logits_small.shape
     d = hidden.shape[1]
     assert hidden.shape[0] == B * K and w_t.shape == (V, d)
-    dev = hidden.device
-    out = dict(zip(("accept_len", "next_token"), _rows(dev, torch.int32, (B,), 2)))
     want_resid = want_rows if want_resid is None else want_resid
-    names = (("div",) if want_rows else ()) + (("resid_mass",) if want_resid else ())
-    if names:
-        out.update(zip(names, _rows(dev, torch.float32, (B, K), len(names))))
+    n = 2 + bool(want_rows) + bool(want_resid)
+    made = _new_tensors(hidden, 2, B, 0, 2, B, 0, *(1, B, K) * (n - 2))
+    out = dict(zip(("accept_len", "next_token") + (("div",) if want_rows else ()) + (("resid_mass",) if want_resid else ()), made))
     rc = load_library().packed_verify_fused_lmhead_ex(_LMHEAD.pack(
         _LMHEAD.size, int(mode),
         _dev_ptr(hidden, torch.bfloat16, "hidden") or 0, _dev_ptr(w_t, torch.bfloat16, "w_t") or 0,
         _dev_ptr(logits_small, torch.bfloat16, "logits_small") or 0, _dev_ptr(tokens, torch.int32, "tokens") or 0,
         B, K, d, V, float(threshold), int(tile_variant or 0), int(div_kind), 0,
         int(philox_seed), int(offset), int(seq_index_base),
-        out["accept_len"].data_ptr(), out["next_token"].data_ptr(),
-        out["div"].data_ptr() if want_rows else 0, out["resid_mass"].data_ptr() if want_resid else 0, _stream_handle(stream)))
+        made[n], made[n + 1], made[n + 2] if want_rows else 0, made[2 * n - 1] if want_resid else 0, _stream_handle(stream)))
     out["status"] = rc
     if raise_on_error:
         _check(rc, "pyramidsd_verify_fused_lmhead")
@@ -408,24 +419,28 @@ def verify_stage_ex(logits_small, logits_large, tokens, threshold, mode=FUZZY, p
         B, K, V = logits_small.shape
         assert tuple(logits_large.shape) == (B, K + (1 if large_has_bonus_row else 0), V)
     dt = dtype_code(logits_small)
-    dev = logits_small.device
     want_resid = want_rows if want_resid is None else (want_resid and want_rows)
-    accept_len = torch.empty(B, dtype=torch.int32, device=dev)
-    out = {"accept_len": accept_len, "next_token": torch.empty_like(accept_len)}
     rows = (0, 0, 0, 0, 0)
-    if want_rows:
-        out["row_flags"] = accept_len.new_empty((B, K))
-        out["div"] = div = torch.empty((B, K), dtype=torch.float32, device=dev)
-        out["p_small_tok"], out["p_large_tok"] = torch.empty_like(div), torch.empty_like(div)
-        if want_resid:
-            out["resid_mass"] = torch.empty_like(div)
-        rows = (div.data_ptr(), out["p_small_tok"].data_ptr(), out["p_large_tok"].data_ptr(),
-                out["resid_mass"].data_ptr() if want_resid else 0, out["row_flags"].data_ptr())
+    if not want_rows:
+        accept_len, next_token, accept_at, next_at = _new_tensors(logits_small, 2, B, 0, 2, B, 0)
+        out = {"accept_len": accept_len, "next_token": next_token}
+    elif not want_resid:
+        accept_len, next_token, flags, div, p_small, p_large, accept_at, next_at, *at = _new_tensors(
+            logits_small, 2, B, 0, 2, B, 0, 0, B, K, 1, B, K, 1, B, K, 1, B, K)
+        out = {"accept_len": accept_len, "next_token": next_token, "row_flags": flags, "div": div, "p_small_tok": p_small,
+               "p_large_tok": p_large}
+        rows = (at[1], at[2], at[3], 0, at[0])
+    else:
+        accept_len, next_token, flags, div, p_small, p_large, resid, accept_at, next_at, *at = _new_tensors(
+            logits_small, 2, B, 0, 2, B, 0, 0, B, K, 1, B, K, 1, B, K, 1, B, K, 1, B, K)
+        out = {"accept_len": accept_len, "next_token": next_token, "row_flags": flags, "div": div, "p_small_tok": p_small,
+               "p_large_tok": p_large, "resid_mass": resid}
+        rows = (at[1], at[2], at[3], at[4], at[0])
     rc = load_library().packed_verify_stage_ex(_STAGE.pack(
         _STAGE.size, dt, logits_small.data_ptr(), logits_large.data_ptr(), _dev_ptr(tokens, torch.int32, "tokens") or 0, B, K, V,
         int(mode), int(div_kind), float(threshold), float(inv_temperature), int(seq_stride_small), int(seq_stride_large),
         int(philox_seed), int(offset), _dev_ptr(n_valid, torch.int32, "n_valid") or 0,
-        accept_len.data_ptr(), out["next_token"].data_ptr(), *rows,
+        accept_at, next_at, *rows,
         0 if workspace is None else workspace.data_ptr(),
         0 if workspace is None else workspace.numel() * workspace.element_size(),
         _stream_handle(stream), 1, int(kernel_variant), int(cluster_size), 1 if large_has_bonus_row else 0, 0, int(seq_index_base)))
@@ -466,29 +481,23 @@ def verify_ex(logits_draft, logits_qual, logits_target, draft_tokens, tau_q, tau
     B, K_d, V = logits_draft.shape
     K_q = logits_target.shape[1] - (1 if target_has_bonus_row else 0)
     assert logits_qual.shape == logits_draft.shape and logits_target.shape[0] == B and logits_target.shape[2] == V
-    dev = logits_draft.device
     if out is None:
-        out = {k: torch.empty(B, dtype=torch.int32, device=dev)
-               for k in ("accept_len_q", "next_token_q", "accept_len", "next_token")}
+        out = dict(zip(("accept_len_q", "next_token_q", "accept_len", "next_token"), _new_tensors(logits_draft, *(2, B, 0) * 4)))
     else:
         out = dict(out)
     results = [_dev_ptr(out[k], torch.int32, k) or 0 for k in ("accept_len_q", "next_token_q", "accept_len", "next_token")]
     want_resid = want_rows if want_resid is None else (want_resid and want_rows)
     rows = (0, 0, 0, 0)   # div_q, resid_q, div_t, resid_t
     if want_rows:         # without residual masses the KL divergence takes the one-pass statistics kernel
-        out["div_q"] = div_q = torch.empty((B, K_d), dtype=torch.float32, device=dev)
         if want_resid:
-            out["resid_q"] = torch.empty_like(div_q)
-        out["div_t"] = div_t = div_q.new_empty((B, K_q))
-        if want_resid:
-            out["resid_t"] = torch.empty_like(div_t)
-        rows = (div_q.data_ptr(), out["resid_q"].data_ptr() if want_resid else 0,
-                div_t.data_ptr(), out["resid_t"].data_ptr() if want_resid else 0)
+            out["div_q"], out["resid_q"], out["div_t"], out["resid_t"], *rows = _new_tensors(
+                logits_draft, 1, B, K_d, 1, B, K_d, 1, B, K_q, 1, B, K_q)
+        else:
+            out["div_q"], out["div_t"], at_q, at_t = _new_tensors(logits_draft, 1, B, K_d, 1, B, K_q)
+            rows = (at_q, 0, at_t, 0)
     window = (0, 0)
     if want_window:
-        out["window"] = win = torch.empty((B, K_q), dtype=torch.int32, device=dev)
-        out["n_window"] = n_win = win.new_empty(B)
-        window = (win.data_ptr(), n_win.data_ptr())
+        out["window"], out["n_window"], *window = _new_tensors(logits_draft, 0, B, K_q, 2, B, 0)
     dt = logits_draft.dtype
     rc = load_library().packed_verify_ex(_PYRAMID.pack(
         _PYRAMID.size, dtype_code(logits_draft), _dev_ptr(logits_draft, name="logits_draft") or 0, _dev_ptr(logits_qual, dt, "logits_qual") or 0,

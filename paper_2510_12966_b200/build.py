@@ -1,13 +1,16 @@
-"""Builds the CUDA library in-tree: ``csrc/pyramidsd.cu`` -> ``libpyramidsd.so`` (sm_100a only)."""
+"""Builds the CUDA library in-tree: ``csrc/pyramidsd.cu`` -> ``libpyramidsd.so`` (sm_100a only), and the binding's allocator of
+output tensors: ``csrc/tensors.cpp`` -> ``_tensors.so``."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
+import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
 LIB_PATH = os.path.join(_HERE, "libpyramidsd.so")
+TENSORS_PATH = os.path.join(_HERE, "_tensors.so")
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "--use_fast_math=false", "-Xcompiler", "-fPIC", "-shared"]
 
@@ -17,9 +20,9 @@ def _sources():
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB_PATH):
+    if not os.path.exists(LIB_PATH) or not os.path.exists(TENSORS_PATH):
         return True
-    t = os.path.getmtime(LIB_PATH)
+    t = min(os.path.getmtime(LIB_PATH), os.path.getmtime(TENSORS_PATH))
     deps = glob.glob(os.path.join(CSRC, "*")) + [os.path.join(_HERE, "..", "include", "pyramidsd.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 
@@ -34,7 +37,23 @@ def build(force: bool = False, verbose: bool = False) -> str:
     cmd += _sources() + ["-o", tmp]
     subprocess.check_call(cmd, cwd=CSRC)
     os.replace(tmp, LIB_PATH)
+    _build_tensors()
     return LIB_PATH
+
+
+def _build_tensors() -> None:
+    """A CPython extension against torch's headers; torch's own libraries are in the process before it is loaded."""
+    import torch
+    root = os.path.dirname(torch.__file__)
+    tmp = TENSORS_PATH + f".tmp{os.getpid()}"
+    include = os.path.join(root, "include")
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-w",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-isystem", include, "-isystem", os.path.join(include, "torch", "csrc", "api", "include"),
+           "-isystem", sysconfig.get_paths()["include"], os.path.join(CSRC, "tensors.cpp"), "-o", tmp,
+           "-L", os.path.join(root, "lib"), "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10"]
+    subprocess.check_call(cmd)
+    os.replace(tmp, TENSORS_PATH)
 
 
 if __name__ == "__main__":
