@@ -144,6 +144,13 @@ __device__ __forceinline__ V warp_reduce(V v) {
   return v;
 }
 
+// The warp's largest value in every lane, NaN ignored.
+__device__ __forceinline__ float warp_max(float v) {
+  float r;
+  asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+  return r;
+}
+
 // Reduce over the whole CTA; every thread gets the result. `scratch` holds >= 32 values. Fixed tree, so
 // results are bit-identical from run to run.
 template <typename Op, typename V>

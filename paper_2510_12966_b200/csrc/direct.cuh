@@ -53,11 +53,6 @@ struct DirectParams {
 // First group of a cluster's run `nth` of `n`.
 __device__ __forceinline__ int run_begin(int nth, int n, int n_groups) { return nth * n_groups / n; }
 
-__device__ __forceinline__ float warp_max(float v) {   // NaN ignored
-  float r;
-  asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
-  return r;
-}
 __device__ __forceinline__ float sum_of(const float (&w)[kFinElemsPerThread]) {
   float ts = 0.f;
 #pragma unroll

@@ -531,23 +531,29 @@ lmhead_sweep2sm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
 // weight are the M of the MMA, the call's rows its N (rounded up to 16), so an MMA costs what the rows are worth; a
 // tile's accumulator has a vocabulary index per lane and a row per column, which makes every store to z and every read
 // of the small logits a run of consecutive indices. A tile may load fewer than 128 weight rows (what the MMA makes of the rest
-// of the shared-memory tile is never read), which lets the host cut the vocabulary into equal rounds. A warp keeps the
-// (max, sum) of its columns of a row over all its tiles (lane r: row r of the warp's half) and leaves one partial.
-// Measured at M = 15, d = 2048, V = 32000: the launch 40 -> 29 us (131 MB of weight), the whole call 50.6 -> 35.6 us.
-// Up to 32 rows: the epilogue takes a warp-wide maximum and sum per row, about 2.9 us a row at V = 128256, while a lane of the
-// pairs' epilogue has a row to itself. Whole calls in us, this form / pairs of CTAs: V = 152064, d = 1024: M = 16 92 / 138,
-// 32 134 / 136, 64 215 / 141, 128 385 / 197; V = 128256, d = 4096: 32 244 / 242, 64 256 / 272, 128 422 / 282;
-// V = 50257, d = 768: 32 74 / 95, 64 106 / 101, 128 173 / 118.
-constexpr int kLmFewRows = 32;
+// of the shared-memory tile is never read), which lets the host cut the vocabulary into equal rounds. A warp leaves one
+// (max, sum) per row and model. Measured at M = 15, d = 2048, V = 32000: the launch 40 -> 29 us (131 MB of weight), the whole
+// call 50.6 -> 35.6 us.
+// Which rows go this way, and with which epilogue (lm_few_epilogue). Whole calls in us, sums across the warp / per lane / pairs
+// of CTAs: V = 152064, d = 1024: M = 2 63 / 65, 16 67 / 68, 32 92 / 76, 48 - / 83 / 108, 64 - / 93 / 109, 128 - / 182 / 135; V = 141632, d = 576: 16 51 / 45,
+// 32 77 / 51, 48 - / 60 / 87, 64 - / 70 / 94; V = 32000, d = 2048: 16 38.5 / 37.2, 32 43.5 / 41.6, 64 - / 47.0 / 47.7; V = 128256, d = 4096: 2 187 / 198, 16 194 / 204,
+// 32 202 / 208, 64 - / 243 / 232; V = 7488, d = 1024: 33 - / 29 / 24. Per lane is the cheaper sum, but where the weight is deep and rows few the
+// stream runs 5 % slower with it, for no reason found (with no epilogue at all it runs as slowly, pauses between the polls change nothing).
+// From 33 rows on the hidden rows, read again for every 128 columns of the vocabulary, cost more than the pairs' 256-row tiles once they are deep.
+constexpr int kLmFewDeep = 3072;
+inline int lm_few_epilogue(long long M, int d, int V) {   // -1: pairs of CTAs; 0: sums across the warp; 1: per lane
+  if (M <= 32) return d >= kLmFewDeep ? 0 : 1;
+  return M <= 64 && d <= 1088 && V >= 32000 ? 1 : -1;
+}
+constexpr int kLmFewRows = 64;        // the most
 constexpr int kLmFewMaxStages = 12;
 constexpr int kLmFewRing = 200 * 1024;
-static_assert(2 * kLmFewRows >= 32 && kLmFewRows <= 32, "tensor memory comes in 32 columns or more; a lane per row of a half");
 
 struct LmFewBarriers {
   unsigned long long full[kLmFewMaxStages], empty[kLmFewMaxStages], tmem_full[2], tmem_empty[2];
   unsigned tmem_base;
 };
-constexpr size_t kLmFewSmemBytes = static_cast<size_t>(kLmFewRing) + 1024 + 512;
+constexpr size_t kLmFewSmemBytes = static_cast<size_t>(kLmFewRing) + 1024 + 512 + kLmEpiWarps * (kLmFewRows / 2) * sizeof(float2);
 static_assert(sizeof(LmFewBarriers) <= 512, "the barriers' share of the shared memory");
 
 __device__ __forceinline__ void tma_load_2d_hint(void* smem_dst, const CUtensorMap* map, int x, int y, unsigned long long* bar, unsigned long long policy) {
@@ -555,7 +561,20 @@ __device__ __forceinline__ void tma_load_2d_hint(void* smem_dst, const CUtensorM
                ::"r"(smem_u32(smem_dst)), "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y), "l"(policy) : "memory");
 }
 
-// P.tile_n: weight rows per tile (a multiple of 8, at most 128); `n_rows`: the call's rows rounded up to 16.
+// The (max, sum) of one row over this lane's columns of all tiles, again and against the true maximum: a sum left the range
+// of a float (or the row holds a NaN or +inf). `z` and `x` of tile 0 at this lane's column; by one full warp.
+template <typename Load>
+__device__ __noinline__ float2 few_row_again(Load load, int n_tiles, float c) {
+  float m = -INFINITY, sum = 0.f;
+  for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) m = fmaxf(m, load(t));
+  const float ref = fmaxf(warp_reduce<OpMaxNan>(m == m ? m : -INFINITY) * c, -1e30f);
+  for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) sum += ex2_approx(fmaf(load(t), c, -ref));
+  return make_float2(ref, warp_reduce<OpSum>(sum));
+}
+
+// P.tile_n: weight rows per tile (a multiple of 8, at most 128); `n_rows`: the call's rows rounded up to 16; RW: at least half
+// of them, or 0 for the epilogue that sums across the warp.
+template <int RW>
 __global__ void __launch_bounds__(kLmThreads, 1)
 lmhead_sweep_few_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUtensorMap map_w, const LmParams P, const int n_rows,
                         const int stages) {
@@ -572,7 +591,9 @@ lmhead_sweep_few_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_
     for (int b = 0; b < 2; ++b) { mbar_init(&bars->tmem_full[b], 1); mbar_init(&bars->tmem_empty[b], kLmEpiWarps); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 1) tmem_alloc(&bars->tmem_base, 2 * kLmFewRows);
+  constexpr int kRows = RW == 0 ? 32 : 2 * RW;            // columns of tensor memory of an accumulator
+  constexpr unsigned kColumns = 2 * kRows;
+  if (warp == 1) tmem_alloc(&bars->tmem_base, kColumns);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -627,7 +648,7 @@ lmhead_sweep_few_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_
         if (it >= 2) wait_phase(&bars->tmem_empty[buf], ((it >> 1) - 1) & 1u);   // the epilogue has drained this buffer
         if (dead) break;
         tc_fence_after();
-        const unsigned acc = tmem_base + static_cast<unsigned>(buf) * kLmFewRows;
+        const unsigned acc = tmem_base + static_cast<unsigned>(buf) * kRows;
         for (int ks = 0; ks < k_steps; ++ks) {
           wait_phase(&bars->full[stage], par);
           if (dead) break;   // no MMA on operands that have not arrived
@@ -646,59 +667,170 @@ lmhead_sweep_few_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_
   } else {
     // ================================ epilogue ================================
     const int quarter = warp & 3, half = (warp - 2) >> 2;          // TMEM lanes 32*quarter.., the half's rows
-    const int half_rows = n_rows >> 1, r0 = half * half_rows;      // at most 16 rows: a lane keeps the (max, sum) of one
+    const int half_rows = n_rows >> 1, r0 = half * half_rows;
     const int rows = min(half_rows, P.M - P.row0 - r0);            // rows that exist (<= 0: none)
     const float c = P.c;
-    float ml = -1e30f, sl = 0.f, ms = -1e30f, ss = 0.f;
-    int it = 0;
-    for (int tile = blockIdx.x; tile < P.n_tiles; tile += gridDim.x, ++it) {
-      const int buf = it & 1;
-      wait_phase(&bars->tmem_full[buf], (it >> 1) & 1u);
-      tc_fence_after();
-      const unsigned tacc = tmem_base + static_cast<unsigned>(buf * kLmFewRows + r0) + (static_cast<unsigned>(quarter * 32) << 16);
-      const int in_tile = quarter * 32 + lane, col = tile * P.tile_n + in_tile;
-      const bool col_ok = in_tile < P.tile_n && col < P.V;
+    if constexpr (RW == 0) {   // at most 32 rows: lane r keeps the (max, sum) of the warp's columns of row r over all its tiles
+      float ml = -1e30f, sl = 0.f, ms = -1e30f, ss = 0.f;
+      int it = 0;
+      for (int tile = blockIdx.x; tile < P.n_tiles; tile += gridDim.x, ++it) {
+        const int buf = it & 1;
+        wait_phase(&bars->tmem_full[buf], (it >> 1) & 1u);
+        tc_fence_after();
+        const unsigned tacc = tmem_base + static_cast<unsigned>(buf * kRows + r0) + (static_cast<unsigned>(quarter * 32) << 16);
+        const int in_tile = quarter * 32 + lane, col = tile * P.tile_n + in_tile;
+        const bool col_ok = in_tile < P.tile_n && col < P.V;
 #pragma unroll 1
-      for (int g = 0; g < rows; g += 8) {   // uniform across the warp
-        float z[8], x[8];
+        for (int g = 0; g < rows; g += 8) {   // uniform across the warp
+          float z[8], x[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
-          x[i] = (col_ok && g + i < rows) ? Elem<__nv_bfloat16>::load(P.small + static_cast<size_t>(P.row0 + r0 + g + i) * P.V, col) : -INFINITY;
-        tmem_ld8(tacc + static_cast<unsigned>(g), z);
+          for (int i = 0; i < 8; ++i)
+            x[i] = (col_ok && g + i < rows) ? Elem<__nv_bfloat16>::load(P.small + static_cast<size_t>(P.row0 + r0 + g + i) * P.V, col) : -INFINITY;
+          tmem_ld8(tacc + static_cast<unsigned>(g), z);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            if (g + i >= rows) break;
+            const size_t srow = static_cast<size_t>(P.row0 + r0 + g + i);   // one block: the ring holds every row
+            if (col_ok) P.z[srow * P.ldz + col] = z[i];
+            const float zv = col_ok ? z[i] : -INFINITY;
+            float gl = zv, gs = x[i];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+              gl = fmaxf(gl, __shfl_xor_sync(0xffffffffu, gl, o));
+              gs = fmaxf(gs, __shfl_xor_sync(0xffffffffu, gs, o));
+            }
+            const float rl = fmaxf(gl * c, -1e30f), rs = fmaxf(gs * c, -1e30f);
+            // NaN and +inf logits poison the sums, as they should
+            const float tl = warp_reduce<OpSum>(col_ok ? ex2_approx(fmaf(z[i], c, -rl)) : 0.f);
+            const float ts = warp_reduce<OpSum>(col_ok ? ex2_approx(fmaf(x[i], c, -rs)) : 0.f);
+            if (g + i == lane) { lse_merge(ml, sl, rl, tl); lse_merge(ms, ss, rs, ts); }
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bars->tmem_empty[buf]);   // this warp has read its part of the accumulator
+      }
+      if (lane < rows) {
+        const size_t idx = static_cast<size_t>(P.row0 + r0 + lane) * P.n_part + blockIdx.x * 4 + quarter;
+        P.part_large[idx] = make_float2(ml, sl);
+        P.part_small[idx] = make_float2(ms, ss);
+      }
+    } else {
+      const size_t first = static_cast<size_t>(P.row0 + r0);         // one block: the ring holds every row
+      const int in_tile = quarter * 32 + lane;
+      // A lane sums its own column of every row against a reference per row: that of the warp's columns in its first tile. Only
+      // if a row's sum leaves the range of a float is it taken again (few_row_again). A maximum and a sum across the warp
+      // for each row and tile cost 45 instructions where this takes 10.
+      float2* refs = reinterpret_cast<float2*>(tiles + kLmFewRing + 512) + (warp - 2) * (kLmFewRows / 2);
+      float sl[RW], ss[RW];
+      // The small model's logits, 64 bytes per row, warp and tile, stand behind megabytes of weight in the memory's queues: they
+      // are brought into L2 a tile ahead.
+      auto prefetch = [&](int tile) {
+        const int at = tile * P.tile_n + quarter * 32;
+        if (tile >= P.n_tiles || quarter * 32 >= P.tile_n) return;
+        for (int r = lane >> 1; r < rows; r += 16) {
+          const int column = at + (lane & 1) * 31;
+          if (column < P.V) asm volatile("prefetch.global.L2 [%0];" ::"l"(P.small + (first + r) * P.V + column));
+        }
+      };
+#pragma unroll
+      for (int i = 0; i < RW; ++i) { sl[i] = 0.f; ss[i] = 0.f; }
+      int it = 0;
+      for (int tile = blockIdx.x; tile < P.n_tiles; tile += gridDim.x, ++it) {
+        const int buf = it & 1;
+        const int col = tile * P.tile_n + in_tile;
+        const bool col_ok = in_tile < P.tile_n && col < P.V;
+        const __nv_bfloat16* small = P.small + first * P.V + col;
+        float* zp = P.z + first * P.ldz + col;
+        if (it == 0) prefetch(tile);
+        prefetch(tile + gridDim.x);
+        unsigned short x[2][8];
+        auto fetch = [&](int g, unsigned short (&v)[8]) {   // the small model's logits of rows g .. g + 7
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            v[i] = 0xff80u;   // -inf
+            if (col_ok && g + i < rows) asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(v[i]) : "l"(small + static_cast<size_t>(g + i) * P.V));
+          }
+        };
+        fetch(0, x[0]);
+        wait_phase(&bars->tmem_full[buf], (it >> 1) & 1u);
+        tc_fence_after();
+        const unsigned tacc = tmem_base + static_cast<unsigned>(buf * kRows + r0) + (static_cast<unsigned>(quarter * 32) << 16);
+#pragma unroll
+        for (int g = 0; g < RW; g += 8) {
+          if (g < rows) {   // uniform across the warp
+            if (g + 8 < RW) fetch(g + 8, x[(g / 8 + 1) & 1]);
+            float xg[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) xg[i] = __uint_as_float(static_cast<unsigned>(x[(g / 8) & 1][i]) << 16);
+            float z[8];
+            tmem_ld8(tacc + static_cast<unsigned>(g), z);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              if (col_ok && g + i < rows) zp[static_cast<size_t>(g + i) * P.ldz] = z[i];
+              z[i] = col_ok ? z[i] : -INFINITY;
+            }
+            if (it == 0) {
+#pragma unroll
+              for (int i = 0; i < 8; ++i) {
+                const float rl = fmaxf(warp_max(z[i]) * c, -1e30f), rs = fmaxf(warp_max(xg[i]) * c, -1e30f);
+                if (lane == 0) refs[g + i] = make_float2(rl, rs);
+              }
+              __syncwarp();
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const float2 r = refs[g + i];
+              sl[g + i] += ex2_approx(fmaf(z[i], c, -r.x));   // NaN and +inf logits poison the sums, as they should
+              ss[g + i] += ex2_approx(fmaf(xg[i], c, -r.y));
+            }
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bars->tmem_empty[buf]);   // this warp has read its part of the accumulator
+      }
+      __syncwarp();
+      const size_t part0 = blockIdx.x * 4 + quarter;
+#pragma unroll
+      for (int g = 0; g < RW; g += 8) {
+        if (g >= rows) break;
+        float tl[8], ts[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) { tl[i] = warp_reduce<OpSum>(sl[g + i]); ts[i] = warp_reduce<OpSum>(ss[g + i]); }
+        float worst = 0.f;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-          if (g + i >= rows) break;
-          const size_t srow = static_cast<size_t>(P.row0 + r0 + g + i);   // one block: the ring holds every row
-          if (col_ok) P.z[srow * P.ldz + col] = z[i];
-          const float zv = col_ok ? z[i] : -INFINITY;
-          float gl = zv, gs = x[i];
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) {
-            gl = fmaxf(gl, __shfl_xor_sync(0xffffffffu, gl, o));
-            gs = fmaxf(gs, __shfl_xor_sync(0xffffffffu, gs, o));
+          if (g + i < rows) {
+            worst += tl[i] + ts[i];   // not finite if one of them is not
+            if (lane == 0) {
+              const float2 r = refs[g + i];
+              P.part_large[(first + g + i) * P.n_part + part0] = make_float2(r.x, tl[i]);
+              P.part_small[(first + g + i) * P.n_part + part0] = make_float2(r.y, ts[i]);
+            }
           }
-          const float rl = fmaxf(gl * c, -1e30f), rs = fmaxf(gs * c, -1e30f);
-          // NaN and +inf logits poison the sums, as they should
-          const float tl = warp_reduce<OpSum>(col_ok ? ex2_approx(fmaf(z[i], c, -rl)) : 0.f);
-          const float ts = warp_reduce<OpSum>(col_ok ? ex2_approx(fmaf(x[i], c, -rs)) : 0.f);
-          if (g + i == lane) { lse_merge(ml, sl, rl, tl); lse_merge(ms, ss, rs, ts); }
+        }
+        if (!(worst < INFINITY)) {   // the group's rows again
+          for (int i = g; i < min(g + 8, rows); ++i) {
+            const float* z = P.z + (first + i) * P.ldz;
+            const __nv_bfloat16* x = P.small + (first + i) * P.V;
+            auto inside = [&](int t) { return in_tile < P.tile_n && t * P.tile_n + in_tile < P.V; };
+            const float2 pl = few_row_again([&](int t) { return inside(t) ? __ldcg(z + t * P.tile_n + in_tile) : -INFINITY; }, P.n_tiles, c);
+            const float2 ps = few_row_again([&](int t) { return inside(t) ? Elem<__nv_bfloat16>::load(x, t * P.tile_n + in_tile) : -INFINITY; }, P.n_tiles, c);
+            if (lane == 0) {
+              P.part_large[(first + i) * P.n_part + part0] = pl;
+              P.part_small[(first + i) * P.n_part + part0] = ps;
+            }
+          }
         }
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&bars->tmem_empty[buf]);   // this warp has read its part of the accumulator
-    }
-    if (lane < rows) {
-      const size_t idx = static_cast<size_t>(P.row0 + r0 + lane) * P.n_part + blockIdx.x * 4 + quarter;
-      P.part_large[idx] = make_float2(ml, sl);
-      P.part_small[idx] = make_float2(ms, ss);
     }
   }
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, 2 * kLmFewRows);
+    tmem_dealloc(tmem_base, kColumns);
   }
 }
 

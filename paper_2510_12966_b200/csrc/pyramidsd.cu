@@ -1079,7 +1079,8 @@ int pyramidsd_verify_fused_lmhead_ex(const psd_lmhead_args* args) {
   if (sms <= 0) sms = 1;
   // the two-SM (cta_group::2) sweep is the default, unless the call has so few rows that the weight is streamed faster
   // than its 256-row tiles multiply
-  const bool use_few = args->tile_variant == PSD_LMHEAD_TILES_AUTO && M <= psd::kLmFewRows;
+  const int few = args->tile_variant == PSD_LMHEAD_TILES_AUTO ? psd::lm_few_epilogue(M, d_model, V) : -1;
+  const bool use_few = few >= 0;
   const bool use_pair = !use_few && args->tile_variant != PSD_LMHEAD_TILES_ONE_SM;
   // Columns per tile of the pair: the weight is streamed in rounds of one tile per pair, so a width that leaves fewer
   // columns per pair in all is taken (V = 32000: two rounds of 224 instead of two of 256, the second of them two thirds
@@ -1169,7 +1170,10 @@ int pyramidsd_verify_fused_lmhead_ex(const psd_lmhead_args* args) {
         cudaFuncSetAttribute(psd::lmhead_sweep_kernel<true>, at, one) != cudaSuccess ||
         cudaFuncSetAttribute(psd::lmhead_sweep2sm_kernel<false>, at, two) != cudaSuccess ||
         cudaFuncSetAttribute(psd::lmhead_sweep2sm_kernel<true>, at, two) != cudaSuccess ||
-        cudaFuncSetAttribute(psd::lmhead_sweep_few_kernel, at, static_cast<int>(psd::kLmFewSmemBytes)) != cudaSuccess) {
+        cudaFuncSetAttribute(psd::lmhead_sweep_few_kernel<8>, at, static_cast<int>(psd::kLmFewSmemBytes)) != cudaSuccess ||
+        cudaFuncSetAttribute(psd::lmhead_sweep_few_kernel<16>, at, static_cast<int>(psd::kLmFewSmemBytes)) != cudaSuccess ||
+        cudaFuncSetAttribute(psd::lmhead_sweep_few_kernel<32>, at, static_cast<int>(psd::kLmFewSmemBytes)) != cudaSuccess ||
+        cudaFuncSetAttribute(psd::lmhead_sweep_few_kernel<0>, at, static_cast<int>(psd::kLmFewSmemBytes)) != cudaSuccess) {
       cudaGetLastError();
       return PSD_ERR_CUDA;
     }
@@ -1190,7 +1194,11 @@ int pyramidsd_verify_fused_lmhead_ex(const psd_lmhead_args* args) {
       const int stage = 128 * psd::kLmK * 2 + n_rows16 * psd::kLmK * 2, fit = psd::kLmFewRing / stage;
       cfg.gridDim = dim3(static_cast<unsigned>(n_ctas));
       cfg.dynamicSmemBytes = psd::kLmFewSmemBytes;
-      return cudaLaunchKernelEx(&cfg, psd::lmhead_sweep_few_kernel, map_h, map_w, L, n_rows16, fit < psd::kLmFewMaxStages ? fit : psd::kLmFewMaxStages);
+      const int stages = fit < psd::kLmFewMaxStages ? fit : psd::kLmFewMaxStages;
+      return few == 0         ? cudaLaunchKernelEx(&cfg, psd::lmhead_sweep_few_kernel<0>, map_h, map_w, L, n_rows16, stages)
+             : n_rows16 <= 16 ? cudaLaunchKernelEx(&cfg, psd::lmhead_sweep_few_kernel<8>, map_h, map_w, L, n_rows16, stages)
+             : n_rows16 <= 32 ? cudaLaunchKernelEx(&cfg, psd::lmhead_sweep_few_kernel<16>, map_h, map_w, L, n_rows16, stages)
+                              : cudaLaunchKernelEx(&cfg, psd::lmhead_sweep_few_kernel<32>, map_h, map_w, L, n_rows16, stages);
     }
     if (!use_pair) {
       cfg.gridDim = dim3(static_cast<unsigned>(n_ctas));

@@ -139,3 +139,37 @@ def test_scratch_is_one_block_of_logits():
         taken = before - torch.cuda.mem_get_info()[0]
     psd.release_stream(stream)
     assert taken < 200 << 20, taken
+
+
+@pytest.mark.parametrize("M,K,V,d", [(1, 1, 3000, 64), (6, 2, 20001, 128), (16, 4, 19000, 64), (17, 1, 33000, 192), (32, 8, 40000, 64),
+                                     (33, 3, 33001, 64), (48, 4, 50000, 128), (64, 8, 32000, 64)])
+def test_few_rows_whose_first_columns_say_nothing_of_the_rest(M, K, V, d):
+    """The epilogues of the form for few rows, either side of 4, 16, 32 and 64 rows: per row the first 128 columns' logits lie
+    some 250 nats below the rest's, so that sums against their maximum overflow and are taken again; others above."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2510_12966_b200 import binding as psd
+    g = torch.Generator(device="cuda").manual_seed(M + V)
+    B = M // K
+    h = torch.randn((M, d), generator=g, device="cuda").bfloat16()
+    w = (torch.randn((V, d), generator=g, device="cuda") * 0.1).bfloat16()
+    h[:, 0] = 1.0
+    w[:, 0] = 0.0
+    w[:128, 0] = -250.0
+    h[::3, 0] = -0.03                                        # every third row: the first columns weigh more
+    z = h.double() @ w.double().T
+    zs = (z + torch.randn((M, V), generator=g, device="cuda") * 0.5).bfloat16().view(B, K, V)
+    zs[0, 0, :100] = -float("inf")
+    tok = torch.randint(0, V, (B, K), generator=g, device="cuda", dtype=torch.int32)
+    out = psd.verify_fused_lmhead(h, w, zs, tok, 0.1, psd.FUZZY, 3, 1)
+    torch.cuda.synchronize()
+    assert psd.last_status() == 0
+    p, q = torch.log_softmax(z, -1).view(B, K, V), torch.log_softmax(zs.double(), -1)
+    m = torch.logaddexp(p, q) - 0.6931471805599453
+    term = lambda a: torch.where(a > -1e300, a.exp() * (a - m), 0.0)
+    js, resid = 0.5 * (term(p) + term(q)).sum(-1), (p.exp() - q.exp()).clamp_min(0).sum(-1)
+    # the logits' own error: single-precision sums of up to d products of size |z| (250 here), 2^-24 |z| sqrt(d) in the exponent
+    tol = 1e-5 + 250 * d ** 0.5 * 2.0 ** -24
+    assert (out["div"].double() - js).abs().max() < tol and (out["resid_mass"].double() - resid).abs().max() < tol
+    accept = (out["div"] <= 0.1).int().cumprod(1).sum(1)
+    assert torch.equal(out["accept_len"], accept.int()) and bool(((out["next_token"] >= 0) == (accept < K)).all())
