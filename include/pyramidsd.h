@@ -288,8 +288,8 @@ int pyramidsd_verify_fused_lmhead(const void* hidden, const void* w_t, const voi
 
 /* The same call with every option exposed. Zero-initialise, set struct_size, fill what you need.
  *   seq_index_base  as in psd_stage_args.
- *   tile_variant    PSD_LMHEAD_TILES_AUTO (few rows (32, or 64 of a shallow weight): one CTA per 128 rows of the weight; more: pairs of CTAs on
- *                   256 x 256 tiles, tcgen05 cta_group::2) or
+ *   tile_variant    PSD_LMHEAD_TILES_AUTO (few rows -- 32, or 64 of a shallow weight --: one CTA per 128 rows of the
+ *                   weight; more: pairs of CTAs on 256 x 256 tiles, tcgen05 cta_group::2) or
  *                   PSD_LMHEAD_TILES_ONE_SM (one CTA per 256 x 128 tile); same results within rounding.
  *   div_kind        PSD_DIV_JS or PSD_DIV_KL (KL(large || small)). */
 #define PSD_LMHEAD_TILES_AUTO 0

@@ -534,15 +534,18 @@ lmhead_sweep2sm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
 // of the shared-memory tile is never read), which lets the host cut the vocabulary into equal rounds. A warp leaves one
 // (max, sum) per row and model. Measured at M = 15, d = 2048, V = 32000: the launch 40 -> 29 us (131 MB of weight), the whole
 // call 50.6 -> 35.6 us.
-// Which rows go this way, and with which epilogue (lm_few_epilogue). Whole calls in us, sums across the warp / per lane / pairs
-// of CTAs: V = 152064, d = 1024: M = 2 63 / 65, 16 67 / 68, 32 92 / 76, 48 - / 83 / 108, 64 - / 93 / 109, 128 - / 182 / 135; V = 141632, d = 576: 16 51 / 45,
-// 32 77 / 51, 48 - / 60 / 87, 64 - / 70 / 94; V = 32000, d = 2048: 16 38.5 / 37.2, 32 43.5 / 41.6, 64 - / 47.0 / 47.7; V = 128256, d = 4096: 2 187 / 198, 16 194 / 204,
-// 32 202 / 208, 64 - / 243 / 232; V = 7488, d = 1024: 33 - / 29 / 24. Per lane is the cheaper sum, but where the weight is deep and rows few the
-// stream runs 5 % slower with it, for no reason found (with no epilogue at all it runs as slowly, pauses between the polls change nothing).
-// From 33 rows on the hidden rows, read again for every 128 columns of the vocabulary, cost more than the pairs' 256-row tiles once they are deep.
+// Which rows go this way, and with which epilogue (lm_few_epilogue). Whole calls in us, sums across the warp / per lane /
+// pairs of CTAs: V = 152064, d = 1024: M = 2 63 / 65, 16 67 / 68, 32 92 / 76, 48 - / 83 / 108, 64 - / 93 / 109, 128 - / 182 / 135;
+// V = 141632, d = 576: 16 51 / 45, 32 77 / 51, 48 - / 60 / 87, 64 - / 70 / 94; V = 32000, d = 2048: 16 38.5 / 37.2, 32 43.5 / 41.6, 64
+// - / 47.0 / 47.7; V = 128256, d = 4096: 2 187 / 198, 16 194 / 204, 32 202 / 208, 64 - / 243 / 232; V = 7488, d = 1024: 33 - / 29 / 24.
+// Per lane is the cheaper sum, but where the weight is deep, or the rows are a handful, the stream runs up to 6 % slower
+// with it, for no reason found (with no epilogue at all it runs as slowly; pauses between the polls and other ring depths
+// change nothing). The small logits have to be brought into L2 a tile ahead: M = 64, d = 1024, V = 152064 151 -> 98 us. From 33
+// rows on the hidden rows, read again for every 128 columns of the vocabulary, cost more than the pairs' 256-row tiles
+// once they are deep.
 constexpr int kLmFewDeep = 3072;
 inline int lm_few_epilogue(long long M, int d, int V) {   // -1: pairs of CTAs; 0: sums across the warp; 1: per lane
-  if (M <= 32) return d >= kLmFewDeep ? 0 : 1;
+  if (M <= 32) return d >= kLmFewDeep || M <= 4 ? 0 : 1;
   return M <= 64 && d <= 1088 && V >= 32000 ? 1 : -1;
 }
 constexpr int kLmFewRows = 64;        // the most
