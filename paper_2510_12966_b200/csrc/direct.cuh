@@ -566,22 +566,28 @@ inline cudaError_t launch_direct(const DirectParams& D, int dtype, unsigned item
 // 17.2, 14.8, 31 24.1, 19.9 / 27.8, 25.5. Rows that the ring kernel takes logit by logit (unaligned): V = 32001 bf16 two
 // stages B = 10 31.7 / 18.7, 83 96.1 / 85.9; one stage B = 16 25.9 / 18.8, 62 54.3 / 49.4. fp32 logits, twice the bytes to copy and
 // to hold, turn earlier. `onepass`: the KL kernel that reads every logit once would take the call.
-inline bool direct_applies(int V, int dtype, int n_stages, long long rows, bool unaligned, bool ragged, bool bonus, bool onepass) {
+// Two stages with everything accepted, which costs the other way's finalisation least: V = 5440 bf16 16 M pairs 48.2 / 49.8, 33 M
+// 87.7 / 95.9. Ragged windows (n_valid), half of the positions valid, mixed outcomes: V = 8320 bf16 B = 80 28.3 / 18.8, 160 39.9 / 31.2;
+// V = 16384 B = 10 16.6 / 12.0, 41 20.1 / 19.0; V = 64001 B = 5 27.1 / 15.6, 21 52.3 / 34.2; V = 32000 fp32 B = 21 27.4 / 20.6, 42 32.6 / 41.2; from 96
+// sequences on the other way deals its valid rows over whole rounds of the device.
+inline bool direct_applies(int V, int dtype, int n_stages, int B, long long rows, bool unaligned, bool ragged, bool bonus, bool onepass) {
   const double pairs = static_cast<double>(rows) * V;
   if (V < 2048) return false;
   double most;
   if (n_stages == 2) {
     if (onepass) most = V <= 16384 ? 8.2e6 : 4.1e6;
-    else if (dtype == 1) most = unaligned ? 33e6 : (V <= 8192 || V >= 49152) ? 16.5e6 : 8.2e6;
+    else if (dtype == 1) most = unaligned ? 33e6 : V >= 49152 ? 16.5e6 : V <= 12288 ? 12e6 : 8.2e6;
     else if (unaligned) most = V <= 65536 ? 16.5e6 : 4.8e6;
-    else most = V > 4096 && V <= 16384 ? 4.1e6 : 8.2e6;
+    else most = V <= 4096 ? 6.5e6 : V <= 16384 ? 4.1e6 : 8.2e6;
   } else {
     if (onepass) most = 0.0;
+    else if (ragged) most = dtype == 1 ? (unaligned ? 16.5e6 : V <= 8704 ? 12e6 : V >= 49152 ? 8.2e6 : V >= 24576 ? 4e6 : 2.2e6)
+                                       : unaligned || V >= 24576 ? 8.2e6 : 4.1e6;
     else if (dtype == 1) most = unaligned ? min(33e6, 5.2e11 / V) : min(8.2e6, 6.6e10 / V);
     else if (V <= 4608) most = unaligned ? 16.5e6 : 4.1e6;
     else most = min(2.2e6, 1.3e11 / V);
     if (bonus) most *= 2.0;                  // a draw more from a row that the ring kernel has not seen
-    if (ragged) most = min(most, 4.0e6);     // the ring kernel deals out the valid rows alone
+    if (ragged && B >= 96) most = min(most, 4e6);
   }
   return pairs <= most;
 }
