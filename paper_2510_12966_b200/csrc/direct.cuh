@@ -28,7 +28,7 @@
 
 namespace psd {
 
-constexpr int kDirMaxRanks = 8;
+constexpr int kDirMaxRanks = 16;
 constexpr int kDirThreads = 256;
 constexpr int kDirWarps = kDirThreads / 32;
 constexpr int kDirCtasPerSm = 4;
@@ -527,6 +527,7 @@ inline cudaError_t direct_launch_typed(const DirectParams& D, unsigned items, cu
   if (dev < 0 || dev >= kClMaxDevices) return cudaErrorInvalidDevice;
   if (!prepared[dev]) {
     e = cudaFuncSetAttribute(direct_kernel<T, DIV>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDirMaxSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(direct_kernel<T, DIV>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     prepared[dev] = true;
   }
@@ -594,13 +595,15 @@ inline bool direct_applies(int V, int dtype, int n_stages, int B, long long rows
 
 // CTAs per row pair: what lets four CTAs share an SM, and more while all CTAs are resident at once and every warp has 256
 // indices (0: rows too long for the kernel). V = 32000 bf16, K = 8, one stage, clusters of 2 / 4 / 8: B = 4 11.1 / 10.0 / 8.9 us,
-// 8 11.3 / 11.7 / 11.0, 16 18.0 / 14.5 / 18.6.
+// 8 11.3 / 11.7 / 11.0, 16 18.0 / 14.5 / 18.6. Sixteen where that leaves two CTAs per SM and every warp two groups: one sequence
+// through the pyramid, K = 8 / 4, V = 128256 bf16, clusters of 8 / 16: 14.7 / 12.2 us, with a bonus row 15.4 / 12.5; V = 65536 10.6 / 9.2.
 inline int direct_cluster_size(int V, int dtype, long long items) {
   const int es = dtype == 0 ? 4 : 2, sms = cluster_sm_count(), groups = (V + kFinPart - 1) / kFinPart;
   int cs = 1;
-  while (cs < kDirMaxRanks && direct_smem_bytes(V, es, cs) > kDirSmemForFour) ++cs;
+  while (cs < 8 && direct_smem_bytes(V, es, cs) > kDirSmemForFour) ++cs;
   if (direct_smem_bytes(V, es, cs) > kDirMaxSmem) return 0;
-  while (cs < kDirMaxRanks && (cs + 1) * kDirWarps <= groups && items * (cs + 1) <= static_cast<long long>(kDirCtasPerSm) * sms) ++cs;
+  while (cs < 8 && (cs + 1) * kDirWarps <= groups && items * (cs + 1) <= static_cast<long long>(kDirCtasPerSm) * sms) ++cs;
+  if (cs == 8 && items * 16 <= 2 * sms && groups >= 32 * kDirWarps) cs = 16;
   return cs;
 }
 
